@@ -1,9 +1,10 @@
 """Thin Python binding of the C-ABI library ``libqarl.so`` (see ``include/qarl.h``).
 
 Argument marshalling only: every step of the quantized forward runs in the library's CUDA
-kernels.  torch is used for device memory and streams.  There is no CPU path: loading fails
-loudly if the library has not been built, and creating a context fails without an sm_100
-device.
+kernels.  torch is used for device memory and streams.  The calls a decode step or a training
+step makes are marshalled in C++ (``_native.so``, ``csrc/native_binding.cpp``), the others and
+the debug forms through ctypes.  There is no CPU path: loading fails loudly if the library has
+not been built, and creating a context fails without an sm_100 device.
 """
 from __future__ import annotations
 
@@ -14,6 +15,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libqarl.so")
+NATIVE_PATH = os.path.join(_HERE, "_native.so")
 
 QARL_OK = 0
 STATUS_NAMES = {
@@ -63,18 +65,21 @@ class MoeDebug(C.Structure):
 
 
 _lib = None
+_native = None
 
 
 def load() -> C.CDLL:
     """Load libqarl.so and declare its signatures.  Raises if the library is not built."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
-    if not os.path.exists(LIB_PATH):
-        raise RuntimeError(
-            f"{LIB_PATH} is missing: build it with `python -m paper_2604_07853_b200.build` "
-            "(there is no CPU fallback)")
+    for path in (LIB_PATH, NATIVE_PATH):
+        if not os.path.exists(path):
+            raise RuntimeError(
+                f"{path} is missing: build it with `python -m paper_2604_07853_b200.build` "
+                "(there is no CPU fallback)")
     L = C.CDLL(LIB_PATH)
+    from . import _native
     i64, p, sz = C.c_int64, C.c_void_p, C.c_size_t
     L.qarl_create.restype = C.c_int
     L.qarl_create.argtypes = [C.POINTER(p), C.c_int]
@@ -192,12 +197,14 @@ class Context:
         if rc != QARL_OK:
             raise QarlError(rc)
         self.h = h
+        self._hv = h.value  # what the C++ marshalling reads
         self._ws: torch.Tensor | None = None
 
     def close(self):
         if getattr(self, "h", None):
             self.lib.qarl_destroy(self.h)
             self.h = None
+            self._hv = 0
 
     def __del__(self):
         try:
@@ -279,40 +286,15 @@ class Context:
     # ------------------------------------------------------------------ calls
     def quantize_weight(self, w: torch.Tensor, codes=None, scales=None):
         """w bf16 [E, N, K] or [N, K] -> (codes u8 same shape, scales f32 [.., N/128, K/128])."""
-        assert w.dtype == torch.bfloat16 and w.is_cuda and w.is_contiguous()
-        shape = w.shape
-        E, N, K = (1, *shape) if w.dim() == 2 else shape
-        if codes is None:
-            codes = torch.empty(shape, dtype=torch.uint8, device=w.device)
-        if scales is None:
-            scales = torch.empty((*shape[:-2], N // 128, K // 128), dtype=torch.float32, device=w.device)
-        self._check(self.lib.qarl_quantize_weight(self.h, _ptr(w), E, N, K, _ptr(codes), _ptr(scales), _stream()))
-        return codes, scales
+        return _native.quantize_weight(self, w, codes, scales, None, None)
 
     def quantize_act(self, x: torch.Tensor, codes=None, scales=None):
         """x bf16 [M, K] (rows may be strided) -> (codes u8 [M, K], scales f32 [M, K/128])."""
-        assert x.dtype == torch.bfloat16 and x.is_cuda and x.dim() == 2 and x.stride(1) == 1
-        M, K = x.shape
-        ldx = x.stride(0) if M > 1 else K
-        if codes is None:
-            codes = torch.empty((M, K), dtype=torch.uint8, device=x.device)
-        if scales is None:
-            scales = torch.empty((M, K // 128), dtype=torch.float32, device=x.device)
-        self._check(self.lib.qarl_quantize_act(self.h, _ptr(x), M, K, ldx, _ptr(codes), _ptr(scales), _stream()))
-        return codes, scales
+        return _native.quantize_act(self, x, codes, scales)
 
     def linear_fwd(self, x, w_codes, w_scales, out=None, want_f32: bool = False):
         """y = blockscaled(quantize_act(x), W) -> y bf16 [M, N] (and the fp32 accumulator)."""
-        assert x.dtype == torch.bfloat16 and x.is_contiguous()
-        M, K = x.shape
-        N = w_codes.shape[0]
-        y = out if out is not None else torch.empty((M, N), dtype=torch.bfloat16, device=x.device)
-        y32 = torch.empty((M, N), dtype=torch.float32, device=x.device) if want_f32 else None
-        nbytes = int(self.lib.qarl_linear_workspace_bytes(M, N, K))
-        ws = self.workspace(nbytes)
-        self._check(self.lib.qarl_linear_fwd(self.h, _ptr(x), M, K, _ptr(w_codes), _ptr(w_scales), N,
-                                             _ptr(y), _ptr(y32), _ptr(ws), ws.numel(), _stream()))
-        return (y, y32) if want_f32 else y
+        return _native.linear_fwd(self, x, w_codes, w_scales, out, want_f32)
 
     def linear_fwd_static(self, x, w_codes, w_scales, out):
         """qarl_linear_fwd_static: the dense projection for callers that cannot allocate device
@@ -346,6 +328,10 @@ class Context:
         """One routed-expert FFN layer -> out bf16 [M, H] (and a dict of dumps if debug).
         save: dict(gate_up=bf16 [P, 2I], h=bf16 [P, I]) of caller-owned tensors that receive the
         activations the backward needs (expert-sorted order), without the other dumps."""
+        if not debug:
+            gate_up, h = (save["gate_up"], save["h"]) if save is not None else (None, None)
+            return _native.moe_fwd(self, x, topk_ids, topk_weights, w13_codes, w13_scales, w2_codes, w2_scales, out,
+                                   workspace, gate_up, h)
         assert x.dtype == torch.bfloat16 and x.is_contiguous()
         assert topk_ids.dtype == torch.int32 and topk_weights.dtype == torch.float32
         M, H = x.shape
@@ -356,26 +342,21 @@ class Context:
         y = out if out is not None else torch.empty((M, H), dtype=torch.bfloat16, device=x.device)
         nbytes = self.moe_workspace_bytes(M, H, I, E, k)
         ws = workspace if workspace is not None else self.workspace(nbytes)
-        d, dbg = None, None
-        if save is not None:
-            dbg = MoeDebug(None, None, save["gate_up"].data_ptr(), save["h"].data_ptr(), None, None, None)
-        if debug:
-            dev = x.device
-            d = dict(expert_offsets=torch.zeros(E + 1, dtype=torch.int32, device=dev),
-                     sorted_pair=torch.zeros(P, dtype=torch.int32, device=dev),
-                     gate_up=torch.zeros((P, 2 * I), dtype=torch.bfloat16, device=dev),
-                     h=torch.zeros((P, I), dtype=torch.bfloat16, device=dev),
-                     h_codes=torch.zeros((P, I), dtype=torch.uint8, device=dev),
-                     h_scales=torch.zeros((P, I // 128), dtype=torch.float32, device=dev),
-                     down_f32=torch.zeros((P, H), dtype=torch.float32, device=dev))
-            dbg = MoeDebug(d["expert_offsets"].data_ptr(), d["sorted_pair"].data_ptr(),
-                           d["gate_up"].data_ptr(), d["h"].data_ptr(), d["h_codes"].data_ptr(),
-                           d["h_scales"].data_ptr(), d["down_f32"].data_ptr())
+        dev = x.device
+        d = dict(expert_offsets=torch.zeros(E + 1, dtype=torch.int32, device=dev),
+                 sorted_pair=torch.zeros(P, dtype=torch.int32, device=dev),
+                 gate_up=torch.zeros((P, 2 * I), dtype=torch.bfloat16, device=dev),
+                 h=torch.zeros((P, I), dtype=torch.bfloat16, device=dev),
+                 h_codes=torch.zeros((P, I), dtype=torch.uint8, device=dev),
+                 h_scales=torch.zeros((P, I // 128), dtype=torch.float32, device=dev),
+                 down_f32=torch.zeros((P, H), dtype=torch.float32, device=dev))
+        dbg = MoeDebug(d["expert_offsets"].data_ptr(), d["sorted_pair"].data_ptr(),
+                       d["gate_up"].data_ptr(), d["h"].data_ptr(), d["h_codes"].data_ptr(),
+                       d["h_scales"].data_ptr(), d["down_f32"].data_ptr())
         self._check(self.lib.qarl_moe_fwd(self.h, _ptr(x), _ptr(topk_ids), _ptr(topk_weights), M, H, I, E, k,
                                           _ptr(w13_codes), _ptr(w13_scales), _ptr(w2_codes), _ptr(w2_scales),
-                                          _ptr(y), _ptr(ws), ws.numel(),
-                                          C.byref(dbg) if dbg is not None else None, _stream()))
-        return (y, d) if debug else y
+                                          _ptr(y), _ptr(ws), ws.numel(), C.byref(dbg), _stream()))
+        return y, d
 
     # ------------------------------------------------------------------ expert-parallel stages
     def moe_dispatch(self, x, topk_ids, topk_weights, E: int):
@@ -467,6 +448,8 @@ class Context:
     def moe_fwd_w4a16(self, x, topk_ids, topk_weights, w13, w2, out=None, debug: bool = False,
                       workspace: torch.Tensor | None = None):
         """One routed-expert FFN layer on W4A16 weights; w13 and w2 are (packed, scales, zeros)."""
+        if not debug:
+            return _native.moe_fwd_4bit(self, x, topk_ids, topk_weights, w13, w2, out, workspace)
         assert x.dtype == torch.bfloat16 and x.is_contiguous()
         assert topk_ids.dtype == torch.int32 and topk_weights.dtype == torch.float32
         M, H = x.shape
@@ -476,22 +459,20 @@ class Context:
         P = M * k
         y = out if out is not None else torch.empty((M, H), dtype=torch.bfloat16, device=x.device)
         ws = workspace if workspace is not None else self.workspace(self.moe_w4a16_workspace_bytes(M, H, I, E, k))
-        d, dbg = None, None
-        if debug:
-            dev = x.device
-            d = dict(expert_offsets=torch.zeros(E + 1, dtype=torch.int32, device=dev),
-                     sorted_pair=torch.zeros(P, dtype=torch.int32, device=dev),
-                     gate_up=torch.zeros((P, 2 * I), dtype=torch.bfloat16, device=dev),
-                     h=torch.zeros((P, I), dtype=torch.bfloat16, device=dev),
-                     down_f32=torch.zeros((P, H), dtype=torch.float32, device=dev))
-            dbg = MoeDebug(d["expert_offsets"].data_ptr(), d["sorted_pair"].data_ptr(),
-                           d["gate_up"].data_ptr(), d["h"].data_ptr(), None, None, d["down_f32"].data_ptr())
+        dev = x.device
+        d = dict(expert_offsets=torch.zeros(E + 1, dtype=torch.int32, device=dev),
+                 sorted_pair=torch.zeros(P, dtype=torch.int32, device=dev),
+                 gate_up=torch.zeros((P, 2 * I), dtype=torch.bfloat16, device=dev),
+                 h=torch.zeros((P, I), dtype=torch.bfloat16, device=dev),
+                 down_f32=torch.zeros((P, H), dtype=torch.float32, device=dev))
+        dbg = MoeDebug(d["expert_offsets"].data_ptr(), d["sorted_pair"].data_ptr(),
+                       d["gate_up"].data_ptr(), d["h"].data_ptr(), None, None, d["down_f32"].data_ptr())
         self._check(self.lib.qarl_moe_fwd_w4a16(self.h, _ptr(x), _ptr(topk_ids), _ptr(topk_weights), M, H, I, E, k,
                                                 _ptr(w13[0]), _ptr(w13[1]), _ptr(w13[2]),
                                                 _ptr(w2[0]), _ptr(w2[1]), _ptr(w2[2]),
                                                 _ptr(y), _ptr(ws), ws.numel(),
-                                                C.byref(dbg) if dbg is not None else None, _stream()))
-        return (y, d) if debug else y
+                                                C.byref(dbg), _stream()))
+        return y, d
 
     # ------------------------------------------------------------------ FP4A16 (e2m1 weights)
     def quantize_weight_fp4(self, w: torch.Tensor, out=None, pub=None):
@@ -525,6 +506,8 @@ class Context:
     def moe_fwd_fp4a16(self, x, topk_ids, topk_weights, w13, w2, out=None, debug: bool = False,
                        workspace: torch.Tensor | None = None):
         """One routed-expert FFN layer on e2m1 weights; w13 and w2 are (packed, scales)."""
+        if not debug:
+            return _native.moe_fwd_4bit(self, x, topk_ids, topk_weights, w13, w2, out, workspace)
         assert x.dtype == torch.bfloat16 and x.is_contiguous()
         assert topk_ids.dtype == torch.int32 and topk_weights.dtype == torch.float32
         M, H = x.shape
@@ -534,45 +517,29 @@ class Context:
         P = M * k
         y = out if out is not None else torch.empty((M, H), dtype=torch.bfloat16, device=x.device)
         ws = workspace if workspace is not None else self.workspace(self.moe_w4a16_workspace_bytes(M, H, I, E, k))
-        d, dbg = None, None
-        if debug:
-            dev = x.device
-            d = dict(expert_offsets=torch.zeros(E + 1, dtype=torch.int32, device=dev),
-                     sorted_pair=torch.zeros(P, dtype=torch.int32, device=dev),
-                     gate_up=torch.zeros((P, 2 * I), dtype=torch.bfloat16, device=dev),
-                     h=torch.zeros((P, I), dtype=torch.bfloat16, device=dev),
-                     down_f32=torch.zeros((P, H), dtype=torch.float32, device=dev))
-            dbg = MoeDebug(d["expert_offsets"].data_ptr(), d["sorted_pair"].data_ptr(),
-                           d["gate_up"].data_ptr(), d["h"].data_ptr(), None, None, d["down_f32"].data_ptr())
+        dev = x.device
+        d = dict(expert_offsets=torch.zeros(E + 1, dtype=torch.int32, device=dev),
+                 sorted_pair=torch.zeros(P, dtype=torch.int32, device=dev),
+                 gate_up=torch.zeros((P, 2 * I), dtype=torch.bfloat16, device=dev),
+                 h=torch.zeros((P, I), dtype=torch.bfloat16, device=dev),
+                 down_f32=torch.zeros((P, H), dtype=torch.float32, device=dev))
+        dbg = MoeDebug(d["expert_offsets"].data_ptr(), d["sorted_pair"].data_ptr(),
+                       d["gate_up"].data_ptr(), d["h"].data_ptr(), None, None, d["down_f32"].data_ptr())
         self._check(self.lib.qarl_moe_fwd_fp4a16(self.h, _ptr(x), _ptr(topk_ids), _ptr(topk_weights), M, H, I, E, k,
                                                  _ptr(w13[0]), _ptr(w13[1]), _ptr(w2[0]), _ptr(w2[1]),
                                                  _ptr(y), _ptr(ws), ws.numel(),
-                                                 C.byref(dbg) if dbg is not None else None, _stream()))
-        return (y, d) if debug else y
+                                                 C.byref(dbg), _stream()))
+        return y, d
 
     def quantize_weight_publish(self, w, codes, scales, pub_codes, pub_scales):
         """quantize_weight writing a second, published copy of codes and scales in the same launch."""
-        assert w.dtype == torch.bfloat16 and w.is_cuda and w.is_contiguous()
-        E, N, K = (1, *w.shape) if w.dim() == 2 else w.shape
-        self._check(self.lib.qarl_quantize_weight_publish(self.h, _ptr(w), E, N, K, _ptr(codes), _ptr(scales),
-                                                          _ptr(pub_codes), _ptr(pub_scales), _stream()))
-        return codes, scales
+        return _native.quantize_weight(self, w, codes, scales, pub_codes, pub_scales)
 
     # ------------------------------------------------------------------ backward
     def linear_bwd(self, dy, x, w, want_dx_f32: bool = False, dx: bool = True, dw: bool = True):
         """Straight-through backward of y = x . W^T on the bf16 masters ->
         (dX bf16 [M, K] or None, dX fp32 or None, dW fp32 [N, K] or None)."""
-        for t in (dy, x, w):
-            assert t.dtype == torch.bfloat16 and t.is_cuda and t.is_contiguous()
-        M, N = dy.shape
-        K = x.shape[1]
-        assert x.shape == (M, K) and w.shape == (N, K)
-        dxo = torch.empty((M, K), dtype=torch.bfloat16, device=dy.device) if dx else None
-        dx32 = torch.empty((M, K), dtype=torch.float32, device=dy.device) if (dx and want_dx_f32) else None
-        dwo = torch.empty((N, K), dtype=torch.float32, device=dy.device) if dw else None
-        self._check(self.lib.qarl_linear_bwd(self.h, _ptr(dy), _ptr(x), _ptr(w), M, N, K, _ptr(dxo), _ptr(dx32),
-                                             _ptr(dwo), _stream()))
-        return dxo, dx32, dwo
+        return _native.linear_bwd(self, dy, x, w, want_dx_f32, dx, dw)
 
     def grouped_linear_bwd(self, dy, x, w, offsets, want_dx_f32: bool = False, dx: bool = True, dw: bool = True):
         """Backward of an expert projection on expert-sorted rows: dy [P, N], x [P, K], w [E, N, K] bf16,
@@ -615,33 +582,10 @@ class Context:
                   delta_h=7e-4, cap=2.0, want_grad: bool = True, out=None, workspace=None):
         """Sequence-level TBPO surrogate over B packed responses -> dict(r, w, J f64 [B], flags i32 [B],
         grad f32 [T] or None, loss f64 [1]) of device tensors.  out: an earlier result to overwrite."""
-        for t in (lp_cur, lp_old_learner, lp_old_sampler, adv):
-            assert t.dtype == torch.float32 and t.is_cuda and t.is_contiguous()
-        assert offsets.dtype == torch.int64 and offsets.is_cuda
-        B, T = adv.shape[0], lp_cur.shape[0]
-        dev = lp_cur.device
-        if out is None:
-            out = dict(r=torch.empty(B, dtype=torch.float64, device=dev), w=torch.empty(B, dtype=torch.float64, device=dev),
-                       J=torch.empty(B, dtype=torch.float64, device=dev), flags=torch.empty(B, dtype=torch.int32, device=dev),
-                       grad=torch.empty(T, dtype=torch.float32, device=dev) if want_grad else None,
-                       loss=torch.empty(1, dtype=torch.float64, device=dev))
-        ws = workspace if workspace is not None else self.workspace(max(int(self.lib.qarl_tbpo_workspace_bytes(B, T)), 256))
-        prm = TbpoParams(eps_h, delta_l, delta_h, cap)
-        self._check(self.lib.qarl_tbpo_loss(self.h, _ptr(lp_cur), _ptr(lp_old_learner), _ptr(lp_old_sampler),
-                                            _ptr(offsets), _ptr(adv), B, T, C.byref(prm), _ptr(out["r"]), _ptr(out["w"]),
-                                            _ptr(out["J"]), _ptr(out["flags"]), _ptr(out["grad"]), _ptr(out["loss"]),
-                                            _ptr(ws), ws.numel(), _stream()))
-        return out
+        return _native.tbpo_loss(self, lp_cur, lp_old_learner, lp_old_sampler, offsets, adv, eps_h, delta_l, delta_h, cap,
+                                 want_grad, out, workspace)
 
     # ------------------------------------------------------------------ router
     def router_fwd(self, x, w_router, k: int):
         """x bf16 [M, H], w_router bf16 [E, H] -> (logits f32 [M, E], ids i32 [M, k], weights f32 [M, k])."""
-        assert x.dtype == torch.bfloat16 and w_router.dtype == torch.bfloat16 and x.is_contiguous() and w_router.is_contiguous()
-        M, H = x.shape
-        E = w_router.shape[0]
-        logits = torch.empty((M, E), dtype=torch.float32, device=x.device)
-        ids = torch.empty((M, k), dtype=torch.int32, device=x.device)
-        wts = torch.empty((M, k), dtype=torch.float32, device=x.device)
-        self._check(self.lib.qarl_router_fwd(self.h, _ptr(x), M, H, _ptr(w_router), E, k, _ptr(logits), _ptr(ids),
-                                             _ptr(wts), _stream()))
-        return logits, ids, wts
+        return _native.router_fwd(self, x, w_router, k)
