@@ -83,6 +83,27 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, unsigned block, size
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// The same in clusters of `cluster` CTAs (grid a multiple of it).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, unsigned cluster, unsigned block, size_t smem,
+                               cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // pub_codes / pub_scales: optional second destination (the copy published to the rollout engine)
 cudaError_t launch_quantize_weight(const Launch& L, const uint16_t* w, int64_t E, int64_t N, int64_t K,
                                    uint8_t* codes, float* scales, uint8_t* pub_codes = nullptr,
@@ -238,6 +259,13 @@ bool router_fused_applies(int64_t E, int64_t k);
 cudaError_t launch_router_fused(const Launch& L, EncodeTiledFn encode, const uint16_t* x, int64_t M, int64_t H,
                                 const uint16_t* wr, int64_t E, int64_t k, float* logits, int32_t* ids, float* wts,
                                 CUresult* cu_err);
+
+// The same for fewer tokens, the experts of a token tile split over the CTAs of a cluster
+// (router_cluster_sm100.cu); the entry point picks it when router_cluster_applies.
+bool router_cluster_applies(const Launch& L, int64_t M, int64_t E);
+cudaError_t launch_router_cluster(const Launch& L, EncodeTiledFn encode, const uint16_t* x, int64_t M, int64_t H,
+                                  const uint16_t* wr, int64_t E, int64_t k, float* logits, int32_t* ids, float* wts,
+                                  CUresult* cu_err);
 
 // ---- TBPO sequence-level loss ------------------------------------------------------------------
 struct TbpoArgs {

@@ -225,7 +225,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   };
 
   if (warp == kTmaWarp) {
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
       uint32_t armed = 0, armed_parity = 0;
@@ -268,51 +268,66 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       }
     }
   } else if (warp == kMmaWarp) {
-    // The whole warp follows the pipeline (so that it can zero the overhang rows of a ragged
-    // contraction step together); lane 0 issues the MMAs and commits.
+    // One thread waits, issues and commits.  Only the last step of a ragged contraction is the whole warp's:
+    // the lanes zero the overhang rows of the staged A tile together before that step's MMAs.
     constexpr uint32_t idesc = umma_idesc_bf16_f32_major(BM, BN, A_MN, B_MN);
     int stage = 0, acc = 0;
     uint32_t phase = 0, acc_phase = 0;
     bool ok = true;
     int cur_e = 0;
+    auto issue = [&](uint32_t d_tmem, int stage, bool first, bool last, int acc) {
+      tc_fence_after_sync();
+      const uint32_t a_addr = smem_u32(smem + static_cast<size_t>(stage) * kStageBytes);
+      const uint32_t b_addr = a_addr + kABytes;
+      const uint64_t a_desc = A_MN ? umma_desc_mn_sw128(a_addr, kBlockBytes) : umma_desc_k_sw128(a_addr);
+      const uint64_t b_desc = B_MN ? umma_desc_mn_sw128(b_addr, kBlockBytes) : umma_desc_k_sw128(b_addr);
+      // 16 contraction elements further on: 32 bytes inside a K-major row, 16 rows of 128 bytes
+      // in an MN-major block (start-address field counts 16-byte units)
+      constexpr uint32_t a_step = A_MN ? (16 * 128) >> 4 : 32 >> 4;
+      constexpr uint32_t b_step = B_MN ? (16 * 128) >> 4 : 32 >> 4;
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt)  // the 128-row halves of A share the B tile
+#pragma unroll
+        for (int k4 = 0; k4 < BK / 16; ++k4)
+          umma_bf16(d_tmem + mt * BN, a_desc + mt * (kAHalfBytes >> 4) + a_step * k4, b_desc + b_step * k4, idesc,
+                    (!first || k4 > 0) ? 1u : 0u);
+      umma_commit(&s->empty[stage]);
+      if (last) umma_commit(&s->tmem_full[acc]);
+    };
     for (int T = blockIdx.x; ok && T < total_tiles; T += grid) {
       const Tile t = tile_of(T, cur_e);
       if (t.KS == 0) continue;  // an expert without rows: the epilogue writes zeros, no accumulator is used
-      if (!warp_wait_or_abort(&s->tmem_empty[acc], acc_phase ^ 1, s, p)) { ok = false; break; }
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * MT) * BN;
-      for (int ks = 0; ks < t.KS; ++ks) {
+      const bool ragged = GROUP == kGroupedContraction && t.last_valid < BK;
+      const int whole = t.KS - (ragged ? 1 : 0);  // steps without overhang rows
+      if (elect_one()) {
+        ok = wait_or_abort(&s->tmem_empty[acc], acc_phase ^ 1, s, p);
+        int st = stage;
+        uint32_t ph = phase;
+        for (int ks = 0; ok && ks < whole; ++ks) {
+          if (!wait_or_abort(&s->full[st], ph, s, p)) { ok = false; break; }
+          issue(d_tmem, st, ks == 0, ks == t.KS - 1, acc);
+          if (++st == kStages) { st = 0; ph ^= 1; }
+        }
+      }
+      ok = __all_sync(0xFFFFFFFFu, ok);
+      if (!ok) break;
+      const int n = stage + whole;
+      phase ^= static_cast<uint32_t>(n / kStages) & 1u;
+      stage = n % kStages;
+      if (GROUP == kGroupedContraction && ragged) {
         if (!warp_wait_or_abort(&s->full[stage], phase, s, p)) { ok = false; break; }
+        // rows last_valid .. 63 of every 64-column block of A belong to the next expert: make them zero
         uint8_t* a_tile = smem + static_cast<size_t>(stage) * kStageBytes;
-        if (GROUP == kGroupedContraction && ks == t.KS - 1 && t.last_valid < BK) {
-          // rows last_valid .. 63 of both 64-column blocks of A belong to the next expert: make them zero
-          const int nrows = BK - t.last_valid;
-          for (int idx = lane; idx < (TM / 64) * nrows * 8; idx += 32) {
-            const int blk = idx / (nrows * 8), rem = idx % (nrows * 8);
-            *reinterpret_cast<uint4*>(a_tile + blk * kBlockBytes + (t.last_valid + rem / 8) * 128 + (rem % 8) * 16) =
-                make_uint4(0, 0, 0, 0);
-          }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        const int nrows = BK - t.last_valid;
+        for (int idx = lane; idx < (TM / 64) * nrows * 8; idx += 32) {
+          const int blk = idx / (nrows * 8), rem = idx % (nrows * 8);
+          *reinterpret_cast<uint4*>(a_tile + blk * kBlockBytes + (t.last_valid + rem / 8) * 128 + (rem % 8) * 16) =
+              make_uint4(0, 0, 0, 0);
         }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
-        if (lane == 0) {
-          tc_fence_after_sync();
-          const uint32_t a_addr = smem_u32(a_tile);
-          const uint32_t b_addr = a_addr + kABytes;
-          const uint64_t a_desc = A_MN ? umma_desc_mn_sw128(a_addr, kBlockBytes) : umma_desc_k_sw128(a_addr);
-          const uint64_t b_desc = B_MN ? umma_desc_mn_sw128(b_addr, kBlockBytes) : umma_desc_k_sw128(b_addr);
-          // 16 contraction elements further on: 32 bytes inside a K-major row, 16 rows of 128 bytes
-          // in an MN-major block (start-address field counts 16-byte units)
-          constexpr uint32_t a_step = A_MN ? (16 * 128) >> 4 : 32 >> 4;
-          constexpr uint32_t b_step = B_MN ? (16 * 128) >> 4 : 32 >> 4;
-#pragma unroll
-          for (int mt = 0; mt < MT; ++mt)  // the 128-row halves of A share the B tile
-#pragma unroll
-            for (int k4 = 0; k4 < BK / 16; ++k4)
-              umma_bf16(d_tmem + mt * BN, a_desc + mt * (kAHalfBytes >> 4) + a_step * k4, b_desc + b_step * k4, idesc,
-                        (ks > 0 || k4 > 0) ? 1u : 0u);
-          umma_commit(&s->empty[stage]);
-          if (ks == t.KS - 1) umma_commit(&s->tmem_full[acc]);
-        }
+        if (elect_one()) issue(d_tmem, stage, whole == 0, true, acc);
         __syncwarp();
         if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
@@ -320,7 +335,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     }
     // Nothing of this CTA's tensor work may be in flight when its TMEM and shared memory go
     // away: after an abort some MMAs may still be executing, so wait (bounded) for them.
-    if (!ok && lane == 0) {
+    if (!ok && elect_one()) {
       umma_commit(&s->teardown);
       mbar_wait_bounded(&s->teardown, 0, 20000000ull);
     }

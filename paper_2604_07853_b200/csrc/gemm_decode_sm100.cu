@@ -399,7 +399,7 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   if (warp >= kPromoWarps + kEpiWarps) {
     if (warp == kTmaWarp) {
       // =============================== TMA producer =======================================
-      if (lane == 0) {
+      if (elect_one()) {
         int stage = 0, armed_total = 0, cur = 0, sslot = 0;
         uint32_t phase = 0, armed = 0, armed_parity = 0, sphase = 0;
         bool ok = true;
@@ -457,7 +457,7 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       // One thread per weight block of the pair: each feeds its own 32 columns of the accumulator, so the
       // two never write the same TMEM columns, and the fixed cost per K-block of waiting, issuing and
       // committing (which holds the shared-memory stage, i.e. bytes in flight from HBM) is halved.
-      if (lane == 0) {
+      if (elect_one()) {
         const int half = warp - kMmaWarp;
         constexpr uint32_t idesc = umma_idesc_e4m3_f32(BW, NT);
         int stage = 0, ks = 0, cur = 0, sslot = 0;

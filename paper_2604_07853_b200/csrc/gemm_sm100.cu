@@ -289,7 +289,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
   if (warp >= kPromoWarps + kEpiWarps) {
     if (warp == kTmaWarp) {
       // =============================== TMA producer =====================================
-      if (lane == 0) {
+      if (elect_one()) {
         int stage = 0;
         uint32_t phase = 0;
         uint32_t armed = 0, armed_parity = 0;  // per-stage: has a load in flight / its parity
@@ -336,7 +336,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
       // issued by thread n % 2 into accumulator n % 2.  Every K-block starts a fresh accumulator, so
       // the two never write the same columns, and the fixed cost per K-block of one thread waiting,
       // issuing and committing (about as long as the MMAs themselves take) is spread over two.
-      if (lane == 0) {
+      if (elect_one()) {
         constexpr uint32_t idesc = umma_idesc_e4m3_f32(BM, BN);
         const int me = warp - kMmaWarp;
         uint32_t n = 0;  // K-blocks of this CTA so far

@@ -232,7 +232,7 @@ gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Decod
     // (this warp only started the first tile's codes on their way to L2, above)
   } else if (warp == kTokenWarp) {
     // =============================== producer of the token rows =======================
-    if (lane == 0) {
+    if (elect_one()) {
       int xs = 0, cur_e = 0;
       uint32_t x_phase = 0, x_armed = 0, x_armed_parity = 0;
       bool ok = true;
@@ -259,7 +259,7 @@ gemm_w4a16_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Decod
     // =============================== MMA issuers ======================================
     // One thread per weight block: each feeds its own 32 TMEM columns in ascending k, so the two never
     // touch the same accumulator, and the per-stage cost of waiting, issuing and committing is shared.
-    if (lane == 0) {
+    if (elect_one()) {
       const int h = warp - kMmaWarp0;
       constexpr uint32_t idesc = umma_idesc_bf16_f32(BW, NT);
       int xs = 0, ds = 0, acc = 0;

@@ -223,7 +223,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_a, const W4Params p) {
 
   if (warp == kTmaWarp) {
     // =============================== TMA producer =====================================
-    if (lane == 0) {
+    if (elect_one()) {
       int as = 0, qs = 0;
       uint32_t a_phase = 0, q_phase = 0;
       uint32_t a_armed = 0, a_armed_parity = 0, q_armed = 0, q_armed_parity = 0;
@@ -268,7 +268,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_a, const W4Params p) {
     }
   } else if (warp == kMmaWarp) {
     // =============================== MMA issuer =======================================
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = umma_idesc_bf16_f32(BM, BN);
       int ls = 0, ds = 0, acc = 0;
       uint32_t ld_phase = 0, dq_phase = 0, acc_phase = 0;

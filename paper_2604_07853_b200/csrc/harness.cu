@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(128, 1) fp8_mma_peak_kernel(int kblocks, int* 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ uint64_t done[2];
   __shared__ uint32_t taddr;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     ptx::mbar_init(&done[0], 1);
     ptx::mbar_init(&done[1], 1);
@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(128, 1) fp8_mma_peak_kernel(int kblocks, int* 
   ptx::tc_fence_before_sync();
   __syncthreads();
   ptx::tc_fence_after_sync();
-  if (warp == 1 && lane == 0) {
+  if (warp == 1 && ptx::elect_one()) {
     constexpr uint32_t idesc = ptx::umma_idesc_e4m3_f32(128, 256);
     uint32_t ph[2] = {0, 0};
     bool ok = true;

@@ -3,15 +3,12 @@
 // keeps experts l, l + 32, ... in registers; k rounds of a warp arg-max.  The logits come from the
 // bf16 tensor-core GEMM (x . W_r^T, fp32 accumulation in a fixed order), so a token's routing
 // depends only on that token's row -- the same invariance the expert GEMMs have (App. C).
-#include <math.h>
-
-#include "common.cuh"
+#include "router_select.cuh"
 
 namespace qarl {
 namespace {
 
-// PER = experts per lane (E <= 32 PER), a compile-time bound so that the selection loops unroll to
-// exactly the work the expert count needs.
+// PER = experts per lane (E <= 32 PER).
 template <int PER>
 __global__ void __launch_bounds__(256) router_topk_kernel(const float* __restrict__ logits, int64_t M, int E, int k,
                                                           int32_t* __restrict__ ids, float* __restrict__ wts) {
@@ -27,47 +24,7 @@ __global__ void __launch_bounds__(256) router_topk_kernel(const float* __restric
     const int e = lane + 32 * j;
     v[j] = e < E ? row[e] : -INFINITY;
   }
-  uint32_t taken = 0;  // bit j: this lane's j-th expert was selected
-  float sel = 0.0f;    // lane j < k ends up holding the j-th selected logit
-  int sel_id = 0;
-  for (int r = 0; r < k; ++r) {
-    float best = -INFINITY;
-    int best_e = 0x7FFFFFFF;
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-      if (!((taken >> j) & 1u)) {
-        const int e = lane + 32 * j;
-        if (e < E && (v[j] > best || best_e == 0x7FFFFFFF)) {  // ascending e within a lane: strict > keeps the lower id
-          best = v[j];
-          best_e = e;
-        }
-      }
-    }
-    // Warp arg-max in two reductions instead of a five-step butterfly on (value, id) pairs: the largest
-    // value through an order-preserving map of its bits to unsigned (-0 first folded onto +0, so equal
-    // values map to equal keys), then the lowest id among the lanes that hold it.
-    const uint32_t bits = __float_as_uint(best + 0.0f);
-    const uint32_t key = best_e == 0x7FFFFFFF ? 0u : ((bits & 0x80000000u) ? ~bits : (bits | 0x80000000u));
-    const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, key);
-    const int win_e = static_cast<int>(__reduce_min_sync(0xFFFFFFFFu, key == top ? static_cast<uint32_t>(best_e) : 0x7FFFFFFFu));
-    const float win = __shfl_sync(0xFFFFFFFFu, best, win_e & 31);
-    best = win;
-    best_e = win_e;
-    if ((best_e & 31) == lane) taken |= 1u << (best_e >> 5);
-    if (lane == r) {
-      sel = best;
-      sel_id = best_e;
-    }
-  }
-  // softmax over the k selected logits, in double: exp(l - max) / sum, rounded to fp32
-  const double mx = static_cast<double>(__shfl_sync(0xFFFFFFFFu, sel, 0));
-  double ex = lane < k ? exp(static_cast<double>(sel) - mx) : 0.0;
-  double den = 0.0;  // summed in selection order (the one-launch router adds them as it selects)
-  for (int j = 0; j < k; ++j) den += __shfl_sync(0xFFFFFFFFu, ex, j);
-  if (lane < k) {
-    ids[m * k + lane] = sel_id;
-    wts[m * k + lane] = static_cast<float>(ex / den);
-  }
+  select_topk<PER>(v, E, k, lane, ids + m * k, wts + m * k);
 }
 
 }  // namespace

@@ -138,7 +138,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
   const int grid = gridDim.x;
 
   if (warp == kTmaWarp) {
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
       uint32_t armed = 0, armed_parity = 0;
@@ -164,7 +164,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
       }
     }
   } else if (warp == kMmaWarp) {
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = umma_idesc_bf16_f32_major(RM, RN, false, false);
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
