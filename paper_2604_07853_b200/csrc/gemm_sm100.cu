@@ -12,21 +12,28 @@
 // [n_hi, n_hi+128) of the weight -- adjacent for linear/down, gate rows and the matching up
 // rows for gate_up so that SwiGLU and the 1x128 re-quantization of h need no second pass.
 //
-// Structure of a CTA (512 threads = 4 warpgroups, one CTA per SM, persistent, static tile list):
-//   warp 12     TMA producer: per K-block one stage = A box 128x128 B + two B boxes 128x128 B
-//               (SWIZZLE_128B) into a 3-deep shared-memory ring;
-//   warp 13     MMA issuer: 4 x tcgen05.mma kind::f8f6f4 per K-block into one of two
+// Structure of a CTA (384 threads = 3 warpgroups, one CTA per SM, persistent, static tile list):
+//   warp 8      TMA producer: per K-block one stage = A box 128x128 B + two B boxes 128x128 B
+//               (SWIZZLE_128B) into a ring of 48 KB stages;
+//   warp 9      MMA issuer: 4 x tcgen05.mma kind::f8f6f4 per K-block into one of two
 //               256-column TMEM accumulators (overwrite on the first), then tcgen05.commit to
 //               free the smem stage and to publish the accumulator;
-//   warps 0-7   promotion (208 registers each via setmaxnreg): warp w reads TMEM lanes
+//   warps 10-11 scales: fl(s_x s_w) of every row and half for the K-block in each accumulator;
+//   warps 0-7   promotion (224 registers each via setmaxnreg): warp w reads TMEM lanes
 //               32*(w%4).. (its hardware quadrant) and the 64-column slice (w/4) of each half,
-//               in 16-column double-buffered chunks, releases the accumulator, and adds
-//               scale * partial into fp32 registers; MMA of block kb+1 overlaps promotion of kb.  At the
-//               end of a tile it rounds its 128 values to bf16 into a shared-memory staging
-//               tile and goes straight on to the next tile;
-//   warps 8-11  epilogue: read the staged bf16 tile (coalesced, several rows per pass) and
-//               finish it while the next tile's main loop runs: plain store (linear),
-//               scatter by pair id (down), or SwiGLU + 1x128 amax/scale/e4m3 codes (gate_up).
+//               releases the accumulator, and adds scale * partial into fp32 registers; the
+//               MMA of block kb+1 overlaps the promotion of kb.  At the end of a tile it finishes
+//               its 128 values itself: gate_up = SwiGLU, 1x128 amax / scale / e4m3 codes from registers;
+//               linear, down = bf16 rows through a swizzled staging box and a TMA store.
+//
+// What bounds it: the promotion next to the MMA.  Per K-block it reads 128 KB of TMEM and does 32768 FMAs
+// (256 clocks of the FP32 pipes; reads and FMAs alone measure 360) against 512 clocks of MMAs, so what it must
+// not do is wait or spill.  With scale loads, waits and separate epilogue warps inline a K-block took ~1210
+// clocks; as below ~960 (dense M = 8192, N = 5120, K = 2048: 103 -> 84 us on the same part, at the clock
+// the power cap allows).  What did it: scales from two warps of their own through shared memory, one stream
+// of TMEM reads across K-blocks (the first chunk of the next accumulator is on its way before the last chunk
+// of this one is accumulated), two FMAs per instruction, the loop body without spills (32-column chunks
+// spill and lose), and no epilogue warps (their registers and polling cost more than they hid).
 //
 // Every wait on an mbarrier is bounded; on expiry the thread records
 // QARL_ERR_DEVICE_TIMEOUT, raises a CTA-wide abort flag that all other waits poll, and the
@@ -46,24 +53,23 @@ constexpr int BM = 128;           // rows per tile (UMMA M)
 constexpr int BNH = 128;          // columns per half tile
 constexpr int BN = 2 * BNH;       // UMMA N
 constexpr int BK = 128;           // one K-block = one 128-byte swizzle span of e4m3
-constexpr int kStages = 3;        // shared-memory ring of 48 KB stages
 constexpr int kAccBufs = 2;       // TMEM accumulators of 256 columns
 constexpr int kPromoWarps = 8;    // warps 0-7
-constexpr int kEpiWarps = 4;      // warps 8-11
-constexpr int kTmaWarp = 12;
-constexpr int kMmaWarp = 13;      // and 14: two issuers; warp 15 idle (setmaxnreg works on whole warpgroups)
-constexpr int kThreads = 16 * 32;
-// register re-allocation: 256 x 208 + 128 x 56 + 128 x 40 = 65536 = 512 x 128 (the launch allocation)
-constexpr int kPromoRegs = 208;
-constexpr int kEpiRegs = 56;
-constexpr int kAuxRegs = 40;
+constexpr int kTmaWarp = 8;
+constexpr int kMmaWarp = 9;
+constexpr int kScaleWarp = 10;    // and 11
+constexpr int kThreads = 12 * 32;
+// register re-allocation: 256 x 224 + 128 x 56 = 64512 = 384 x 168 (the launch allocation)
+constexpr int kPromoRegs = 224;
+constexpr int kAuxRegs = 56;
 constexpr int kSliceCols = 64;    // columns of each half owned by one promotion warp
 constexpr uint32_t kABytes = BM * BK;
 constexpr uint32_t kBBytes = BN * BK;
 constexpr uint32_t kStageBytes = kABytes + kBBytes;  // 48 KB
 constexpr uint32_t kTmemCols = 512;
-constexpr int kOutPitch = BN * 2 + 16;  // bytes per row of the bf16 staging tile (padded: conflict-free)
-constexpr uint32_t kOutBytes = BM * kOutPitch;
+// a promotion warp's bf16 rows on their way out: two boxes of 32 rows x 128 bytes (128-byte swizzle)
+constexpr uint32_t kOutBoxBytes = 32 * 128;
+constexpr uint32_t kOutBytes = kPromoWarps * 2 * kOutBoxBytes;
 constexpr int kMaxExperts = 1024;
 
 struct GemmParams {
@@ -82,29 +88,39 @@ struct GemmParams {
   uint8_t* h_codes;
   float* h_scales;
   uint16_t* h_bf16;
-  const int32_t* sorted_pair;
+  int h_vec32;             // h_bf16 is 32-byte aligned
   const float* pair_weights;  // down: combine weight of each sorted position
   int* status;
   unsigned long long wait_limit_ns;
   int stop_after_stages;   // test harness only (< 0: off): the TMA producer stops arming stages after this many
 };
 
+// SAVE (gate_up only): the call also wants the bf16 gate_up and / or h rows (a training forward, tests)
+template <int MODE, bool SAVE>
+struct Cfg {
+  static constexpr bool kStaged = MODE != kModeGateUp || SAVE;  // rows leave through the staging boxes
+  static constexpr int kStages = kStaged ? 3 : 4;
+  static constexpr uint32_t kStaging = kStaged ? kOutBytes : 0;
+};
+
 struct __align__(8) SmemTail {
-  uint64_t full[kStages];
-  uint64_t empty[kStages];
+  uint64_t full[4];
+  uint64_t empty[4];
   uint64_t tmem_full[kAccBufs];
   uint64_t tmem_empty[kAccBufs];
-  uint64_t out_full;
-  uint64_t out_empty;
-  uint64_t teardown[2];
+  uint64_t amax_full[4];       // gate_up: the two warps of a TMEM quadrant have exchanged their row maxima
+  uint64_t teardown;
+  float2 scale[kAccBufs][BM];  // products of the K-block in each accumulator: row scale x (lo, hi) weight scale
+  uint32_t amax[2][2][BM];     // gate_up: [tile parity][column slice][row] |h| maxima (bf16 bits)
   uint32_t tmem_addr;
   int abort_flag;
   int32_t off[kMaxExperts + 1];
   int32_t prefix[kMaxExperts + 1];
 };
 
-constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(kStages) * kStageBytes + kOutBytes + sizeof(SmemTail);
-static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
+template <int MODE, bool SAVE>
+constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(Cfg<MODE, SAVE>::kStages) * kStageBytes + Cfg<MODE, SAVE>::kStaging + sizeof(SmemTail);
+static_assert(kSmemBytes<kModeGateUp, false> <= 227 * 1024 && kSmemBytes<kModeGateUp, true> <= 227 * 1024, "shared memory budget");
 
 struct TileCoord {
   int e, n_tile, m0, m_end;
@@ -127,13 +143,13 @@ __device__ __forceinline__ TileCoord decode_tile(const SmemTail* s, int T, int& 
 
 // Bounded wait of one thread.  False: the limit ran out here (the error is recorded and the
 // CTA-wide abort flag raised) or another thread raised the flag; the caller leaves its loop.
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, SmemTail* s, const GemmParams& p) {
-  if (mbar_try_wait(bar, parity)) return true;
+__device__ __forceinline__ bool wait_or_abort_at(uint32_t bar, uint32_t parity, SmemTail* s, const GemmParams& p) {
+  if (mbar_try_wait_at(bar, parity)) return true;
   const uint64_t t0 = globaltimer_ns();
   for (;;) {
 #pragma unroll 1
     for (int i = 0; i < 128; ++i)
-      if (mbar_try_wait(bar, parity)) return true;
+      if (mbar_try_wait_at(bar, parity)) return true;
     if (*reinterpret_cast<volatile int*>(&s->abort_flag)) return false;
     if (globaltimer_ns() - t0 > p.wait_limit_ns) {
       set_status(p.status, QARL_ERR_DEVICE_TIMEOUT);
@@ -141,6 +157,9 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, Sm
       return false;
     }
   }
+}
+__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, SmemTail* s, const GemmParams& p) {
+  return wait_or_abort_at(smem_u32(bar), parity, s, p);
 }
 
 // The same for a whole warp: every lane polls (one polling lane with 31 parked at a shuffle
@@ -157,13 +176,11 @@ __device__ __forceinline__ float silu_mul(float g, float u) {
   return __fdividef(g, 1.0f + __expf(-g)) * u;
 }
 
-// acc[j] = fmaf(sc, v[j], acc[j]) for 16 values (8 float2 accumulators).
+// acc[j] = fmaf(sc, v[j], acc[j]) for 16 values (8 float2 accumulators), two per instruction.
 __device__ __forceinline__ void promote16(float2* acc, const uint32_t (&v)[16], float sc) {
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    acc[j].x = __fmaf_rn(sc, __uint_as_float(v[2 * j]), acc[j].x);
-    acc[j].y = __fmaf_rn(sc, __uint_as_float(v[2 * j + 1]), acc[j].y);
-  }
+  for (int j = 0; j < 8; ++j)
+    acc[j] = __ffma2_rn(make_float2(sc, sc), make_float2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1])), acc[j]);
 }
 
 __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
@@ -171,14 +188,255 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&b);
 }
 
-template <int MODE>
+// 32 bytes to global memory, 32-byte aligned
+__device__ __forceinline__ void st_global_v8(void* dst, const uint32_t (&v)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+               "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+// the same for a pointer that is only 16-byte aligned (caller-owned dumps)
+__device__ __forceinline__ void st_global_2x16(void* dst, const uint32_t (&v)[8]) {
+  uint4* d = static_cast<uint4*>(dst);
+  d[0] = make_uint4(v[0], v[1], v[2], v[3]);
+  d[1] = make_uint4(v[4], v[5], v[6], v[7]);
+}
+
+// The promotion warps (see the header).  What they need is read again here instead of being carried over from
+// the kernel's set-up: with 160 registers of sums and partial sums every long-lived value counts.
+template <int MODE, bool SAVE>
+__device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const GemmParams& p, uint8_t* smem, SmemTail* s,
+                                               const int first_tile, const int num_ctas, const int total_tiles) {
+  uint32_t tid;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+  const int warp = tid >> 5, lane = tid & 31;
+  const int q = warp & 3;          // TMEM lane quadrant this warp may read
+  const int hs = warp >> 2;        // which 64-column slice of each half tile
+  const int r = q * 32 + lane;     // row within the tile
+  const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&s->tmem_addr) + (static_cast<uint32_t>(q * 32) << 16) +
+                        static_cast<uint32_t>(hs * kSliceCols);
+  const uint32_t full_bar = smem_u32(&s->tmem_full[0]), empty_bar = smem_u32(&s->tmem_empty[0]);
+  const uint32_t scale_at = smem_u32(&s->scale[0][r]);
+  const int KB = p.kblocks;
+  int ks = 0;
+  uint32_t acc_phase = 0;
+  int cur_e = 0;
+  uint32_t tile_iter = 0;
+
+  auto full_wait = [&]() -> bool { return __all_sync(0xFFFFFFFFu, wait_or_abort_at(full_bar + 8 * ks, acc_phase, s, p)) != 0; };
+  auto release = [&]() {  // this warp's reads of accumulator ks are done: hand it back to the MMA warp
+    tc_fence_before_sync();
+    __syncwarp();
+    if (lane == 0) mbar_arrive_at(empty_bar + 8 * ks);
+    if (++ks == kAccBufs) { ks = 0; acc_phase ^= 1; }
+  };
+
+  // bf16 rows leave through this warp's two boxes: 64 columns each, 16-byte chunk j of a row at j ^ (row % 8)
+  uint8_t* boxes = smem + static_cast<size_t>(Cfg<MODE, SAVE>::kStages) * kStageBytes + static_cast<size_t>(warp) * 2 * kOutBoxBytes;
+  auto box_chunk = [&](int box, int j) { return reinterpret_cast<uint4*>(boxes + box * kOutBoxBytes + lane * 128 + ((j ^ (lane & 7)) << 4)); };
+  auto boxes_free = [&]() {  // the previous tile's boxes have been read
+    if (lane == 0) bulk_wait_group_read_all();
+    __syncwarp();
+  };
+  auto send_boxes = [&](int row0, int m_end, int col0, int col1) {
+    if (MODE == kModeLinear || row0 + 32 <= m_end) {  // (a dense tile's rows past M are clipped by the tensor map)
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        tma_store_2d(&tm_o, boxes, col0, row0);
+        if (col1 < p.N) tma_store_2d(&tm_o, boxes + kOutBoxBytes, col1, row0);
+        bulk_commit_group();
+      }
+    } else {  // the rows past the group's end are the next expert's: 8 lanes per row and box, 2 rows at a time
+      __syncwarp();
+      const int box = (lane >> 3) & 1, chunk = lane & 7;
+      const int col = (box ? col1 : col0) + 8 * chunk;
+      for (int rr = lane >> 4; row0 + rr < m_end; rr += 2) {
+        const uint4 v = *reinterpret_cast<const uint4*>(boxes + box * kOutBoxBytes + rr * 128 + ((chunk ^ (rr & 7)) << 4));
+        if (col < p.N) *reinterpret_cast<uint4*>(p.out_bf16 + static_cast<int64_t>(row0 + rr) * p.N + col) = v;
+      }
+      __syncwarp();
+    }
+  };
+
+  for (int T = first_tile; T < total_tiles; T += num_ctas, ++tile_iter) {
+    const TileCoord c = decode_tile(s, T, cur_e);
+    // a warp whose 32 rows all lie past the group's end (ragged tails, decode-sized groups)
+    // keeps the barrier protocol going but reads and accumulates nothing
+    const bool warp_live = c.m0 + q * 32 < c.m_end;
+    float2 acc_lo[32], acc_hi[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) acc_lo[j] = acc_hi[j] = make_float2(0.0f, 0.0f);
+
+    if (!warp_live) {
+      for (int kb = 0; kb < KB; ++kb) {
+        if (!full_wait()) return;
+        release();
+      }
+    } else {
+      // The 16-column chunks of the accumulators are one stream across the K-blocks of the tile: while a
+      // chunk is accumulated the next one is on its way from TMEM, and behind the last chunk of a K-block
+      // that is the first one of the next (whose barrier was polled a chunk earlier).
+      uint32_t va[16], vb[16];
+      float2 scale;
+      auto read_scale = [&]() {
+        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(scale.x), "=f"(scale.y)
+                     : "r"(scale_at + static_cast<uint32_t>(ks) * static_cast<uint32_t>(sizeof(s->scale[0]))) : "memory");
+      };
+      auto all_but_last = [&]() {  // chunks 0-6 of accumulator ks but for the sums of chunk 6; on return chunk 7 is in flight
+        const uint32_t t0 = tmem + static_cast<uint32_t>(ks * BN);
+        tmem_ld_wait();
+#pragma unroll
+        for (int c = 0; c < 6; c += 2) {
+          tmem_ld_x16(t0 + (c < 4 ? 16 * (c + 1) : BNH + 16 * (c - 3)), vb);
+          promote16(c < 4 ? acc_lo + 8 * c : acc_hi + 8 * (c - 4), va, c < 4 ? scale.x : scale.y);
+          tmem_ld_wait();
+          tmem_ld_x16(t0 + (c < 2 ? 16 * (c + 2) : BNH + 16 * (c - 2)), va);
+          promote16(c < 4 ? acc_lo + 8 * (c + 1) : acc_hi + 8 * (c - 3), vb, c < 4 ? scale.x : scale.y);
+          tmem_ld_wait();
+        }
+        tmem_ld_x16(t0 + BNH + 48, vb);
+      };
+      if (!full_wait()) return;
+      tc_fence_after_sync();
+      tmem_ld_x16(tmem + static_cast<uint32_t>(ks * BN), va);
+      read_scale();
+#pragma unroll 1
+      for (int kb = 1; kb < KB; ++kb) {
+        all_but_last();
+        // the other accumulator's barrier: the answer is needed one chunk later
+        const bool next_ready = mbar_try_wait_at(full_bar + 8 * (ks ^ 1), acc_phase ^ static_cast<uint32_t>(ks));
+        promote16(acc_hi + 16, va, scale.y);
+        tmem_ld_wait();
+        release();
+        if (!__all_sync(0xFFFFFFFFu, next_ready) && !full_wait()) return;
+        tc_fence_after_sync();
+        tmem_ld_x16(tmem + static_cast<uint32_t>(ks * BN), va);
+        promote16(acc_hi + 24, vb, scale.y);
+        read_scale();
+      }
+      all_but_last();
+      promote16(acc_hi + 16, va, scale.y);
+      tmem_ld_wait();
+      release();
+      promote16(acc_hi + 24, vb, scale.y);
+    }
+
+    // ---- the tile is complete: finish it ------------------------------------------------
+    const int row = c.m0 + r;
+    const bool valid = row < c.m_end;
+    if ((MODE == kModeLinear || MODE == kModeDown) && p.out_f32 && valid) {  // debug fp32 dump
+      const int col_lo = c.n_tile * BN + hs * kSliceCols;
+      const int col_hi = col_lo + BNH;
+      float2* d_lo = reinterpret_cast<float2*>(p.out_f32 + static_cast<int64_t>(row) * p.N + col_lo);
+      float2* d_hi = reinterpret_cast<float2*>(p.out_f32 + static_cast<int64_t>(row) * p.N + col_hi);
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        d_lo[j] = acc_lo[j];
+        if (col_hi < p.N) d_hi[j] = acc_hi[j];
+      }
+    }
+    if (MODE == kModeDown) {  // contribution = bf16( fl(w * y) )
+      const float w = valid ? __ldg(p.pair_weights + row) : 0.0f;
+      const float2 w2 = make_float2(w, w);
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        acc_lo[j] = __fmul2_rn(w2, acc_lo[j]);
+        acc_hi[j] = __fmul2_rn(w2, acc_hi[j]);
+      }
+    }
+    if (MODE == kModeGateUp) {
+      // This thread holds gate columns [64 hs, 64 hs + 64) of its row in acc_lo and the up columns of the
+      // same h columns in acc_hi.  h = bf16(silu(bf16 gate) * bf16 up); the other warp of the quadrant
+      // (w ^ 4) holds the rest of the row's 128-wide quantization group: only the maxima are exchanged.
+      uint32_t hb[32];
+      uint32_t m = 0;
+      const int64_t col = c.n_tile * BNH + hs * kSliceCols;
+      if (warp_live) {
+        if (SAVE && p.out_bf16) boxes_free();
+#pragma unroll
+        for (int j8 = 0; j8 < 4; ++j8) {  // 16 columns at a time
+          uint32_t gw[8], uw[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            gw[j] = bf16x2_bits(acc_lo[8 * j8 + j].x, acc_lo[8 * j8 + j].y);
+            uw[j] = bf16x2_bits(acc_hi[8 * j8 + j].x, acc_hi[8 * j8 + j].y);
+            const float h0 = silu_mul(bf16_bits_to_f32(gw[j] & 0xFFFFu), bf16_bits_to_f32(uw[j] & 0xFFFFu));
+            const float h1 = silu_mul(__uint_as_float(gw[j] & 0xFFFF0000u), __uint_as_float(uw[j] & 0xFFFF0000u));
+            hb[8 * j8 + j] = bf16x2_bits(h0, h1);
+            m = __vmaxu2(m, hb[8 * j8 + j] & 0x7FFF7FFFu);  // |bf16| bit patterns: exact, order-free max
+          }
+          if (SAVE && p.out_bf16) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+              *box_chunk(0, 2 * j8 + k) = make_uint4(gw[4 * k], gw[4 * k + 1], gw[4 * k + 2], gw[4 * k + 3]);
+              *box_chunk(1, 2 * j8 + k) = make_uint4(uw[4 * k], uw[4 * k + 1], uw[4 * k + 2], uw[4 * k + 3]);
+            }
+          }
+        }
+        if (SAVE && p.out_bf16) send_boxes(c.m0 + q * 32, c.m_end, static_cast<int>(col), static_cast<int>(col) + p.I);
+      }
+      m = max(m & 0xFFFFu, m >> 16);
+      const uint32_t par = tile_iter & 1u;
+      s->amax[par][hs][r] = m;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&s->amax_full[q]);
+      if (!warp_wait_or_abort(&s->amax_full[q], par, s, p)) return;
+      m = max(m, s->amax[par][hs ^ 1][r]);
+      float inv;
+      const float sc = block_scale(bf16_bits_to_f32(m), &inv);
+      if (valid) {
+        uint8_t* hc = p.h_codes + static_cast<int64_t>(row) * p.I + col;
+#pragma unroll
+        for (int j8 = 0; j8 < 2; ++j8) {
+          uint32_t cw[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const uint32_t x0 = hb[16 * j8 + 2 * j], x1 = hb[16 * j8 + 2 * j + 1];
+            cw[j] = cvt_e4m3x4(__fmul_rn(bf16_bits_to_f32(x0 & 0xFFFFu), inv), __fmul_rn(__uint_as_float(x0 & 0xFFFF0000u), inv),
+                               __fmul_rn(bf16_bits_to_f32(x1 & 0xFFFFu), inv), __fmul_rn(__uint_as_float(x1 & 0xFFFF0000u), inv));
+          }
+          st_global_v8(hc + 32 * j8, cw);
+        }
+        if (hs == 0) p.h_scales[static_cast<int64_t>(row) * (p.I / BNH) + c.n_tile] = sc;
+        if (SAVE && p.h_bf16) {
+          uint16_t* hd = p.h_bf16 + static_cast<int64_t>(row) * p.I + col;
+#pragma unroll
+          for (int j8 = 0; j8 < 4; ++j8) {
+            uint32_t w8[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w8[j] = hb[8 * j8 + j];
+            if (p.h_vec32) st_global_v8(hd + 16 * j8, w8);
+            else st_global_2x16(hd + 16 * j8, w8);
+          }
+        }
+      }
+    } else if (warp_live) {
+      boxes_free();
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        *box_chunk(0, j) =
+            make_uint4(bf16x2_bits(acc_lo[4 * j].x, acc_lo[4 * j].y), bf16x2_bits(acc_lo[4 * j + 1].x, acc_lo[4 * j + 1].y),
+                       bf16x2_bits(acc_lo[4 * j + 2].x, acc_lo[4 * j + 2].y), bf16x2_bits(acc_lo[4 * j + 3].x, acc_lo[4 * j + 3].y));
+        *box_chunk(1, j) =
+            make_uint4(bf16x2_bits(acc_hi[4 * j].x, acc_hi[4 * j].y), bf16x2_bits(acc_hi[4 * j + 1].x, acc_hi[4 * j + 1].y),
+                       bf16x2_bits(acc_hi[4 * j + 2].x, acc_hi[4 * j + 2].y), bf16x2_bits(acc_hi[4 * j + 3].x, acc_hi[4 * j + 3].y));
+      }
+      const int col_lo = c.n_tile * BN + hs * kSliceCols;
+      send_boxes(c.m0 + q * 32, c.m_end, col_lo, col_lo + BNH);
+    }
+  }
+  if (Cfg<MODE, SAVE>::kStaged && lane == 0) bulk_wait_group_all();  // this warp's rows are written
+}
+
+template <int MODE, bool SAVE>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
-                        const GemmParams p) {
+                        const __grid_constant__ CUtensorMap tm_o, const GemmParams p) {
+  constexpr int kStages = Cfg<MODE, SAVE>::kStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* out_tile = smem + static_cast<size_t>(kStages) * kStageBytes;
-  SmemTail* s = reinterpret_cast<SmemTail*>(out_tile + kOutBytes);
+  SmemTail* s = reinterpret_cast<SmemTail*>(out_tile + Cfg<MODE, SAVE>::kStaging);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   // ---- set-up: barriers, TMEM, tile list ------------------------------------------------
@@ -189,19 +447,18 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
       mbar_init(&s->empty[i], 1);
     }
     for (int i = 0; i < kAccBufs; ++i) {
-      mbar_init(&s->tmem_full[i], 1);
+      mbar_init(&s->tmem_full[i], 3);  // the MMA commit and the two scale warps
       mbar_init(&s->tmem_empty[i], kPromoWarps);
     }
-    mbar_init(&s->out_full, kPromoWarps);
-    mbar_init(&s->out_empty, kEpiWarps);
-    mbar_init(&s->teardown[0], 1);
-    mbar_init(&s->teardown[1], 1);
+    for (int i = 0; i < 4; ++i) mbar_init(&s->amax_full[i], 2);
+    mbar_init(&s->teardown, 1);
     s->abort_flag = 0;
     fence_mbar_init();
   }
   if (warp == kTmaWarp && lane == 0) {
     prefetch_tensormap(&tm_a);
     prefetch_tensormap(&tm_b);
+    if (Cfg<MODE, SAVE>::kStaged) prefetch_tensormap(&tm_o);
   }
   if (warp == kMmaWarp) {
     tmem_alloc(&s->tmem_addr, kTmemCols);
@@ -283,10 +540,8 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
   const int KB = p.kblocks;
   const int NB = p.N / BNH;  // weight scale block-rows per expert
 
-  if (warp >= kPromoWarps + kEpiWarps) setmaxnreg_dec<kAuxRegs>();
-  else if (warp >= kPromoWarps) setmaxnreg_dec<kEpiRegs>();
-  else setmaxnreg_inc<kPromoRegs>();
-  if (warp >= kPromoWarps + kEpiWarps) {
+  if (warp >= kPromoWarps) {
+    setmaxnreg_dec<kAuxRegs>();
     if (warp == kTmaWarp) {
       // =============================== TMA producer =====================================
       if (elect_one()) {
@@ -330,290 +585,94 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
             if (armed & (1u << i)) mbar_wait_bounded(&s->full[i], (armed_parity >> i) & 1u, 20000000ull);
         }
       }
-    } else if (warp == kMmaWarp || warp == kMmaWarp + 1) {
-      // =============================== MMA issuers ======================================
-      // Two threads, one per TMEM accumulator: K-block n of this CTA (counted across its tiles) is
-      // issued by thread n % 2 into accumulator n % 2.  Every K-block starts a fresh accumulator, so
-      // the two never write the same columns, and the fixed cost per K-block of one thread waiting,
-      // issuing and committing (about as long as the MMAs themselves take) is spread over two.
+    } else if (warp == kMmaWarp) {
+      // =============================== MMA issuer =======================================
       if (elect_one()) {
         constexpr uint32_t idesc = umma_idesc_e4m3_f32(BM, BN);
-        const int me = warp - kMmaWarp;
-        uint32_t n = 0;  // K-blocks of this CTA so far
+        int stage = 0, ks = 0;
+        uint32_t phase = 0, acc_phase = 0;
         bool ok = true;
         for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
-          for (int kb = 0; kb < KB; ++kb, ++n) {
-            if (static_cast<int>(n & 1u) != me) continue;
-            const uint32_t stage = n % kStages, phase = (n / kStages) & 1u;
-            const uint32_t ks = n & 1u, acc_phase = (n >> 1) & 1u;
+          for (int kb = 0; kb < KB; ++kb) {
             if (!wait_or_abort(&s->tmem_empty[ks], acc_phase ^ 1, s, p)) { ok = false; break; }
             if (!wait_or_abort(&s->full[stage], phase, s, p)) { ok = false; break; }
             tc_fence_after_sync();
             const uint32_t a_addr = smem_u32(smem + static_cast<size_t>(stage) * kStageBytes);
             const uint64_t a_desc = umma_desc_k_sw128(a_addr);
             const uint64_t b_desc = umma_desc_k_sw128(a_addr + kABytes);
-            const uint32_t d_tmem = tmem_base + ks * BN;
+            const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(ks * BN);
 #pragma unroll
             for (int k4 = 0; k4 < BK / 32; ++k4)  // +32 bytes of K = +2 in the 16-byte address field
               umma_f8(d_tmem, a_desc + 2 * k4, b_desc + 2 * k4, idesc, k4 > 0 ? 1u : 0u);
             umma_commit(&s->empty[stage]);
             umma_commit(&s->tmem_full[ks]);
+            if (++stage == kStages) { stage = 0; phase ^= 1; }
+            if (++ks == kAccBufs) { ks = 0; acc_phase ^= 1; }
           }
         }
         // Nothing of this CTA's tensor work may be in flight when its TMEM and shared memory
         // go away: after a normal run every MMA has been consumed already; after an abort
         // some may still be executing, so wait (bounded) for all of them.
         if (!ok) {
-          umma_commit(&s->teardown[me]);
-          mbar_wait_bounded(&s->teardown[me], 0, 20000000ull);
+          umma_commit(&s->teardown);
+          mbar_wait_bounded(&s->teardown, 0, 20000000ull);
         }
       }
-    }
-  } else if (warp >= kPromoWarps) {
-    // =============================== epilogue warps ===================================
-    const int ew = warp - kPromoWarps;
-    int cur_e = 0;
-    uint32_t tile_iter = 0;
-    for (int T = first_tile; T < total_tiles; T += num_ctas, ++tile_iter) {
-      const TileCoord c = decode_tile(s, T, cur_e);
-      int my_pair = 0;  // down: destination (flat pair id) of the lane-th row this warp handles
-      if (MODE == kModeDown) {
-        const int row = c.m0 + ew + kEpiWarps * lane;
-        // no pair map: the contribution stays at its sorted position (expert-parallel use)
-        if (row < c.m_end)
-          my_pair = p.sorted_pair ? min(max(__ldg(p.sorted_pair + row), 0), p.rows_total - 1) : row;  // in bounds even after bad ids
-      }
-      if (!warp_wait_or_abort(&s->out_full, tile_iter & 1u, s, p)) break;
-      if (MODE == kModeGateUp) {
-        // 8 lanes per row, 4 rows per pass.  Lane `sub` owns h columns [8 sub, 8 sub + 8) and
-        // [64 + 8 sub, 64 + 8 sub + 8) of the row's 128-wide quantization group, so that a
-        // quarter-warp reads 128 contiguous bytes of the staging tile (conflict-free).
-        const int sub = lane & 7, rsel = lane >> 3;
-        const int IB = p.I / BNH;
-#pragma unroll 2
-        for (int i = 0; i < BM / (kEpiWarps * 4); ++i) {
-          const int r0 = (i * kEpiWarps + ew) * 4;
-          if (c.m0 + r0 >= c.m_end) break;  // warp-uniform: rows ascend with i
-          const int rr = r0 + rsel;
-          const int row = c.m0 + rr;
-          const bool live = row < c.m_end;
-          const uint8_t* src = out_tile + rr * kOutPitch + sub * 16;
-          uint4 g[2], u[2];
-          g[0] = *reinterpret_cast<const uint4*>(src);
-          g[1] = *reinterpret_cast<const uint4*>(src + 128);
-          u[0] = *reinterpret_cast<const uint4*>(src + BNH * 2);
-          u[1] = *reinterpret_cast<const uint4*>(src + BNH * 2 + 128);
-          uint32_t hb[8];
-          uint32_t m = 0;
-#pragma unroll
-          for (int t = 0; t < 2; ++t) {
-            const uint32_t gw[4] = {g[t].x, g[t].y, g[t].z, g[t].w};
-            const uint32_t uw[4] = {u[t].x, u[t].y, u[t].z, u[t].w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const float h0 = silu_mul(bf16_bits_to_f32(gw[j] & 0xFFFFu), bf16_bits_to_f32(uw[j] & 0xFFFFu));
-              const float h1 = silu_mul(__uint_as_float(gw[j] & 0xFFFF0000u), __uint_as_float(uw[j] & 0xFFFF0000u));
-              hb[4 * t + j] = bf16x2_bits(h0, h1);
-              m = __vmaxu2(m, hb[4 * t + j] & 0x7FFF7FFFu);  // |bf16| bit patterns: exact, order-free max
-            }
-          }
-          m = max(m & 0xFFFFu, m >> 16);
-#pragma unroll
-          for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-          float inv;
-          const float sc = block_scale(bf16_bits_to_f32(m), &inv);
-          uint32_t cw[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint32_t x0 = hb[2 * j], x1 = hb[2 * j + 1];
-            cw[j] = cvt_e4m3x4(__fmul_rn(bf16_bits_to_f32(x0 & 0xFFFFu), inv), __fmul_rn(__uint_as_float(x0 & 0xFFFF0000u), inv),
-                               __fmul_rn(bf16_bits_to_f32(x1 & 0xFFFFu), inv), __fmul_rn(__uint_as_float(x1 & 0xFFFF0000u), inv));
-          }
-          if (live) {
-            const int col = c.n_tile * BNH + 8 * sub;
-            uint8_t* hc = p.h_codes + static_cast<int64_t>(row) * p.I + col;
-            *reinterpret_cast<uint2*>(hc) = make_uint2(cw[0], cw[1]);
-            *reinterpret_cast<uint2*>(hc + 64) = make_uint2(cw[2], cw[3]);
-            if (sub == 0) p.h_scales[static_cast<int64_t>(row) * IB + c.n_tile] = sc;
-            if (p.h_bf16) {
-              uint16_t* hd = p.h_bf16 + static_cast<int64_t>(row) * p.I + col;
-              *reinterpret_cast<uint4*>(hd) = make_uint4(hb[0], hb[1], hb[2], hb[3]);
-              *reinterpret_cast<uint4*>(hd + 64) = make_uint4(hb[4], hb[5], hb[6], hb[7]);
-            }
-            if (p.out_bf16) {  // debug dump of the bf16 gate_up row
-              uint16_t* gd = p.out_bf16 + static_cast<int64_t>(row) * p.N + col;
-              *reinterpret_cast<uint4*>(gd) = g[0];
-              *reinterpret_cast<uint4*>(gd + 64) = g[1];
-              *reinterpret_cast<uint4*>(gd + p.I) = u[0];
-              *reinterpret_cast<uint4*>(gd + p.I + 64) = u[1];
-            }
-          }
+    } else {
+      // =============================== scale warps ======================================
+      // Two warps, 64 rows each, form the products fl(s_x s_w) of every K-block next to its accumulator: the
+      // slot is free when the accumulator is and published with it (tmem_full counts the MMA and these
+      // warps), so the promotion warps wait for nothing more than before and keep their registers for sums.
+      const int r0 = (warp - kScaleWarp) * 64 + lane;
+      int ks = 0, cur_e = 0;
+      uint32_t acc_phase = 0;
+      const float *x0 = nullptr, *x1 = nullptr, *wl = nullptr, *wh = nullptr;
+      float n0 = 0.f, n1 = 0.f, nl = 0.f, nh = 0.f;  // of the next K-block: its loads fly during this one
+      auto open_tile = [&](int T) {
+        const TileCoord c = decode_tile(s, T, cur_e);
+        int nb_lo, nb_hi;
+        if (MODE == kModeGateUp) {
+          nb_lo = c.n_tile;
+          nb_hi = c.n_tile + p.I / BNH;
+        } else {
+          nb_lo = 2 * c.n_tile;
+          nb_hi = min(2 * c.n_tile + 1, NB - 1);
         }
-      } else {
-        // the tile's 256 columns are contiguous in the output row: 512 bytes per row, 16 per lane
-        const int col = c.n_tile * BN + 8 * lane;
-        const bool col_ok = col < p.N;
-#pragma unroll 4
-        for (int i = 0; i < BM / kEpiWarps; ++i) {
-          const int rr = ew + kEpiWarps * i;
-          const int row = c.m0 + rr;
-          if (row >= c.m_end) break;
-          const uint4 v = *reinterpret_cast<const uint4*>(out_tile + rr * kOutPitch + lane * 16);
-          int64_t out_row = row;
-          if (MODE == kModeDown) out_row = __shfl_sync(0xFFFFFFFFu, my_pair, i);  // lane i holds row i's pair id
-          if (col_ok) *reinterpret_cast<uint4*>(p.out_bf16 + out_row * p.N + col) = v;
+        x0 = p.a_scales + static_cast<int64_t>(min(c.m0 + r0, p.rows_total - 1)) * KB;
+        x1 = p.a_scales + static_cast<int64_t>(min(c.m0 + r0 + 32, p.rows_total - 1)) * KB;
+        wl = p.b_scales + (static_cast<int64_t>(c.e) * NB + nb_lo) * KB;
+        wh = p.b_scales + (static_cast<int64_t>(c.e) * NB + nb_hi) * KB;
+        n0 = __ldg(x0);
+        n1 = __ldg(x1);
+        nl = __ldg(wl);
+        nh = __ldg(wh);
+      };
+      if (first_tile < total_tiles) open_tile(first_tile);
+      bool ok = true;
+      for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
+        for (int kb = 0; kb < KB; ++kb) {
+          const float2 v0 = make_float2(__fmul_rn(n0, nl), __fmul_rn(n0, nh)), v1 = make_float2(__fmul_rn(n1, nl), __fmul_rn(n1, nh));
+          if (kb + 1 < KB) {
+            n0 = __ldg(x0 + kb + 1);
+            n1 = __ldg(x1 + kb + 1);
+            nl = __ldg(wl + kb + 1);
+            nh = __ldg(wh + kb + 1);
+          } else if (T + num_ctas < total_tiles) {
+            open_tile(T + num_ctas);
+          }
+          if (!warp_wait_or_abort(&s->tmem_empty[ks], acc_phase ^ 1, s, p)) { ok = false; break; }
+          s->scale[ks][r0] = v0;
+          s->scale[ks][r0 + 32] = v1;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&s->tmem_full[ks]);
+          if (++ks == kAccBufs) { ks = 0; acc_phase ^= 1; }
         }
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&s->out_empty);
     }
   } else {
     // =============================== promotion warps ==================================
-    const int q = warp & 3;          // TMEM lane quadrant this warp may read
-    const int hs = warp >> 2;        // which 64-column slice of each half tile
-    const int r = q * 32 + lane;     // row within the tile
-    const uint32_t lane_addr = static_cast<uint32_t>(q * 32) << 16;
-    int ks = 0;
-    uint32_t acc_phase = 0;
-    int cur_e = 0;
-    uint32_t tile_iter = 0;
-
-    // scale pointers of a tile for this thread's row: s_x[row, :], s_w[lo block-row, :] and
-    // the offset from the lo to the hi block-row
-    auto scale_ptrs = [&](const TileCoord& c, const float*& sx, const float*& swl, int& hi_off) {
-      const int row_c = min(c.m0 + r, p.rows_total - 1);
-      int nb_lo, nb_hi;
-      if (MODE == kModeGateUp) {
-        nb_lo = c.n_tile;
-        nb_hi = c.n_tile + p.I / BNH;
-      } else {
-        nb_lo = 2 * c.n_tile;
-        nb_hi = min(2 * c.n_tile + 1, NB - 1);
-      }
-      sx = p.a_scales + static_cast<int64_t>(row_c) * KB;
-      swl = p.b_scales + (static_cast<int64_t>(c.e) * NB + nb_lo) * KB;
-      hi_off = (nb_hi - nb_lo) * KB;
-    };
-
-    int T = first_tile;
-    if (T < total_tiles) {
-      TileCoord c = decode_tile(s, T, cur_e);
-      const float *sx_ptr, *sw_lo_ptr;
-      int sw_hi_off;
-      scale_ptrs(c, sx_ptr, sw_lo_ptr, sw_hi_off);
-      float sx_next = __ldg(sx_ptr), swl_next = __ldg(sw_lo_ptr), swh_next = __ldg(sw_lo_ptr + sw_hi_off);
-      bool ok = true;
-      for (;;) {
-        const int row = c.m0 + r;
-        const bool valid = row < c.m_end;
-        // a warp whose 32 rows all lie past the group's end (ragged tails, decode-sized groups)
-        // keeps the barrier protocol going but reads and accumulates nothing
-        const bool warp_live = c.m0 + q * 32 < c.m_end;
-        const int Tn = T + num_ctas;
-        const bool has_next = Tn < total_tiles;
-        TileCoord cn = c;
-        float w = 0.0f;  // down: the pair's combine weight (sorted order), used at the end of the tile
-        if (MODE == kModeDown && valid) w = __ldg(p.pair_weights + row);
-
-        float2 acc_lo[32], acc_hi[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) acc_lo[j] = acc_hi[j] = make_float2(0.0f, 0.0f);
-
-        for (int kb = 0; kb < KB; ++kb) {
-          const float sc_lo = __fmul_rn(sx_next, swl_next);
-          const float sc_hi = __fmul_rn(sx_next, swh_next);
-          if (kb + 1 < KB) {
-            sx_next = __ldg(sx_ptr + kb + 1);
-            swl_next = __ldg(sw_lo_ptr + kb + 1);
-            swh_next = __ldg(sw_lo_ptr + sw_hi_off + kb + 1);
-          } else if (has_next) {  // first scales of the next tile: their latency hides behind this block
-            cn = decode_tile(s, Tn, cur_e);
-            scale_ptrs(cn, sx_ptr, sw_lo_ptr, sw_hi_off);
-            sx_next = __ldg(sx_ptr);
-            swl_next = __ldg(sw_lo_ptr);
-            swh_next = __ldg(sw_lo_ptr + sw_hi_off);
-          }
-          if (!warp_wait_or_abort(&s->tmem_full[ks], acc_phase, s, p)) { ok = false; break; }
-          tc_fence_after_sync();
-          if (!warp_live) {
-            tc_fence_before_sync();
-            if (lane == 0) mbar_arrive(&s->tmem_empty[ks]);
-          } else {
-            const uint32_t t0 = tmem_base + lane_addr + static_cast<uint32_t>(ks * BN + hs * kSliceCols);
-            // 16-column chunks, double-buffered: the load of chunk c+1 is in flight while chunk c
-            // is accumulated; small enough that nothing spills under the register budget.
-            uint32_t va[16], vb[16];
-            tmem_ld_x16(t0, va);
-            tmem_ld_wait();
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              const uint32_t next = (c < 3) ? t0 + 16 * (c + 1) : t0 + BNH;
-              if (c & 1) { tmem_ld_x16(next, va); promote16(acc_lo + 8 * c, vb, sc_lo); }
-              else       { tmem_ld_x16(next, vb); promote16(acc_lo + 8 * c, va, sc_lo); }
-              tmem_ld_wait();
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              if (c < 3) {
-                if (c & 1) tmem_ld_x16(t0 + BNH + 16 * (c + 1), va);
-                else       tmem_ld_x16(t0 + BNH + 16 * (c + 1), vb);
-              }
-              if (c & 1) promote16(acc_hi + 8 * c, vb, sc_hi);
-              else       promote16(acc_hi + 8 * c, va, sc_hi);
-              if (c < 3) tmem_ld_wait();
-              if (c == 2) {
-                // (the last chunk is in registers after this wait): this warp's reads of the
-                // accumulator are done, hand it back to the MMA warp
-                tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&s->tmem_empty[ks]);
-              }
-            }
-          }
-          if (++ks == kAccBufs) { ks = 0; acc_phase ^= 1; }
-        }
-        if (!ok) break;
-
-        // ---- hand the tile to the epilogue warps as bf16 -----------------------------------
-        if ((MODE == kModeLinear || MODE == kModeDown) && p.out_f32 && valid) {  // debug fp32 dump
-          const int col_lo = c.n_tile * BN + hs * kSliceCols;
-          const int col_hi = col_lo + BNH;
-          float2* d_lo = reinterpret_cast<float2*>(p.out_f32 + static_cast<int64_t>(row) * p.N + col_lo);
-          float2* d_hi = reinterpret_cast<float2*>(p.out_f32 + static_cast<int64_t>(row) * p.N + col_hi);
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            d_lo[j] = acc_lo[j];
-            if (col_hi < p.N) d_hi[j] = acc_hi[j];
-          }
-        }
-        if (MODE == kModeDown) {  // contribution = bf16( fl(w * y) )
-          const float2 w2 = make_float2(w, w);
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            acc_lo[j] = __fmul2_rn(w2, acc_lo[j]);
-            acc_hi[j] = __fmul2_rn(w2, acc_hi[j]);
-          }
-        }
-        if (!warp_wait_or_abort(&s->out_empty, (tile_iter & 1u) ^ 1u, s, p)) break;  // previous tile drained
-        if (warp_live) {
-          uint4* d_lo = reinterpret_cast<uint4*>(out_tile + r * kOutPitch + hs * (kSliceCols * 2));
-          uint4* d_hi = reinterpret_cast<uint4*>(out_tile + r * kOutPitch + BNH * 2 + hs * (kSliceCols * 2));
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            d_lo[j] = make_uint4(bf16x2_bits(acc_lo[4 * j].x, acc_lo[4 * j].y), bf16x2_bits(acc_lo[4 * j + 1].x, acc_lo[4 * j + 1].y),
-                                 bf16x2_bits(acc_lo[4 * j + 2].x, acc_lo[4 * j + 2].y), bf16x2_bits(acc_lo[4 * j + 3].x, acc_lo[4 * j + 3].y));
-            d_hi[j] = make_uint4(bf16x2_bits(acc_hi[4 * j].x, acc_hi[4 * j].y), bf16x2_bits(acc_hi[4 * j + 1].x, acc_hi[4 * j + 1].y),
-                                 bf16x2_bits(acc_hi[4 * j + 2].x, acc_hi[4 * j + 2].y), bf16x2_bits(acc_hi[4 * j + 3].x, acc_hi[4 * j + 3].y));
-          }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&s->out_full);
-        if (!has_next) break;
-        T = Tn;
-        c = cn;
-        ++tile_iter;
-      }
-    }
+    setmaxnreg_inc<kPromoRegs>();
+    promotion_role<MODE, SAVE>(tm_o, p, smem, s, first_tile, num_ctas, total_tiles);
   }
 
   // ---- teardown ---------------------------------------------------------------------------
@@ -630,6 +689,17 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
 
 namespace {
 
+// Output bf16 [rows, cols]: box of 64 columns x 32 rows, 128-byte swizzle.
+CUresult make_out_tmap(EncodeTiledFn encode, CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols) {
+  const cuuint64_t dims[2] = {cols, rows};
+  const cuuint64_t strides[1] = {cols * 2};
+  const cuuint32_t box[2] = {64, 32};
+  const cuuint32_t estr[2] = {1, 1};
+  return encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
+
 CUresult make_tmap(EncodeTiledFn encode, CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols) {
   // u8 tensor [rows, cols] row-major; box = 128 bytes x 128 rows, 128-byte swizzle, zero fill.
   const cuuint64_t dims[2] = {cols, rows};
@@ -641,21 +711,21 @@ CUresult make_tmap(EncodeTiledFn encode, CUtensorMap* m, const void* base, uint6
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
-template <int MODE>
-cudaError_t launch_mode(const Launch& L, const CUtensorMap& ta, const CUtensorMap& tb, const GemmParams& p,
-                        int grid) {
+template <int MODE, bool SAVE>
+cudaError_t launch_mode(const Launch& L, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to,
+                        const GemmParams& p, int grid) {
   // sticky per function and device; atomic: contexts on several host threads may launch at once (both
   // would set the same value)
   static std::atomic<bool> attr_set_dev[64];
   std::atomic<bool>& attr_set = attr_set_dev[L.device & 63];
   if (!attr_set.load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_blockscaled_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kSmemBytes));
+    cudaError_t e = cudaFuncSetAttribute(gemm_blockscaled_kernel<MODE, SAVE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(kSmemBytes<MODE, SAVE>));
     if (e != cudaSuccess) return e;
     attr_set.store(true, std::memory_order_release);
   }
   ++*L.launches;
-  return launch_pdl(gemm_blockscaled_kernel<MODE>, static_cast<unsigned>(grid), kThreads, kSmemBytes, L.stream, ta, tb, p);
+  return launch_pdl(gemm_blockscaled_kernel<MODE, SAVE>, static_cast<unsigned>(grid), kThreads, kSmemBytes<MODE, SAVE>, L.stream, ta, tb, to, p);
 }
 
 }  // namespace
@@ -666,10 +736,12 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
   // decode-sized groups: the swapped-operand kernel (bitwise the same rows, bound by the weight stream)
   if (L.gemm_path == 2 ? ((a.offsets != nullptr || a.E == 1) && a.K / BK <= 64) : (L.gemm_path == 0 && gemm_decode_applies(a)))
     return launch_gemm_decode(L, encode, a, cu_err);
-  CUtensorMap ta, tb;
+  CUtensorMap ta, tb, to{};
   CUresult r = make_tmap(encode, &ta, a.a_codes, static_cast<uint64_t>(a.rows_total), static_cast<uint64_t>(a.K));
   if (r == CUDA_SUCCESS)
     r = make_tmap(encode, &tb, a.b_codes, static_cast<uint64_t>(a.E * a.N), static_cast<uint64_t>(a.K));
+  if (r == CUDA_SUCCESS && a.out_bf16 != nullptr)
+    r = make_out_tmap(encode, &to, a.out_bf16, static_cast<uint64_t>(a.rows_total), static_cast<uint64_t>(a.N));
   if (r != CUDA_SUCCESS) {
     *cu_err = r;
     return cudaErrorUnknown;
@@ -689,7 +761,7 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
   p.h_codes = a.h_codes;
   p.h_scales = a.h_scales;
   p.h_bf16 = a.h_bf16;
-  p.sorted_pair = a.sorted_pair;
+  p.h_vec32 = (reinterpret_cast<uintptr_t>(a.h_bf16) & 31u) == 0;
   p.pair_weights = a.pair_weights;
   p.status = L.d_status;
   p.wait_limit_ns = L.wait_limit_ns ? L.wait_limit_ns : 2000000000ull;
@@ -705,9 +777,11 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
   const int64_t m_tiles_max = a.rows_total / BM + a.E;
   const int grid = static_cast<int>(std::min<int64_t>(L.sm_count, m_tiles_max * p.n_tiles));
   switch (a.mode) {
-    case kModeLinear: return launch_mode<kModeLinear>(L, ta, tb, p, grid);
-    case kModeGateUp: return launch_mode<kModeGateUp>(L, ta, tb, p, grid);
-    case kModeDown: return launch_mode<kModeDown>(L, ta, tb, p, grid);
+    case kModeLinear: return launch_mode<kModeLinear, false>(L, ta, tb, to, p, grid);
+    case kModeGateUp:
+      return a.out_bf16 || a.h_bf16 ? launch_mode<kModeGateUp, true>(L, ta, tb, to, p, grid)
+                                    : launch_mode<kModeGateUp, false>(L, ta, tb, to, p, grid);
+    case kModeDown: return launch_mode<kModeDown, false>(L, ta, tb, to, p, grid);
   }
   return cudaErrorInvalidValue;
 }
