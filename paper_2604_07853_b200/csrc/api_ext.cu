@@ -484,7 +484,7 @@ int qarl_moe_bwd(qarl_ctx* ctx, const void* x, const int32_t* ids, const float* 
   if ((e = launch_swiglu_bwd(L, static_cast<const uint16_t*>(gate_up), dh, P, I, dgu)) != cudaSuccess)
     return cuda_fail(ctx, e, "swiglu_bwd");
   mark(ctx, L.stream, QARL_STAGE_BWD_ELEMENTWISE);
-  {  // dXs = dGU . W13_e, stored by flat pair id for the combine
+  {  // dXs = dGU . W13_e, left in sorted order (dense row blocks); the combine finds a token's rows by position
     GemmBf16Args a{};
     a.group = 1;
     a.a = dgu;
@@ -495,7 +495,6 @@ int qarl_moe_bwd(qarl_ctx* ctx, const void* x, const int32_t* ids, const float* 
     a.Kc = 2 * I;
     a.E = E;
     a.offsets = pb.offsets;
-    a.out_rows = pb.sorted_pair;
     a.c_bf16 = dxs;
     if ((rc = gemm(a, "moe_bwd dXs", QARL_STAGE_BWD_DX)) != QARL_OK) return rc;
   }
@@ -514,7 +513,7 @@ int qarl_moe_bwd(qarl_ctx* ctx, const void* x, const int32_t* ids, const float* 
     a.c_f32 = dw13;
     if ((rc = gemm(a, "moe_bwd dW13", QARL_STAGE_BWD_DW)) != QARL_OK) return rc;
   }
-  if ((e = launch_combine(L, dxs, ids, M, k, H, E, static_cast<uint16_t*>(dx))) != cudaSuccess)
+  if ((e = launch_combine(L, dxs, ids, M, k, H, E, static_cast<uint16_t*>(dx), pb.pos_of_pair)) != cudaSuccess)
     return cuda_fail(ctx, e, "combine");
   mark(ctx, L.stream, QARL_STAGE_COMBINE);
   return QARL_OK;

@@ -239,7 +239,6 @@ struct GemmBf16Args {
   const int32_t* offsets = nullptr;  // [E + 1], device
   int64_t E = 1;
   int64_t rows_total = 0;
-  const int32_t* out_rows = nullptr;  // group = 1: C row of sorted row p is out_rows[p] (e.g. the flat pair id)
 };
 cudaError_t launch_gemm_bf16(const Launch& L, EncodeTiledFn encode, const GemmBf16Args& a, CUresult* cu_err);
 

@@ -22,11 +22,14 @@
 //                        with zeros (generic stores + proxy fence) before it issues the step, so
 //                        they contribute nothing whatever B holds there.
 //
-// Tile 128 x 256 x 64.  TMA stages both operands with the 128-byte swizzle (a K-major tile is
+// Tile 128 x 256 x 64 (or 256 x 256, 128 x 192: see the host).  TMA stages both operands with the 128-byte swizzle (a K-major tile is
 // one box of R rows x 128 bytes; an MN-major tile is one box of 64 c-rows x 128 bytes per 64
 // output indices); one thread issues 4 x tcgen05.mma kind::f16 (128 x 256 x 16) per stage with
 // the matching operand-major bits; two 256-column TMEM accumulators let the epilogue of a tile
-// overlap the main loop of the next.  Static persistent schedule, row tiles fastest.  One fixed
+// overlap the main loop of the next.  The epilogue writes through shared-memory boxes of 32 rows x 128 bytes and
+// TMA stores: rows stored straight from registers (16 bytes of 32 different rows per instruction, half
+// sectors) took four times as long as the MMAs of a short contraction -- expert dW of 8192 tokens (128 experts,
+// 1536 x 2048, 1.6 GB out) 1010 us of which the stores need 250.  Static persistent schedule, row tiles fastest.  One fixed
 // order of accumulation: a result does not depend on the grid or on the other rows.
 // Every wait is bounded (status word + CTA-wide abort flag), as in the other GEMMs.
 #include <algorithm>
@@ -41,32 +44,35 @@ namespace {
 
 using namespace ptx;
 
-constexpr int BM = 128, BN = 256, BK = 64;
-constexpr int kMaxStages = 4, kMaxAccBufs = 2;
+constexpr int BM = 128, BK = 64;
+constexpr int kMaxStages = 5, kMaxAccBufs = 2;
 constexpr int kEpiWarps = 4;   // warps 0-3 (TMEM quadrant = warp index)
 constexpr int kTmaWarp = 4;
 constexpr int kMmaWarp = 5;
 constexpr int kThreads = 6 * 32;
 constexpr uint32_t kAHalfBytes = BM * BK * 2;   // 16 KB: 128 output rows x 64 contraction elements
-constexpr uint32_t kBBytes = BN * BK * 2;   // 32 KB
+// an epilogue warp's rows on their way out: boxes of 32 rows x 128 bytes (128-byte swizzle)
+constexpr uint32_t kOutBoxBytes = 32 * 128;
 // A tile holds MT x 128 output rows.  The kernel is bound by the bytes it can keep in flight from
 // L2/HBM (shared-memory capacity over load latency: throughput grew linearly with the ring depth),
 // so MT = 2 -- both 128-row halves share one B tile, a third fewer bytes per flop -- is the default;
 // it leaves one set of accumulators, i.e. an epilogue that is not overlapped, which only pays when
 // the contraction is long enough (MT = 1 for the ragged contraction of the grouped dW).
-template <int MT>
+enum { kDense = 0, kGroupedRows = 1, kGroupedContraction = 2 };
+template <int GROUP, int MT, int BN>
 struct Cfg {
   static constexpr int kRows = MT * BM;
   static constexpr uint32_t kABytes = MT * kAHalfBytes;
+  static constexpr uint32_t kBBytes = BN * BK * 2;
   static constexpr uint32_t kStageBytes = kABytes + kBBytes;
-  static constexpr int kStages = MT == 1 ? 4 : 3;
+  static constexpr int kStages = MT == 2 ? 3 : BN == 192 ? 5 : 4;
   static constexpr int kAccBufs = MT == 1 ? 2 : 1;
+  static constexpr int kBoxes = GROUP == kGroupedRows || BN == 192 ? 1 : 2;  // per epilogue warp, as the shared memory allows
+  static constexpr uint32_t kOutBytes = kEpiWarps * kBoxes * kOutBoxBytes;
 };
 constexpr uint32_t kBlockBytes = 64 * BK * 2;  // one MN-major block: 64 output indices x 64 c-rows
 constexpr uint32_t kTmemCols = 512;
 constexpr int kMaxExperts = 1024;
-enum { kDense = 0, kGroupedRows = 1, kGroupedContraction = 2 };
-
 struct Bf16Params {
   int Mo, No, Kc;           // grouped rows: Mo = total rows P;  grouped contraction: Kc unused (from offsets)
   const int32_t* offsets;   // [E + 1] (grouped forms)
@@ -74,7 +80,6 @@ struct Bf16Params {
   int rows_total;           // grouped contraction: P
   int a3d, b3d;             // MN-major operand staged by one 3-D TMA box (64 columns x 64 rows x blocks)
   int col_fastest;          // dense: consecutive tiles walk the column tiles of a row tile (else the row tiles of a column tile)
-  const int32_t* out_rows;  // grouped rows: output row of each sorted row (nullptr: the row itself)
   uint16_t* c_bf16;   // [Mo, No] or nullptr
   float* c_f32;       // [Mo, No] or nullptr
   int* status;
@@ -89,12 +94,20 @@ struct __align__(8) SmemTail {
   uint64_t teardown;
   uint32_t tmem_addr;
   int abort_flag;
+};
+struct SmemLists {  // grouped rows: the tile list
   int32_t off[kMaxExperts + 1];
   int32_t prefix[kMaxExperts + 1];
 };
-template <int MT>
-constexpr size_t smem_bytes() { return 1024 + static_cast<size_t>(Cfg<MT>::kStages) * Cfg<MT>::kStageBytes + sizeof(SmemTail); }
-static_assert(smem_bytes<1>() <= 227 * 1024 && smem_bytes<2>() <= 227 * 1024, "shared memory budget");
+template <int GROUP, int MT, int BN>
+constexpr size_t smem_bytes() {
+  using C = Cfg<GROUP, MT, BN>;
+  return 1024 + static_cast<size_t>(C::kStages) * C::kStageBytes + C::kOutBytes + sizeof(SmemTail) +
+         (GROUP == kGroupedRows ? sizeof(SmemLists) : 0);
+}
+static_assert(smem_bytes<kDense, 1, 256>() <= 227 * 1024 && smem_bytes<kDense, 1, 192>() <= 227 * 1024 &&
+                  smem_bytes<kDense, 2, 256>() <= 227 * 1024 && smem_bytes<kGroupedRows, 1, 256>() <= 227 * 1024,
+              "shared memory budget");
 
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, SmemTail* s, const Bf16Params& p) {
   if (mbar_try_wait(bar, parity)) return true;
@@ -124,16 +137,19 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&b);
 }
 
-template <bool A_MN, bool B_MN, int GROUP, int MT>
+template <bool A_MN, bool B_MN, int GROUP, int MT, int BN>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
+                 const __grid_constant__ CUtensorMap tm_f32, const __grid_constant__ CUtensorMap tm_bf16,
                  const Bf16Params p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  using C = Cfg<MT>;
+  using C = Cfg<GROUP, MT, BN>;
   constexpr int kStages = C::kStages, kAccBufs = C::kAccBufs, TM = C::kRows;
   constexpr uint32_t kABytes = C::kABytes, kStageBytes = C::kStageBytes;
-  SmemTail* s = reinterpret_cast<SmemTail*>(smem + static_cast<size_t>(kStages) * kStageBytes);
+  uint8_t* out_boxes = smem + static_cast<size_t>(kStages) * kStageBytes;
+  SmemTail* s = reinterpret_cast<SmemTail*>(out_boxes + C::kOutBytes);
+  SmemLists* lists = reinterpret_cast<SmemLists*>(s + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   pdl_trigger();
@@ -162,28 +178,39 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   const int n_tiles = (p.No + BN - 1) / BN;
   const int m_tiles = GROUP == kGroupedRows ? 1 : (p.Mo + TM - 1) / TM;  // grouped rows: tiles come from the offsets
   if (GROUP == kGroupedRows) {
-    build_tile_list(s->off, s->prefix, p.offsets, p.Mo, p.E, TM, n_tiles);
-  } else if (GROUP == kGroupedContraction) {
-    for (int e = threadIdx.x; e <= p.E; e += kThreads) s->off[e] = min(max(p.offsets[e], 0), p.rows_total);
+    build_tile_list(lists->off, lists->prefix, p.offsets, p.Mo, p.E, TM, n_tiles);
   }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = s->tmem_addr;
-  const int total_tiles = GROUP == kGroupedRows ? s->prefix[p.E]
+  const int total_tiles = GROUP == kGroupedRows ? lists->prefix[p.E]
                         : GROUP == kGroupedContraction ? p.E * m_tiles * n_tiles : m_tiles * n_tiles;
   const int grid = gridDim.x;
 
   // Everything a role needs to know about tile T.  i0 / j0: first output row / column; a_c0 / b_c0:
   // first contraction coordinate of A / B; KS: 64-element contraction steps; last_valid: contraction
   // elements of the last step that belong to this tile (64 = all); row_end: end of the rows that
-  // may be stored; c_off: element offset of this tile's output matrix.
+  // may be stored.
   struct Tile {
     int i0, j0, a_c0, b_c0, KS, last_valid, row_end;
-    int64_t c_off;
+    int e;       // grouped contraction: whose output matrix
     int b_row0;  // K-major B: first row of the expert's block
   };
-  auto tile_of = [&](int T, int& cur_e) {
+  // `cur`: where the caller's walk over the list stands; for the grouped contraction the caller's next pair
+  // of group boundaries, loaded one tile ahead.
+  struct Walk {
+    int cur_e = 0;
+    int lo = 0, hi = 0;
+  };
+  auto bounds_of = [&](int T, Walk& w) {
+    if (GROUP == kGroupedContraction && T < total_tiles) {
+      const int e = T / (m_tiles * n_tiles);
+      w.lo = __ldg(p.offsets + e);
+      w.hi = __ldg(p.offsets + e + 1);
+    }
+  };
+  auto tile_of = [&](int T, Walk& w) {
     Tile t{};
     t.last_valid = BK;
     if (GROUP == kDense) {
@@ -201,7 +228,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       t.KS = (p.Kc + BK - 1) / BK;  // a ragged last step reads zeros (TMA out-of-range fill)
       t.row_end = p.Mo;
     } else if (GROUP == kGroupedRows) {
-      const TileCoord c = decode_tile(s->off, s->prefix, TM, T, cur_e);
+      const TileCoord c = decode_tile(lists->off, lists->prefix, TM, T, w.cur_e);
       t.i0 = c.m0;
       t.j0 = c.n_tile * BN;
       t.KS = p.Kc / BK;             // Kc is a multiple of 64 here: a step never runs into the next expert's weights
@@ -214,12 +241,14 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       const int e = T / per_e, r = T % per_e;
       t.i0 = (r % m_tiles) * TM;
       t.j0 = (r / m_tiles) * BN;
-      const int rows = s->off[e + 1] - s->off[e];
+      const int first = min(max(w.lo, 0), p.rows_total);
+      const int rows = max(min(max(w.hi, 0), p.rows_total) - first, 0);
+      bounds_of(T + grid, w);
       t.KS = (rows + BK - 1) / BK;
       t.last_valid = rows - (t.KS - 1) * BK;
-      t.a_c0 = t.b_c0 = s->off[e];
+      t.a_c0 = t.b_c0 = first;
       t.row_end = p.Mo;
-      t.c_off = static_cast<int64_t>(e) * p.Mo * p.No;
+      t.e = e;
     }
     return t;
   };
@@ -230,9 +259,10 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       uint32_t phase = 0;
       uint32_t armed = 0, armed_parity = 0;
       bool ok = true;
-      int cur_e = 0;
+      Walk walk;
+      bounds_of(blockIdx.x, walk);
       for (int T = blockIdx.x; ok && T < total_tiles; T += grid) {
-        const Tile t = tile_of(T, cur_e);
+        const Tile t = tile_of(T, walk);
         const int i0 = t.i0, j0 = t.j0;
         for (int ks = 0; ks < t.KS; ++ks) {
           if (!wait_or_abort(&s->empty[stage], phase ^ 1, s, p)) { ok = false; break; }
@@ -274,7 +304,8 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     int stage = 0, acc = 0;
     uint32_t phase = 0, acc_phase = 0;
     bool ok = true;
-    int cur_e = 0;
+    Walk walk;
+    bounds_of(blockIdx.x, walk);
     auto issue = [&](uint32_t d_tmem, int stage, bool first, bool last, int acc) {
       tc_fence_after_sync();
       const uint32_t a_addr = smem_u32(smem + static_cast<size_t>(stage) * kStageBytes);
@@ -295,7 +326,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       if (last) umma_commit(&s->tmem_full[acc]);
     };
     for (int T = blockIdx.x; ok && T < total_tiles; T += grid) {
-      const Tile t = tile_of(T, cur_e);
+      const Tile t = tile_of(T, walk);
       if (t.KS == 0) continue;  // an expert without rows: the epilogue writes zeros, no accumulator is used
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * MT) * BN;
       const bool ragged = GROUP == kGroupedContraction && t.last_valid < BK;
@@ -340,64 +371,99 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       mbar_wait_bounded(&s->teardown, 0, 20000000ull);
     }
   } else if (warp < kEpiWarps) {
-    const int r = warp * 32 + lane;
+    // =============================== epilogue warps: TMEM -> box -> TMA store ==========
     const uint32_t lane_addr = static_cast<uint32_t>(warp * 32) << 16;
-    int acc = 0;
+    uint8_t* my_boxes = out_boxes + static_cast<size_t>(warp) * C::kBoxes * kOutBoxBytes;
+    int acc = 0, box = 0;
     uint32_t acc_phase = 0;
-    int cur_e = 0;
+    Walk walk;
+    bounds_of(blockIdx.x, walk);
     for (int T = blockIdx.x; T < total_tiles; T += grid) {
-      const Tile t = tile_of(T, cur_e);
-      const int j0 = t.j0;
-      const bool have_acc = t.KS > 0;
+      const Tile t = tile_of(T, walk);
+      const bool have_acc = t.KS > 0;  // an expert without rows gets zeros
       if (have_acc) {
         if (!warp_wait_or_abort(&s->tmem_full[acc], acc_phase, s, p)) break;
         tc_fence_after_sync();
       }
 #pragma unroll 1
       for (int mt = 0; mt < MT; ++mt) {
-      const int i0 = t.i0 + mt * BM;
-      const int row = i0 + r;
-      const bool valid = row < t.row_end;
-      const bool warp_live = i0 + warp * 32 < t.row_end;
-      const uint32_t t0 = tmem_base + lane_addr + static_cast<uint32_t>((acc * MT + mt) * BN);
-      if (warp_live) {
-#pragma unroll 1
-        for (int ch = 0; ch < BN / 16; ++ch) {
-          const int col = j0 + 16 * ch;
-          if (col >= p.No) break;
-          uint32_t v[16];
+        const int row0 = t.i0 + mt * BM + warp * 32;
+        if (row0 >= t.row_end) continue;
+        const uint32_t t0 = tmem_base + lane_addr + static_cast<uint32_t>((acc * MT + mt) * BN);
+        // rows past a group's end are the next expert's: then the box is copied row by row
+        const bool whole = GROUP != kGroupedRows || row0 + 32 <= t.row_end;
+        auto columns = [&](int col, uint32_t (&v)[32]) {
           if (have_acc) {
-            tmem_ld_x16(t0 + 16 * ch, v);
+            tmem_ld_x32(t0 + col, v);
             tmem_ld_wait();
           } else {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = 0u;
+            for (int j = 0; j < 32; ++j) v[j] = 0u;
           }
-          if (valid) {
-            const bool whole = col + 16 <= p.No;  // No is a multiple of 8: a ragged last chunk holds 8 columns
-            int64_t orow = row;
-            if (GROUP == kGroupedRows && p.out_rows) orow = min(max(__ldg(p.out_rows + row), 0), p.Mo - 1);
-            const int64_t at = t.c_off + orow * p.No + col;
-            if (p.c_f32) {
-              float4* fd = reinterpret_cast<float4*>(p.c_f32 + at);
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                if (j < 2 || whole)
-                  fd[j] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                                      __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
+        };
+        // the next box of this warp, once TMA has read what it held
+        auto next_box = [&]() {
+          if (lane == 0) {
+            if (C::kBoxes == 2) bulk_wait_group_read_1();
+            else bulk_wait_group_read_all();
+          }
+          __syncwarp();
+          uint8_t* b = my_boxes + (C::kBoxes == 2 ? box : 0) * kOutBoxBytes;
+          box ^= 1;
+          return b;
+        };
+        auto put = [&](uint8_t* b, int j, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
+          *reinterpret_cast<uint4*>(b + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_uint4(w0, w1, w2, w3);
+        };
+        // box of 32 rows x 128 bytes at output column `col` (element size `es`)
+        auto send = [&](uint8_t* b, const CUtensorMap* m, void* base, int col, int es) {
+          if (whole) {
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+              tma_store_3d(m, b, col, row0, GROUP == kGroupedContraction ? t.e : 0);
+              bulk_commit_group();
             }
-            if (p.c_bf16) {
-              uint32_t ob[8];
-#pragma unroll
-              for (int j = 0; j < 8; ++j) ob[j] = bf16x2_bits(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
-              uint4* od = reinterpret_cast<uint4*>(p.c_bf16 + at);
-              od[0] = make_uint4(ob[0], ob[1], ob[2], ob[3]);
-              if (whole) od[1] = make_uint4(ob[4], ob[5], ob[6], ob[7]);
+          } else {
+            __syncwarp();
+            const int chunk = lane & 7, c = col + chunk * (16 / es);
+            for (int rr = lane >> 3; row0 + rr < t.row_end; rr += 4) {
+              const uint4 v = *reinterpret_cast<const uint4*>(b + rr * 128 + ((chunk ^ (rr & 7)) << 4));
+              if (c < p.No)
+                *reinterpret_cast<uint4*>(static_cast<uint8_t*>(base) + (static_cast<int64_t>(row0 + rr) * p.No + c) * es) = v;
             }
+            __syncwarp();
+          }
+        };
+        if (p.c_f32) {
+#pragma unroll 2
+          for (int c = 0; c < BN && t.j0 + c < p.No; c += 32) {
+            uint32_t v[32];
+            columns(c, v);
+            uint8_t* b = next_box();
+#pragma unroll
+            for (int j = 0; j < 8; ++j) put(b, j, v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+            send(b, &tm_f32, p.c_f32, t.j0 + c, 4);
+          }
+        }
+        if (p.c_bf16) {
+#pragma unroll 2
+          for (int c = 0; c < BN && t.j0 + c < p.No; c += 64) {
+            uint32_t w[32];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              uint32_t v[32];
+              columns(c + 32 * h, v);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) w[16 * h + j] = bf16x2_bits(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+            }
+            uint8_t* b = next_box();
+#pragma unroll
+            for (int j = 0; j < 8; ++j) put(b, j, w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+            send(b, &tm_bf16, p.c_bf16, t.j0 + c, 2);
           }
         }
       }
-      }  // mt
       if (have_acc) {
         tc_fence_before_sync();
         __syncwarp();
@@ -405,6 +471,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
         if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1; }
       }
     }
+    if (lane == 0) bulk_wait_group_all();  // this warp's rows are written
   }
 
   tc_fence_before_sync();
@@ -441,16 +508,30 @@ CUresult make_tmap_mn3d(EncodeTiledFn encode, CUtensorMap* m, const void* base, 
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
-template <bool A_MN, bool B_MN, int GROUP, int MT>
-cudaError_t launch_variant(const Launch& L, const CUtensorMap& ta, const CUtensorMap& tb, const Bf16Params& p,
-                           int64_t tiles) {
+// Output matrices [count][rows, cols] of elements of `es` bytes: box of 128 bytes x 32 rows, 128-byte swizzle.
+CUresult make_out_tmap(EncodeTiledFn encode, CUtensorMap* m, const void* base, uint64_t count, uint64_t rows, uint64_t cols, uint32_t es) {
+  const cuuint64_t dims[3] = {cols, rows, count};
+  const cuuint64_t strides[2] = {cols * es, rows * cols * es};
+  const cuuint32_t box[3] = {128 / es, 32, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return encode(m, es == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims,
+                strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
+
+struct Maps {
+  CUtensorMap a, b, f32, bf16;
+};
+
+template <bool A_MN, bool B_MN, int GROUP, int MT, int BN>
+cudaError_t launch_variant(const Launch& L, const Maps& tm, const Bf16Params& p, int64_t tiles) {
   // sticky per function and device; atomic: contexts on several host threads may launch at once (both
   // would set the same value)
   static std::atomic<bool> attr_set_dev[64];
   std::atomic<bool>& attr_set = attr_set_dev[L.device & 63];
   if (!attr_set.load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_bf16_kernel<A_MN, B_MN, GROUP, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem_bytes<MT>()));
+    cudaError_t e = cudaFuncSetAttribute(gemm_bf16_kernel<A_MN, B_MN, GROUP, MT, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(smem_bytes<GROUP, MT, BN>()));
     if (e != cudaSuccess) return e;
     attr_set.store(true, std::memory_order_release);
   }
@@ -459,7 +540,17 @@ cudaError_t launch_variant(const Launch& L, const CUtensorMap& ta, const CUtenso
   const int64_t rounds = std::max<int64_t>(1, (tiles + L.sm_count - 1) / L.sm_count);
   const int grid = static_cast<int>(std::max<int64_t>(1, (tiles + rounds - 1) / rounds));
   ++*L.launches;
-  return launch_pdl(gemm_bf16_kernel<A_MN, B_MN, GROUP, MT>, static_cast<unsigned>(grid), kThreads, smem_bytes<MT>(), L.stream, ta, tb, p);
+  return launch_pdl(gemm_bf16_kernel<A_MN, B_MN, GROUP, MT, BN>, static_cast<unsigned>(grid), kThreads, smem_bytes<GROUP, MT, BN>(), L.stream,
+                    tm.a, tm.b, tm.f32, tm.bf16, p);
+}
+
+template <int GROUP, int MT, int BN>
+cudaError_t launch_majors(const Launch& L, const Maps& tm, const Bf16Params& p, int64_t tiles, bool a_mn, bool b_mn) {
+  if constexpr (GROUP == kGroupedContraction) return launch_variant<true, true, GROUP, MT, BN>(L, tm, p, tiles);
+  if constexpr (GROUP != kGroupedRows)  // (grouped rows: A is K-major)
+    if (a_mn)
+      return b_mn ? launch_variant<true, true, GROUP, MT, BN>(L, tm, p, tiles) : launch_variant<true, false, GROUP, MT, BN>(L, tm, p, tiles);
+  return b_mn ? launch_variant<false, true, GROUP, MT, BN>(L, tm, p, tiles) : launch_variant<false, false, GROUP, MT, BN>(L, tm, p, tiles);
 }
 
 }  // namespace
@@ -468,29 +559,35 @@ cudaError_t launch_gemm_bf16(const Launch& L, EncodeTiledFn encode, const GemmBf
   *cu_err = CUDA_SUCCESS;
   if (a.Mo == 0 || a.No == 0) return cudaSuccess;
   const bool grouped_rows = a.group == 1, grouped_k = a.group == 2;
-  // 256-row tiles pay (measured: 13 % less time per unit of work) when the tile count still fills the
-  // SMs' rounds; the grouped forms keep 128-row tiles (ragged groups waste more of a 256-row tile and
-  // the single accumulator set exposes the epilogue of short tiles).
-  int MT = 1;
-  if (a.group == 0 && a.Mo > BM) {
-    const int64_t n_t = (a.No + BN - 1) / BN;
-    const int64_t t1 = (a.Mo + BM - 1) / BM * n_t, t2 = (a.Mo + 2 * BM - 1) / (2 * BM) * n_t;
-    const double cost1 = static_cast<double>((t1 + L.sm_count - 1) / L.sm_count);
-    const double cost2 = static_cast<double>((t2 + L.sm_count - 1) / L.sm_count) * 2.0 * 0.87;
-    if (cost2 < cost1) MT = 2;
+  // Tile of the dense form: the one whose full rounds over the SMs cost least.  A round of 128 x 256 tiles is the
+  // unit; 256 x 256 tiles move a third fewer operand bytes (measured: 13 % less time per unit of work), 128 x 192
+  // tiles cost in proportion.  The grouped forms keep 128 x 256 (ragged groups waste more of a 256-row tile
+  // and its single accumulator set exposes the epilogue of short contractions).
+  int MT = 1, BN = 256;
+  if (a.group == 0) {
+    auto cost = [&](int rows, int cols, double unit) {
+      const int64_t tiles = ((a.Mo + rows - 1) / rows) * ((a.No + cols - 1) / cols);
+      return static_cast<double>((tiles + L.sm_count - 1) / L.sm_count) * unit;
+    };
+    double best = cost(BM, 256, 1.0);
+    if (const double c = cost(2 * BM, 256, 2.0 * 0.87); c < best) { best = c; MT = 2; }
+    if (const double c = cost(BM, 192, 0.77); c < best) { best = c; MT = 1; BN = 192; }
   }
   const int TM = MT * BM;
   // rows of the tensors as TMA sees them
   const int64_t a_rows = a.a_mn_major ? (grouped_k ? a.rows_total : a.Kc) : a.Mo;
   const int64_t b_rows = a.b_mn_major ? (grouped_k ? a.rows_total : (grouped_rows ? a.E * a.Kc : a.Kc))
                                       : (grouped_rows ? a.E * a.No : a.No);
-  CUtensorMap ta, tb;
+  Maps tm{};
   const bool a3d = a.a_mn_major && a.Mo % 64 == 0, b3d = a.b_mn_major && a.No % 64 == 0;
-  CUresult r = a3d ? make_tmap_mn3d(encode, &ta, a.a, a_rows, a.Mo, TM / 64)
-             : a.a_mn_major ? make_tmap(encode, &ta, a.a, a_rows, a.Mo, 64, BK) : make_tmap(encode, &ta, a.a, a_rows, a.Kc, BK, TM);
+  CUresult r = a3d ? make_tmap_mn3d(encode, &tm.a, a.a, a_rows, a.Mo, TM / 64)
+             : a.a_mn_major ? make_tmap(encode, &tm.a, a.a, a_rows, a.Mo, 64, BK) : make_tmap(encode, &tm.a, a.a, a_rows, a.Kc, BK, TM);
   if (r == CUDA_SUCCESS)
-    r = b3d ? make_tmap_mn3d(encode, &tb, a.b, b_rows, a.No, BN / 64)
-      : a.b_mn_major ? make_tmap(encode, &tb, a.b, b_rows, a.No, 64, BK) : make_tmap(encode, &tb, a.b, b_rows, a.Kc, BK, BN);
+    r = b3d ? make_tmap_mn3d(encode, &tm.b, a.b, b_rows, a.No, BN / 64)
+      : a.b_mn_major ? make_tmap(encode, &tm.b, a.b, b_rows, a.No, 64, BK) : make_tmap(encode, &tm.b, a.b, b_rows, a.Kc, BK, BN);
+  const uint64_t out_count = grouped_k ? static_cast<uint64_t>(a.E) : 1;
+  if (r == CUDA_SUCCESS && a.c_f32) r = make_out_tmap(encode, &tm.f32, a.c_f32, out_count, a.Mo, a.No, 4);
+  if (r == CUDA_SUCCESS && a.c_bf16) r = make_out_tmap(encode, &tm.bf16, a.c_bf16, out_count, a.Mo, a.No, 2);
   if (r != CUDA_SUCCESS) {
     *cu_err = r;
     return cudaErrorUnknown;
@@ -502,7 +599,6 @@ cudaError_t launch_gemm_bf16(const Launch& L, EncodeTiledFn encode, const GemmBf
   p.offsets = a.offsets;
   p.E = static_cast<int>(a.E);
   p.rows_total = static_cast<int>(a.rows_total);
-  p.out_rows = a.out_rows;
   p.a3d = a3d;
   p.b3d = b3d;
   p.col_fastest = a.group == 0 && a.Mo >= a.No;  // A (Mo x Kc) is the larger operand: re-read B, not A
@@ -511,22 +607,14 @@ cudaError_t launch_gemm_bf16(const Launch& L, EncodeTiledFn encode, const GemmBf
   p.status = L.d_status;
   p.wait_limit_ns = 2000000000ull;
   const int64_t n_tiles = (a.No + BN - 1) / BN;
-  if (grouped_rows) {  // A K-major; each expert adds at most one partial row tile
-    const int64_t tiles = (a.Mo / TM + a.E) * n_tiles;
-    return a.b_mn_major ? launch_variant<false, true, kGroupedRows, 1>(L, ta, tb, p, tiles)
-                        : launch_variant<false, false, kGroupedRows, 1>(L, ta, tb, p, tiles);
-  }
   const int64_t m_tiles = (a.Mo + TM - 1) / TM;
-  if (grouped_k) return launch_variant<true, true, kGroupedContraction, 1>(L, ta, tb, p, a.E * m_tiles * n_tiles);
+  if (grouped_rows)  // each expert adds at most one partial row tile
+    return launch_majors<kGroupedRows, 1, 256>(L, tm, p, (a.Mo / TM + a.E) * n_tiles, false, a.b_mn_major);
+  if (grouped_k) return launch_majors<kGroupedContraction, 1, 256>(L, tm, p, a.E * m_tiles * n_tiles, true, true);
   const int64_t tiles = m_tiles * n_tiles;
-  if (MT == 2) {
-    if (a.a_mn_major)
-      return a.b_mn_major ? launch_variant<true, true, kDense, 2>(L, ta, tb, p, tiles) : launch_variant<true, false, kDense, 2>(L, ta, tb, p, tiles);
-    return a.b_mn_major ? launch_variant<false, true, kDense, 2>(L, ta, tb, p, tiles) : launch_variant<false, false, kDense, 2>(L, ta, tb, p, tiles);
-  }
-  if (a.a_mn_major)
-    return a.b_mn_major ? launch_variant<true, true, kDense, 1>(L, ta, tb, p, tiles) : launch_variant<true, false, kDense, 1>(L, ta, tb, p, tiles);
-  return a.b_mn_major ? launch_variant<false, true, kDense, 1>(L, ta, tb, p, tiles) : launch_variant<false, false, kDense, 1>(L, ta, tb, p, tiles);
+  if (MT == 2) return launch_majors<kDense, 2, 256>(L, tm, p, tiles, a.a_mn_major, a.b_mn_major);
+  if (BN == 192) return launch_majors<kDense, 1, 192>(L, tm, p, tiles, a.a_mn_major, a.b_mn_major);
+  return launch_majors<kDense, 1, 256>(L, tm, p, tiles, a.a_mn_major, a.b_mn_major);
 }
 
 }  // namespace qarl
