@@ -18,8 +18,8 @@
 //   grouped contraction  C_e = sum over the expert's rows p of A[p, :]^T B[p, :]  (dW of an
 //                        expert projection: both operands MN-major, the contraction runs over a
 //                        ragged row range).  The last 64-row step of an expert also holds rows of
-//                        the next expert: the MMA warp overwrites those rows of the staged A tile
-//                        with zeros (generic stores + proxy fence) before it issues the step, so
+//                        the next expert: a warp overwrites those rows of the staged A tile with zeros
+//                        (generic stores + proxy fence) before the step is issued, so
 //                        they contribute nothing whatever B holds there.
 //
 // Tile 128 x 256 x 64 (or 256 x 256, 128 x 192: see the host).  TMA stages both operands with the 128-byte swizzle (a K-major tile is
@@ -45,11 +45,7 @@ namespace {
 using namespace ptx;
 
 constexpr int BM = 128, BK = 64;
-constexpr int kMaxStages = 5, kMaxAccBufs = 2;
-constexpr int kEpiWarps = 4;   // warps 0-3 (TMEM quadrant = warp index)
-constexpr int kTmaWarp = 4;
-constexpr int kMmaWarp = 5;
-constexpr int kThreads = 6 * 32;
+constexpr int kMaxStages = 4, kMaxAccBufs = 2;
 constexpr uint32_t kAHalfBytes = BM * BK * 2;   // 16 KB: 128 output rows x 64 contraction elements
 // an epilogue warp's rows on their way out: boxes of 32 rows x 128 bytes (128-byte swizzle)
 constexpr uint32_t kOutBoxBytes = 32 * 128;
@@ -65,10 +61,16 @@ struct Cfg {
   static constexpr uint32_t kABytes = MT * kAHalfBytes;
   static constexpr uint32_t kBBytes = BN * BK * 2;
   static constexpr uint32_t kStageBytes = kABytes + kBBytes;
-  static constexpr int kStages = MT == 2 ? 3 : BN == 192 ? 5 : 4;
+  static constexpr int kStages = MT == 2 ? 3 : 4;
   static constexpr int kAccBufs = MT == 1 ? 2 : 1;
-  static constexpr int kBoxes = GROUP == kGroupedRows || BN == 192 ? 1 : 2;  // per epilogue warp, as the shared memory allows
-  static constexpr uint32_t kOutBytes = kEpiWarps * kBoxes * kOutBoxBytes;
+  // Warps 0 .. kEpiWarps - 1: TMEM quadrant = warp % 4; with eight, two share a quadrant and take the 128-byte
+  // column chunks in turn (each has one box; grouped rows need the shared memory for the tile list).
+  static constexpr int kEpiWarps = GROUP == kGroupedRows ? 4 : 8;
+  static constexpr int kTmaWarp = kEpiWarps;
+  static constexpr int kMmaWarp = kEpiWarps + 1;
+  static constexpr int kFixWarp = kEpiWarps + 2;
+  static constexpr int kThreads = (kEpiWarps + 3) * 32;
+  static constexpr uint32_t kOutBytes = kEpiWarps * kOutBoxBytes;
 };
 constexpr uint32_t kBlockBytes = 64 * BK * 2;  // one MN-major block: 64 output indices x 64 c-rows
 constexpr uint32_t kTmemCols = 512;
@@ -89,6 +91,7 @@ struct Bf16Params {
 struct __align__(8) SmemTail {
   uint64_t full[kMaxStages];
   uint64_t empty[kMaxStages];
+  uint64_t fixed[kMaxStages];  // grouped contraction: the overhang rows of a ragged step are zero
   uint64_t tmem_full[kMaxAccBufs];
   uint64_t tmem_empty[kMaxAccBufs];
   uint64_t teardown;
@@ -138,7 +141,7 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
 }
 
 template <bool A_MN, bool B_MN, int GROUP, int MT, int BN>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(Cfg<GROUP, MT, BN>::kThreads, 1)
 gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                  const __grid_constant__ CUtensorMap tm_f32, const __grid_constant__ CUtensorMap tm_bf16,
                  const Bf16Params p) {
@@ -147,6 +150,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   using C = Cfg<GROUP, MT, BN>;
   constexpr int kStages = C::kStages, kAccBufs = C::kAccBufs, TM = C::kRows;
   constexpr uint32_t kABytes = C::kABytes, kStageBytes = C::kStageBytes;
+  constexpr int kEpiWarps = C::kEpiWarps, kTmaWarp = C::kTmaWarp, kMmaWarp = C::kMmaWarp;
   uint8_t* out_boxes = smem + static_cast<size_t>(kStages) * kStageBytes;
   SmemTail* s = reinterpret_cast<SmemTail*>(out_boxes + C::kOutBytes);
   SmemLists* lists = reinterpret_cast<SmemLists*>(s + 1);
@@ -156,7 +160,8 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) {
       mbar_init(&s->full[i], 1);
-      mbar_init(&s->empty[i], 1);
+      mbar_init(&s->empty[i], GROUP == kGroupedContraction ? 2 : 1);  // the MMAs (and the warp that follows ragged steps)
+      mbar_init(&s->fixed[i], 1);
     }
     for (int i = 0; i < kAccBufs; ++i) {
       mbar_init(&s->tmem_full[i], 1);
@@ -298,83 +303,97 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       }
     }
   } else if (warp == kMmaWarp) {
-    // One thread waits, issues and commits.  Only the last step of a ragged contraction is the whole warp's:
-    // the lanes zero the overhang rows of the staged A tile together before that step's MMAs.
-    constexpr uint32_t idesc = umma_idesc_bf16_f32_major(BM, BN, A_MN, B_MN);
-    int stage = 0, acc = 0;
-    uint32_t phase = 0, acc_phase = 0;
-    bool ok = true;
+    if (elect_one()) {
+      constexpr uint32_t idesc = umma_idesc_bf16_f32_major(BM, BN, A_MN, B_MN);
+      int stage = 0, acc = 0;
+      uint32_t phase = 0, acc_phase = 0, fix_phase = 0;  // fix_phase: a bit per stage, it flips only when the stage held a ragged step
+      bool ok = true;
+      Walk walk;
+      bounds_of(blockIdx.x, walk);
+      for (int T = blockIdx.x; ok && T < total_tiles; T += grid) {
+        const Tile t = tile_of(T, walk);
+        if (t.KS == 0) continue;  // an expert without rows: the epilogue writes zeros, no accumulator is used
+        if (!wait_or_abort(&s->tmem_empty[acc], acc_phase ^ 1, s, p)) { ok = false; break; }
+        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * MT) * BN;
+        for (int ks = 0; ks < t.KS; ++ks) {
+          if (!wait_or_abort(&s->full[stage], phase, s, p)) { ok = false; break; }
+          const bool ragged = GROUP == kGroupedContraction && ks == t.KS - 1 && t.last_valid < BK;
+          if (ragged) {
+            if (!wait_or_abort(&s->fixed[stage], (fix_phase >> stage) & 1u, s, p)) { ok = false; break; }
+            fix_phase ^= 1u << stage;
+          }
+          tc_fence_after_sync();
+          const uint32_t a_addr = smem_u32(smem + static_cast<size_t>(stage) * kStageBytes);
+          const uint32_t b_addr = a_addr + kABytes;
+          const uint64_t a_desc = A_MN ? umma_desc_mn_sw128(a_addr, kBlockBytes) : umma_desc_k_sw128(a_addr);
+          const uint64_t b_desc = B_MN ? umma_desc_mn_sw128(b_addr, kBlockBytes) : umma_desc_k_sw128(b_addr);
+          // 16 contraction elements further on: 32 bytes inside a K-major row, 16 rows of 128 bytes
+          // in an MN-major block (start-address field counts 16-byte units)
+          constexpr uint32_t a_step = A_MN ? (16 * 128) >> 4 : 32 >> 4;
+          constexpr uint32_t b_step = B_MN ? (16 * 128) >> 4 : 32 >> 4;
+          if (!ragged) {
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)  // the 128-row halves of A share the B tile
+#pragma unroll
+              for (int k4 = 0; k4 < BK / 16; ++k4)
+                umma_bf16(d_tmem + mt * BN, a_desc + mt * (kAHalfBytes >> 4) + a_step * k4, b_desc + b_step * k4, idesc,
+                          (ks > 0 || k4 > 0) ? 1u : 0u);
+          } else {  // (MT is 1 in this form) only the slices that hold rows of the expert
+            for (int k4 = 0; 16 * k4 < t.last_valid; ++k4)
+              umma_bf16(d_tmem, a_desc + a_step * k4, b_desc + b_step * k4, idesc, (ks > 0 || k4 > 0) ? 1u : 0u);
+          }
+          umma_commit(&s->empty[stage]);
+          if (ks == t.KS - 1) umma_commit(&s->tmem_full[acc]);
+          if (++stage == kStages) { stage = 0; phase ^= 1; }
+        }
+        if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1; }
+      }
+      // Nothing of this CTA's tensor work may be in flight when its TMEM and shared memory go
+      // away: after an abort some MMAs may still be executing, so wait (bounded) for them.
+      if (!ok) {
+        umma_commit(&s->teardown);
+        mbar_wait_bounded(&s->teardown, 0, 20000000ull);
+      }
+    }
+  } else if (GROUP == kGroupedContraction && warp == C::kFixWarp) {
+    // =============================== ragged steps =====================================
+    // The last 64-row step of an expert also holds rows of the next one.  This warp zeroes what the last 16-row
+    // slice holds of them in the staged A tile as soon as the step has landed, ahead of the MMA thread (which
+    // did this itself once: ~2000 clocks of a tile's ~12000).
+    int stage = 0;
+    uint32_t phase = 0;
     Walk walk;
     bounds_of(blockIdx.x, walk);
-    auto issue = [&](uint32_t d_tmem, int stage, bool first, bool last, int acc) {
-      tc_fence_after_sync();
-      const uint32_t a_addr = smem_u32(smem + static_cast<size_t>(stage) * kStageBytes);
-      const uint32_t b_addr = a_addr + kABytes;
-      const uint64_t a_desc = A_MN ? umma_desc_mn_sw128(a_addr, kBlockBytes) : umma_desc_k_sw128(a_addr);
-      const uint64_t b_desc = B_MN ? umma_desc_mn_sw128(b_addr, kBlockBytes) : umma_desc_k_sw128(b_addr);
-      // 16 contraction elements further on: 32 bytes inside a K-major row, 16 rows of 128 bytes
-      // in an MN-major block (start-address field counts 16-byte units)
-      constexpr uint32_t a_step = A_MN ? (16 * 128) >> 4 : 32 >> 4;
-      constexpr uint32_t b_step = B_MN ? (16 * 128) >> 4 : 32 >> 4;
-#pragma unroll
-      for (int mt = 0; mt < MT; ++mt)  // the 128-row halves of A share the B tile
-#pragma unroll
-        for (int k4 = 0; k4 < BK / 16; ++k4)
-          umma_bf16(d_tmem + mt * BN, a_desc + mt * (kAHalfBytes >> 4) + a_step * k4, b_desc + b_step * k4, idesc,
-                    (!first || k4 > 0) ? 1u : 0u);
-      umma_commit(&s->empty[stage]);
-      if (last) umma_commit(&s->tmem_full[acc]);
-    };
-    for (int T = blockIdx.x; ok && T < total_tiles; T += grid) {
+    for (int T = blockIdx.x; T < total_tiles; T += grid) {
       const Tile t = tile_of(T, walk);
-      if (t.KS == 0) continue;  // an expert without rows: the epilogue writes zeros, no accumulator is used
-      const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * MT) * BN;
-      const bool ragged = GROUP == kGroupedContraction && t.last_valid < BK;
-      const int whole = t.KS - (ragged ? 1 : 0);  // steps without overhang rows
-      if (elect_one()) {
-        ok = wait_or_abort(&s->tmem_empty[acc], acc_phase ^ 1, s, p);
-        int st = stage;
-        uint32_t ph = phase;
-        for (int ks = 0; ok && ks < whole; ++ks) {
-          if (!wait_or_abort(&s->full[st], ph, s, p)) { ok = false; break; }
-          issue(d_tmem, st, ks == 0, ks == t.KS - 1, acc);
-          if (++st == kStages) { st = 0; ph ^= 1; }
-        }
-      }
-      ok = __all_sync(0xFFFFFFFFu, ok);
-      if (!ok) break;
-      const int n = stage + whole;
-      phase ^= static_cast<uint32_t>(n / kStages) & 1u;
-      stage = n % kStages;
-      if (GROUP == kGroupedContraction && ragged) {
+      if (t.KS == 0) continue;
+      // every step is followed (and counted in `empty`): a parity wait tells neighbouring fills apart, no more
+      bool ok = true;
+      for (int ks = 0; ks < t.KS; ++ks) {
         if (!warp_wait_or_abort(&s->full[stage], phase, s, p)) { ok = false; break; }
-        // rows last_valid .. 63 of every 64-column block of A belong to the next expert: make them zero
-        uint8_t* a_tile = smem + static_cast<size_t>(stage) * kStageBytes;
-        const int nrows = BK - t.last_valid;
-        for (int idx = lane; idx < (TM / 64) * nrows * 8; idx += 32) {
-          const int blk = idx / (nrows * 8), rem = idx % (nrows * 8);
-          *reinterpret_cast<uint4*>(a_tile + blk * kBlockBytes + (t.last_valid + rem / 8) * 128 + (rem % 8) * 16) =
-              make_uint4(0, 0, 0, 0);
+        if (ks == t.KS - 1 && t.last_valid < BK) {
+          uint8_t* a_tile = smem + static_cast<size_t>(stage) * kStageBytes;
+          const int nrows = -t.last_valid & 15;
+          for (int idx = lane; idx < (TM / 64) * nrows * 8; idx += 32) {
+            const int blk = idx / (nrows * 8), rem = idx % (nrows * 8);
+            *reinterpret_cast<uint4*>(a_tile + blk * kBlockBytes + (t.last_valid + rem / 8) * 128 + (rem % 8) * 16) =
+                make_uint4(0, 0, 0, 0);
+          }
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&s->fixed[stage]);
         }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (elect_one()) issue(d_tmem, stage, whole == 0, true, acc);
-        __syncwarp();
+        if (lane == 0) mbar_arrive(&s->empty[stage]);
         if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
-      if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1; }
-    }
-    // Nothing of this CTA's tensor work may be in flight when its TMEM and shared memory go
-    // away: after an abort some MMAs may still be executing, so wait (bounded) for them.
-    if (!ok && elect_one()) {
-      umma_commit(&s->teardown);
-      mbar_wait_bounded(&s->teardown, 0, 20000000ull);
+      if (!ok) break;
     }
   } else if (warp < kEpiWarps) {
     // =============================== epilogue warps: TMEM -> box -> TMA store ==========
-    const uint32_t lane_addr = static_cast<uint32_t>(warp * 32) << 16;
-    uint8_t* my_boxes = out_boxes + static_cast<size_t>(warp) * C::kBoxes * kOutBoxBytes;
-    int acc = 0, box = 0;
+    const uint32_t lane_addr = static_cast<uint32_t>((warp & 3) * 32) << 16;
+    uint8_t* my_box = out_boxes + static_cast<size_t>(warp) * kOutBoxBytes;
+    constexpr int kTurns = kEpiWarps / 4;  // warps that share a quadrant's columns
+    int acc = 0;
     uint32_t acc_phase = 0;
     Walk walk;
     bounds_of(blockIdx.x, walk);
@@ -387,80 +406,80 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       }
 #pragma unroll 1
       for (int mt = 0; mt < MT; ++mt) {
-        const int row0 = t.i0 + mt * BM + warp * 32;
+        const int row0 = t.i0 + mt * BM + (warp & 3) * 32;
         if (row0 >= t.row_end) continue;
         const uint32_t t0 = tmem_base + lane_addr + static_cast<uint32_t>((acc * MT + mt) * BN);
         // rows past a group's end are the next expert's: then the box is copied row by row
         const bool whole = GROUP != kGroupedRows || row0 + 32 <= t.row_end;
-        auto columns = [&](int col, uint32_t (&v)[32]) {
+        auto start = [&](int col, uint32_t (&v)[32]) {
           if (have_acc) {
             tmem_ld_x32(t0 + col, v);
-            tmem_ld_wait();
           } else {
 #pragma unroll
             for (int j = 0; j < 32; ++j) v[j] = 0u;
           }
         };
-        // the next box of this warp, once TMA has read what it held
-        auto next_box = [&]() {
-          if (lane == 0) {
-            if (C::kBoxes == 2) bulk_wait_group_read_1();
-            else bulk_wait_group_read_all();
-          }
+        auto box_free = [&]() {  // TMA has read what the box held
+          if (lane == 0) bulk_wait_group_read_all();
           __syncwarp();
-          uint8_t* b = my_boxes + (C::kBoxes == 2 ? box : 0) * kOutBoxBytes;
-          box ^= 1;
-          return b;
         };
-        auto put = [&](uint8_t* b, int j, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
-          *reinterpret_cast<uint4*>(b + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_uint4(w0, w1, w2, w3);
+        auto put = [&](int j, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
+          *reinterpret_cast<uint4*>(my_box + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_uint4(w0, w1, w2, w3);
         };
         // box of 32 rows x 128 bytes at output column `col` (element size `es`)
-        auto send = [&](uint8_t* b, const CUtensorMap* m, void* base, int col, int es) {
+        auto send = [&](const CUtensorMap* m, void* base, int col, int es) {
           if (whole) {
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
-              tma_store_3d(m, b, col, row0, GROUP == kGroupedContraction ? t.e : 0);
+              tma_store_3d(m, my_box, col, row0, GROUP == kGroupedContraction ? t.e : 0);
               bulk_commit_group();
             }
           } else {
             __syncwarp();
             const int chunk = lane & 7, c = col + chunk * (16 / es);
             for (int rr = lane >> 3; row0 + rr < t.row_end; rr += 4) {
-              const uint4 v = *reinterpret_cast<const uint4*>(b + rr * 128 + ((chunk ^ (rr & 7)) << 4));
+              const uint4 v = *reinterpret_cast<const uint4*>(my_box + rr * 128 + ((chunk ^ (rr & 7)) << 4));
               if (c < p.No)
                 *reinterpret_cast<uint4*>(static_cast<uint8_t*>(base) + (static_cast<int64_t>(row0 + rr) * p.No + c) * es) = v;
             }
             __syncwarp();
           }
         };
+        const int cols = min(BN, p.No - t.j0);
         if (p.c_f32) {
+          // the next chunk is on its way from TMEM while this one is written out
+          constexpr int kStep = 32 * kTurns;
+          uint32_t v[2][32];
+          const int first = (warp >> 2) * 32;
+          if (first < cols) start(first, v[0]);
 #pragma unroll 2
-          for (int c = 0; c < BN && t.j0 + c < p.No; c += 32) {
-            uint32_t v[32];
-            columns(c, v);
-            uint8_t* b = next_box();
+          for (int i = 0; first + i * kStep < cols; ++i) {
+            const int c = first + i * kStep;
+            tmem_ld_wait();
+            if (c + kStep < cols) start(c + kStep, v[(i + 1) & 1]);
+            box_free();
+            const uint32_t(&u)[32] = v[i & 1];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) put(b, j, v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-            send(b, &tm_f32, p.c_f32, t.j0 + c, 4);
+            for (int j = 0; j < 8; ++j) put(j, u[4 * j], u[4 * j + 1], u[4 * j + 2], u[4 * j + 3]);
+            send(&tm_f32, p.c_f32, t.j0 + c, 4);
           }
+          tmem_ld_wait();
         }
         if (p.c_bf16) {
-#pragma unroll 2
-          for (int c = 0; c < BN && t.j0 + c < p.No; c += 64) {
-            uint32_t w[32];
+          for (int c = (warp >> 2) * 64; c < cols; c += 64 * kTurns) {
+            uint32_t v[2][32];
+            start(c, v[0]);
+            start(c + 32, v[1]);
+            tmem_ld_wait();
+            box_free();
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              uint32_t v[32];
-              columns(c + 32 * h, v);
-#pragma unroll
-              for (int j = 0; j < 16; ++j) w[16 * h + j] = bf16x2_bits(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+            for (int j = 0; j < 8; ++j) {
+              const uint32_t* u = &v[j >> 2][8 * (j & 3)];
+              put(j, bf16x2_bits(__uint_as_float(u[0]), __uint_as_float(u[1])), bf16x2_bits(__uint_as_float(u[2]), __uint_as_float(u[3])),
+                  bf16x2_bits(__uint_as_float(u[4]), __uint_as_float(u[5])), bf16x2_bits(__uint_as_float(u[6]), __uint_as_float(u[7])));
             }
-            uint8_t* b = next_box();
-#pragma unroll
-            for (int j = 0; j < 8; ++j) put(b, j, w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
-            send(b, &tm_bf16, p.c_bf16, t.j0 + c, 2);
+            send(&tm_bf16, p.c_bf16, t.j0 + c, 2);
           }
         }
       }
@@ -540,7 +559,7 @@ cudaError_t launch_variant(const Launch& L, const Maps& tm, const Bf16Params& p,
   const int64_t rounds = std::max<int64_t>(1, (tiles + L.sm_count - 1) / L.sm_count);
   const int grid = static_cast<int>(std::max<int64_t>(1, (tiles + rounds - 1) / rounds));
   ++*L.launches;
-  return launch_pdl(gemm_bf16_kernel<A_MN, B_MN, GROUP, MT, BN>, static_cast<unsigned>(grid), kThreads, smem_bytes<GROUP, MT, BN>(), L.stream,
+  return launch_pdl(gemm_bf16_kernel<A_MN, B_MN, GROUP, MT, BN>, static_cast<unsigned>(grid), Cfg<GROUP, MT, BN>::kThreads, smem_bytes<GROUP, MT, BN>(), L.stream,
                     tm.a, tm.b, tm.f32, tm.bf16, p);
 }
 
