@@ -132,10 +132,11 @@ struct __align__(8) SmemTail {
   int ready_flag;
   int peek_T;
   int token_T;
-  int pad_;
   int32_t order[1][kMaxTopK];  // combine: contribution row of the rank-th smallest expert id of a token
+  int n_slots;
   int32_t off[kMaxExperts + 1];
   int32_t prefix[kMaxExperts + kDepSlots + 1];
+  int16_t slot[kMaxExperts + kDepSlots];  // layer: the slot of each list entry
 };
 
 constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(kStages) * kStageBytes + kOutBytes + 2 * sizeof(Slab) + sizeof(SmemTail);
@@ -250,14 +251,17 @@ __device__ __forceinline__ void tile_blocks(const DecodeParams& p, const Tile& t
 }
 
 // Layer mode.  Slot s of the list holds the gate_up tiles of expert s (s < E) followed by the down
-// tiles of expert s - D (s >= D), D = min(kDepSlots, E): E + D slots.  prefix[s] = tiles before slot s.
-__device__ __forceinline__ void build_layer_list(int32_t* off, int32_t* prefix, const DecodeParams& p, int D) {
+// tiles of expert s - D (s >= D), D = min(kDepSlots, E): E + D slots.  Only slots that hold tiles are
+// listed (one token of 8 experts leaves 16 of 192, and every role walks the list from its start): entry i is
+// slot[i], with prefix[i] tiles before it.
+__device__ __forceinline__ void build_layer_list(SmemTail* s, const DecodeParams& p, int D) {
+  int32_t* off = s->off;
   for (int e = threadIdx.x; e <= p.E; e += blockDim.x)
     off[e] = p.offsets ? min(max(p.offsets[e], 0), p.rows_total) : (e == 0 ? 0 : p.rows_total);
   __syncthreads();
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x, S = p.E + D;
-    int carry = 0;
+    int carry = 0, n = 0;
     for (int base = 0; base < S; base += 32) {
       const int sl = base + lane;
       int v = 0;
@@ -265,16 +269,26 @@ __device__ __forceinline__ void build_layer_list(int32_t* off, int32_t* prefix, 
         if (sl < p.E) v += chunks_of(off, sl) * p.pj[0].n_pairs;
         if (sl >= D) v += chunks_of(off, sl - D) * p.pj[1].n_pairs;
       }
+      const uint32_t some = __ballot_sync(0xFFFFFFFFu, v > 0);
+      if (some == 0) continue;
       int inc = v;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int u = __shfl_up_sync(0xFFFFFFFFu, inc, o);
         if (lane >= o) inc += u;
       }
-      if (sl < S) prefix[sl] = carry + inc - v;
+      if (v > 0) {
+        const int i = n + __popc(some & ((1u << lane) - 1u));
+        s->slot[i] = static_cast<int16_t>(sl);
+        s->prefix[i] = carry + inc - v;
+      }
+      n += __popc(some);
       carry += __shfl_sync(0xFFFFFFFFu, inc, 31);
     }
-    if (lane == 0) prefix[S] = carry;
+    if (lane == 0) {
+      s->prefix[n] = carry;
+      s->n_slots = n;
+    }
   }
   __syncthreads();
 }
@@ -294,13 +308,14 @@ __device__ __forceinline__ Tile tile_at(const SmemTail* s, const DecodeParams& p
   } else {
     while (T >= s->prefix[cur + 1]) ++cur;
     int local = T - s->prefix[cur];
-    const int gt = cur < p.E ? chunks_of(s->off, cur) * p.pj[0].n_pairs : 0;
+    const int sl = s->slot[cur];
+    const int gt = sl < p.E ? chunks_of(s->off, sl) * p.pj[0].n_pairs : 0;
     if (local < gt) {
       t.mode = kModeGateUp;
-      t.e = cur;
+      t.e = sl;
     } else {
       t.mode = kModeDown;
-      t.e = cur - D;
+      t.e = sl - D;
       local -= gt;
     }
     const int ch = chunks_of(s->off, t.e);
@@ -380,13 +395,18 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     }
   }
   pdl_wait();
-  if (kLayer) build_layer_list(s->off, s->prefix, p, D);
+  int first_draw = 0;  // layer: this CTA's first tile number, drawn while the list is built
+  if (kLayer && warp == kTmaWarp) {
+    if (lane == 0) first_draw = atomicAdd(p.sync, 1);
+    first_draw = __shfl_sync(0xFFFFFFFFu, first_draw, 0);
+  }
+  if (kLayer) build_layer_list(s, p, D);
   else build_tile_list(s->off, s->prefix, p.offsets, p.rows_total, p.E, NT, p.pj[0].n_pairs);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = s->tmem_addr;
-  const int total_tiles = s->prefix[kLayer ? p.E + D : p.E];
+  const int total_tiles = s->prefix[kLayer ? s->n_slots : p.E];
   // Which tiles a CTA runs.  Single projection: tile blockIdx.x, then every gridDim.x-th (every SM
   // streams: the tiles are equal and small, the last round costs little).  Layer: the tiles differ in
   // size (a gate_up tile streams 2.7 x the bytes of a down tile), so the CTAs draw tile numbers from a
@@ -412,7 +432,7 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             return t < total_tiles ? t : -1;
           } else {
             if (!wait_or_abort(&s->sched_empty[sslot], sphase ^ 1, s, p)) { ok = false; return -1; }
-            int t = atomicAdd(p.sync, 1);
+            int t = prev < 0 ? first_draw : atomicAdd(p.sync, 1);
             if (t >= total_tiles) t = -1;
             *reinterpret_cast<volatile int*>(&s->sched_T[sslot]) = t;
             mbar_arrive(&s->sched_full[sslot]);  // release: the number is visible to whoever sees the phase flip
@@ -427,12 +447,17 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
           tile_blocks<MODE>(p, c, row_lo, row_hi, nb_lo, nb_hi);
           const CUtensorMap* mx = pi ? &tm_x2 : &tm_x;
           const CUtensorMap* mw = pi ? &tm_w2 : &tm_w;
-          if (kLayer && c.mode == kModeDown) {
-            // the h codes of this expert are written by gate_up tiles of this launch (other CTAs)
-            if (!counter_wait_or_abort(p.sync + 1 + c.e, chunks_of(s->off, c.e) * p.pj[0].n_pairs, s, p)) { ok = false; break; }
-            fence_proxy_async_global();
-          }
+          // A down tile's h codes are written by gate_up tiles of this launch (other CTAs).  Its weights are not:
+          // while the expert is incomplete they fill the ring on their own, the token rows follow.
           const int KB = p.pj[pi].kblocks;
+          const int* ctr = kLayer && c.mode == kModeDown ? p.sync + 1 + c.e : nullptr;
+          const int target = ctr ? chunks_of(s->off, c.e) * p.pj[0].n_pairs : 0;
+          int ahead = 0;  // leading K-blocks of the tile whose token rows are still to be loaded
+          if (ctr) {
+            if (ld_acquire_gpu(ctr) >= target) fence_proxy_async_global();
+            else ahead = min(KB, kStages);
+          }
+          const int stage0 = stage;
           for (int kb = 0; kb < KB; ++kb) {
             if (p.stop_after_stages >= 0 && armed_total >= p.stop_after_stages) { ok = false; break; }
             ++armed_total;
@@ -441,10 +466,18 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
             tma_load_2d_hint(a_dst, mw, &s->full[stage], kb * BK, row_lo, stream_once);
             tma_load_2d_hint(a_dst + kABytes / 2, mw, &s->full[stage], kb * BK, row_hi, stream_once);
-            tma_load_2d(a_dst + kABytes, mx, &s->full[stage], kb * BK, c.m0);
+            if (kb >= ahead) tma_load_2d(a_dst + kABytes, mx, &s->full[stage], kb * BK, c.m0);
             armed |= 1u << stage;
             armed_parity = (armed_parity & ~(1u << stage)) | (phase << stage);
             if (++stage == kStages) { stage = 0; phase ^= 1; }
+            if (kb + 1 == ahead) {
+              if (!counter_wait_or_abort(ctr, target, s, p)) { ok = false; break; }
+              fence_proxy_async_global();
+              for (int i = 0, st = stage0; i < ahead; ++i) {
+                tma_load_2d(smem + static_cast<size_t>(st) * kStageBytes + kABytes, mx, &s->full[st], i * BK, c.m0);
+                if (++st == kStages) st = 0;
+              }
+            }
           }
         }
         if (!ok) {  // let copies in flight land before the CTA's shared memory is released
@@ -987,7 +1020,9 @@ cudaError_t launch_moe_decode_layer(const Launch& L, EncodeTiledFn encode, const
   p.status = L.d_status;
   p.wait_limit_ns = L.wait_limit_ns ? L.wait_limit_ns : 2000000000ull;
   p.stop_after_stages = L.stop_after_stages;
-  p.early_prefetch = early_prefetch_tiles(L, p.pj[0].kblocks);
+  // The guess behind the prefetch (every expert has tokens) holds for 1 - (1 - 1/E)^P of the experts: below
+  // E / 2 pairs most of it is bandwidth taken from the tiles (one token: 32.6 us with it, 30.2 without).
+  p.early_prefetch = 2 * g.rows_total >= g.E ? early_prefetch_tiles(L, p.pj[0].kblocks) : 0;
   // every SM takes part: the CTAs share the combine even when the tiles are few
   return launch_mode<kModeLayer>(L, tx, tw, tx2, tw2, p, L.sm_count);
 }

@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(kThreads) permute_single_cta_kernel(const int3
 constexpr int kPrepThreads = 512;
 constexpr int kPrepWarps = kPrepThreads / 32;
 constexpr int kPrepPairsPerWarp = kChunk / kPrepWarps;
+constexpr int kFewPairs = 256;  // up to here positions are counted pair against pair
 __global__ void __launch_bounds__(kPrepThreads) moe_prep_small_kernel(
     const int32_t* __restrict__ ids, int64_t P, int E, int fanout, const uint16_t* __restrict__ x, int64_t M, int64_t K,
     const float* __restrict__ pair_w, int32_t* __restrict__ offsets, int32_t* __restrict__ sorted_pair,
@@ -224,8 +225,8 @@ __global__ void __launch_bounds__(kPrepThreads) moe_prep_small_kernel(
   if (blockIdx.x == 0)
     for (int i = threadIdx.x; i < zero_count; i += kPrepThreads) zero[i] = 0;
   int32_t* whist = sm;                 // [kPrepWarps][E]
-  int32_t* total = sm + kPrepWarps * E;    // [E]
-  int32_t* scratch = total + E;        // [33]
+  int32_t* total = sm + kPrepWarps * E;    // [max(E, kFewPairs)] (kPrepWarps E words in: 16-byte aligned)
+  int32_t* scratch = total + max(E, kFewPairs);  // [33]
   int32_t* spos = scratch + 33;        // [kChunk] sorted position of every pair (-1: bad id)
   const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
   const bool publish = blockIdx.x == 0;
@@ -244,72 +245,122 @@ __global__ void __launch_bounds__(kPrepThreads) moe_prep_small_kernel(
     v1 = __ldg(src + 1);
   }
 
-  // ---- the grouping (as permute_single_cta_kernel), positions kept in shared memory
-  constexpr int kRounds = kPrepPairsPerWarp / 32;
-  const int64_t p0 = static_cast<int64_t>(wid) * kPrepPairsPerWarp + lane;
-  int my[kRounds];
-  bool bad = false;
-#pragma unroll
-  for (int r = 0; r < kRounds; ++r) {
-    const int64_t p = p0 + r * 32;
-    int e = -1;
-    if (p < P) {
-      e = __ldg(ids + p);
-      if (e < 0 || e >= E) { bad = true; e = -1; }
+  if (P <= kFewPairs) {
+    // Few pairs: a pair's position is the number of pairs that sort before it, an expert's offset the number of
+    // pairs with a lower id -- counted directly, two block barriers in all where the histogram, scan and
+    // scatter below need eight and cost ~5 us however few the pairs are.
+    if (tid < kFewPairs) {
+      int e = 0x7FFFFFFF;  // none, or a bad id: never counted
+      if (tid < P) {
+        e = __ldg(ids + tid);
+        if (e < 0 || e >= E) {
+          e = 0x7FFFFFFF;
+          if (publish) set_status(status, QARL_ERR_BAD_EXPERT_ID);
+        }
+      }
+      total[tid] = e;
     }
-    my[r] = e;
-  }
-  if (bad && publish) set_status(status, QARL_ERR_BAD_EXPERT_ID);
-  for (int i = tid; i < kPrepWarps * E; i += kPrepThreads) whist[i] = 0;
-  for (int i = tid; i < kChunk; i += kPrepThreads) spos[i] = -1;
-  __syncthreads();
-  int32_t* hist_w = whist + wid * E;
-#pragma unroll
-  for (int r = 0; r < kRounds; ++r) {
-    const int e = my[r];
-    const uint32_t peers = match_id(e);
-    if (e >= 0 && (__ffs(peers) - 1) == lane) hist_w[e] += __popc(peers);
-    __syncwarp();
-  }
-  __syncthreads();
-  for (int e = tid; e < E; e += kPrepThreads) {
-    int s = 0;
-    for (int w = 0; w < kPrepWarps; ++w) s += whist[w * E + e];
-    total[e] = s;
-  }
-  __syncthreads();
-  const int all = block_exclusive_scan(total, E, scratch);
-  for (int e = tid; e < E; e += kPrepThreads) {
-    int run = total[e];
-    if (publish) offsets[e] = run;
-    for (int w = 0; w < kPrepWarps; ++w) {
-      const int c = whist[w * E + e];
-      whist[w * E + e] = run;
-      run += c;
-    }
-  }
-  if (publish && tid == 0) offsets[E] = all;
-  __syncthreads();
-  const uint32_t lt = (1u << lane) - 1u;
-#pragma unroll
-  for (int r = 0; r < kRounds; ++r) {
-    const int e = my[r];
-    const uint32_t peers = match_id(e);
-    int pos = -1;
-    if (e >= 0) pos = hist_w[e] + __popc(peers & lt);
-    __syncwarp();
-    if (e >= 0 && (__ffs(peers) - 1) == lane) hist_w[e] += __popc(peers);
-    __syncwarp();
-    if (e >= 0) {
-      const int64_t p = p0 + r * 32;
-      spos[p] = pos;
-      if (publish) {
-        sorted_pair[pos] = static_cast<int32_t>(p);
-        pos_of_pair[p] = pos;
+    __syncthreads();
+    const int4* all_ids = reinterpret_cast<const int4*>(total);
+    const int quads = static_cast<int>((P + 3) >> 2);
+    if (tid < kFewPairs) {
+      if (tid < P) {
+        const int mine = total[tid];
+        int pos = 0;
+#pragma unroll 4
+        for (int i = 0; i < quads; ++i) {
+          const int4 o = all_ids[i];
+          const int q = 4 * i;
+          pos += (o.x < mine || (o.x == mine && q < tid)) + (o.y < mine || (o.y == mine && q + 1 < tid)) +
+                 (o.z < mine || (o.z == mine && q + 2 < tid)) + (o.w < mine || (o.w == mine && q + 3 < tid));
+        }
+        const bool good = mine != 0x7FFFFFFF;
+        spos[tid] = good ? pos : -1;
+        if (publish && good) {
+          sorted_pair[pos] = tid;
+          pos_of_pair[tid] = pos;
+        }
+      }
+    } else if (publish) {
+      for (int e = tid - kFewPairs; e <= E; e += kPrepThreads - kFewPairs) {
+        int below = 0;
+#pragma unroll 4
+        for (int i = 0; i < quads; ++i) {
+          const int4 o = all_ids[i];
+          below += (o.x < e) + (o.y < e) + (o.z < e) + (o.w < e);
+        }
+        offsets[e] = below;
       }
     }
+    __syncthreads();
+  } else {
+    // ---- the grouping (as permute_single_cta_kernel), positions kept in shared memory
+    constexpr int kRounds = kPrepPairsPerWarp / 32;
+    const int64_t p0 = static_cast<int64_t>(wid) * kPrepPairsPerWarp + lane;
+    int my[kRounds];
+    bool bad = false;
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) {
+      const int64_t p = p0 + r * 32;
+      int e = -1;
+      if (p < P) {
+        e = __ldg(ids + p);
+        if (e < 0 || e >= E) { bad = true; e = -1; }
+      }
+      my[r] = e;
+    }
+    if (bad && publish) set_status(status, QARL_ERR_BAD_EXPERT_ID);
+    for (int i = tid; i < kPrepWarps * E; i += kPrepThreads) whist[i] = 0;
+    for (int i = tid; i < kChunk; i += kPrepThreads) spos[i] = -1;
+    __syncthreads();
+    int32_t* hist_w = whist + wid * E;
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) {
+      const int e = my[r];
+      const uint32_t peers = match_id(e);
+      if (e >= 0 && (__ffs(peers) - 1) == lane) hist_w[e] += __popc(peers);
+      __syncwarp();
+    }
+    __syncthreads();
+    for (int e = tid; e < E; e += kPrepThreads) {
+      int s = 0;
+      for (int w = 0; w < kPrepWarps; ++w) s += whist[w * E + e];
+      total[e] = s;
+    }
+    __syncthreads();
+    const int all = block_exclusive_scan(total, E, scratch);
+    for (int e = tid; e < E; e += kPrepThreads) {
+      int run = total[e];
+      if (publish) offsets[e] = run;
+      for (int w = 0; w < kPrepWarps; ++w) {
+        const int c = whist[w * E + e];
+        whist[w * E + e] = run;
+        run += c;
+      }
+    }
+    if (publish && tid == 0) offsets[E] = all;
+    __syncthreads();
+    const uint32_t lt = (1u << lane) - 1u;
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) {
+      const int e = my[r];
+      const uint32_t peers = match_id(e);
+      int pos = -1;
+      if (e >= 0) pos = hist_w[e] + __popc(peers & lt);
+      __syncwarp();
+      if (e >= 0 && (__ffs(peers) - 1) == lane) hist_w[e] += __popc(peers);
+      __syncwarp();
+      if (e >= 0) {
+        const int64_t p = p0 + r * 32;
+        spos[p] = pos;
+        if (publish) {
+          sorted_pair[pos] = static_cast<int32_t>(p);
+          pos_of_pair[p] = pos;
+        }
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
 
   // ---- quantize this thread's group and scatter it to the token's sorted rows
   uint32_t m = fold_halves(absmax_u4(absmax_u4(0, v0), v1));
@@ -434,7 +485,7 @@ cudaError_t launch_moe_prep_small(const Launch& L, const int32_t* ids, int64_t M
                                   const PermuteBuffers& b, const uint16_t* x, int64_t K, const float* pair_w,
                                   uint8_t* codes, float* scales, float* sorted_w, int32_t* zero, int zero_count) {
   const int e = static_cast<int>(E);
-  const size_t smem = (static_cast<size_t>(kPrepWarps) * e + e + 33 + kChunk) * sizeof(int32_t);
+  const size_t smem = (static_cast<size_t>(kPrepWarps) * e + std::max(e, kFewPairs) + 33 + kChunk) * sizeof(int32_t);
   if (smem > 48 * 1024) {
     cudaError_t err = cudaFuncSetAttribute(moe_prep_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            static_cast<int>(smem));
