@@ -27,7 +27,7 @@
 //
 // The whole decode-sized MoE layer also runs as ONE launch of this kernel (kModeLayer): the tile
 // list holds the gate_up tiles and the down tiles of every expert, the down tiles of expert e
-// kDepSlots experts after its gate_up tiles, so the weight stream never stops between the two
+// kDepSlots experts (that have rows) after its gate_up tiles, so the weight stream never stops between the two
 // projections; a down tile starts once a per-expert counter says the h rows it reads are written
 // (release by the writers, acquire + proxy fence by the readers, every spin bounded); tiles are
 // drawn from a counter (they differ in size), and a CTA that has run out of tiles draws tokens
@@ -68,7 +68,7 @@ constexpr int kMaxExperts = 1024;
 constexpr int kOutRowBytes = 2 * BW * 2 + 16;  // bf16 row of 256 outputs, padded
 constexpr uint32_t kOutBytes = NT * kOutRowBytes;
 constexpr int kModeLayer = 3;     // gate_up tiles + down tiles + combine in one launch (this file only)
-constexpr int kDepSlots = 64;     // the down tiles of expert e are listed with the gate_up tiles of expert e + kDepSlots
+constexpr int kDepSlots = 64;     // the down tiles of an expert are listed with the gate_up tiles of the 64th next one
 constexpr int kMaxTopK = 32;
 constexpr int kSchedSlots = 4;    // layer: tile numbers the producer has drawn and the other roles have not yet read
 
@@ -133,10 +133,10 @@ struct __align__(8) SmemTail {
   int peek_T;
   int token_T;
   int32_t order[1][kMaxTopK];  // combine: contribution row of the rank-th smallest expert id of a token
-  int n_slots;
+  int n_active;               // layer: experts with rows
   int32_t off[kMaxExperts + 1];
   int32_t prefix[kMaxExperts + kDepSlots + 1];
-  int16_t slot[kMaxExperts + kDepSlots];  // layer: the slot of each list entry
+  int16_t active[kMaxExperts];  // their ids, ascending
 };
 
 constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(kStages) * kStageBytes + kOutBytes + 2 * sizeof(Slab) + sizeof(SmemTail);
@@ -250,44 +250,47 @@ __device__ __forceinline__ void tile_blocks(const DecodeParams& p, const Tile& t
   row_hi = t.e * N + nb_hi * BW;
 }
 
-// Layer mode.  Slot s of the list holds the gate_up tiles of expert s (s < E) followed by the down
-// tiles of expert s - D (s >= D), D = min(kDepSlots, E): E + D slots.  Only slots that hold tiles are
-// listed (one token of 8 experts leaves 16 of 192, and every role walks the list from its start): entry i is
-// slot[i], with prefix[i] tiles before it.
-__device__ __forceinline__ void build_layer_list(SmemTail* s, const DecodeParams& p, int D) {
+// Layer mode.  The list runs over the n experts that have rows: slot i holds the gate_up tiles of the i-th
+// of them (i < n) followed by the down tiles of the (i - D)-th (i >= D), D = min(kDepSlots, n): n + D slots.
+// prefix[i] = tiles before slot i.  Counting only experts with rows keeps the list short (one token of 8
+// experts: 16 slots) and the distance between the projections real: with down tiles 64 expert IDS behind, CTAs
+// of a sparse batch drew down tiles of the first experts and sat on them while gate_up tiles were left
+// (4 tokens: the last gate_up tile began 20 us into a 41 us launch).
+__device__ __forceinline__ int dep_slots(int n_active) { return min(kDepSlots, n_active); }
+
+__device__ __forceinline__ void build_layer_list(SmemTail* s, const DecodeParams& p) {
   int32_t* off = s->off;
-  for (int e = threadIdx.x; e <= p.E; e += blockDim.x)
-    off[e] = p.offsets ? min(max(p.offsets[e], 0), p.rows_total) : (e == 0 ? 0 : p.rows_total);
+  for (int e = threadIdx.x; e <= p.E; e += blockDim.x) off[e] = min(max(p.offsets[e], 0), p.rows_total);
   __syncthreads();
   if (threadIdx.x < 32) {
-    const int lane = threadIdx.x, S = p.E + D;
-    int carry = 0, n = 0;
+    const int lane = threadIdx.x;
+    int n = 0;
+    for (int base = 0; base < p.E; base += 32) {
+      const int e = base + lane;
+      const uint32_t some = __ballot_sync(0xFFFFFFFFu, e < p.E && off[e + 1] > off[e]);
+      if (e < p.E && off[e + 1] > off[e]) s->active[n + __popc(some & ((1u << lane) - 1u))] = static_cast<int16_t>(e);
+      n += __popc(some);
+    }
+    __syncwarp();
+    const int D = dep_slots(n), S = n + D;
+    int carry = 0;
     for (int base = 0; base < S; base += 32) {
       const int sl = base + lane;
       int v = 0;
-      if (sl < S) {
-        if (sl < p.E) v += chunks_of(off, sl) * p.pj[0].n_pairs;
-        if (sl >= D) v += chunks_of(off, sl - D) * p.pj[1].n_pairs;
-      }
-      const uint32_t some = __ballot_sync(0xFFFFFFFFu, v > 0);
-      if (some == 0) continue;
+      if (sl < n) v += chunks_of(off, s->active[sl]) * p.pj[0].n_pairs;
+      if (sl >= D && sl < S) v += chunks_of(off, s->active[sl - D]) * p.pj[1].n_pairs;
       int inc = v;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int u = __shfl_up_sync(0xFFFFFFFFu, inc, o);
         if (lane >= o) inc += u;
       }
-      if (v > 0) {
-        const int i = n + __popc(some & ((1u << lane) - 1u));
-        s->slot[i] = static_cast<int16_t>(sl);
-        s->prefix[i] = carry + inc - v;
-      }
-      n += __popc(some);
+      if (sl < S) s->prefix[sl] = carry + inc - v;
       carry += __shfl_sync(0xFFFFFFFFu, inc, 31);
     }
     if (lane == 0) {
-      s->prefix[n] = carry;
-      s->n_slots = n;
+      s->prefix[S] = carry;
+      s->n_active = n;
     }
   }
   __syncthreads();
@@ -295,7 +298,7 @@ __device__ __forceinline__ void build_layer_list(SmemTail* s, const DecodeParams
 
 // Tile T of the list (T ascending per caller: `cur` only moves forward).
 template <int MODE>
-__device__ __forceinline__ Tile tile_at(const SmemTail* s, const DecodeParams& p, int D, int T, int& cur) {
+__device__ __forceinline__ Tile tile_at(const SmemTail* s, const DecodeParams& p, int T, int& cur) {
   Tile t;
   if constexpr (MODE != kModeLayer) {
     const TileCoord c = decode_tile(s->off, s->prefix, NT, T, cur);
@@ -308,14 +311,14 @@ __device__ __forceinline__ Tile tile_at(const SmemTail* s, const DecodeParams& p
   } else {
     while (T >= s->prefix[cur + 1]) ++cur;
     int local = T - s->prefix[cur];
-    const int sl = s->slot[cur];
-    const int gt = sl < p.E ? chunks_of(s->off, sl) * p.pj[0].n_pairs : 0;
+    const int n = s->n_active;
+    const int gt = cur < n ? chunks_of(s->off, s->active[cur]) * p.pj[0].n_pairs : 0;
     if (local < gt) {
       t.mode = kModeGateUp;
-      t.e = sl;
+      t.e = s->active[cur];
     } else {
       t.mode = kModeDown;
-      t.e = sl - D;
+      t.e = s->active[cur - dep_slots(n)];
       local -= gt;
     }
     const int ch = chunks_of(s->off, t.e);
@@ -338,7 +341,6 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   SmemTail* s = reinterpret_cast<SmemTail*>(slab + 2);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr bool kLayer = MODE == kModeLayer;
-  const int D = kLayer ? min(kDepSlots, p.E) : 0;
 
   pdl_trigger();
   if (threadIdx.x == 0) {
@@ -400,13 +402,13 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     if (lane == 0) first_draw = atomicAdd(p.sync, 1);
     first_draw = __shfl_sync(0xFFFFFFFFu, first_draw, 0);
   }
-  if (kLayer) build_layer_list(s, p, D);
+  if (kLayer) build_layer_list(s, p);
   else build_tile_list(s->off, s->prefix, p.offsets, p.rows_total, p.E, NT, p.pj[0].n_pairs);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = s->tmem_addr;
-  const int total_tiles = s->prefix[kLayer ? s->n_slots : p.E];
+  const int total_tiles = s->prefix[kLayer ? s->n_active + dep_slots(s->n_active) : p.E];
   // Which tiles a CTA runs.  Single projection: tile blockIdx.x, then every gridDim.x-th (every SM
   // streams: the tiles are equal and small, the last round costs little).  Layer: the tiles differ in
   // size (a gate_up tile streams 2.7 x the bytes of a down tile), so the CTAs draw tile numbers from a
@@ -441,7 +443,7 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
           }
         };
         for (int T = draw(-1); ok && T >= 0; T = draw(T)) {
-          const Tile c = tile_at<MODE>(s, p, D, T, cur);
+          const Tile c = tile_at<MODE>(s, p, T, cur);
           const int pi = proj_of<MODE>(c.mode);
           int row_lo, row_hi, nb_lo, nb_hi;
           tile_blocks<MODE>(p, c, row_lo, row_hi, nb_lo, nb_hi);
@@ -510,7 +512,7 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         };
         for (int T = take(-1); ok && T >= 0; T = take(T)) {
           int KB = p.pj[0].kblocks;
-          if (kLayer) KB = p.pj[proj_of<MODE>(tile_at<MODE>(s, p, D, T, cur).mode)].kblocks;
+          if (kLayer) KB = p.pj[proj_of<MODE>(tile_at<MODE>(s, p, T, cur).mode)].kblocks;
           for (int kb = 0; kb < KB; ++kb) {
             if (!wait_or_abort(&s->tmem_empty[ks], acc_phase ^ 1, s, p)) { ok = false; break; }
             if (!wait_or_abort(&s->full[stage], phase, s, p)) { ok = false; break; }
@@ -616,7 +618,7 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     // of a tile, and a warp whose wait ran out inside a tile skips the work but not the barriers.
     int T = take(-1);
     if (T >= 0) {
-      Tile c = tile_at<MODE>(s, p, D, T, cur);
+      Tile c = tile_at<MODE>(s, p, T, cur);
       bool filled = false;  // is the current tile's slab on its way?
       for (;;) {
         if (!filled) ok = fill_slab(sb, c, true, filled) && ok;
@@ -641,7 +643,7 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         }
         bool next_filled = false;
         if (Tn >= 0) {
-          cn = tile_at<MODE>(s, p, D, Tn, cur);
+          cn = tile_at<MODE>(s, p, Tn, cur);
           fill_slab(sb ^ 1, cn, false, next_filled);  // next tile's scales fly while this tile computes
         }
         const Slab& sl = slab[sb];
@@ -710,7 +712,7 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         ++tile_iter;
         if (kLayer && Tn == -2) {  // the producer had not drawn the next tile when this one began: wait for it now
           Tn = take(T);
-          if (Tn >= 0) cn = tile_at<MODE>(s, p, D, Tn, cur);
+          if (Tn >= 0) cn = tile_at<MODE>(s, p, Tn, cur);
         }
         if (Tn < 0) break;
         T = Tn;
@@ -744,7 +746,7 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       }
     };
     for (int T = take(-1); T >= 0; T = take(T), ++tile_iter) {
-      const Tile c = tile_at<MODE>(s, p, D, T, cur);
+      const Tile c = tile_at<MODE>(s, p, T, cur);
       const int rows = min(NT, c.m_end - c.m0);
       const int N = p.pj[proj_of<MODE>(c.mode)].N;
       const int j = c.j;
@@ -795,8 +797,8 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       if (kLayer) {
         // Other CTAs read what this tile wrote once the expert's counter says so -- the h codes by TMA
         // and their scales by plain loads (gate_up), the contribution rows in the k-sum (down): every
-        // writer orders its stores (both proxies), then one thread bumps the counter.
-        __threadfence();
+        // writer orders its stores for the async proxy, and after the barrier one thread bumps the counter with a
+        // release, which covers the stores of all of them (a fence per thread as well cost ~0.5 us per tile).
         if (c.mode == kModeGateUp) fence_proxy_async_global();
         named_bar_sync(4, kEpiThreads);
         if (et == 0) red_release_gpu_add(p.sync + (c.mode == kModeGateUp ? 1 : 1 + p.E) + c.e, 1);
