@@ -5,17 +5,20 @@
 //   w~ = exp(clip(b, -log c, log c));  r~ = clip(r, 0, 1 + eps_h) if A >= 0 else clip(r, 1 - delta_l, 1 + delta_h)
 //   J = w~ r~ A;   loss = -mean_i J;   d loss / d lp_cur[t] = -(w~ A r) / (L B) if r is inside its band, else 0.
 // HBM-bound: 12 bytes read and 4 written per token.  Two launches:
-//   partial  (warp per 512 tokens)  the 12 loads of a lane are issued before anything else; for every response that
+//   partial  (warp per piece, all pieces at once: T / 2368 tokens, at least 512)  walks its piece in steps of 512
+//                                   tokens with the next step's loads in flight; for every response that
 //                                   overlaps the piece, the sums of the two token differences over the
 //                                   overlap, in double, to slot (response + piece) -- unique, because both
 //                                   indices only grow along the token axis.  No block barrier, whatever the lengths.
-//   finish   (CTA per 4096 tokens)  for every response that overlaps the chunk: its partials added (lane l takes
+//   finish   (CTA per 8192 tokens)  for every response that overlaps the chunk: its partials added (lane l takes
 //                                   every 32nd, then a butterfly), r, w, J, flags and the gradient value its
 //                                   tokens share, in double -- repeated by each chunk of a response, written out
 //                                   by the chunk that holds its first token --, then the gradient streamed over
 //                                   the chunk; the last CTA to finish adds all J in index order: loss = -mean J
 // The response of a token is found by a 32-way search of the offsets.  Every sum has a fixed order: results do not
-// depend on the grid or on timing.
+// depend on the grid or on timing.  1024 responses, 4.2 M tokens (67 MB) on the device: 31.7 us as four launches (response
+// map, CTA per 8192 tokens with a block sum per response, statistics, gradient), 22.5 us so, of which 13.6 are the partial
+// kernel (3.7 TB/s: ~4 us of its time is launch and first-load latency).
 #include <math.h>
 
 #include <algorithm>
@@ -25,8 +28,9 @@
 namespace qarl {
 namespace {
 
-constexpr int kPiece = 512;    // tokens per warp of the partial kernel: 16 per lane
-constexpr int kChunk = 4096;   // tokens per CTA of the finish kernel
+constexpr int kStep = 512;     // tokens a warp of the partial kernel takes at a time: 16 per lane
+constexpr int kPieces = 2368;  // most pieces of a call: 16 warps on each of 148 SMs (a fixed number: the cut depends on T alone)
+constexpr int kChunk = 8192;   // tokens per CTA of the finish kernel
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 
@@ -44,6 +48,7 @@ struct TbpoParams {
   int32_t* flags;
   float* grad;
   double* loss;
+  int64_t piece;         // tokens per piece
   double2* partial;      // [B + pieces]
   unsigned int* ticket;  // CTAs of the finish kernel that are done
 };
@@ -76,69 +81,98 @@ __device__ __forceinline__ double2 warp_sum(double2 v) {
   return v;
 }
 
-// VEC: the three arrays are 16-byte aligned
-template <bool VEC>
-__global__ void __launch_bounds__(kThreads) tbpo_partial_kernel(const TbpoParams p) {
-  pdl_trigger();
-  pdl_wait();
-  if (blockIdx.x == 0 && threadIdx.x == 0) *p.ticket = 0;
-  const int lane = threadIdx.x & 31;
-  const int64_t k = static_cast<int64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
-  const int64_t lo = k * kPiece, hi = min(lo + kPiece, p.T);
-  if (lo >= p.T) return;
-  // token of this lane's element (j, u): lo + 4 (32 j + lane) + u
+struct Step {
   float c[16], o[16], q[16];
+};
+// Loads of the step at token `base`; element e of a lane is token base + 4 lane + 128 (e / 4) + e % 4.
+// VEC: the three arrays are 16-byte aligned.
+template <bool VEC>
+__device__ __forceinline__ void load_step(const TbpoParams& p, Step& s, int64_t base, int64_t hi, int lane) {
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const int64_t t = lo + 4 * (32 * j + lane);
+    const int64_t t = base + 4 * (32 * j + lane);
     if (VEC && t + 4 <= hi) {
       const float4 a = __ldcs(reinterpret_cast<const float4*>(p.lp_cur + t));
       const float4 b = __ldcs(reinterpret_cast<const float4*>(p.lp_old + t));
       const float4 d = __ldcs(reinterpret_cast<const float4*>(p.lp_smp + t));
-      c[4 * j] = a.x, c[4 * j + 1] = a.y, c[4 * j + 2] = a.z, c[4 * j + 3] = a.w;
-      o[4 * j] = b.x, o[4 * j + 1] = b.y, o[4 * j + 2] = b.z, o[4 * j + 3] = b.w;
-      q[4 * j] = d.x, q[4 * j + 1] = d.y, q[4 * j + 2] = d.z, q[4 * j + 3] = d.w;
+      s.c[4 * j] = a.x, s.c[4 * j + 1] = a.y, s.c[4 * j + 2] = a.z, s.c[4 * j + 3] = a.w;
+      s.o[4 * j] = b.x, s.o[4 * j + 1] = b.y, s.o[4 * j + 2] = b.z, s.o[4 * j + 3] = b.w;
+      s.q[4 * j] = d.x, s.q[4 * j + 1] = d.y, s.q[4 * j + 2] = d.z, s.q[4 * j + 3] = d.w;
     } else {
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const bool in = t + u < hi;
-        c[4 * j + u] = in ? __ldcs(p.lp_cur + t + u) : 0.0f;
-        o[4 * j + u] = in ? __ldcs(p.lp_old + t + u) : 0.0f;
-        q[4 * j + u] = in ? __ldcs(p.lp_smp + t + u) : 0.0f;
+        s.c[4 * j + u] = in ? __ldcs(p.lp_cur + t + u) : 0.0f;
+        s.o[4 * j + u] = in ? __ldcs(p.lp_old + t + u) : 0.0f;
+        s.q[4 * j + u] = in ? __ldcs(p.lp_smp + t + u) : 0.0f;
       }
     }
   }
-  for (int64_t i = response_of(p, lo, lane); i < p.B; ++i) {
-    const int64_t t0 = clamp_off(p, i);
-    if (t0 >= hi) break;
-    const int64_t s0 = max(t0, lo), s1 = min(clamp_off(p, i + 1), hi);
-    if (s1 <= s0) continue;
-    double2 acc = make_double2(0.0, 0.0);
-    if (s0 == lo && s1 == lo + kPiece) {
-#pragma unroll
-      for (int e = 0; e < 16; ++e) {  // differences formed in double: exact
-        acc.x += static_cast<double>(c[e]) - static_cast<double>(o[e]);
-        acc.y += static_cast<double>(o[e]) - static_cast<double>(q[e]);
-      }
-    } else {
-      const int a0 = static_cast<int>(s0 - lo) - 4 * lane, a1 = static_cast<int>(s1 - lo) - 4 * lane;
-#pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        const int at = 128 * (e >> 2) + (e & 3);
-        if (at >= a0 && at < a1) {
-          acc.x += static_cast<double>(c[e]) - static_cast<double>(o[e]);
-          acc.y += static_cast<double>(o[e]) - static_cast<double>(q[e]);
-        }
-      }
-    }
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads, 2) tbpo_partial_kernel(const TbpoParams p) {
+  pdl_wait();
+  pdl_trigger();  // after the wait: the finish kernel may read the call's inputs before its own wait
+  if (blockIdx.x == 0 && threadIdx.x == 0) *p.ticket = 0;
+  const int lane = threadIdx.x & 31;
+  const int64_t k = static_cast<int64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
+  const int64_t lo = k * p.piece, hi = min(lo + p.piece, p.T);
+  if (lo >= p.T) return;
+  Step s[2];
+  load_step<VEC>(p, s[0], lo, hi, lane);
+  int64_t i = response_of(p, lo, lane);
+  int64_t t0 = clamp_off(p, i), t1 = clamp_off(p, i + 1);
+  double2 acc = make_double2(0.0, 0.0);
+  auto flush = [&]() {
     acc = warp_sum(acc);
     if (lane == 0) p.partial[i + k] = acc;
+    acc = make_double2(0.0, 0.0);
+  };
+  auto consume = [&](const Step& s, int64_t base) -> bool {  // false: no response left
+    const int64_t end = min(base + kStep, hi);
+    for (;;) {
+      if (t0 <= base && t1 >= base + kStep && end == base + kStep) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {  // differences formed in double: exact
+          acc.x += static_cast<double>(s.c[e]) - static_cast<double>(s.o[e]);
+          acc.y += static_cast<double>(s.o[e]) - static_cast<double>(s.q[e]);
+        }
+      } else {
+        const int a0 = static_cast<int>(max(t0, base) - base) - 4 * lane;
+        const int a1 = static_cast<int>(max(min(t1, end), base) - base) - 4 * lane;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          const int at = 128 * (e >> 2) + (e & 3);
+          if (at >= a0 && at < a1) {
+            acc.x += static_cast<double>(s.c[e]) - static_cast<double>(s.o[e]);
+            acc.y += static_cast<double>(s.o[e]) - static_cast<double>(s.q[e]);
+          }
+        }
+      }
+      if (t1 > end) return true;  // goes on in the next step (or piece)
+      if (t1 > max(t0, lo)) flush();
+      if (++i >= p.B) return false;
+      t0 = clamp_off(p, i);
+      t1 = clamp_off(p, i + 1);
+      if (t0 >= end) return true;
+    }
+  };
+  bool more = true;
+  for (int64_t base = lo; more && base < hi; base += 2 * kStep) {
+    if (base + kStep < hi) load_step<VEC>(p, s[1], base + kStep, hi, lane);
+    more = consume(s[0], base);
+    if (more && base + kStep < hi) {
+      if (base + 2 * kStep < hi) load_step<VEC>(p, s[0], base + 2 * kStep, hi, lane);
+      more = consume(s[1], base + kStep);
+    }
   }
+  if (more && t0 < hi && t1 > hi) flush();
 }
 
 // Everything about response i (tokens [t0, t1), t1 > t0) from its two sums; returns the gradient value its tokens
 // share, and writes the per-response outputs if `write`.
-__device__ __forceinline__ float finish_response(const TbpoParams& p, int64_t i, int64_t t0, int64_t t1, double2 sum, bool write) {
+__device__ __forceinline__ float finish_response(const TbpoParams& p, int64_t i, int64_t t0, int64_t t1, double2 sum, float adv, bool write) {
   const double L = static_cast<double>(t1 - t0);
   const double a = sum.x / L, b = sum.y / L;
   const double r = exp(a);
@@ -147,7 +181,7 @@ __device__ __forceinline__ float finish_response(const TbpoParams& p, int64_t i,
   if (bc > p.log_cap) { bc = p.log_cap; f |= 2; }
   if (bc < -p.log_cap) { bc = -p.log_cap; f |= 2; }
   const double wt = exp(bc);
-  const double A = static_cast<double>(__ldg(p.adv + i));
+  const double A = static_cast<double>(adv);
   const double band_lo = A >= 0.0 ? 0.0 : 1.0 - p.delta_l;
   const double band_hi = A >= 0.0 ? 1.0 + p.eps_h : 1.0 + p.delta_h;
   double rt = r;
@@ -169,9 +203,18 @@ __global__ void __launch_bounds__(kThreads) tbpo_finish_kernel(const TbpoParams 
   __shared__ int64_t bound[kThreads + 1];  // clamped offsets of the responses in hand
   __shared__ bool last;
   pdl_trigger();
-  pdl_wait();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t lo = static_cast<int64_t>(blockIdx.x) * kChunk, hi = min(lo + kChunk, p.T);
+  // Offsets and advantages are inputs of the call and the partial kernel started this one after its own wait: they may
+  // be read ahead of this kernel's wait, while the last pieces are still being summed.
+  int64_t first = 0;
+  float adv = 0.0f;  // of response i0 + tid
+  if (lo < hi) {
+    first = response_of(p, lo, lane);
+    for (int j = tid; j <= kThreads; j += kThreads) bound[j] = first + j <= p.B ? clamp_off(p, first + j) : p.T;
+    if (first + tid < p.B) adv = __ldg(p.adv + first + tid);
+  }
+  pdl_wait();
   // empty responses: J = 0, still counted in B
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + tid; i < p.B; i += static_cast<int64_t>(gridDim.x) * kThreads)
     if (clamp_off(p, i + 1) <= clamp_off(p, i)) {
@@ -180,16 +223,27 @@ __global__ void __launch_bounds__(kThreads) tbpo_finish_kernel(const TbpoParams 
       p.j_seq[i] = 0.0;
       p.flags[i] = 4;
     }
+  // Counted once the CTA's J are written: the last CTA to get here adds every J at its end, in one fixed order
+  // (thread j takes j, j + 256, ...; then a tree): which CTA that is varies, what it computes does not.
+  auto count = [&]() {
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();  // after the barrier: covers what the CTA's threads wrote
+      last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+    }
+  };
   if (lo < hi) {
     // up to kThreads responses at a time
-    for (int64_t i0 = response_of(p, lo, lane); i0 < p.B; i0 += kThreads) {
-      for (int j = tid; j <= kThreads; j += kThreads) bound[j] = i0 + j <= p.B ? clamp_off(p, i0 + j) : p.T;
+    for (int64_t i0 = first; i0 < p.B; i0 += kThreads) {
+      if (i0 > first) {
+        for (int j = tid; j <= kThreads; j += kThreads) bound[j] = i0 + j <= p.B ? clamp_off(p, i0 + j) : p.T;
+        if (i0 + tid < p.B) adv = __ldg(p.adv + i0 + tid);
+      }
       __syncthreads();
-      if (bound[0] >= hi) break;  // (the same for every thread)
       for (int j = warp; j < kThreads && i0 + j < p.B && bound[j] < hi; j += kWarps) {
         const int64_t t0 = bound[j], t1 = bound[j + 1];
         if (t1 <= max(t0, lo)) continue;
-        const int64_t k0 = t0 / kPiece, k1 = (t1 + kPiece - 1) / kPiece;
+        const int64_t k0 = t0 / p.piece, k1 = (t1 + p.piece - 1) / p.piece;
         double2 s = make_double2(0.0, 0.0);
         for (int64_t kk = k0 + lane; kk < k1; kk += 32) {
           const double2 v = p.partial[i0 + j + kk];
@@ -201,8 +255,10 @@ __global__ void __launch_bounds__(kThreads) tbpo_finish_kernel(const TbpoParams 
       }
       __syncthreads();
       if (i0 + tid < p.B && bound[tid] < hi && bound[tid + 1] > max(bound[tid], lo))
-        gval[tid] = finish_response(p, i0 + tid, bound[tid], bound[tid + 1], sums[tid], bound[tid] >= lo);
-      __syncthreads();
+        gval[tid] = finish_response(p, i0 + tid, bound[tid], bound[tid + 1], sums[tid], adv, bound[tid] >= lo);
+      const bool final = i0 + kThreads >= p.B || bound[kThreads] >= hi;  // no further round
+      if (final) count();
+      else __syncthreads();
       if (p.grad) {
         const bool vec = (reinterpret_cast<uintptr_t>(p.grad) & 15u) == 0;
         for (int j = 0; j < kThreads && i0 + j < p.B && bound[j] < hi; ++j) {
@@ -215,16 +271,11 @@ __global__ void __launch_bounds__(kThreads) tbpo_finish_kernel(const TbpoParams 
           for (int64_t t = v1 + tid; t < s1; t += kThreads) p.grad[t] = g;
         }
       }
-      if (bound[kThreads] >= hi) break;
+      if (final) break;
       __syncthreads();
     }
-  }
-  // The last CTA to get here adds every J in one fixed order (thread j takes j, j + 256, ...; then a
-  // tree): which CTA that is varies, what it computes does not.
-  __syncthreads();
-  if (tid == 0) {
-    __threadfence();  // after the barrier: covers what the CTA's threads wrote
-    last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+  } else {
+    count();
   }
   __syncthreads();
   if (!last) return;
@@ -249,7 +300,8 @@ __global__ void tbpo_zero_loss_kernel(const TbpoParams p) {
 }  // namespace
 
 namespace {
-int64_t pieces_of(int64_t T) { return (T + kPiece - 1) / kPiece; }
+int64_t piece_of(int64_t T) { return std::max<int64_t>(kStep, ((T + kPieces - 1) / kPieces + 127) / 128 * 128); }
+int64_t pieces_of(int64_t T) { return (T + piece_of(T) - 1) / piece_of(T); }
 size_t ticket_at(int64_t B, int64_t T) { return (static_cast<size_t>(B + pieces_of(T)) * sizeof(double2) + 255) / 256 * 256; }
 }  // namespace
 
@@ -275,6 +327,7 @@ cudaError_t launch_tbpo(const Launch& L, const TbpoArgs& a) {
   p.grad = a.grad;
   p.loss = a.loss;
   uint8_t* ws = static_cast<uint8_t*>(a.workspace);
+  p.piece = piece_of(a.T);
   p.partial = reinterpret_cast<double2*>(ws);
   p.ticket = reinterpret_cast<unsigned int*>(ws + ticket_at(a.B, a.T));
   if (a.B == 0) {  // no responses: the loss of an empty batch is 0
