@@ -16,13 +16,15 @@
 //
 // A tile = (expert e, pair of weight blocks j, chunk of <= NT rows of the expert's group):
 //   gate_up: blocks j (gate rows) and j + I/128 (the matching up rows); down/linear: blocks 2j, 2j+1.
-// CTA = 704 threads: warps 0-3 epilogue (thread = weight row: TMEM -> SwiGLU / weighting -> bf16, transposed through
-// shared memory so that global stores are whole token rows), warps 4-19 dequantization in two groups that take
-// 64-element K-steps in turn (thread = one of the pair's 256 weight rows, 64 codes; codes, scale and zero point come
-// straight from global memory into registers, three of the thread's steps ahead), warp 20 producer of the token
-// rows (TMA), warp 21 MMA issuer.
-// TMEM: two accumulators of 2 NT columns (the epilogue of a tile overlaps the next tile), the rest stages of 64
-// columns (two blocks x 64 k).
+// CTA = 896 threads: warps 0-7 epilogue (thread = weight row, half of the tokens: TMEM -> SwiGLU / weighting -> bf16,
+// transposed through shared memory so that global stores are whole token rows), warps 8-23 dequantization in two
+// groups that take A stages in turn (thread = one of the pair's 256 weight rows), warp 24 producer of the codes
+// (bulk copies into a shared-memory ring, scales and zero points copied alongside), warp 25 producer of the token
+// rows (TMA), warps 26 / 27 MMA issuers of the two blocks.
+// TMEM: two accumulators of 2 NT columns (the epilogue of a tile overlaps the next tile), the rest A stages.
+// What the hand-offs cost decides the stage sizes: a step of one issuing thread (two waits, its MMAs, the
+// commits) takes 300-450 clocks whatever the MMAs, so codes and token rows move in 128-element quantization groups, and
+// with NT = 32 an A stage is a whole group too (NT = 96: half of one, its MMAs take 384 clocks).
 // Every barrier wait is bounded; an expired wait aborts the CTA cleanly.
 #include <algorithm>
 #include <atomic>
@@ -39,31 +41,37 @@ using namespace ptx;
 
 constexpr int BW = 128;            // weight rows per block (UMMA M)
 constexpr int BK = 64;             // bf16 elements per K-step (128 bytes)
-constexpr int kEpiWarps = 4;       // warps 0-3
-constexpr int kDqWarps = 16;       // warps 4-19: two groups of eight
-constexpr int kTokenWarp = 20;     // producer of the token rows
-constexpr int kMmaWarp = 21;
-constexpr int kThreads = 22 * 32;
+constexpr int kEpiWarps = 8;       // warps 0-7: TMEM quadrant = warp % 4, token half = warp / 4
+constexpr int kDqWarps = 16;       // warps 8-23: two groups of eight
+constexpr int kCodeWarp = 24;      // producer of the codes
+constexpr int kTokenWarp = 25;     // producer of the token rows
+constexpr int kMmaWarp = 26;       // and 27: one issuer per weight block
+constexpr int kThreads = 28 * 32;
 constexpr uint32_t kQStepBytes = BW * BK / 2;  // 4 KB: 128 rows x 32 bytes of codes (one K-step of one block)
 constexpr uint32_t kTmemCols = 512;
 constexpr int kAccBufs = 2;
-constexpr int kStageCols = 64;                 // two blocks x 64 bf16
 constexpr int kMaxExperts = 1024;
 constexpr int kOutRowBytes = 2 * BW * 2 + 16;  // bf16 row of 256 outputs, padded
 constexpr uint32_t kPrefetchChunk = 32768;     // bytes per L2 prefetch instruction
-constexpr int kMaxXStages = 16, kMaxAStages = 6;
+constexpr int kMaxStages = 8;
+// one quantization group of a pair of blocks in the ring: codes, then scales [2][128] bf16, zero points [2][128]
+constexpr uint32_t kCodeBytes = 2 * 2 * kQStepBytes;
+constexpr uint32_t kGroupBytes = kCodeBytes + 2 * BW * 2 + 2 * BW;
 
 // NT = 32 for groups of a few rows (decode), kWide for larger ones.
 constexpr int kNarrow = 32;
 constexpr int kWide = 96;
 template <int NT>
 struct Cfg {
-  static constexpr uint32_t kXBytes = NT * BK * 2;
-  static constexpr int kXStages = NT == kNarrow ? 16 : 8;
+  static constexpr uint32_t kXBytes = 2 * NT * BK * 2;               // token rows of one group: two boxes of 64 elements
+  static constexpr int kXStages = NT == kNarrow ? 4 : 3;
+  static constexpr int kQStages = NT == kNarrow ? 8 : 5;
+  static constexpr int kAK = NT == kNarrow ? 2 : 1;                  // K-steps of 64 per A stage
+  static constexpr int kStageCols = 2 * 32 * kAK;                    // two blocks
   static constexpr int kAStages = (static_cast<int>(kTmemCols) - kAccBufs * 2 * NT) / kStageCols;
   static constexpr uint32_t kABase = kAccBufs * 2 * NT;
 };
-static_assert(Cfg<kNarrow>::kAStages <= kMaxAStages && Cfg<kWide>::kAStages >= 2, "TMEM budget");
+static_assert(Cfg<kNarrow>::kAStages >= 2 && Cfg<kWide>::kAStages >= 2, "TMEM budget");
 
 struct W4Params {
   const uint8_t* b_packed;   // tile-major 4 KB chunks [E][N/128][K/64]
@@ -86,13 +94,15 @@ struct W4Params {
 };
 
 struct __align__(8) SmemTail {
-  uint64_t x_full[kMaxXStages];
-  uint64_t x_empty[kMaxXStages];
-  uint64_t a_full[kMaxAStages];
-  uint64_t a_empty[kMaxAStages];
+  uint64_t x_full[kMaxStages];
+  uint64_t x_empty[kMaxStages];
+  uint64_t q_full[kMaxStages];
+  uint64_t q_empty[kMaxStages];
+  uint64_t a_full[kMaxStages];
+  uint64_t a_empty[kMaxStages];
   uint64_t tmem_full[kAccBufs];
   uint64_t tmem_empty[kAccBufs];
-  uint64_t teardown;
+  uint64_t teardown[2];
   uint32_t tmem_addr;
   int abort_flag;
   int32_t off[kMaxExperts + 1];
@@ -100,7 +110,8 @@ struct __align__(8) SmemTail {
 };
 
 template <int NT>
-constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(Cfg<NT>::kXStages) * Cfg<NT>::kXBytes + static_cast<size_t>(NT) * kOutRowBytes + sizeof(SmemTail);
+constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(Cfg<NT>::kXStages) * Cfg<NT>::kXBytes + static_cast<size_t>(Cfg<NT>::kQStages) * kGroupBytes +
+                              static_cast<size_t>(NT) * kOutRowBytes + sizeof(SmemTail);
 static_assert(kSmemBytes<kNarrow> <= 227 * 1024 && kSmemBytes<kWide> <= 227 * 1024, "shared memory budget");
 
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, SmemTail* s, const W4Params& p) {
@@ -158,11 +169,12 @@ template <int MODE, int FMT, int NT>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
   using C = Cfg<NT>;
-  constexpr int kXStages = C::kXStages, kAStages = C::kAStages;
+  constexpr int kXStages = C::kXStages, kQStages = C::kQStages, kAStages = C::kAStages, kAK = C::kAK, kStageCols = C::kStageCols;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* x_base = smem;  // [stage][NT rows x 128 bytes], swizzled
-  uint8_t* out_tile = x_base + static_cast<size_t>(kXStages) * C::kXBytes;
+  uint8_t* x_base = smem;  // [stage][K-step][NT rows x 128 bytes], swizzled
+  uint8_t* q_base = x_base + static_cast<size_t>(kXStages) * C::kXBytes;
+  uint8_t* out_tile = q_base + static_cast<size_t>(kQStages) * kGroupBytes;
   SmemTail* s = reinterpret_cast<SmemTail*>(out_tile + NT * kOutRowBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -171,17 +183,22 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
   if (threadIdx.x == 0) {
     for (int i = 0; i < kXStages; ++i) {
       mbar_init(&s->x_full[i], 1);
-      mbar_init(&s->x_empty[i], 1);
+      mbar_init(&s->x_empty[i], 2);                                  // the commits of the two issuers
+    }
+    for (int i = 0; i < kQStages; ++i) {
+      mbar_init(&s->q_full[i], 2);                                   // the bulk copies, the scales
+      mbar_init(&s->q_empty[i], kAK == 2 ? kDqWarps / 2 : kDqWarps);  // the warps that read it
     }
     for (int i = 0; i < kAStages; ++i) {
       mbar_init(&s->a_full[i], kDqWarps / 2);
-      mbar_init(&s->a_empty[i], 1);
+      mbar_init(&s->a_empty[i], 2);
     }
     for (int i = 0; i < kAccBufs; ++i) {
-      mbar_init(&s->tmem_full[i], 1);
+      mbar_init(&s->tmem_full[i], 2);
       mbar_init(&s->tmem_empty[i], kEpiWarps);
     }
-    mbar_init(&s->teardown, 1);
+    mbar_init(&s->teardown[0], 1);
+    mbar_init(&s->teardown[1], 1);
     s->abort_flag = 0;
     fence_mbar_init();
   }
@@ -200,7 +217,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
     q_lo = p.b_packed + (static_cast<int64_t>(e) * NB + nb_lo) * KS * kQStepBytes;
     q_hi = p.b_packed + (static_cast<int64_t>(e) * NB + nb_hi) * KS * kQStepBytes;
   };
-  if (warp == kTokenWarp && lane == 0 && p.early_prefetch) {
+  if (warp == kCodeWarp && lane == 0 && p.early_prefetch) {
     // The weights do not depend on the kernels before this one in the stream: start pulling this CTA's
     // first tile (guessed as expert T / n_pairs, pair T % n_pairs: exact when every expert has one chunk).
     const int T = blockIdx.x;
@@ -232,10 +249,12 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
       bool ok = true;
       for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
         const TileCoord c = decode_tile(s->off, s->prefix, NT, T, cur_e);
-        for (int ks = 0; ks < KS; ++ks) {
+        for (int g = 0; g < KG; ++g) {
           if (!wait_or_abort(&s->x_empty[xs], x_phase ^ 1, s, p)) { ok = false; break; }
           mbar_arrive_expect_tx(&s->x_full[xs], C::kXBytes);
-          tma_load_2d(x_base + static_cast<size_t>(xs) * C::kXBytes, &tm_x, &s->x_full[xs], ks * BK, c.m0);
+          uint8_t* dst = x_base + static_cast<size_t>(xs) * C::kXBytes;
+          tma_load_2d(dst, &tm_x, &s->x_full[xs], 2 * g * BK, c.m0);
+          tma_load_2d(dst + C::kXBytes / 2, &tm_x, &s->x_full[xs], (2 * g + 1) * BK, c.m0);
           armed |= 1u << xs;
           armed_parity = (armed_parity & ~(1u << xs)) | (x_phase << xs);
           if (++xs == kXStages) { xs = 0; x_phase ^= 1; }
@@ -246,134 +265,156 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
           if (armed & (1u << i)) mbar_wait_bounded(&s->x_full[i], (armed_parity >> i) & 1u, 20000000ull);
       }
     }
-  } else if (warp == kMmaWarp) {
-    // =============================== MMA issuer =======================================
+  } else if (warp == kCodeWarp) {
+    // =============================== producer of the codes ============================
+    // Per quantization group: two bulk copies of 8 KB, and the 256 scales and zero points (no 16-byte alignment is
+    // promised for those: plain loads, lane l rows l, l + 32, ..., written to the stage by this warp).  The ring is
+    // deep enough to hide the latency of both.
+    int qs = 0, cur_e = 0;
+    uint32_t q_phase = 0, armed = 0, armed_parity = 0;
+    bool ok = true;
+    for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
+      const TileCoord c = decode_tile(s->off, s->prefix, NT, T, cur_e);
+      const uint8_t *q_lo, *q_hi;
+      tile_codes(c.e, c.n_tile, q_lo, q_hi);
+      int nb_lo, nb_hi;
+      tile_blocks<MODE>(p, c.n_tile, nb_lo, nb_hi);
+      int64_t sz = static_cast<int64_t>(c.e) * KG * p.N + lane;
+      for (int g = 0; g < KG; ++g, sz += p.N) {
+        uint16_t sc[8];
+        uint8_t z[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const int64_t at = sz + (r < 4 ? nb_lo : nb_hi) * BW + 32 * (r & 3);
+          sc[r] = __ldg(p.b_scales + at);
+          if constexpr (FMT == kFmtInt4) z[r] = __ldg(p.b_zeros + at);
+        }
+        if (!warp_wait_or_abort(&s->q_empty[qs], q_phase ^ 1, s, p)) { ok = false; break; }
+        uint8_t* dst = q_base + static_cast<size_t>(qs) * kGroupBytes;
+        if (lane == 0) {
+          mbar_arrive_expect_tx(&s->q_full[qs], kCodeBytes);
+          bulk_load_1d(dst, q_lo + static_cast<int64_t>(g) * (2 * kQStepBytes), 2 * kQStepBytes, &s->q_full[qs]);
+          bulk_load_1d(dst + kCodeBytes / 2, q_hi + static_cast<int64_t>(g) * (2 * kQStepBytes), 2 * kQStepBytes, &s->q_full[qs]);
+        }
+        uint16_t* sdst = reinterpret_cast<uint16_t*>(dst + kCodeBytes);
+        uint8_t* zdst = dst + kCodeBytes + 2 * BW * 2;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          sdst[32 * r + lane] = sc[r];
+          if constexpr (FMT == kFmtInt4) zdst[32 * r + lane] = z[r];
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&s->q_full[qs]);
+        armed |= 1u << qs;
+        armed_parity = (armed_parity & ~(1u << qs)) | (q_phase << qs);
+        if (++qs == kQStages) { qs = 0; q_phase ^= 1; }
+      }
+    }
+    if (!ok && lane == 0) {
+      for (int i = 0; i < kQStages; ++i)
+        if (armed & (1u << i)) mbar_wait_bounded(&s->q_full[i], (armed_parity >> i) & 1u, 20000000ull);
+    }
+  } else if (warp >= kMmaWarp) {
+    // =============================== MMA issuers ======================================
+    // One thread per weight block, each with its own NT accumulator columns and its half of an A stage.
     if (elect_one()) {
+      const int h = warp - kMmaWarp;
       constexpr uint32_t idesc = umma_idesc_bf16_f32(BW, NT);
       int xs = 0, as = 0, acc = 0;
       uint32_t x_phase = 0, a_phase = 0, acc_phase = 0;
       bool ok = true;
       for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
         if (!wait_or_abort(&s->tmem_empty[acc], acc_phase ^ 1, s, p)) { ok = false; break; }
-        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc) * (2 * NT);
-        for (int ks = 0; ks < KS; ++ks) {
+        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc) * (2 * NT) + static_cast<uint32_t>(h) * NT;
+        for (int g = 0; ok && g < KG; ++g) {
           if (!wait_or_abort(&s->x_full[xs], x_phase, s, p)) { ok = false; break; }
-          if (!wait_or_abort(&s->a_full[as], a_phase, s, p)) { ok = false; break; }
-          tc_fence_after_sync();
-          const uint64_t x_desc = umma_desc_k_sw128(smem_u32(x_base + static_cast<size_t>(xs) * C::kXBytes));
-          const uint32_t a_tmem = tmem_base + C::kABase + static_cast<uint32_t>(as) * kStageCols;
+          const uint32_t x_addr = smem_u32(x_base + static_cast<size_t>(xs) * C::kXBytes);
 #pragma unroll
-          for (int k4 = 0; k4 < BK / 16; ++k4)  // +16 elements: 8 TMEM columns of A, 2 in the 16-byte address field of B
+          for (int u0 = 0; u0 < 2; u0 += kAK) {
+            if (!wait_or_abort(&s->a_full[as], a_phase, s, p)) { ok = false; break; }
+            tc_fence_after_sync();
+            const uint32_t a_tmem = tmem_base + C::kABase + static_cast<uint32_t>(as * kStageCols + h * (kStageCols / 2));
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
-              umma_bf16_ts(d_tmem + h * NT, a_tmem + h * (kStageCols / 2) + 8 * k4, x_desc + 2 * k4, idesc, (ks > 0 || k4 > 0) ? 1u : 0u);
-          umma_commit(&s->a_empty[as]);
+            for (int u = 0; u < kAK; ++u) {
+              const uint64_t x_desc = umma_desc_k_sw128(x_addr + (u0 + u) * (C::kXBytes / 2));
+#pragma unroll
+              for (int k4 = 0; k4 < BK / 16; ++k4)  // +16 elements: 8 TMEM columns of A, 2 in the 16-byte address field of B
+                umma_bf16_ts(d_tmem, a_tmem + 32 * u + 8 * k4, x_desc + 2 * k4, idesc, (g > 0 || u0 + u > 0 || k4 > 0) ? 1u : 0u);
+            }
+            umma_commit(&s->a_empty[as]);
+            if (++as == kAStages) { as = 0; a_phase ^= 1; }
+          }
+          if (!ok) break;
           umma_commit(&s->x_empty[xs]);
-          if (ks == KS - 1) umma_commit(&s->tmem_full[acc]);
+          if (g == KG - 1) umma_commit(&s->tmem_full[acc]);
           if (++xs == kXStages) { xs = 0; x_phase ^= 1; }
-          if (++as == kAStages) { as = 0; a_phase ^= 1; }
         }
         if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1; }
       }
       if (!ok) {  // after an abort MMAs may still be executing: wait (bounded) before TMEM goes away
-        umma_commit(&s->teardown);
-        mbar_wait_bounded(&s->teardown, 0, 20000000ull);
+        umma_commit(&s->teardown[h]);
+        mbar_wait_bounded(&s->teardown[h], 0, 20000000ull);
       }
     }
   } else if (warp >= kEpiWarps) {
     // =============================== dequantization warps =============================
-    const int grp = (warp - kEpiWarps) >> 3;         // takes K-steps ks with ks % 2 == grp (a tile has an even number)
+    // A stage of kAK K-steps is filled by one group of eight warps; the groups take stages in turn (a tile has an
+    // even number of K-steps; with kAK = 2 the turn goes on across tiles).
+    const int grp = (warp - kEpiWarps) >> 3;
     const int h = ((warp - kEpiWarps) >> 2) & 1;     // weight block of the pair
     const int nr = (warp & 3) * 32 + lane;           // weight row of the block = TMEM lane
-    const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16) + C::kABase + static_cast<uint32_t>(h) * (kStageCols / 2);
-    // A thread's i-th step of a tile is K-step 2i + grp, inside quantization group i: 32 bytes of codes (consecutive
-    // threads read consecutive 16-byte pieces of a 4 KB chunk, [word quad 0..1][row][16 bytes]; read once: streaming
-    // loads), a scale and a zero point, all loaded three steps ahead.
-    struct Ahead {
-      uint4 q0, q1;
-      uint32_t s, z;
-    };
-    int pfT = first_tile, pfi = 0, pf_e = 0;
-    const uint8_t* pf_q = nullptr;
-    int64_t pf_sz = 0;
-    auto pf_set_tile = [&]() {
-      if (pfT < total_tiles) {
-        const TileCoord t = decode_tile(s->off, s->prefix, NT, pfT, pf_e);
-        const uint8_t *q_lo, *q_hi;
-        tile_codes(t.e, t.n_tile, q_lo, q_hi);
-        pf_q = (h ? q_hi : q_lo) + grp * kQStepBytes + nr * 16;
-        int nb_lo, nb_hi;
-        tile_blocks<MODE>(p, t.n_tile, nb_lo, nb_hi);
-        pf_sz = static_cast<int64_t>(t.e) * KG * p.N + (h ? nb_hi : nb_lo) * BW + nr;
-      }
-    };
-    auto pf_load = [&](Ahead& a) {
-      if (pfT < total_tiles) {
-        const uint4* src = reinterpret_cast<const uint4*>(pf_q);
-        a.q0 = __ldcs(src);
-        a.q1 = __ldcs(src + kQStepBytes / 32);
-        a.s = __ldg(p.b_scales + pf_sz);
-        if constexpr (FMT == kFmtInt4) a.z = __ldg(p.b_zeros + pf_sz);
-        pf_q += 2 * kQStepBytes;
-        pf_sz += p.N;
-        if (++pfi == KG) {
-          pfi = 0;
-          pfT += num_ctas;
-          pf_set_tile();
-        }
-      }
-    };
-    pf_set_tile();
-    Ahead a[3] = {};
-    pf_load(a[0]);
-    pf_load(a[1]);
-    pf_load(a[2]);
-    uint32_t n = static_cast<uint32_t>(grp);  // K-steps of this CTA so far, this group's next one
-    const int steps = first_tile < total_tiles ? ((total_tiles - 1 - first_tile) / num_ctas + 1) * KG : 0;  // of this thread
-    auto expand = [&](Ahead& cur) -> bool {
+    const uint32_t a_base = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16) + C::kABase + static_cast<uint32_t>(h) * (kStageCols / 2);
+    const int groups = first_tile < total_tiles ? ((total_tiles - 1 - first_tile) / num_ctas + 1) * KG : 0;  // of this CTA
+    // group index in the ring / A stage index, both counted over the CTA's life
+    for (int g = kAK == 2 ? grp : 0; g < groups; g += kAK) {
+      const int qs = g % kQStages;
+      const uint32_t n = static_cast<uint32_t>(kAK == 2 ? g : 2 * g + grp);
+      const int as = static_cast<int>(n % kAStages);
+      if (!warp_wait_or_abort(&s->q_full[qs], static_cast<uint32_t>(g / kQStages) & 1u, s, p)) break;
+      const uint8_t* q = q_base + static_cast<size_t>(qs) * kGroupBytes;
       uint32_t s2, zc2;  // integer: s and 128 + z as bf16x2; e2m1: the two per-group factors
+      const uint32_t sb = *reinterpret_cast<const uint16_t*>(q + kCodeBytes + 2 * (h * BW + nr));
       if constexpr (FMT == kFmtInt4) {
-        s2 = cur.s | (cur.s << 16);
-        zc2 = (0x4300u | cur.z) * 0x00010001u;
+        s2 = sb | (sb << 16);
+        zc2 = (0x4300u | q[kCodeBytes + 4 * BW + h * BW + nr]) * 0x00010001u;
       } else {
-        fp4_group_consts(cur.s, zc2, s2);
+        fp4_group_consts(sb, zc2, s2);
       }
-      const uint32_t stage = n % kAStages, phase = (n / kAStages) & 1u;
-      if (!warp_wait_or_abort(&s->a_empty[stage], phase ^ 1, s, p)) return false;
-      tc_fence_after_sync();
-      const uint32_t dst = lane_addr + stage * kStageCols;
-      const uint32_t words[8] = {cur.q0.x, cur.q0.y, cur.q0.z, cur.q0.w, cur.q1.x, cur.q1.y, cur.q1.z, cur.q1.w};
+      // [block][K-step][word quad 0..1][row][16 bytes]
+      const uint8_t* src = q + h * (2 * kQStepBytes) + (kAK == 2 ? 0 : grp) * kQStepBytes + nr * 16;
+      uint4 w[2 * kAK];
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
+      for (int i = 0; i < 2 * kAK; ++i) w[i] = *reinterpret_cast<const uint4*>(src + i * (kQStepBytes / 2));
+      if (!warp_wait_or_abort(&s->a_empty[as], ((n / kAStages) & 1u) ^ 1u, s, p)) break;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&s->q_empty[qs]);  // every lane has its codes
+      tc_fence_after_sync();
+      const uint32_t dst = a_base + static_cast<uint32_t>(as) * kStageCols;
+#pragma unroll
+      for (int i = 0; i < 2 * kAK; ++i) {
+        const uint32_t words[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
         uint32_t r[16];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const uint4 v = FMT == kFmtInt4 ? dequant_word(words[4 * half + i], zc2, s2) : dequant_word_fp4(words[4 * half + i], zc2, s2);
-          r[4 * i] = v.x;
-          r[4 * i + 1] = v.y;
-          r[4 * i + 2] = v.z;
-          r[4 * i + 3] = v.w;
+        for (int j = 0; j < 4; ++j) {
+          const uint4 v = FMT == kFmtInt4 ? dequant_word(words[j], zc2, s2) : dequant_word_fp4(words[j], zc2, s2);
+          r[4 * j] = v.x;
+          r[4 * j + 1] = v.y;
+          r[4 * j + 2] = v.z;
+          r[4 * j + 3] = v.w;
         }
-        tmem_st_x16(dst + 16 * half, r);
+        tmem_st_x16(dst + 16 * i, r);
       }
-      pf_load(cur);  // refilled for the step after the next two
       tmem_st_wait();
       tc_fence_before_sync();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&s->a_full[stage]);
-      n += 2;
-      return true;
-    };
-    for (int i = 0; i < steps; i += 3) {  // three register sets in turn
-      if (!expand(a[0])) break;
-      if (i + 1 < steps && !expand(a[1])) break;
-      if (i + 2 < steps && !expand(a[2])) break;
+      if (lane == 0) mbar_arrive(&s->a_full[as]);
     }
   } else {
     // =============================== epilogue warps ===================================
-    const int wr = warp * 32 + lane;  // weight row within a block = TMEM lane
+    const int wr = (warp & 3) * 32 + lane;  // weight row within a block = TMEM lane
+    const int tc0 = (warp >> 2) * (NT / 2);  // this warp's half of the tokens
     constexpr uint32_t kEpiThreads = kEpiWarps * 32;
-    const uint32_t lane_addr = static_cast<uint32_t>(warp * 32) << 16;
+    const uint32_t lane_addr = static_cast<uint32_t>((warp & 3) * 32) << 16;
     int acc = 0, cur_e = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
@@ -391,12 +432,12 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
       const bool hi_ok = col_hi < p.N;
       // 16 token columns at a time (the register budget of the CTA)
 #pragma unroll 1
-      for (int tc = 0; tc < NT; tc += 16) {
+      for (int tc = tc0; tc < tc0 + NT / 2; tc += 16) {
         uint32_t vl[16], vh[16];
         tmem_ld_x16(t0 + tc, vl);
         tmem_ld_x16(t0 + NT + tc, vh);
         tmem_ld_wait();
-        if (tc + 16 == NT) {  // the accumulator is in registers: hand it back
+        if (tc + 16 == tc0 + NT / 2) {  // this warp's share of the accumulator is in registers: hand it back
           tc_fence_before_sync();
           __syncwarp();
           if (lane == 0) mbar_arrive(&s->tmem_empty[acc]);
