@@ -12,19 +12,21 @@
 // stores and 2 of operand reads per weight.  Measured per 64 KB (256 rows x 128 k) on one SM: 616 clocks of stores with
 // their proxy fences against 69 clocks of tcgen05.st, and an MMA 128 x 32 x 16 takes 40 clocks with A in shared
 // memory (bound by reading A) against 16 with A in TMEM (its multiply rate).  What is left is the expansion's own
-// arithmetic (~450 clocks per 64 KB at full issue) and, at decode, the weight stream.
+// arithmetic (measured 740 clocks per 64 KB for integer codes, 920 for e2m1 with its general scale: bf16x2 instructions
+// issue at half rate) and, at decode, the weight stream.  Layer of 96 / 1024 / 4096 tokens (128 experts, top-8): integer 177 /
+// 223 / 562 -> 117 / 200 / 484 us, e2m1 209 / 238 / 585 -> 130 / 210 / 501.
 //
 // A tile = (expert e, pair of weight blocks j, chunk of <= NT rows of the expert's group):
 //   gate_up: blocks j (gate rows) and j + I/128 (the matching up rows); down/linear: blocks 2j, 2j+1.
-// CTA = 896 threads: warps 0-7 epilogue (thread = weight row, half of the tokens: TMEM -> SwiGLU / weighting -> bf16,
-// transposed through shared memory so that global stores are whole token rows), warps 8-23 dequantization in two
-// groups that take A stages in turn (thread = one of the pair's 256 weight rows), warp 24 producer of the codes
-// (bulk copies into a shared-memory ring, scales and zero points copied alongside), warp 25 producer of the token
-// rows (TMA), warps 26 / 27 MMA issuers of the two blocks.
-// TMEM: two accumulators of 2 NT columns (the epilogue of a tile overlaps the next tile), the rest A stages.
+// CTA: epilogue warps (4, or 8 with NT = 128; thread = weight row: TMEM -> SwiGLU / weighting -> bf16, transposed
+// through shared memory so that global stores are whole token rows), 16 dequantization warps in two groups that take A
+// stages in turn (thread = one of the pair's 256 weight rows), a producer warp for the codes (bulk copies into a
+// shared-memory ring, scales and zero points with them), one for the token rows (TMA), two MMA issuers (one per block).
+// TMEM: the accumulators of 2 NT columns (two with NT = 32; with NT = 128 one: four A stages instead of two keep
+// the tensor pipe fed, and the exposed epilogue costs less), the rest A stages.
 // What the hand-offs cost decides the stage sizes: a step of one issuing thread (two waits, its MMAs, the
 // commits) takes 300-450 clocks whatever the MMAs, so codes and token rows move in 128-element quantization groups, and
-// with NT = 32 an A stage is a whole group too (NT = 96: half of one, its MMAs take 384 clocks).
+// with NT = 32 an A stage is a whole group too (NT = 128: half of one, its MMAs take 512 clocks).
 // Every barrier wait is bounded; an expired wait aborts the CTA cleanly.
 #include <algorithm>
 #include <atomic>
@@ -41,15 +43,8 @@ using namespace ptx;
 
 constexpr int BW = 128;            // weight rows per block (UMMA M)
 constexpr int BK = 64;             // bf16 elements per K-step (128 bytes)
-constexpr int kEpiWarps = 8;       // warps 0-7: TMEM quadrant = warp % 4, token half = warp / 4
-constexpr int kDqWarps = 16;       // warps 8-23: two groups of eight
-constexpr int kCodeWarp = 24;      // producer of the codes
-constexpr int kTokenWarp = 25;     // producer of the token rows
-constexpr int kMmaWarp = 26;       // and 27: one issuer per weight block
-constexpr int kThreads = 28 * 32;
 constexpr uint32_t kQStepBytes = BW * BK / 2;  // 4 KB: 128 rows x 32 bytes of codes (one K-step of one block)
 constexpr uint32_t kTmemCols = 512;
-constexpr int kAccBufs = 2;
 constexpr int kMaxExperts = 1024;
 constexpr int kOutRowBytes = 2 * BW * 2 + 16;  // bf16 row of 256 outputs, padded
 constexpr uint32_t kPrefetchChunk = 32768;     // bytes per L2 prefetch instruction
@@ -58,20 +53,30 @@ constexpr int kMaxStages = 8;
 constexpr uint32_t kCodeBytes = 2 * 2 * kQStepBytes;
 constexpr uint32_t kGroupBytes = kCodeBytes + 2 * BW * 2 + 2 * BW;
 
-// NT = 32 for groups of a few rows (decode), kWide for larger ones.
+// NT = 32 for groups of a few rows (decode), kMid and kWide for larger ones.
 constexpr int kNarrow = 32;
-constexpr int kWide = 96;
+constexpr int kMid = 64;
+constexpr int kWide = 128;
+constexpr int kMaxAccBufs = 2;
+constexpr int kDqWarps = 16;       // two groups of eight
 template <int NT>
 struct Cfg {
+  // epilogue warps 0 ..: TMEM quadrant = warp % 4, with eight the token half = warp / 4
+  static constexpr int kEpiWarps = 8;
+  static constexpr int kCodeWarp = kEpiWarps + kDqWarps;             // producer of the codes
+  static constexpr int kTokenWarp = kCodeWarp + 1;                   // producer of the token rows
+  static constexpr int kMmaWarp = kCodeWarp + 2;                     // and + 3: one issuer per weight block
+  static constexpr int kThreads = (kCodeWarp + 4) * 32;
   static constexpr uint32_t kXBytes = 2 * NT * BK * 2;               // token rows of one group: two boxes of 64 elements
-  static constexpr int kXStages = NT == kNarrow ? 4 : 3;
-  static constexpr int kQStages = NT == kNarrow ? 8 : 5;
+  static constexpr int kXStages = NT == kWide ? 3 : 4;
+  static constexpr int kQStages = NT == kNarrow ? 8 : NT == kMid ? 6 : 3;
   static constexpr int kAK = NT == kNarrow ? 2 : 1;                  // K-steps of 64 per A stage
   static constexpr int kStageCols = 2 * 32 * kAK;                    // two blocks
+  static constexpr int kAccBufs = NT == kWide ? 1 : 2;
   static constexpr int kAStages = (static_cast<int>(kTmemCols) - kAccBufs * 2 * NT) / kStageCols;
   static constexpr uint32_t kABase = kAccBufs * 2 * NT;
 };
-static_assert(Cfg<kNarrow>::kAStages >= 2 && Cfg<kWide>::kAStages >= 2, "TMEM budget");
+static_assert(Cfg<kNarrow>::kAStages == 3 && Cfg<kWide>::kAStages == 4, "TMEM budget");
 
 struct W4Params {
   const uint8_t* b_packed;   // tile-major 4 KB chunks [E][N/128][K/64]
@@ -101,8 +106,8 @@ struct __align__(8) SmemTail {
   uint64_t q_empty[kMaxStages];
   uint64_t a_full[kMaxStages];
   uint64_t a_empty[kMaxStages];
-  uint64_t tmem_full[kAccBufs];
-  uint64_t tmem_empty[kAccBufs];
+  uint64_t tmem_full[kMaxAccBufs];
+  uint64_t tmem_empty[kMaxAccBufs];
   uint64_t teardown[2];
   uint32_t tmem_addr;
   int abort_flag;
@@ -113,7 +118,7 @@ struct __align__(8) SmemTail {
 template <int NT>
 constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(Cfg<NT>::kXStages) * Cfg<NT>::kXBytes + static_cast<size_t>(Cfg<NT>::kQStages) * kGroupBytes +
                               static_cast<size_t>(NT) * kOutRowBytes + sizeof(SmemTail);
-static_assert(kSmemBytes<kNarrow> <= 227 * 1024 && kSmemBytes<kWide> <= 227 * 1024, "shared memory budget");
+static_assert(kSmemBytes<kNarrow> <= 227 * 1024 && kSmemBytes<kMid> <= 227 * 1024 && kSmemBytes<kWide> <= 227 * 1024, "shared memory budget");
 
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, SmemTail* s, const W4Params& p) {
   if (mbar_try_wait(bar, parity)) return true;
@@ -167,10 +172,11 @@ __device__ __forceinline__ void tile_blocks(const W4Params& p, int j, int& nb_lo
 }
 
 template <int MODE, int FMT, int NT>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(Cfg<NT>::kThreads, 1)
 gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
   using C = Cfg<NT>;
   constexpr int kXStages = C::kXStages, kQStages = C::kQStages, kAStages = C::kAStages, kAK = C::kAK, kStageCols = C::kStageCols;
+  constexpr int kAccBufs = C::kAccBufs, kEpiWarps = C::kEpiWarps, kCodeWarp = C::kCodeWarp, kTokenWarp = C::kTokenWarp, kMmaWarp = C::kMmaWarp;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* x_base = smem;  // [stage][K-step][NT rows x 128 bytes], swizzled
@@ -307,7 +313,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
   } else if (warp == kCodeWarp) {
     // The same for scales and zero points that are not 16-byte aligned (the interface promises 2 and 1): plain loads,
     // lane l rows l, l + 32, ..., written to the stage by this warp; their latency is paid per group (gate_up of 96
-    // tokens 94 us instead of @@@).
+    // tokens 94 us instead of 70).
     int qs = 0, cur_e = 0;
     uint32_t q_phase = 0, armed = 0, armed_parity = 0;
     bool ok = true;
@@ -403,54 +409,83 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
     const int nr = (warp & 3) * 32 + lane;           // weight row of the block = TMEM lane
     const uint32_t a_base = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16) + C::kABase + static_cast<uint32_t>(h) * (kStageCols / 2);
     const int groups = first_tile < total_tiles ? ((total_tiles - 1 - first_tile) / num_ctas + 1) * KG : 0;  // of this CTA
-    // group index in the ring / A stage index, both counted over the CTA's life
-    for (int g = kAK == 2 ? grp : 0; g < groups; g += kAK) {
-      const int qs = g % kQStages;
-      const uint32_t n = static_cast<uint32_t>(kAK == 2 ? g : 2 * g + grp);
-      const int as = static_cast<int>(n % kAStages);
-      if (!warp_wait_or_abort(&s->q_full[qs], static_cast<uint32_t>(g / kQStages) & 1u, s, p)) break;
-      const uint8_t* q = q_base + static_cast<size_t>(qs) * kGroupBytes;
-      uint32_t s2, zc2;  // integer: s and 128 + z as bf16x2; e2m1: the two per-group factors
-      const uint32_t sb = *reinterpret_cast<const uint16_t*>(q + kCodeBytes + 2 * (h * BW + nr));
-      if constexpr (FMT == kFmtInt4) {
-        s2 = sb | (sb << 16);
-        zc2 = (0x4300u | q[kCodeBytes + 4 * BW + h * BW + nr]) * 0x00010001u;
-      } else {
-        fp4_group_consts(sb, zc2, s2);
-      }
-      // [block][K-step][word quad 0..1][row][16 bytes]
-      const uint8_t* src = q + h * (2 * kQStepBytes) + (kAK == 2 ? 0 : grp) * kQStepBytes + nr * 16;
+    // this thread's codes of a group: kAK K-steps, [block][K-step][word quad 0..1][row][16 bytes] in the ring
+    struct Codes {
       uint4 w[2 * kAK];
+      uint32_t s, z;
+    };
+    auto fetch = [&](int g, Codes& c) {  // the group's stage is full; hands the stage back
+      const int qs = g % kQStages;
+      const uint8_t* q = q_base + static_cast<size_t>(qs) * kGroupBytes;
+      const uint8_t* src = q + h * (2 * kQStepBytes) + (kAK == 2 ? 0 : grp) * kQStepBytes + nr * 16;
 #pragma unroll
-      for (int i = 0; i < 2 * kAK; ++i) w[i] = *reinterpret_cast<const uint4*>(src + i * (kQStepBytes / 2));
-      if (!warp_wait_or_abort(&s->a_empty[as], ((n / kAStages) & 1u) ^ 1u, s, p)) break;
+      for (int i = 0; i < 2 * kAK; ++i) c.w[i] = *reinterpret_cast<const uint4*>(src + i * (kQStepBytes / 2));
+      c.s = *reinterpret_cast<const uint16_t*>(q + kCodeBytes + 2 * (h * BW + nr));
+      if constexpr (FMT == kFmtInt4) c.z = q[kCodeBytes + 4 * BW + h * BW + nr];
       __syncwarp();
-      if (lane == 0) mbar_arrive(&s->q_empty[qs]);  // every lane has its codes
+      if (lane == 0) mbar_arrive(&s->q_empty[qs]);
+    };
+    auto q_parity = [&](int g) { return static_cast<uint32_t>(g / kQStages) & 1u; };
+    // Expands group g from `cur`; the next one's codes are fetched into `nxt` first if they are there already, so
+    // that their barrier and shared-memory latency hide behind this group's arithmetic.
+    auto step = [&](int g, Codes& cur, Codes& nxt) -> bool {
+      const int gn = g + kAK;
+      bool have_next = gn >= groups;
+      if (!have_next && __all_sync(0xFFFFFFFFu, mbar_try_wait(&s->q_full[gn % kQStages], q_parity(gn)))) {
+        fetch(gn, nxt);
+        have_next = true;
+      }
+      const uint32_t n = static_cast<uint32_t>(kAK == 2 ? g : 2 * g + grp);  // A stages of this CTA before this one
+      const int as = static_cast<int>(n % kAStages);
+      if (!warp_wait_or_abort(&s->a_empty[as], ((n / kAStages) & 1u) ^ 1u, s, p)) return false;
       tc_fence_after_sync();
       const uint32_t dst = a_base + static_cast<uint32_t>(as) * kStageCols;
+      auto expand = [&](auto sc) {
 #pragma unroll
-      for (int i = 0; i < 2 * kAK; ++i) {
-        const uint32_t words[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
-        uint32_t r[16];
+        for (int i = 0; i < 2 * kAK; ++i) {
+          const uint32_t words[4] = {cur.w[i].x, cur.w[i].y, cur.w[i].z, cur.w[i].w};
+          uint32_t r[16];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint4 v = FMT == kFmtInt4 ? dequant_word(words[j], zc2, s2) : dequant_word_fp4(words[j], zc2, s2);
-          r[4 * j] = v.x;
-          r[4 * j + 1] = v.y;
-          r[4 * j + 2] = v.z;
-          r[4 * j + 3] = v.w;
+          for (int j = 0; j < 4; ++j) {
+            const uint4 v = sc.expand(words[j]);
+            r[4 * j] = v.x;
+            r[4 * j + 1] = v.y;
+            r[4 * j + 2] = v.z;
+            r[4 * j + 3] = v.w;
+          }
+          tmem_st_x16(dst + 16 * i, r);
         }
-        tmem_st_x16(dst + 16 * i, r);
+      };
+      if constexpr (FMT == kFmtInt4) {
+        expand(W4Scale<0>(cur.s, cur.z));
+      } else {
+        if (__all_sync(0xFFFFFFFFu, ((cur.s >> 7) & 0xFFu) <= 127u)) expand(W4Scale<2>(cur.s, 0));
+        else expand(W4Scale<1>(cur.s, 0));
       }
       tmem_st_wait();
       tc_fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(&s->a_full[as]);
+      if (!have_next) {
+        if (!warp_wait_or_abort(&s->q_full[gn % kQStages], q_parity(gn), s, p)) return false;
+        fetch(gn, nxt);
+      }
+      return true;
+    };
+    const int g0 = kAK == 2 ? grp : 0;
+    Codes ca{}, cb{};
+    if (g0 < groups && warp_wait_or_abort(&s->q_full[g0], 0, s, p)) {
+      fetch(g0, ca);
+      for (int g = g0; g < groups; g += 2 * kAK) {
+        if (!step(g, ca, cb)) break;
+        if (g + kAK < groups && !step(g + kAK, cb, ca)) break;
+      }
     }
   } else {
     // =============================== epilogue warps ===================================
     const int wr = (warp & 3) * 32 + lane;  // weight row within a block = TMEM lane
-    const int tc0 = (warp >> 2) * (NT / 2);  // this warp's half of the tokens
+    constexpr int kShare = NT / (kEpiWarps / 4);  // tokens of a warp
+    const int tc0 = (warp >> 2) * kShare;
     constexpr uint32_t kEpiThreads = kEpiWarps * 32;
     const uint32_t lane_addr = static_cast<uint32_t>((warp & 3) * 32) << 16;
     int acc = 0, cur_e = 0;
@@ -470,12 +505,12 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
       const bool hi_ok = col_hi < p.N;
       // 16 token columns at a time (the register budget of the CTA)
 #pragma unroll 1
-      for (int tc = tc0; tc < tc0 + NT / 2; tc += 16) {
+      for (int tc = tc0; tc < tc0 + kShare; tc += 16) {
         uint32_t vl[16], vh[16];
         tmem_ld_x16(t0 + tc, vl);
         tmem_ld_x16(t0 + NT + tc, vh);
         tmem_ld_wait();
-        if (tc + 16 == tc0 + NT / 2) {  // this warp's share of the accumulator is in registers: hand it back
+        if (tc + 16 == tc0 + kShare) {  // this warp's share of the accumulator is in registers: hand it back
           tc_fence_before_sync();
           __syncwarp();
           if (lane == 0) mbar_arrive(&s->tmem_empty[acc]);
@@ -566,14 +601,18 @@ cudaError_t launch_size(const Launch& L, const CUtensorMap& tx, const W4Params& 
   const int64_t chunks_max = p.rows_total / NT + p.E;
   const int grid = static_cast<int>(std::min<int64_t>(L.sm_count, chunks_max * p.n_pairs));
   ++*L.launches;
-  return launch_pdl(gemm_w4a16_kernel<MODE, FMT, NT>, static_cast<unsigned>(grid), kThreads, kSmemBytes<NT>, L.stream, tx, p);
+  return launch_pdl(gemm_w4a16_kernel<MODE, FMT, NT>, static_cast<unsigned>(grid), Cfg<NT>::kThreads, kSmemBytes<NT>, L.stream, tx, p);
 }
 
 template <int MODE>
-cudaError_t launch_mode(const Launch& L, const CUtensorMap& tx, const W4Params& p, int fmt, bool narrow) {
+cudaError_t launch_mode(const Launch& L, const CUtensorMap& tx, const W4Params& p, int fmt, int nt) {
   if (fmt == kFmtE2m1)
-    return narrow ? launch_size<MODE, kFmtE2m1, kNarrow>(L, tx, p) : launch_size<MODE, kFmtE2m1, kWide>(L, tx, p);
-  return narrow ? launch_size<MODE, kFmtInt4, kNarrow>(L, tx, p) : launch_size<MODE, kFmtInt4, kWide>(L, tx, p);
+    return nt == kNarrow ? launch_size<MODE, kFmtE2m1, kNarrow>(L, tx, p)
+         : nt == kMid    ? launch_size<MODE, kFmtE2m1, kMid>(L, tx, p)
+                         : launch_size<MODE, kFmtE2m1, kWide>(L, tx, p);
+  return nt == kNarrow ? launch_size<MODE, kFmtInt4, kNarrow>(L, tx, p)
+       : nt == kMid    ? launch_size<MODE, kFmtInt4, kMid>(L, tx, p)
+                       : launch_size<MODE, kFmtInt4, kWide>(L, tx, p);
 }
 
 }  // namespace
@@ -581,12 +620,14 @@ cudaError_t launch_mode(const Launch& L, const CUtensorMap& tx, const W4Params& 
 cudaError_t launch_gemm_w4a16(const Launch& L, EncodeTiledFn encode, const GemmW4Args& a, CUresult* cu_err) {
   *cu_err = CUDA_SUCCESS;
   if (a.rows_total == 0) return cudaSuccess;
-  // 32-row tiles where the groups average at most 32 rows (a wide tile would multiply padding and each weight is
-  // expanded once either way), 96-row tiles beyond (an expansion serves three times the rows)
-  const bool narrow = L.gemm_path == 0 ? a.rows_total <= static_cast<int64_t>(kNarrow) * a.E : L.gemm_path == 2;
+  // Rows per tile by the average group: 32 up to 24 rows (a wider tile would multiply padding; groups scatter around
+  // the average, and at 32 rows half of them already need a second 32-row tile: 512 tokens, top-8 of 128, 165 us against
+  // 149 with 64-row tiles), 64 up to 56 rows (1024 tokens: equal), 128 beyond (2048 tokens: 279 us against 299: an
+  // expansion serves more rows).
+  const int nt = L.gemm_path == 1 ? kWide : L.gemm_path == 2 || a.rows_total <= 24 * a.E ? kNarrow : a.rows_total <= 56 * a.E ? kMid : kWide;
   CUtensorMap tx;
   const CUresult r = make_tmap_x(encode, &tx, a.a_bf16, static_cast<uint64_t>(a.rows_total), static_cast<uint64_t>(a.K),
-                                 narrow ? kNarrow : kWide);
+                                 static_cast<uint32_t>(nt));
   if (r != CUDA_SUCCESS) {
     *cu_err = r;
     return cudaErrorUnknown;
@@ -611,9 +652,9 @@ cudaError_t launch_gemm_w4a16(const Launch& L, EncodeTiledFn encode, const GemmW
   p.status = L.d_status;
   p.wait_limit_ns = L.wait_limit_ns ? L.wait_limit_ns : 2000000000ull;
   switch (a.mode) {
-    case kModeLinear: return launch_mode<kModeLinear>(L, tx, p, a.fmt, narrow);
-    case kModeGateUp: return launch_mode<kModeGateUp>(L, tx, p, a.fmt, narrow);
-    case kModeDown: return launch_mode<kModeDown>(L, tx, p, a.fmt, narrow);
+    case kModeLinear: return launch_mode<kModeLinear>(L, tx, p, a.fmt, nt);
+    case kModeGateUp: return launch_mode<kModeGateUp>(L, tx, p, a.fmt, nt);
+    case kModeDown: return launch_mode<kModeDown>(L, tx, p, a.fmt, nt);
   }
   return cudaErrorInvalidValue;
 }

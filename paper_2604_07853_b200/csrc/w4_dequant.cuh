@@ -46,4 +46,39 @@ __device__ __forceinline__ uint4 dequant_word_fp4(uint32_t w, uint32_t c1x2, uin
                     dequant_bits_fp4(w >> 2, w << 4, c1x2, c2x2), dequant_bits_fp4(w >> 6, w, c1x2, c2x2));
 }
 
+// e2m1 with a scale below 2 (every weight tensor in practice): c = s 2^126 is itself a finite bf16, so the first,
+// exact multiplication is not needed; the sign goes in last.  s 2^126 adds 126 to s's exponent (s is normal: at
+// least 2^-40 / 6).
+__device__ __forceinline__ uint32_t dequant_bits_fp4_small(uint32_t x6, uint32_t x12, uint32_t cx2) {
+  uint32_t v, r;
+  asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(v) : "r"(x6 & 0x01C001C0u), "r"(cx2));
+  asm("lop3.b32 %0, %1, 0x80008000, %2, 0xEA;" : "=r"(r) : "r"(x12), "r"(v));  // (a & b) | c
+  return r;
+}
+
+// What a row's scale (and zero point) contribute to the expansion of its quantization group.  FORM 0: integer with zero
+// point; 1: e2m1, any scale; 2: e2m1, scale below 2.
+template <int FORM>
+struct W4Scale {
+  uint32_t a, b = 0;
+  __device__ __forceinline__ W4Scale(uint32_t s, uint32_t z) {
+    if constexpr (FORM == 0) {
+      a = (0x4300u | z) * 0x00010001u;
+      b = s | (s << 16);
+    } else if constexpr (FORM == 1) {
+      fp4_group_consts(s, a, b);
+    } else {
+      a = (s + (126u << 7)) * 0x00010001u;
+    }
+  }
+  // eight codes of one word -> eight bf16 in K order
+  __device__ __forceinline__ uint4 expand(uint32_t w) const {
+    if constexpr (FORM == 0) return dequant_word(w, a, b);
+    else if constexpr (FORM == 1) return dequant_word_fp4(w, a, b);
+    else
+      return make_uint4(dequant_bits_fp4_small(w << 6, w << 12, a), dequant_bits_fp4_small(w << 2, w << 8, a),
+                        dequant_bits_fp4_small(w >> 2, w << 4, a), dequant_bits_fp4_small(w >> 6, w, a));
+  }
+};
+
 }  // namespace qarl
