@@ -54,6 +54,7 @@ constexpr int BNH = 128;          // columns per half tile
 constexpr int BN = 2 * BNH;       // UMMA N
 constexpr int BK = 128;           // one K-block = one 128-byte swizzle span of e4m3
 constexpr int kMaxAccBufs = 4;
+constexpr int kMaxStages = 16;
 constexpr int kPromoWarps = 8;    // warps 0-7
 constexpr int kTmaWarp = 8;
 constexpr int kMmaWarp = 9;
@@ -62,7 +63,6 @@ constexpr int kThreads = 12 * 32;
 // register re-allocation: 256 x 224 + 128 x 56 = 64512 = 384 x 168 (the launch allocation)
 constexpr int kPromoRegs = 224;
 constexpr int kAuxRegs = 56;
-constexpr int kSliceCols = 64;    // columns of each half owned by one promotion warp
 constexpr uint32_t kABytes = BM * BK;
 constexpr uint32_t kBHalfBytes = BNH * BK;
 constexpr uint32_t kTmemCols = 512;
@@ -80,6 +80,7 @@ struct GemmParams {
   int E;
   int n_tiles;             // column tiles per expert
   int I;                   // gate_up: intermediate size (N = 2I)
+  int a_rows, stages;      // COLS = 64: rows of the token box, stages of a_rows x 128 + 8192 bytes
   int early_prefetch;      // decode-sized calls: weight tiles to pull into L2 before the predecessor finishes
   uint16_t* out_bf16;
   float* out_f32;
@@ -94,20 +95,22 @@ struct GemmParams {
 };
 
 // SAVE (gate_up only): the call also wants the bf16 gate_up and / or h rows (a training forward, tests)
-// HALVES (linear): 2 = tiles of 128 x 256; 1 = tiles of 128 x 128 for calls that do not fill the SMs with the others
-template <int MODE, bool SAVE, int HALVES>
+// COLS: columns of a tile, 256 (two halves); 128 and 64 are for dense calls that do not fill the SMs with 256
+template <int MODE, bool SAVE, int COLS>
 struct Cfg {
   static constexpr bool kStaged = MODE != kModeGateUp || SAVE;  // rows leave through the staging boxes
-  static constexpr int kStages = HALVES == 1 ? 5 : kStaged ? 3 : 4;
-  static constexpr uint32_t kStageBytes = kABytes + HALVES * kBHalfBytes;  // 48 or 32 KB
-  static constexpr uint32_t kStaging = kStaged ? kPromoWarps * HALVES * kOutBoxBytes : 0;
-  static constexpr int kCols = HALVES * BNH;                    // UMMA N
-  static constexpr int kAccBufs = static_cast<int>(kTmemCols) / kCols;
+  static constexpr int kHalves = COLS == 256 ? 2 : 1;
+  static constexpr int kSlice = COLS / kHalves / 2;             // columns of each half owned by one promotion warp
+  // ring: fixed 48 or 32 KB stages; with 64 columns as many as fit (a decode call's token box is a few rows, see the host)
+  static constexpr int kStages = COLS == 64 ? 0 : COLS == 128 ? 5 : kStaged ? 3 : 4;
+  static constexpr uint32_t kStageBytes = kABytes + COLS * BK;
+  static constexpr uint32_t kStaging = kStaged && COLS > 64 ? kPromoWarps * kHalves * kOutBoxBytes : 0;
+  static constexpr int kAccBufs = COLS == 256 ? 2 : 4;
 };
 
 struct __align__(8) SmemTail {
-  uint64_t full[5];
-  uint64_t empty[5];
+  uint64_t full[kMaxStages];
+  uint64_t empty[kMaxStages];
   uint64_t tmem_full[kMaxAccBufs];
   uint64_t tmem_empty[kMaxAccBufs];
   uint64_t amax_full[4];       // gate_up: the two warps of a TMEM quadrant have exchanged their row maxima
@@ -120,11 +123,12 @@ struct __align__(8) SmemTail {
   int32_t prefix[kMaxExperts + 1];
 };
 
-template <int MODE, bool SAVE, int HALVES>
-constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(Cfg<MODE, SAVE, HALVES>::kStages) * Cfg<MODE, SAVE, HALVES>::kStageBytes +
-                              Cfg<MODE, SAVE, HALVES>::kStaging + sizeof(SmemTail);
-static_assert(kSmemBytes<kModeGateUp, false, 2> <= 227 * 1024 && kSmemBytes<kModeGateUp, true, 2> <= 227 * 1024 &&
-                  kSmemBytes<kModeLinear, false, 1> <= 227 * 1024,
+template <int MODE, bool SAVE, int COLS>
+constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(Cfg<MODE, SAVE, COLS>::kStages) * Cfg<MODE, SAVE, COLS>::kStageBytes +
+                              Cfg<MODE, SAVE, COLS>::kStaging + sizeof(SmemTail);
+constexpr size_t kSmemLimit = 227 * 1024;
+static_assert(kSmemBytes<kModeGateUp, false, 256> <= kSmemLimit && kSmemBytes<kModeGateUp, true, 256> <= kSmemLimit &&
+                  kSmemBytes<kModeLinear, false, 128> <= kSmemLimit,
               "shared memory budget");
 
 struct TileCoord {
@@ -208,11 +212,12 @@ __device__ __forceinline__ void st_global_2x16(void* dst, const uint32_t (&v)[8]
 
 // The promotion warps (see the header).  What they need is read again here instead of being carried over from
 // the kernel's set-up: with 160 registers of sums and partial sums every long-lived value counts.
-template <int MODE, bool SAVE, int HALVES>
+template <int MODE, bool SAVE, int COLS>
 __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const GemmParams& p, uint8_t* smem, SmemTail* s,
                                                const int first_tile, const int num_ctas, const int total_tiles) {
-  using C = Cfg<MODE, SAVE, HALVES>;
-  constexpr int kAccBufs = C::kAccBufs, kChunks = 4 * HALVES;  // 16-column chunks of this warp's slice
+  using C = Cfg<MODE, SAVE, COLS>;
+  constexpr int kAccBufs = C::kAccBufs, HALVES = C::kHalves, kSliceCols = C::kSlice;
+  constexpr int kPerHalf = kSliceCols / 16, kChunks = kPerHalf * HALVES;  // 16-column chunks of this warp's slices
   uint32_t tid;
   asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
   const int warp = tid >> 5, lane = tid & 31;
@@ -270,9 +275,9 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
     // a warp whose 32 rows all lie past the group's end (ragged tails, decode-sized groups)
     // keeps the barrier protocol going but reads and accumulates nothing
     const bool warp_live = c.m0 + q * 32 < c.m_end;
-    float2 acc[32 * HALVES];  // columns of the low half, then of the high half
+    float2 acc[8 * kChunks];  // columns of the low half, then of the high half
 #pragma unroll
-    for (int j = 0; j < 32 * HALVES; ++j) acc[j] = make_float2(0.0f, 0.0f);
+    for (int j = 0; j < 8 * kChunks; ++j) acc[j] = make_float2(0.0f, 0.0f);
     float2* const acc_lo = acc;
     float2* const acc_hi = acc + (HALVES == 2 ? 32 : 0);
 
@@ -291,10 +296,10 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
         asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(scale.x), "=f"(scale.y)
                      : "r"(scale_at + static_cast<uint32_t>(ks) * static_cast<uint32_t>(sizeof(s->scale[0]))) : "memory");
       };
-      auto chunk_at = [&](uint32_t t0, int c) { return t0 + (c >> 2) * BNH + 16 * (c & 3); };
-      auto add = [&](int c, const uint32_t (&v)[16]) { promote16(acc + 8 * c, v, c < 4 ? scale.x : scale.y); };
+      auto chunk_at = [&](uint32_t t0, int c) { return t0 + (c / kPerHalf) * BNH + 16 * (c % kPerHalf); };
+      auto add = [&](int c, const uint32_t (&v)[16]) { promote16(acc + 8 * c, v, c < kPerHalf ? scale.x : scale.y); };
       auto all_but_last = [&]() {  // every chunk of accumulator ks but the last two sums; on return the last is in flight
-        const uint32_t t0 = tmem + static_cast<uint32_t>(ks * C::kCols);
+        const uint32_t t0 = tmem + static_cast<uint32_t>(ks * COLS);
         tmem_ld_wait();
 #pragma unroll
         for (int c = 0; c < kChunks - 2; c += 2) {
@@ -309,7 +314,7 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
       };
       if (!full_wait()) return;
       tc_fence_after_sync();
-      tmem_ld_x16(tmem + static_cast<uint32_t>(ks * C::kCols), va);
+      tmem_ld_x16(tmem + static_cast<uint32_t>(ks * COLS), va);
       read_scale();
 #pragma unroll 1
       for (int kb = 1; kb < KB; ++kb) {
@@ -323,7 +328,7 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
         release();
         if (!__all_sync(0xFFFFFFFFu, next_ready) && !full_wait()) return;
         tc_fence_after_sync();
-        tmem_ld_x16(tmem + static_cast<uint32_t>(ks * C::kCols), va);
+        tmem_ld_x16(tmem + static_cast<uint32_t>(ks * COLS), va);
         promote16(acc + 8 * (kChunks - 1), vb, last_scale);
         read_scale();
       }
@@ -338,12 +343,12 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
     const int row = c.m0 + r;
     const bool valid = row < c.m_end;
     if ((MODE == kModeLinear || MODE == kModeDown) && p.out_f32 && valid) {  // debug fp32 dump
-      const int col_lo = c.n_tile * C::kCols + hs * kSliceCols;
+      const int col_lo = c.n_tile * COLS + hs * kSliceCols;
       const int col_hi = col_lo + BNH;
       float2* d_lo = reinterpret_cast<float2*>(p.out_f32 + static_cast<int64_t>(row) * p.N + col_lo);
       float2* d_hi = reinterpret_cast<float2*>(p.out_f32 + static_cast<int64_t>(row) * p.N + col_hi);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
+      for (int j = 0; j < kSliceCols / 2; ++j) {
         d_lo[j] = acc_lo[j];
         if (HALVES == 2 && col_hi < p.N) d_hi[j] = acc_hi[j];
       }
@@ -352,12 +357,12 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
       const float w = valid ? __ldg(p.pair_weights + row) : 0.0f;
       const float2 w2 = make_float2(w, w);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
+      for (int j = 0; j < kSliceCols / 2; ++j) {
         acc_lo[j] = __fmul2_rn(w2, acc_lo[j]);
         if (HALVES == 2) acc_hi[j] = __fmul2_rn(w2, acc_hi[j]);
       }
     }
-    if (MODE == kModeGateUp) {
+    if constexpr (MODE == kModeGateUp) {
       // This thread holds gate columns [64 hs, 64 hs + 64) of its row in acc_lo and the up columns of the
       // same h columns in acc_hi.  h = bf16(silu(bf16 gate) * bf16 up); the other warp of the quadrant
       // (w ^ 4) holds the rest of the row's 128-wide quantization group: only the maxima are exchanged.
@@ -423,6 +428,14 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
           }
         }
       }
+    } else if constexpr (COLS == 64) {  // a few rows: 64 bytes of each straight from the registers
+      if (valid) {
+        uint4* d = reinterpret_cast<uint4*>(p.out_bf16 + static_cast<int64_t>(row) * p.N + c.n_tile * COLS + hs * kSliceCols);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          d[j] = make_uint4(bf16x2_bits(acc_lo[4 * j].x, acc_lo[4 * j].y), bf16x2_bits(acc_lo[4 * j + 1].x, acc_lo[4 * j + 1].y),
+                            bf16x2_bits(acc_lo[4 * j + 2].x, acc_lo[4 * j + 2].y), bf16x2_bits(acc_lo[4 * j + 3].x, acc_lo[4 * j + 3].y));
+      }
     } else if (warp_live) {
       boxes_free();
 #pragma unroll
@@ -435,23 +448,27 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
               make_uint4(bf16x2_bits(acc_hi[4 * j].x, acc_hi[4 * j].y), bf16x2_bits(acc_hi[4 * j + 1].x, acc_hi[4 * j + 1].y),
                          bf16x2_bits(acc_hi[4 * j + 2].x, acc_hi[4 * j + 2].y), bf16x2_bits(acc_hi[4 * j + 3].x, acc_hi[4 * j + 3].y));
       }
-      const int col_lo = c.n_tile * C::kCols + hs * kSliceCols;
+      const int col_lo = c.n_tile * COLS + hs * kSliceCols;
       send_boxes(c.m0 + q * 32, c.m_end, col_lo, col_lo + BNH);
     }
   }
-  if (C::kStaged && lane == 0) bulk_wait_group_all();  // this warp's rows are written
+  if (C::kStaging > 0 && lane == 0) bulk_wait_group_all();  // this warp's rows are written
 }
 
-template <int MODE, bool SAVE, int HALVES>
+template <int MODE, bool SAVE, int COLS>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                         const __grid_constant__ CUtensorMap tm_o, const GemmParams p) {
-  using C = Cfg<MODE, SAVE, HALVES>;
-  constexpr int kStages = C::kStages, kAccBufs = C::kAccBufs;
-  constexpr uint32_t kStageBytes = C::kStageBytes;
+  using C = Cfg<MODE, SAVE, COLS>;
+  constexpr int kAccBufs = C::kAccBufs, HALVES = C::kHalves;
+  const int kStages = COLS == 64 ? p.stages : C::kStages;
+  const uint32_t a_bytes = COLS == 64 ? static_cast<uint32_t>(p.a_rows) * BK : kABytes;
+  const uint32_t kStageBytes = a_bytes + COLS * BK;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* out_tile = smem + static_cast<size_t>(kStages) * kStageBytes;
+  // (COLS = 64: the MMA reads 128 token rows from a stage whatever its box holds; what lies behind the box must be shared
+  // memory too, and an output row depends on its own row only)
+  uint8_t* out_tile = smem + static_cast<size_t>(kStages) * kStageBytes + (COLS == 64 ? kABytes : 0);
   SmemTail* s = reinterpret_cast<SmemTail*>(out_tile + C::kStaging);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -474,7 +491,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
   if (warp == kTmaWarp && lane == 0) {
     prefetch_tensormap(&tm_a);
     prefetch_tensormap(&tm_b);
-    if (C::kStaged) prefetch_tensormap(&tm_o);
+    if (C::kStaging > 0) prefetch_tensormap(&tm_o);
   }
   if (warp == kMmaWarp) {
     tmem_alloc(&s->tmem_addr, kTmemCols);
@@ -495,7 +512,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
         row_lo = e * p.N + n_tile * BNH;
         row_hi = row_lo + p.I;
       } else {
-        row_lo = e * p.N + n_tile * C::kCols;
+        row_lo = e * p.N + n_tile * COLS;
         row_hi = row_lo + BNH;
       }
       for (int kb = 0; kb < p.kblocks; ++kb) {
@@ -573,7 +590,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
             row_lo = c.e * p.N + c.n_tile * BNH;
             row_hi = row_lo + p.I;
           } else {
-            row_lo = c.e * p.N + c.n_tile * C::kCols;
+            row_lo = c.e * p.N + c.n_tile * COLS;
             row_hi = row_lo + BNH;
           }
         };
@@ -586,7 +603,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
             ++armed_total;
             if (!wait_or_abort(&s->empty[stage], phase ^ 1, s, p)) { ok = false; break; }
             uint8_t* a_dst = smem + static_cast<size_t>(stage) * kStageBytes;
-            uint8_t* b_dst = a_dst + kABytes;
+            uint8_t* b_dst = a_dst + a_bytes;
             mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
             tma_load_2d(a_dst, &tm_a, &s->full[stage], kb * BK, c.m0);
             tma_load_2d(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo);
@@ -604,7 +621,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
     } else if (warp == kMmaWarp) {
       // =============================== MMA issuer =======================================
       if (elect_one()) {
-        constexpr uint32_t idesc = umma_idesc_e4m3_f32(BM, C::kCols);
+        constexpr uint32_t idesc = umma_idesc_e4m3_f32(BM, COLS);
         int stage = 0, ks = 0;
         uint32_t phase = 0, acc_phase = 0;
         bool ok = true;
@@ -615,8 +632,8 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
             tc_fence_after_sync();
             const uint32_t a_addr = smem_u32(smem + static_cast<size_t>(stage) * kStageBytes);
             const uint64_t a_desc = umma_desc_k_sw128(a_addr);
-            const uint64_t b_desc = umma_desc_k_sw128(a_addr + kABytes);
-            const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(ks * C::kCols);
+            const uint64_t b_desc = umma_desc_k_sw128(a_addr + a_bytes);
+            const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(ks * COLS);
 #pragma unroll
             for (int k4 = 0; k4 < BK / 32; ++k4)  // +32 bytes of K = +2 in the 16-byte address field
               umma_f8(d_tmem, a_desc + 2 * k4, b_desc + 2 * k4, idesc, k4 > 0 ? 1u : 0u);
@@ -651,8 +668,8 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
           nb_lo = c.n_tile;
           nb_hi = c.n_tile + p.I / BNH;
         } else {
-          nb_lo = HALVES * c.n_tile;
-          nb_hi = min(HALVES * c.n_tile + HALVES - 1, NB - 1);
+          nb_lo = COLS == 64 ? c.n_tile / 2 : HALVES * c.n_tile;
+          nb_hi = min(nb_lo + HALVES - 1, NB - 1);
         }
         x0 = p.a_scales + static_cast<int64_t>(min(c.m0 + r0, p.rows_total - 1)) * KB;
         x1 = p.a_scales + static_cast<int64_t>(min(c.m0 + r0 + 32, p.rows_total - 1)) * KB;
@@ -688,7 +705,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
   } else {
     // =============================== promotion warps ==================================
     setmaxnreg_inc<kPromoRegs>();
-    promotion_role<MODE, SAVE, HALVES>(tm_o, p, smem, s, first_tile, num_ctas, total_tiles);
+    promotion_role<MODE, SAVE, COLS>(tm_o, p, smem, s, first_tile, num_ctas, total_tiles);
   }
 
   // ---- teardown ---------------------------------------------------------------------------
@@ -716,18 +733,18 @@ CUresult make_out_tmap(EncodeTiledFn encode, CUtensorMap* m, const void* base, u
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
-CUresult make_tmap(EncodeTiledFn encode, CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols) {
-  // u8 tensor [rows, cols] row-major; box = 128 bytes x 128 rows, 128-byte swizzle, zero fill.
+CUresult make_tmap(EncodeTiledFn encode, CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+  // u8 tensor [rows, cols] row-major; box = 128 bytes x box_rows rows, 128-byte swizzle, zero fill.
   const cuuint64_t dims[2] = {cols, rows};
   const cuuint64_t strides[1] = {cols};
-  const cuuint32_t box[2] = {BK, BM};
+  const cuuint32_t box[2] = {BK, box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return encode(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
-template <int MODE, bool SAVE, int HALVES>
+template <int MODE, bool SAVE, int COLS>
 cudaError_t launch_mode(const Launch& L, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to,
                         const GemmParams& p, int grid) {
   // sticky per function and device; atomic: contexts on several host threads may launch at once (both
@@ -735,13 +752,15 @@ cudaError_t launch_mode(const Launch& L, const CUtensorMap& ta, const CUtensorMa
   static std::atomic<bool> attr_set_dev[64];
   std::atomic<bool>& attr_set = attr_set_dev[L.device & 63];
   if (!attr_set.load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_blockscaled_kernel<MODE, SAVE, HALVES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kSmemBytes<MODE, SAVE, HALVES>));
+    cudaError_t e = cudaFuncSetAttribute(gemm_blockscaled_kernel<MODE, SAVE, COLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(COLS == 64 ? kSmemLimit : kSmemBytes<MODE, SAVE, COLS>));
     if (e != cudaSuccess) return e;
     attr_set.store(true, std::memory_order_release);
   }
+  size_t smem = kSmemBytes<MODE, SAVE, COLS>;
+  if (COLS == 64) smem += kABytes + static_cast<size_t>(p.stages) * (p.a_rows + COLS) * BK;
   ++*L.launches;
-  return launch_pdl(gemm_blockscaled_kernel<MODE, SAVE, HALVES>, static_cast<unsigned>(grid), kThreads, kSmemBytes<MODE, SAVE, HALVES>, L.stream, ta, tb, to, p);
+  return launch_pdl(gemm_blockscaled_kernel<MODE, SAVE, COLS>, static_cast<unsigned>(grid), kThreads, smem, L.stream, ta, tb, to, p);
 }
 
 }  // namespace
@@ -749,20 +768,44 @@ cudaError_t launch_mode(const Launch& L, const CUtensorMap& ta, const CUtensorMa
 cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a, CUresult* cu_err) {
   *cu_err = CUDA_SUCCESS;
   if (a.rows_total == 0) return cudaSuccess;
-  // decode-sized groups: the swapped-operand kernel (bitwise the same rows, bound by the weight stream)
-  if (L.gemm_path == 2 ? ((a.offsets != nullptr || a.E == 1) && a.K / BK <= 64) : (L.gemm_path == 0 && gemm_decode_applies(a)))
+  // decode-sized calls: the swapped-operand kernel (bitwise the same rows, bound by the weight stream).  A dense call
+  // whose 64-column tiles fit on the SMs in one round stays here: each CTA streams one tile and nobody waits for the
+  // drawing of tiles (N = 2048, K = 4096, one token, by graph replay: 14.4 us there, 10.2 here; N = 16384, K = 2048:
+  // 10.9 there, 13.6 here).
+  const bool one_round = a.offsets == nullptr && a.N / 64 <= L.sm_count;
+  if (L.gemm_path == 2 ? ((a.offsets != nullptr || a.E == 1) && a.K / BK <= 64)
+                       : (L.gemm_path == 0 && !one_round && gemm_decode_applies(a)))
     return launch_gemm_decode(L, encode, a, cu_err);
+  // Columns per tile of a dense call: the width whose full rounds over the SMs cost least.  Per round 128 columns take
+  // ~0.6 of what 256 take, 64 ~0.45 (M = 777, N = 2048, K = 4096: 56 tiles of 256 on 148 SMs 23.6 us, 112 of 128
+  // columns 16.5; M = 65: 12.9 us with 128 columns, 11.6 with 64).
+  int cols = BN;
+  if (a.mode == kModeLinear && a.offsets == nullptr) {
+    auto cost = [&](int c, double unit) {
+      const int64_t tiles = ((a.rows_total + BM - 1) / BM) * ((a.N + c - 1) / c);
+      return static_cast<double>((tiles + L.sm_count - 1) / L.sm_count) * unit;
+    };
+    double best = cost(BN, 1.0);
+    if (const double c = cost(128, 0.6); c < best) { best = c; cols = 128; }
+    if (const double c = cost(64, 0.45); c < best) { best = c; cols = 64; }
+  }
+  GemmParams p{};
+  if (cols == 64) {
+    p.a_rows = static_cast<int>(std::min<int64_t>(BM, (a.rows_total + 7) / 8 * 8));
+    const size_t room = kSmemLimit - kSmemBytes<kModeLinear, false, 64> - kABytes;
+    p.stages = static_cast<int>(std::min<size_t>({kMaxStages, room / (static_cast<size_t>(p.a_rows + 64) * BK), static_cast<size_t>(a.K / BK)}));
+  }
   CUtensorMap ta, tb, to{};
-  CUresult r = make_tmap(encode, &ta, a.a_codes, static_cast<uint64_t>(a.rows_total), static_cast<uint64_t>(a.K));
+  CUresult r = make_tmap(encode, &ta, a.a_codes, static_cast<uint64_t>(a.rows_total), static_cast<uint64_t>(a.K),
+                         cols == 64 ? static_cast<uint32_t>(p.a_rows) : BM);
   if (r == CUDA_SUCCESS)
-    r = make_tmap(encode, &tb, a.b_codes, static_cast<uint64_t>(a.E * a.N), static_cast<uint64_t>(a.K));
+    r = make_tmap(encode, &tb, a.b_codes, static_cast<uint64_t>(a.E * a.N), static_cast<uint64_t>(a.K), cols == 64 ? 64 : BNH);
   if (r == CUDA_SUCCESS && a.out_bf16 != nullptr)
     r = make_out_tmap(encode, &to, a.out_bf16, static_cast<uint64_t>(a.rows_total), static_cast<uint64_t>(a.N));
   if (r != CUDA_SUCCESS) {
     *cu_err = r;
     return cudaErrorUnknown;
   }
-  GemmParams p{};
   p.a_scales = a.a_scales;
   p.b_scales = a.b_scales;
   p.offsets = a.offsets;
@@ -771,17 +814,7 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
   p.N = static_cast<int>(a.N);
   p.E = static_cast<int>(a.E);
   p.I = static_cast<int>(a.N / 2);
-  // Dense calls of a few hundred rows leave most SMs idle with 256-column tiles; a round of 128-column tiles takes
-  // ~0.6 of the other's time (M = 777, N = 2048, K = 4096: 56 tiles of 148 SMs, 23.6 us, against 112, @@@).
-  bool narrow = false;
-  if (a.mode == kModeLinear && a.offsets == nullptr) {
-    auto rounds = [&](int cols) {
-      const int64_t tiles = ((a.rows_total + BM - 1) / BM) * ((a.N + cols - 1) / cols);
-      return static_cast<double>((tiles + L.sm_count - 1) / L.sm_count);
-    };
-    narrow = 0.6 * rounds(BNH) < rounds(BN);
-  }
-  p.n_tiles = a.mode == kModeGateUp ? static_cast<int>(a.N / 2 / BNH) : static_cast<int>((a.N + (narrow ? BNH : BN) - 1) / (narrow ? BNH : BN));
+  p.n_tiles = a.mode == kModeGateUp ? static_cast<int>(a.N / 2 / BNH) : static_cast<int>((a.N + cols - 1) / cols);
   p.out_bf16 = a.out_bf16;
   p.out_f32 = a.out_f32;
   p.h_codes = a.h_codes;
@@ -804,11 +837,13 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
   const int grid = static_cast<int>(std::min<int64_t>(L.sm_count, m_tiles_max * p.n_tiles));
   switch (a.mode) {
     case kModeLinear:
-      return narrow ? launch_mode<kModeLinear, false, 1>(L, ta, tb, to, p, grid) : launch_mode<kModeLinear, false, 2>(L, ta, tb, to, p, grid);
+      return cols == 64    ? launch_mode<kModeLinear, false, 64>(L, ta, tb, to, p, grid)
+             : cols == 128 ? launch_mode<kModeLinear, false, 128>(L, ta, tb, to, p, grid)
+                           : launch_mode<kModeLinear, false, 256>(L, ta, tb, to, p, grid);
     case kModeGateUp:
-      return a.out_bf16 || a.h_bf16 ? launch_mode<kModeGateUp, true, 2>(L, ta, tb, to, p, grid)
-                                    : launch_mode<kModeGateUp, false, 2>(L, ta, tb, to, p, grid);
-    case kModeDown: return launch_mode<kModeDown, false, 2>(L, ta, tb, to, p, grid);
+      return a.out_bf16 || a.h_bf16 ? launch_mode<kModeGateUp, true, 256>(L, ta, tb, to, p, grid)
+                                    : launch_mode<kModeGateUp, false, 256>(L, ta, tb, to, p, grid);
+    case kModeDown: return launch_mode<kModeDown, false, 256>(L, ta, tb, to, p, grid);
   }
   return cudaErrorInvalidValue;
 }
