@@ -29,7 +29,8 @@
 // overlap the main loop of the next.  The epilogue writes through shared-memory boxes of 32 rows x 128 bytes and
 // TMA stores: rows stored straight from registers (16 bytes of 32 different rows per instruction, half
 // sectors) took four times as long as the MMAs of a short contraction -- expert dW of 8192 tokens (128 experts,
-// 1536 x 2048, 1.6 GB out) 1010 us of which the stores need 250.  Static persistent schedule, row tiles fastest.  One fixed
+// 1536 x 2048, 1.6 GB out) 1010 us of which the stores need 250.  Static persistent schedule, row tiles fastest
+// (grouped contraction: long and short tiles in turn, see the producer).  One fixed
 // order of accumulation: a result does not depend on the grid or on the other rows.
 // Every wait is bounded (status word + CTA-wide abort flag), as in the other GEMMs.
 #include <algorithm>
@@ -75,6 +76,8 @@ struct Cfg {
 constexpr uint32_t kBlockBytes = 64 * BK * 2;  // one MN-major block: 64 output indices x 64 c-rows
 constexpr uint32_t kTmemCols = 512;
 constexpr int kMaxExperts = 1024;
+constexpr int kTurn = 8;  // grouped contraction: steps of the long tile between two short ones:
+// about the time a tile takes to be written (4 .. 20 measure alike)
 struct Bf16Params {
   int Mo, No, Kc;           // grouped rows: Mo = total rows P;  grouped contraction: Kc unused (from offsets)
   const int32_t* offsets;   // [E + 1] (grouped forms)
@@ -98,6 +101,14 @@ struct __align__(8) SmemTail {
   uint32_t tmem_addr;
   int abort_flag;
 };
+// Grouped contraction: experts by falling row count.  (uint16 and at most kMaxSorted of them: what the ring and the
+// boxes leave of shared memory; more experts are taken in index order.)
+constexpr int kMaxSorted = 512;
+struct SmemOrder {
+  uint32_t step[kMaxStages];    // what a staged step is: accumulator | first << 1 | last << 2 | valid rows << 3
+  int32_t tile_at[2][8];        // list index of the tiles opened in each accumulator, the last eight
+  uint16_t order[kMaxSorted];
+};
 struct SmemLists {  // grouped rows: the tile list
   int32_t off[kMaxExperts + 1];
   int32_t prefix[kMaxExperts + 1];
@@ -106,10 +117,11 @@ template <int GROUP, int MT, int BN>
 constexpr size_t smem_bytes() {
   using C = Cfg<GROUP, MT, BN>;
   return 1024 + static_cast<size_t>(C::kStages) * C::kStageBytes + C::kOutBytes + sizeof(SmemTail) +
-         (GROUP == kGroupedRows ? sizeof(SmemLists) : 0);
+         (GROUP == kGroupedRows ? sizeof(SmemLists) : GROUP == kGroupedContraction ? sizeof(SmemOrder) : 0);
 }
 static_assert(smem_bytes<kDense, 1, 256>() <= 227 * 1024 && smem_bytes<kDense, 1, 192>() <= 227 * 1024 &&
-                  smem_bytes<kDense, 2, 256>() <= 227 * 1024 && smem_bytes<kGroupedRows, 1, 256>() <= 227 * 1024,
+                  smem_bytes<kDense, 2, 256>() <= 227 * 1024 && smem_bytes<kGroupedRows, 1, 256>() <= 227 * 1024 &&
+                  smem_bytes<kGroupedContraction, 1, 256>() <= 227 * 1024,
               "shared memory budget");
 
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, SmemTail* s, const Bf16Params& p) {
@@ -135,6 +147,27 @@ __device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parit
   return __all_sync(0xFFFFFFFFu, wait_or_abort(bar, parity, s, p) ? 1 : 0) != 0;
 }
 
+// Which accumulator's tile is complete (the whole warp takes the same answer); -1 after an abort.
+__device__ __forceinline__ int either_full(SmemTail* s, const Bf16Params& p, uint32_t parity0, uint32_t parity1) {
+  unsigned long long t0 = 0;
+  for (int spins = 0;; ++spins) {
+    const bool r0 = mbar_test_wait(&s->tmem_full[0], parity0), r1 = mbar_test_wait(&s->tmem_full[1], parity1);
+    if (__all_sync(0xFFFFFFFFu, r0)) return 0;
+    if (__all_sync(0xFFFFFFFFu, r1)) return 1;
+    if ((spins & 255) == 255) {
+      const unsigned long long now = globaltimer_ns();
+      if (t0 == 0) t0 = now;
+      bool stop = *reinterpret_cast<volatile int*>(&s->abort_flag) != 0;
+      if (now - t0 > p.wait_limit_ns) {
+        set_status(p.status, QARL_ERR_DEVICE_TIMEOUT);
+        *reinterpret_cast<volatile int*>(&s->abort_flag) = 1;
+        stop = true;
+      }
+      if (__any_sync(0xFFFFFFFFu, stop)) return -1;
+    }
+  }
+}
+
 __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
   const __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&b);
@@ -154,6 +187,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   uint8_t* out_boxes = smem + static_cast<size_t>(kStages) * kStageBytes;
   SmemTail* s = reinterpret_cast<SmemTail*>(out_boxes + C::kOutBytes);
   SmemLists* lists = reinterpret_cast<SmemLists*>(s + 1);
+  SmemOrder* list = reinterpret_cast<SmemOrder*>(s + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   pdl_trigger();
@@ -185,6 +219,24 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   if (GROUP == kGroupedRows) {
     build_tile_list(lists->off, lists->prefix, p.offsets, p.Mo, p.E, TM, n_tiles);
   }
+  auto expert_rows = [&](int e, int& first) {  // grouped contraction; whatever the array holds stays inside the tensors
+    first = min(max(__ldg(p.offsets + e), 0), p.rows_total);
+    return max(min(max(__ldg(p.offsets + e + 1), 0), p.rows_total) - first, 0);
+  };
+  if (GROUP == kGroupedContraction && p.E <= kMaxSorted) {
+    int* rows = reinterpret_cast<int*>(out_boxes);  // (free until the first tile is written out)
+    for (int e = threadIdx.x; e < p.E; e += C::kThreads) {
+      int first;
+      rows[e] = expert_rows(e, first);
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < p.E; e += C::kThreads) {
+      const int mine = rows[e];
+      int rank = 0;
+      for (int f = 0; f < p.E; ++f) rank += rows[f] > mine || (rows[f] == mine && f < e);
+      list->order[rank] = static_cast<uint16_t>(e);
+    }
+  }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -202,20 +254,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     int e;       // grouped contraction: whose output matrix
     int b_row0;  // K-major B: first row of the expert's block
   };
-  // `cur`: where the caller's walk over the list stands; for the grouped contraction the caller's next pair
-  // of group boundaries, loaded one tile ahead.
-  struct Walk {
-    int cur_e = 0;
-    int lo = 0, hi = 0;
-  };
-  auto bounds_of = [&](int T, Walk& w) {
-    if (GROUP == kGroupedContraction && T < total_tiles) {
-      const int e = T / (m_tiles * n_tiles);
-      w.lo = __ldg(p.offsets + e);
-      w.hi = __ldg(p.offsets + e + 1);
-    }
-  };
-  auto tile_of = [&](int T, Walk& w) {
+  auto tile_of = [&](int T, int& cur_e) {  // cur_e: where the caller's walk over the groups stands
     Tile t{};
     t.last_valid = BK;
     if (GROUP == kDense) {
@@ -233,7 +272,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       t.KS = (p.Kc + BK - 1) / BK;  // a ragged last step reads zeros (TMA out-of-range fill)
       t.row_end = p.Mo;
     } else if (GROUP == kGroupedRows) {
-      const TileCoord c = decode_tile(lists->off, lists->prefix, TM, T, w.cur_e);
+      const TileCoord c = decode_tile(lists->off, lists->prefix, TM, T, cur_e);
       t.i0 = c.m0;
       t.j0 = c.n_tile * BN;
       t.KS = p.Kc / BK;             // Kc is a multiple of 64 here: a step never runs into the next expert's weights
@@ -241,38 +280,50 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       t.b_c0 = c.e * p.Kc;          // MN-major B: the expert's [Kc, No] block starts at row e Kc
       t.b_row0 = c.e * p.No;        // K-major B: the expert's [No, Kc] block starts at row e No
       t.row_end = c.m_end;
-    } else {
-      const int per_e = m_tiles * n_tiles;
-      const int e = T / per_e, r = T % per_e;
-      t.i0 = (r % m_tiles) * TM;
-      t.j0 = (r / m_tiles) * BN;
-      const int first = min(max(w.lo, 0), p.rows_total);
-      const int rows = max(min(max(w.hi, 0), p.rows_total) - first, 0);
-      bounds_of(T + grid, w);
-      t.KS = (rows + BK - 1) / BK;
-      t.last_valid = rows - (t.KS - 1) * BK;
-      t.a_c0 = t.b_c0 = first;
-      t.row_end = p.Mo;
-      t.e = e;
     }
     return t;
   };
-
+  // Grouped contraction: this CTA's list holds every grid-th tile of the experts by falling row count, the direction
+  // turning round with each lap (so that the CTAs' sums of rows stay close).
+  const int list_len = total_tiles / grid + ((total_tiles / grid & 1 ? grid - 1 - static_cast<int>(blockIdx.x) : static_cast<int>(blockIdx.x)) < total_tiles % grid);
+  auto list_tile = [&](int i) {
+    const int T = i * grid + (i & 1 ? grid - 1 - static_cast<int>(blockIdx.x) : static_cast<int>(blockIdx.x));
+    const int per_e = m_tiles * n_tiles, r = T % per_e;
+    Tile t{};
+    t.e = p.E <= kMaxSorted ? list->order[T / per_e] : T / per_e;
+    t.i0 = (r % m_tiles) * TM;
+    t.j0 = (r / m_tiles) * BN;
+    int first;
+    const int rows = expert_rows(t.e, first);
+    t.KS = (rows + BK - 1) / BK;
+    t.last_valid = rows - (t.KS - 1) * BK;
+    t.a_c0 = t.b_c0 = first;
+    t.row_end = p.Mo;
+    return t;
+  };
+  int live_tiles = 0;  // of the list: with rows
+  if (GROUP == kGroupedContraction) {
+    for (int base = 0; base < list_len; base += 32)
+      live_tiles += __popc(__ballot_sync(0xFFFFFFFFu, base + lane < list_len && list_tile(base + lane).KS > 0));
+  }
   if (warp == kTmaWarp) {
     if (elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
       uint32_t armed = 0, armed_parity = 0;
       bool ok = true;
-      Walk walk;
-      bounds_of(blockIdx.x, walk);
-      for (int T = blockIdx.x; ok && T < total_tiles; T += grid) {
-        const Tile t = tile_of(T, walk);
+      // steps [from, to) of tile t into the ring
+      auto feed = [&](const Tile& t, int from, int to, int acc) {
         const int i0 = t.i0, j0 = t.j0;
-        for (int ks = 0; ks < t.KS; ++ks) {
-          if (!wait_or_abort(&s->empty[stage], phase ^ 1, s, p)) { ok = false; break; }
+        for (int ks = from; ks < to; ++ks) {
+          if (!wait_or_abort(&s->empty[stage], phase ^ 1, s, p)) { ok = false; return; }
           uint8_t* a_dst = smem + static_cast<size_t>(stage) * kStageBytes;
           uint8_t* b_dst = a_dst + kABytes;
+          if (GROUP == kGroupedContraction) {
+            const bool last = ks == t.KS - 1;
+            *reinterpret_cast<volatile uint32_t*>(&list->step[stage]) =
+                acc | (ks == 0 ? 2u : 0u) | (last ? 4u : 0u) | static_cast<uint32_t>(last ? t.last_valid : BK) << 3;
+          }
           mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
           if (A_MN && p.a3d) {
             tma_load_3d(a_dst, &tm_a, &s->full[stage], 0, t.a_c0 + ks * BK, i0 / 64);
@@ -296,6 +347,38 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
           armed_parity = (armed_parity & ~(1u << stage)) | (phase << stage);
           if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
+      };
+      if constexpr (GROUP == kGroupedContraction) {
+        // Two tiles at a time, one per accumulator: long ones from the head of the list in the first, short ones
+        // from its tail in the second, a short one whole after every kTurn steps of the long one.  Every tile writes
+        // 128 KB however few rows its expert has, so a run of short tiles is bound by the stores and a long tile by
+        // its MMAs; taken in turn they overlap (8192 tokens, 128 experts with Zipf popularity 1.1: the two dW GEMMs
+        // 1027 us tile after tile by expert, 844 so; 32768 tokens 2.68 -> 2.28 ms).
+        int head = 0, tail = list_len - 1;
+        uint32_t opened[2] = {0, 0};
+        auto open = [&](int i, int acc) {
+          const Tile t = list_tile(i);
+          if (t.KS > 0) *reinterpret_cast<volatile int32_t*>(&list->tile_at[acc][opened[acc]++ & 7]) = i;
+          return t;
+        };
+        while (ok && head <= tail) {
+          const Tile t = open(head++, 0);
+          for (int ks = 0; ok && ks < t.KS;) {
+            const int to = head <= tail ? min(ks + kTurn, t.KS) : t.KS;
+            feed(t, ks, to, 0);
+            ks = to;
+            if (ok && head <= tail) {
+              const Tile u = open(tail--, 1);
+              feed(u, 0, u.KS, 1);
+            }
+          }
+        }
+      } else {
+        int cur_e = 0;
+        for (int T = blockIdx.x; ok && T < total_tiles; T += grid) {
+          const Tile t = tile_of(T, cur_e);
+          feed(t, 0, t.KS, 0);
+        }
       }
       if (!ok) {
         for (int i = 0; i < kStages; ++i)
@@ -305,48 +388,70 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   } else if (warp == kMmaWarp) {
     if (elect_one()) {
       constexpr uint32_t idesc = umma_idesc_bf16_f32_major(BM, BN, A_MN, B_MN);
-      int stage = 0, acc = 0;
-      uint32_t phase = 0, acc_phase = 0, fix_phase = 0;  // fix_phase: a bit per stage, it flips only when the stage held a ragged step
+      int stage = 0;
+      uint32_t phase = 0;
       bool ok = true;
-      Walk walk;
-      bounds_of(blockIdx.x, walk);
-      for (int T = blockIdx.x; ok && T < total_tiles; T += grid) {
-        const Tile t = tile_of(T, walk);
-        if (t.KS == 0) continue;  // an expert without rows: the epilogue writes zeros, no accumulator is used
-        if (!wait_or_abort(&s->tmem_empty[acc], acc_phase ^ 1, s, p)) { ok = false; break; }
-        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * MT) * BN;
-        for (int ks = 0; ks < t.KS; ++ks) {
+      // the first `slices` 16-element slices of the staged step; 16 contraction elements further on: 32 bytes
+      // inside a K-major row, 16 rows of 128 bytes in an MN-major block (start-address field counts 16-byte units)
+      auto issue = [&](uint32_t d_tmem, bool first, int slices) {
+        tc_fence_after_sync();
+        const uint32_t a_addr = smem_u32(smem + static_cast<size_t>(stage) * kStageBytes);
+        const uint32_t b_addr = a_addr + kABytes;
+        const uint64_t a_desc = A_MN ? umma_desc_mn_sw128(a_addr, kBlockBytes) : umma_desc_k_sw128(a_addr);
+        const uint64_t b_desc = B_MN ? umma_desc_mn_sw128(b_addr, kBlockBytes) : umma_desc_k_sw128(b_addr);
+        constexpr uint32_t a_step = A_MN ? (16 * 128) >> 4 : 32 >> 4;
+        constexpr uint32_t b_step = B_MN ? (16 * 128) >> 4 : 32 >> 4;
+        if (slices == BK / 16) {
+#pragma unroll
+          for (int mt = 0; mt < MT; ++mt)  // the 128-row halves of A share the B tile
+#pragma unroll
+            for (int k4 = 0; k4 < BK / 16; ++k4)
+              umma_bf16(d_tmem + mt * BN, a_desc + mt * (kAHalfBytes >> 4) + a_step * k4, b_desc + b_step * k4, idesc,
+                        (!first || k4 > 0) ? 1u : 0u);
+        } else {  // (MT is 1 in the form that has these)
+          for (int k4 = 0; k4 < slices; ++k4)
+            umma_bf16(d_tmem, a_desc + a_step * k4, b_desc + b_step * k4, idesc, (!first || k4 > 0) ? 1u : 0u);
+        }
+        umma_commit(&s->empty[stage]);
+      };
+      auto next_stage = [&]() {
+        if (++stage == kStages) { stage = 0; phase ^= 1; }
+      };
+      if constexpr (GROUP == kGroupedContraction) {
+        uint32_t acc_phase = 0, fix_phase = 0;  // a bit per accumulator; per stage, flipping only when it held a ragged step
+        for (int done = 0; done < live_tiles;) {
           if (!wait_or_abort(&s->full[stage], phase, s, p)) { ok = false; break; }
-          const bool ragged = GROUP == kGroupedContraction && ks == t.KS - 1 && t.last_valid < BK;
-          if (ragged) {
+          const uint32_t step = *reinterpret_cast<volatile uint32_t*>(&list->step[stage]);
+          const uint32_t acc = step & 1u;
+          const int valid = static_cast<int>(step >> 3);
+          if ((step & 2u) && !wait_or_abort(&s->tmem_empty[acc], ((acc_phase >> acc) & 1u) ^ 1u, s, p)) { ok = false; break; }
+          if (valid < BK) {
             if (!wait_or_abort(&s->fixed[stage], (fix_phase >> stage) & 1u, s, p)) { ok = false; break; }
             fix_phase ^= 1u << stage;
           }
-          tc_fence_after_sync();
-          const uint32_t a_addr = smem_u32(smem + static_cast<size_t>(stage) * kStageBytes);
-          const uint32_t b_addr = a_addr + kABytes;
-          const uint64_t a_desc = A_MN ? umma_desc_mn_sw128(a_addr, kBlockBytes) : umma_desc_k_sw128(a_addr);
-          const uint64_t b_desc = B_MN ? umma_desc_mn_sw128(b_addr, kBlockBytes) : umma_desc_k_sw128(b_addr);
-          // 16 contraction elements further on: 32 bytes inside a K-major row, 16 rows of 128 bytes
-          // in an MN-major block (start-address field counts 16-byte units)
-          constexpr uint32_t a_step = A_MN ? (16 * 128) >> 4 : 32 >> 4;
-          constexpr uint32_t b_step = B_MN ? (16 * 128) >> 4 : 32 >> 4;
-          if (!ragged) {
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt)  // the 128-row halves of A share the B tile
-#pragma unroll
-              for (int k4 = 0; k4 < BK / 16; ++k4)
-                umma_bf16(d_tmem + mt * BN, a_desc + mt * (kAHalfBytes >> 4) + a_step * k4, b_desc + b_step * k4, idesc,
-                          (ks > 0 || k4 > 0) ? 1u : 0u);
-          } else {  // (MT is 1 in this form) only the slices that hold rows of the expert
-            for (int k4 = 0; 16 * k4 < t.last_valid; ++k4)
-              umma_bf16(d_tmem, a_desc + a_step * k4, b_desc + b_step * k4, idesc, (ks > 0 || k4 > 0) ? 1u : 0u);
+          issue(tmem_base + acc * BN, (step & 2u) != 0, (valid + 15) / 16);
+          if (step & 4u) {
+            umma_commit(&s->tmem_full[acc]);
+            acc_phase ^= 1u << acc;
+            ++done;
           }
-          umma_commit(&s->empty[stage]);
-          if (ks == t.KS - 1) umma_commit(&s->tmem_full[acc]);
-          if (++stage == kStages) { stage = 0; phase ^= 1; }
+          next_stage();
         }
-        if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1; }
+      } else {
+        int acc = 0, cur_e = 0;
+        uint32_t acc_phase = 0;
+        for (int T = blockIdx.x; ok && T < total_tiles; T += grid) {
+          const Tile t = tile_of(T, cur_e);
+          if (t.KS == 0) continue;  // an empty contraction: the epilogue writes zeros, no accumulator is used
+          if (!wait_or_abort(&s->tmem_empty[acc], acc_phase ^ 1, s, p)) { ok = false; break; }
+          for (int ks = 0; ks < t.KS; ++ks) {
+            if (!wait_or_abort(&s->full[stage], phase, s, p)) { ok = false; break; }
+            issue(tmem_base + static_cast<uint32_t>(acc * MT) * BN, ks == 0, BK / 16);
+            if (ks == t.KS - 1) umma_commit(&s->tmem_full[acc]);
+            next_stage();
+          }
+          if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1; }
+        }
       }
       // Nothing of this CTA's tensor work may be in flight when its TMEM and shared memory go
       // away: after an abort some MMAs may still be executing, so wait (bounded) for them.
@@ -362,48 +467,34 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     // did this itself once: ~2000 clocks of a tile's ~12000).
     int stage = 0;
     uint32_t phase = 0;
-    Walk walk;
-    bounds_of(blockIdx.x, walk);
-    for (int T = blockIdx.x; T < total_tiles; T += grid) {
-      const Tile t = tile_of(T, walk);
-      if (t.KS == 0) continue;
-      // every step is followed (and counted in `empty`): a parity wait tells neighbouring fills apart, no more
-      bool ok = true;
-      for (int ks = 0; ks < t.KS; ++ks) {
-        if (!warp_wait_or_abort(&s->full[stage], phase, s, p)) { ok = false; break; }
-        if (ks == t.KS - 1 && t.last_valid < BK) {
-          uint8_t* a_tile = smem + static_cast<size_t>(stage) * kStageBytes;
-          const int nrows = -t.last_valid & 15;
-          for (int idx = lane; idx < (TM / 64) * nrows * 8; idx += 32) {
-            const int blk = idx / (nrows * 8), rem = idx % (nrows * 8);
-            *reinterpret_cast<uint4*>(a_tile + blk * kBlockBytes + (t.last_valid + rem / 8) * 128 + (rem % 8) * 16) =
-                make_uint4(0, 0, 0, 0);
-          }
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&s->fixed[stage]);
+    // every step is followed (and counted in `empty`): a parity wait tells neighbouring fills apart, no more
+    for (int done = 0; done < live_tiles;) {
+      if (!warp_wait_or_abort(&s->full[stage], phase, s, p)) break;
+      const uint32_t step = *reinterpret_cast<volatile uint32_t*>(&list->step[stage]);
+      const int valid = static_cast<int>(step >> 3);
+      if (valid < BK) {
+        uint8_t* a_tile = smem + static_cast<size_t>(stage) * kStageBytes;
+        const int nrows = -valid & 15;
+        for (int idx = lane; idx < (TM / 64) * nrows * 8; idx += 32) {
+          const int blk = idx / (nrows * 8), rem = idx % (nrows * 8);
+          *reinterpret_cast<uint4*>(a_tile + blk * kBlockBytes + (valid + rem / 8) * 128 + (rem % 8) * 16) = make_uint4(0, 0, 0, 0);
         }
-        if (lane == 0) mbar_arrive(&s->empty[stage]);
-        if (++stage == kStages) { stage = 0; phase ^= 1; }
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&s->fixed[stage]);
       }
-      if (!ok) break;
+      if (step & 4u) ++done;
+      __syncwarp();  // every lane has read the step's word
+      if (lane == 0) mbar_arrive(&s->empty[stage]);
+      if (++stage == kStages) { stage = 0; phase ^= 1; }
     }
   } else if (warp < kEpiWarps) {
     // =============================== epilogue warps: TMEM -> box -> TMA store ==========
     const uint32_t lane_addr = static_cast<uint32_t>((warp & 3) * 32) << 16;
     uint8_t* my_box = out_boxes + static_cast<size_t>(warp) * kOutBoxBytes;
     constexpr int kTurns = kEpiWarps / 4;  // warps that share a quadrant's columns
-    int acc = 0;
-    uint32_t acc_phase = 0;
-    Walk walk;
-    bounds_of(blockIdx.x, walk);
-    for (int T = blockIdx.x; T < total_tiles; T += grid) {
-      const Tile t = tile_of(T, walk);
-      const bool have_acc = t.KS > 0;  // an expert without rows gets zeros
-      if (have_acc) {
-        if (!warp_wait_or_abort(&s->tmem_full[acc], acc_phase, s, p)) break;
-        tc_fence_after_sync();
-      }
+    // this warp's share of tile t out of accumulator `acc` (have_acc false: an expert without rows gets zeros)
+    auto write_out = [&](const Tile& t, const bool have_acc, const int acc) {
 #pragma unroll 1
       for (int mt = 0; mt < MT; ++mt) {
         const int row0 = t.i0 + mt * BM + (warp & 3) * 32;
@@ -487,6 +578,37 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&s->tmem_empty[acc]);
+      }
+    };
+    if constexpr (GROUP == kGroupedContraction) {
+      if (live_tiles < list_len) {
+        for (int i = 0; i < list_len; ++i) {
+          const Tile t = list_tile(i);
+          if (t.KS == 0) write_out(t, false, 0);
+        }
+      }
+      uint32_t seen[2] = {0, 0};
+      for (int done = 0; done < live_tiles; ++done) {  // whichever accumulator is complete
+        const int acc = either_full(s, p, seen[0] & 1u, seen[1] & 1u);
+        if (acc < 0) break;
+        tc_fence_after_sync();
+        const int i = *reinterpret_cast<volatile int32_t*>(&list->tile_at[acc][(acc ? seen[1] : seen[0]) & 7]);
+        if (acc) ++seen[1];
+        else ++seen[0];
+        write_out(list_tile(i), true, acc);
+      }
+    } else {
+      int acc = 0, cur_e = 0;
+      uint32_t acc_phase = 0;
+      for (int T = blockIdx.x; T < total_tiles; T += grid) {
+        const Tile t = tile_of(T, cur_e);
+        if (t.KS == 0) {
+          write_out(t, false, 0);
+          continue;
+        }
+        if (!warp_wait_or_abort(&s->tmem_full[acc], acc_phase, s, p)) break;
+        tc_fence_after_sync();
+        write_out(t, true, acc);
         if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1; }
       }
     }

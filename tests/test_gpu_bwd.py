@@ -148,6 +148,15 @@ def test_grouped_exact_on_integer_data(ctx):
     check_grouped(ctx, 3, [0, 0, 7, 0], 192, 512, exact=True)
 
 
+@pytest.mark.parametrize("sizes", [
+    [3000] + [1] * 40 + [700, 64, 0, 65],                # one long contraction, many short ones taken between its steps
+    [(7 * e) % 70 if e % 5 else 0 for e in range(512)],  # the largest count of experts that is ordered by rows
+    [(7 * e) % 70 if e % 5 else 0 for e in range(513)],  # one more: index order, empty experts in between
+], ids=["long_and_short", "512", "513"])
+def test_grouped_order_of_tiles(ctx, sizes):
+    check_grouped(ctx, 7, sizes, 128, 520, exact=True)
+
+
 def test_grouped_random_data(ctx):
     check_grouped(ctx, 4, [300, 17, 0, 1000, 64, 129], 256, 512)
 
