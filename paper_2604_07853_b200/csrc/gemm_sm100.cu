@@ -81,6 +81,7 @@ struct GemmParams {
   int n_tiles;             // column tiles per expert
   int I;                   // gate_up: intermediate size (N = 2I)
   int a_rows, stages;      // COLS = 64: rows of the token box, stages of a_rows x 128 + 8192 bytes
+  int weights_once;        // few row tiles per expert: weights are loaded with the evict-first policy
   int early_prefetch;      // decode-sized calls: weight tiles to pull into L2 before the predecessor finishes
   uint16_t* out_bf16;
   float* out_f32;
@@ -515,9 +516,10 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
         row_lo = e * p.N + n_tile * COLS;
         row_hi = row_lo + BNH;
       }
+      const uint64_t stream_once = l2_policy_evict_first();
       for (int kb = 0; kb < p.kblocks; ++kb) {
-        tma_prefetch_2d(&tm_b, kb * BK, row_lo);
-        if (HALVES == 2) tma_prefetch_2d(&tm_b, kb * BK, row_hi);
+        tma_prefetch_2d_hint(&tm_b, kb * BK, row_lo, stream_once);
+        if (HALVES == 2) tma_prefetch_2d_hint(&tm_b, kb * BK, row_hi, stream_once);
       }
     }
   }
@@ -582,6 +584,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
         uint32_t phase = 0;
         uint32_t armed = 0, armed_parity = 0;  // per-stage: has a load in flight / its parity
         int armed_total = 0;
+        const uint64_t stream_once = l2_policy_evict_first();
         int cur_e = 0;
         bool ok = true;
         // weight rows of a tile's two halves
@@ -606,8 +609,13 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
             uint8_t* b_dst = a_dst + a_bytes;
             mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
             tma_load_2d(a_dst, &tm_a, &s->full[stage], kb * BK, c.m0);
-            tma_load_2d(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo);
-            if (HALVES == 2) tma_load_2d(b_dst + kBHalfBytes, &tm_b, &s->full[stage], kb * BK, row_hi);
+            if (p.weights_once) {
+              tma_load_2d_hint(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo, stream_once);
+              if (HALVES == 2) tma_load_2d_hint(b_dst + kBHalfBytes, &tm_b, &s->full[stage], kb * BK, row_hi, stream_once);
+            } else {
+              tma_load_2d(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo);
+              if (HALVES == 2) tma_load_2d(b_dst + kBHalfBytes, &tm_b, &s->full[stage], kb * BK, row_hi);
+            }
             armed |= 1u << stage;
             armed_parity = (armed_parity & ~(1u << stage)) | (phase << stage);
             if (++stage == kStages) { stage = 0; phase ^= 1; }
@@ -825,6 +833,10 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
   p.status = L.d_status;
   p.wait_limit_ns = L.wait_limit_ns ? L.wait_limit_ns : 2000000000ull;
   p.stop_after_stages = L.stop_after_stages;
+  // About one row tile per expert: a weight is read once, and read with the evict-first policy it does not push the
+  // small tensors that pass between the kernels out of L2 (1501 tokens, 128 experts: gate_up 97 -> 91 us, down 60 -> 57,
+  // combine 16 -> 13).
+  p.weights_once = a.offsets != nullptr && a.rows_total <= a.E * BM;
   // decode-sized call (at most one row tile per expert): see the early prefetch in the kernel
   if (a.rows_total <= a.E * BM) {
     const int64_t tile_bytes = static_cast<int64_t>(p.kblocks) * 2 * kBHalfBytes;
