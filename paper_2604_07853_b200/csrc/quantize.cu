@@ -190,33 +190,33 @@ __device__ __forceinline__ uint32_t w4_word(const uint4& v, const W4Group& g) {
 
 // ---- FP4 (e2m1) weights (Sec. 2.2, floating-point quantization): s = amax / 6, W_q = [W / s]_FP4 ----
 // Same groups, code order and storage as the integer format; s = bf16(max(amax, 2^-40) / 6).
-// The magnitude code of |w| / s rounded to the nearest of 0, .5, 1, 1.5, 2, 3, 4, 6 (ties to the even
-// code, saturating) is the number of rounding boundaries b = .25 .75 1.25 1.75 2.5 3.5 5 it passes, where a
-// value exactly on a boundary goes to the neighbour with mantissa bit 0 (so the boundaries are
-// exclusive, inclusive, exclusive, ...).  As above, the sign of |w| - b s from one bf16x2 FMA decides
-// each comparison exactly.  Three levels give the three bits: b = 1.75 (>=); then 3.5 or .75 (>=); then 5,
-// 2.5, 1.25 or .25 (>).  With P1, P2 = +-1 for passed / not passed, the next boundaries are the exact
-// bf16 polynomials  b1 = 2.125 + 1.375 P1  and  b0 = (2.25 + 1.5 P1) + P2 (.875 + .375 P1),  kept negated.
-template <int J>
-__device__ __forceinline__ uint32_t fp4_codes2(uint32_t word, uint32_t w2, uint32_t s2) {
-  const uint32_t a2 = w2 & 0x7FFF7FFFu;
-  uint32_t t = fma_bf2(0xBFE0BFE0u /* -1.75 */, s2, a2) + kTieUp;
-  word |= (~t >> (13 - 4 * J)) & (0x00040004u << (4 * J));
-  const uint32_t p1 = 0x3F803F80u | (t & kSigns);                        // +1 where passed, else -1
-  const uint32_t nb1 = fma_bf2(p1, 0xBFB0BFB0u /* -1.375 */, 0xC008C008u /* -2.125 */);
-  t = fma_bf2(nb1, s2, a2) + kTieUp;
-  word |= (~t >> (14 - 4 * J)) & (0x00020002u << (4 * J));
-  const uint32_t p2 = 0x3F803F80u | (t & kSigns);
-  const uint32_t u = fma_bf2(p1, 0xBFC0BFC0u /* -1.5 */, 0xC010C010u /* -2.25 */);
-  const uint32_t v = fma_bf2(p1, 0xBEC0BEC0u /* -.375 */, 0xBF60BF60u /* -.875 */);
-  t = fma_bf2(fma_bf2(p2, v, u), s2, a2) + kTieDown;
-  word |= (~t >> (15 - 4 * J)) & (0x00010001u << (4 * J));
-  if (J == 3) word |= w2 & 0x80008000u;                                  // sign: bit 3 of the code
-  else word |= (w2 >> (12 - 4 * J)) & (0x00080008u << (4 * J));
-  return word;
+// The code of w / s is its nearest e2m1 value, ties to the even code, saturating: what the conversion instruction
+// gives for an exact quotient.  A multiplication by fl(1 / s) is within 2^-22 of it, which only matters for a quotient
+// exactly on a rounding boundary b (.25 .75 1.25 1.75 2.5 3.5 5: at most 3 significant bits), and there the product
+// rounded to 11 bits is b again: a quotient that is not b differs from it by more than half a unit of 11 bits,
+// because w has 8 bits and b s at most 11, so |w - b s| >= 2^-10 2^k for 2^k <= b s < 2^(k+1), i.e. |w / s - b| > 2^-11 b.
+// The rounding is Veltkamp's splitting (t = q (2^13 + 1), t - (t - q)); it keeps the sign of a zero, and so does the code.
+// One pair took 23 instructions when each boundary was compared by a bf16x2 FMA and the codes were assembled with
+// shifts (half the rate of an FMA each): the kernel was bound by them (403 M elements 239 us, @@@ now; the bytes need 157).
+__device__ __forceinline__ float fp4_quotient(float w, float inv) {
+  const float q = __fmul_rn(w, inv), t = __fmul_rn(q, 8193.0f);
+  return __fsub_rn(t, __fsub_rn(t, q));
 }
-__device__ __forceinline__ uint32_t fp4_word(const uint4& v, uint32_t s2) {
-  return fp4_codes2<3>(fp4_codes2<2>(fp4_codes2<1>(fp4_codes2<0>(0u, v.x, s2), v.y, s2), v.z, s2), v.w, s2);
+__device__ __forceinline__ uint32_t fp4_word(const uint4& v, float inv) {
+  auto lo = [&](uint32_t u) { return fp4_quotient(__uint_as_float(u << 16), inv); };
+  auto hi = [&](uint32_t u) { return fp4_quotient(__uint_as_float(u & 0xFFFF0000u), inv); };
+  uint32_t word;  // bytes e2:e0, e6:e4, e3:e1, e7:e5
+  asm("{\n\t"
+      ".reg .b8 b0, b1, b2, b3;\n\t"
+      "cvt.rn.satfinite.e2m1x2.f32 b0, %3, %1;\n\t"
+      "cvt.rn.satfinite.e2m1x2.f32 b1, %7, %5;\n\t"
+      "cvt.rn.satfinite.e2m1x2.f32 b2, %4, %2;\n\t"
+      "cvt.rn.satfinite.e2m1x2.f32 b3, %8, %6;\n\t"
+      "mov.b32 %0, {b0, b1, b2, b3};\n\t"
+      "}"
+      : "=r"(word)
+      : "f"(lo(v.x)), "f"(hi(v.x)), "f"(lo(v.y)), "f"(hi(v.y)), "f"(lo(v.z)), "f"(hi(v.z)), "f"(lo(v.w)), "f"(hi(v.w)));
+  return word;
 }
 __device__ __forceinline__ __nv_bfloat162 absmax_u4(const uint4& v, __nv_bfloat162 m) {
   m = __hmax2(m, as_bf2(v.x & 0x7FFF7FFFu));
@@ -291,8 +291,8 @@ __global__ void __launch_bounds__(256) quantize_weight_w4_kernel(const uint16_t*
       for (int o = 4; o > 0; o >>= 1) m2 = __hmax2(m2, as_bf2(__shfl_xor_sync(0xFFFFFFFFu, bf2_bits(m2), o)));
       const float amax = fmaxf(fmaxf(__low2float(m2), __high2float(m2)), kAmaxFloor);
       s_bits = f32_to_bf16_bits(__fdiv_rn(amax, 6.0f));
-      const uint32_t s2 = s_bits * 0x00010001u;
-      out = make_uint2(fp4_word(c0, s2), fp4_word(c1, s2));
+      const float inv = __frcp_rn(bf16_bits_to_f32(s_bits));
+      out = make_uint2(fp4_word(c0, inv), fp4_word(c1, inv));
     }
     *reinterpret_cast<uint2*>(packed + at) = out;
     if (pub_packed) *reinterpret_cast<uint2*>(pub_packed + at) = out;  // the rollout engine's copy (Sec. 3.1 item 3)
