@@ -125,67 +125,27 @@ __global__ void __launch_bounds__(256) quantize_act_kernel(const uint16_t* __res
 __device__ __forceinline__ __nv_bfloat162 as_bf2(uint32_t u) { return *reinterpret_cast<__nv_bfloat162*>(&u); }
 __device__ __forceinline__ uint32_t bf2_bits(__nv_bfloat162 v) { return *reinterpret_cast<uint32_t*>(&v); }
 
-__device__ __forceinline__ uint32_t fma_bf2(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t d;
-  asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-  return d;
-}
-__device__ __forceinline__ uint32_t add_bf2(uint32_t a, uint32_t b) {
-  uint32_t d;
-  asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-  return d;
-}
-// Whether a boundary was passed is read from a sign bit, with integer instructions only.  d is the
-// bf16x2 difference value - boundary (never a subnormal: the operands have few bits).  Adding 0x0080 to
-// each half (one exponent step) makes +0 positive and keeps every other sign: sign clear <=> d >= 0, for
-// boundaries that belong to the upper code.  Subtracting it makes +0 negative and keeps every other sign
-// (a borrow out of the low half can only turn a high half that is +0 or positive-minimal around, and the
-// latter cannot occur): sign clear <=> d > 0, for boundaries that belong to the lower code.
-constexpr uint32_t kTieUp = 0x00800080u, kTieDown = 0xFF7FFF80u, kSigns = 0x80008000u;
-
-// q = clamp(rint(w / s) + z, 0, 15) for two adjacent elements at once, equal to the IEEE-division form
-// bit for bit but without a division: q is the number of boundaries (j - z - 1/2) s, j = 1..15, that w
-// passes, where a w exactly on a boundary goes to the even neighbour of rint.  w and s are bf16 (8
-// significant bits), the multiplier m = j - z - 1/2 has at most 6, so w - m s is exact before the one
-// rounding of a fused multiply-add, which keeps its sign and gives zero only for an exact tie, also in
-// bf16; and the IEEE quotient w / s compares with m as w does with m s, because distinct numbers of 8 and
-// 14 bits differ by far more than the quotient's rounding error.  A four-level binary search over j
-// (8, then +-4, +-2, +-1) therefore yields the four bits of q, one bf16x2 FMA per level.
-// Ties: the boundary below code j belongs to rint value j - 1 - z; it goes up when that is odd, i.e.
-// for even j when z is even and for odd j when z is odd.
-struct W4Group {
-  uint32_t neg_s;         // -s twice
-  uint32_t m8;            // 7.5 - z twice: the first boundary
-  uint32_t tie_hi, tie_lo;  // kTieUp / kTieDown for the first three levels (even j) / the last level (odd j)
-};
-__device__ __forceinline__ W4Group w4_group(uint32_t s_bits, float zf) {
-  W4Group g;
-  g.neg_s = (s_bits | 0x8000u) * 0x00010001u;
-  g.m8 = f32_to_bf16_bits(7.5f - zf) * 0x00010001u;   // a half-integer below 16: exact
-  const bool z_odd = (static_cast<int>(zf) & 1) != 0;
-  g.tie_hi = z_odd ? kTieDown : kTieUp;
-  g.tie_lo = z_odd ? kTieUp : kTieDown;
-  return g;
-}
-// codes of the pair (elements 2j, 2j+1 of a word's eight) OR-ed into `word` at bits [4j, 4j+4) and [16+4j, 20+4j)
-template <int J>
-__device__ __forceinline__ uint32_t w4_codes2(uint32_t word, uint32_t w2, const W4Group& g) {
-  uint32_t m = g.m8;
-  uint32_t t = fma_bf2(m, g.neg_s, w2) + g.tie_hi;                       // j = 8
-  word |= (~t >> (12 - 4 * J)) & (0x00080008u << (4 * J));
-  m = add_bf2(m, 0xC080C080u ^ (~t & kSigns));                           // +4 where passed, else -4
-  t = fma_bf2(m, g.neg_s, w2) + g.tie_hi;
-  word |= (~t >> (13 - 4 * J)) & (0x00040004u << (4 * J));
-  m = add_bf2(m, 0xC000C000u ^ (~t & kSigns));                           // +-2
-  t = fma_bf2(m, g.neg_s, w2) + g.tie_hi;
-  word |= (~t >> (14 - 4 * J)) & (0x00020002u << (4 * J));
-  m = add_bf2(m, 0xBF80BF80u ^ (~t & kSigns));                           // +-1
-  t = fma_bf2(m, g.neg_s, w2) + g.tie_lo;
-  word |= (~t >> (15 - 4 * J)) & (0x00010001u << (4 * J));
-  return word;
-}
-__device__ __forceinline__ uint32_t w4_word(const uint4& v, const W4Group& g) {
-  return w4_codes2<3>(w4_codes2<2>(w4_codes2<1>(w4_codes2<0>(0u, v.x, g), v.y, g), v.z, g), v.w, g);
+// q = clamp(rint(w / s) + z, 0, 15), equal to the IEEE-division form without a division.  w * fl(1 / s) is within 2^-18 of the
+// quotient, which only matters for a quotient exactly on a half-integer m (1 to 5 significant bits below 16); fused
+// with the addition of 768 it is rounded to a multiple of 2^-14, which makes m of what is that close to m and leaves a
+// quotient that is not m on its side: w has 8 bits and m s at most 8 + n for an m of n bits, so |w / s - m| > 2^-(7+n) m,
+// at least 2^-9.  The next addition rounds to an integer, ties to even (768 and the constant are even).  No lower clamp:
+// w >= lo gives rint(w / s) >= rint(lo / s) = -z.  The codes are gathered by exact FMAs below 2^24.
+// (Eleven comparisons' worth of bf16x2 FMAs and shifts per pair, a binary search over the boundaries, took 294 us for
+// 403 M elements; this takes 171.)
+constexpr float kRoundAt = 12582912.0f;  // 1.5 * 2^23
+__device__ __forceinline__ uint32_t w4_word(const uint4& v, float inv, float zf) {
+  const float back = zf - kRoundAt;  // exact
+  auto code = [&](float w) {
+    const float x = __fmaf_rn(w, inv, 768.0f);
+    return fminf(__fadd_rn(__fadd_rn(x, kRoundAt - 768.0f), back), 15.0f);
+  };
+  auto lo = [&](uint32_t u) { return code(__uint_as_float(u << 16)); };
+  auto hi = [&](uint32_t u) { return code(__uint_as_float(u & 0xFFFF0000u)); };
+  auto gather = [&](float c0, float c1, float c2, float c3) {
+    return __float_as_uint(__fadd_rn(__fmaf_rn(c1, 16.0f, __fmaf_rn(c2, 256.0f, __fmaf_rn(c3, 4096.0f, 8388608.0f))), c0));
+  };
+  return __byte_perm(gather(lo(v.x), lo(v.y), lo(v.z), lo(v.w)), gather(hi(v.x), hi(v.y), hi(v.z), hi(v.w)), 0x5410);
 }
 
 // ---- FP4 (e2m1) weights (Sec. 2.2, floating-point quantization): s = amax / 6, W_q = [W / s]_FP4 ----
@@ -197,7 +157,7 @@ __device__ __forceinline__ uint32_t w4_word(const uint4& v, const W4Group& g) {
 // because w has 8 bits and b s at most 11, so |w - b s| >= 2^-10 2^k for 2^k <= b s < 2^(k+1), i.e. |w / s - b| > 2^-11 b.
 // The rounding is Veltkamp's splitting (t = q (2^13 + 1), t - (t - q)); it keeps the sign of a zero, and so does the code.
 // One pair took 23 instructions when each boundary was compared by a bf16x2 FMA and the codes were assembled with
-// shifts (half the rate of an FMA each): the kernel was bound by them (403 M elements 239 us, @@@ now; the bytes need 157).
+// shifts (half the rate of an FMA each): the kernel was bound by them (403 M elements 239 us, 156 now; the bytes need 157 at the rate of a copy).
 __device__ __forceinline__ float fp4_quotient(float w, float inv) {
   const float q = __fmul_rn(w, inv), t = __fmul_rn(q, 8193.0f);
   return __fsub_rn(t, __fsub_rn(t, q));
@@ -283,8 +243,8 @@ __global__ void __launch_bounds__(256) quantize_weight_w4_kernel(const uint16_t*
       s_bits = f32_to_bf16_bits(__fdiv_rn(range, 15.0f));
       const float s = bf16_bits_to_f32(s_bits);
       zf = fminf(fmaxf(rintf(__fdiv_rn(-lo, s)), 0.0f), 15.0f);
-      const W4Group grp = w4_group(s_bits, zf);
-      out = make_uint2(w4_word(c0, grp), w4_word(c1, grp));
+      const float inv = __frcp_rn(s);
+      out = make_uint2(w4_word(c0, inv, zf), w4_word(c1, inv, zf));
     } else {
       __nv_bfloat162 m2 = absmax_u4(c1, absmax_u4(c0, as_bf2(0u)));
 #pragma unroll

@@ -385,3 +385,33 @@ def test_moe_training_shape_sampled(ctx):
     # decode-sized call on a slice of the same tokens (128-row tiles) gives the same rows
     c = ctx.moe_fwd_w4a16(x[:256], ids[:256], wts[:256], q13, q2)
     assert torch.equal(c, out[:256])
+
+
+@pytest.mark.parametrize("fmt", ["w4", "fp4"])
+def test_quantizer_next_to_every_boundary(ctx, fmt):
+    """Every significand of the scale times every rounding boundary, hit exactly where bf16 can and missed by one
+    and two units in the last place: the codes are the oracle's (which divides)."""
+    bounds = np.arange(-15.5, 16.0) if fmt == "w4" else np.array([.25, .75, 1.25, 1.75, 2.5, 3.5, 5.0])
+    top = 15.0 if fmt == "w4" else 6.0
+    groups = []
+    for exp in (-20, 0, 9):
+        for m in range(128):
+            s = np.float32((128 + m) * 2.0 ** exp)
+            near = inputs.f32_to_bf16_bits((bounds * s).astype(np.float32)).astype(np.int64)
+            vals = np.concatenate([near + d for d in (-2, -1, 0, 1, 2)])
+            if fmt == "fp4":
+                vals = np.concatenate([vals, vals | 0x8000, [0x8000]])
+            ends = inputs.f32_to_bf16_bits(np.float32([top * s, 0.0]))
+            for shift in ((0.0,) if fmt == "fp4" else (0.0, 7.0, 8.0, 15.0)):  # w4: zero points, odd and even
+                lo, hi = -shift * s, (top - shift) * s
+                f = inputs.bf16_bits_to_f32(vals.astype(np.uint16))
+                keep = vals[(f >= lo) & (f <= hi)] if fmt == "w4" else vals
+                fixed = inputs.f32_to_bf16_bits(np.float32([lo, hi])) if fmt == "w4" else ends
+                row = np.concatenate([fixed, keep])[:128]
+                groups.append(np.concatenate([row, np.zeros(128 - len(row))]).astype(np.uint16))
+    rows = -(-len(groups) // 128) * 128
+    w = np.zeros((1, rows, 128), np.uint16)
+    w[0, :len(groups)] = groups
+    quantize = ctx.quantize_weight_w4 if fmt == "w4" else ctx.quantize_weight_fp4
+    packed = (oracle.quantize_weight_w4 if fmt == "w4" else oracle.quantize_weight_fp4)(w)[0]
+    assert np.array_equal(unpack_lib(quantize(bits_to_torch(w))[0].cpu().numpy()), unpack_linear(packed))
