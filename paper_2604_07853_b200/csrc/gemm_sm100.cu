@@ -4,13 +4,14 @@
 //   acc[m,n] = sum over kb ascending, from 0.0f, of  fmaf( fl(s_x[m,kb] * s_w[n/128,kb]), p_kb[m,n], acc )
 // where p_kb is the tensor-core dot product of the 128 e4m3 codes of K-block kb (Sec. 2.2:
 // Y ~= (s_x s_w)(X_q W_q), applied per block with fp32 accumulation).  The order is the same
-// for every M, group size and tile schedule (App. C): one MMA shape (128 x 256 x 32,
-// cta_group::1), four MMAs per K-block in ascending k, no split-K, no atomics.  A row's
+// for every M, group size, tile width and schedule (App. C): 128-row MMAs of K = 32 (a column's sum does not
+// depend on how many columns the MMA has), four per K-block in ascending k, no split-K, no atomics.  A row's
 // result depends only on that row's codes and scales and on the weight tile.
 //
 // A tile is 128 rows x (128 + 128) columns: two half tiles, rows [n_lo, n_lo+128) and
 // [n_hi, n_hi+128) of the weight -- adjacent for linear/down, gate rows and the matching up
-// rows for gate_up so that SwiGLU and the 1x128 re-quantization of h need no second pass.
+// rows for gate_up so that SwiGLU and the 1x128 re-quantization of h need no second pass.  Dense calls too
+// small for that take tiles of 128 or 64 columns (COLS, see the host).
 //
 // Structure of a CTA (384 threads = 3 warpgroups, one CTA per SM, persistent, static tile list):
 //   warp 8      TMA producer: per K-block one stage = A box 128x128 B + two B boxes 128x128 B

@@ -1,5 +1,4 @@
-// Expansion of packed 4-bit weight codes to bf16 next to the tensor core (Dequant of Sec. 2.2),
-// shared by the wide-tile and the decode-sized W4A16 GEMM kernels: both must produce the same bits.
+// Expansion of packed 4-bit weight codes to bf16 next to the tensor core (Dequant of Sec. 2.2).
 #pragma once
 #include <stdint.h>
 
