@@ -43,6 +43,28 @@ MoePlan plan_moe(int64_t M, int64_t H, int64_t I, int64_t E, int64_t k) {
   return p;
 }
 
+// The dense projection on quantized rows (xc, xs), or on bf16 rows x where linear_fused_applies.
+int run_linear(qarl_ctx* ctx, const uint16_t* x, const uint8_t* xc, const float* xs, int64_t M, int64_t K, const uint8_t* wc,
+               const float* ws, int64_t N, void* y, float* y_f32, void* stream) {
+  GemmArgs a{};
+  a.mode = kModeLinear;
+  a.x = x;
+  a.a_codes = xc;
+  a.a_scales = xs;
+  a.rows_total = M;
+  a.K = K;
+  a.b_codes = wc;
+  a.b_scales = ws;
+  a.N = N;
+  a.E = 1;
+  a.out_bf16 = static_cast<uint16_t*>(y);
+  a.out_f32 = y_f32;
+  mark(ctx, static_cast<cudaStream_t>(stream), -1);
+  const int rc = run_gemm(ctx, make_launch(ctx, stream), a);
+  mark(ctx, static_cast<cudaStream_t>(stream), QARL_STAGE_LINEAR_GEMM);
+  return rc;
+}
+
 }  // namespace
 
 extern "C" {
@@ -211,22 +233,7 @@ int qarl_linear_fwd_q(qarl_ctx* ctx, const uint8_t* xc, const float* xs, int64_t
   if (!aligned16(xc) || !aligned16(wc) || !aligned16(y) || !aligned16(y_f32) ||
       (reinterpret_cast<uintptr_t>(xs) & 3u) || (reinterpret_cast<uintptr_t>(ws) & 3u))
     return QARL_ERR_MISALIGNED;
-  GemmArgs a{};
-  a.mode = kModeLinear;
-  a.a_codes = xc;
-  a.a_scales = xs;
-  a.rows_total = M;
-  a.K = K;
-  a.b_codes = wc;
-  a.b_scales = ws;
-  a.N = N;
-  a.E = 1;
-  a.out_bf16 = static_cast<uint16_t*>(y);
-  a.out_f32 = y_f32;
-  mark(ctx, static_cast<cudaStream_t>(stream), -1);
-  const int rc = run_gemm(ctx, make_launch(ctx, stream), a);
-  mark(ctx, static_cast<cudaStream_t>(stream), QARL_STAGE_LINEAR_GEMM);
-  return rc;
+  return run_linear(ctx, nullptr, xc, xs, M, K, wc, ws, N, y, y_f32, stream);
 }
 
 int qarl_linear_fwd(qarl_ctx* ctx, const void* x, int64_t M, int64_t K, const uint8_t* wc, const float* ws,
@@ -240,9 +247,13 @@ int qarl_linear_fwd(qarl_ctx* ctx, const void* x, int64_t M, int64_t K, const ui
   if (workspace_bytes < qarl_linear_workspace_bytes(M, N, K)) return QARL_ERR_WORKSPACE_TOO_SMALL;
   uint8_t* xc = static_cast<uint8_t*>(workspace);
   float* xs = reinterpret_cast<float*>(xc + align_up(static_cast<size_t>(M) * K, 256));
+  const Launch L = make_launch(ctx, stream);
+  if (linear_fused_applies(L, M, N, K)) {
+    if (!aligned16(wc) || !aligned16(y) || !aligned16(y_f32) || (reinterpret_cast<uintptr_t>(ws) & 3u)) return QARL_ERR_MISALIGNED;
+    return run_linear(ctx, static_cast<const uint16_t*>(x), nullptr, nullptr, M, K, wc, ws, N, y, y_f32, stream);
+  }
   mark(ctx, static_cast<cudaStream_t>(stream), -1);
-  cudaError_t e = launch_quantize_act(make_launch(ctx, stream), static_cast<const uint16_t*>(x), M, K, K, xc, xs,
-                                      nullptr, 1);
+  cudaError_t e = launch_quantize_act(L, static_cast<const uint16_t*>(x), M, K, K, xc, xs, nullptr, 1);
   mark(ctx, static_cast<cudaStream_t>(stream), QARL_STAGE_QUANT_ACT);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "quantize_act");
   return qarl_linear_fwd_q(ctx, xc, xs, M, K, wc, ws, N, y, y_f32, stream);

@@ -168,7 +168,10 @@ struct GemmArgs {
   uint16_t* h_bf16;          // gate_up (debug): [P, I]
   const int32_t* sorted_pair;   // down: [P]
   const float* pair_weights;    // down: [M*k] by sorted position
+  const uint16_t* x;            // linear where linear_fused_applies: the bf16 rows themselves (a_codes, a_scales unused)
 };
+// Whether a dense call of bf16 rows quantizes them inside the GEMM.
+bool linear_fused_applies(const Launch& L, int64_t M, int64_t N, int64_t K);
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

@@ -44,6 +44,7 @@
 
 #include "common.cuh"
 #include "ptx_sm100.cuh"
+#include "quant_device.cuh"
 
 namespace qarl {
 namespace {
@@ -83,6 +84,7 @@ struct GemmParams {
   int I;                   // gate_up: intermediate size (N = 2I)
   int a_rows, stages;      // COLS = 64: rows of the token box, stages of a_rows x 128 + 8192 bytes
   int weights_once;        // few row tiles per expert: weights are loaded with the evict-first policy
+  const uint16_t* x;       // FUSED: the bf16 rows
   int early_prefetch;      // decode-sized calls: weight tiles to pull into L2 before the predecessor finishes
   uint16_t* out_bf16;
   float* out_f32;
@@ -117,6 +119,7 @@ struct __align__(8) SmemTail {
   uint64_t tmem_empty[kMaxAccBufs];
   uint64_t amax_full[4];       // gate_up: the two warps of a TMEM quadrant have exchanged their row maxima
   uint64_t teardown;
+  uint64_t x_ready;            // FUSED: the rows are quantized
   float2 scale[kMaxAccBufs][BM];  // products of the K-block in each accumulator: row scale x (lo, hi) weight scale
   uint32_t amax[2][2][BM];     // gate_up: [tile parity][column slice][row] |h| maxima (bf16 bits)
   uint32_t tmem_addr;
@@ -457,21 +460,62 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
   if (C::kStaging > 0 && lane == 0) bulk_wait_group_all();  // this warp's rows are written
 }
 
-template <int MODE, bool SAVE, int COLS>
+// FUSED (COLS = 64): the 128-element groups of the call's few bf16 rows are quantized by the promotion warps, 8 threads
+// per group, into the operand layout (row r of K-block kb at kb * 1024 + r * 128, 128-byte swizzle) and their
+// scales next to it, while the first weight stages are in flight.
+constexpr int kFusedRows = 8;
+__device__ __forceinline__ void quantize_rows(const GemmParams& p, uint8_t* smem, float* x_scale, SmemTail* s) {
+  const int KB = p.kblocks, groups = p.rows_total * KB, sub = threadIdx.x & 7;
+  constexpr int kStep = kPromoWarps * 4;  // groups per pass
+  auto load = [&](int g, uint4& v0, uint4& v1) {
+    if (g < groups) {
+      const uint4* src = reinterpret_cast<const uint4*>(p.x + static_cast<int64_t>(g) * BK + sub * 16);
+      v0 = __ldg(src);
+      v1 = __ldg(src + 1);
+    }
+  };
+  uint4 v0 = make_uint4(0, 0, 0, 0), v1 = v0;
+  load(static_cast<int>(threadIdx.x) >> 3, v0, v1);
+  for (int base = 0; base < groups; base += kStep) {  // (whole warps: the shuffles below)
+    const int g = base + (static_cast<int>(threadIdx.x) >> 3);
+    const uint4 c0 = v0, c1 = v1;
+    load(g + kStep, v0, v1);
+    uint32_t m = fold_halves(absmax_u4(absmax_u4(0, c0), c1));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+    float inv;
+    const float sc = block_scale(bf16_bits_to_f32(m), &inv);
+    uint4 out;
+    encode8(c0, inv, out.x, out.y);
+    encode8(c1, inv, out.z, out.w);
+    if (g < groups) {
+      const int row = g / KB, kb = g % KB;
+      *reinterpret_cast<uint4*>(smem + kb * 1024 + row * 128 + ((sub ^ row) << 4)) = out;
+      if (sub == 0) x_scale[g] = sc;
+    }
+  }
+  fence_proxy_async_smem();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(&s->x_ready);
+}
+
+template <int MODE, bool SAVE, int COLS, bool FUSED>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                         const __grid_constant__ CUtensorMap tm_o, const GemmParams p) {
   using C = Cfg<MODE, SAVE, COLS>;
   constexpr int kAccBufs = C::kAccBufs, HALVES = C::kHalves;
   const int kStages = COLS == 64 ? p.stages : C::kStages;
-  const uint32_t a_bytes = COLS == 64 ? static_cast<uint32_t>(p.a_rows) * BK : kABytes;
+  const uint32_t a_bytes = FUSED ? 0u : COLS == 64 ? static_cast<uint32_t>(p.a_rows) * BK : kABytes;
   const uint32_t kStageBytes = a_bytes + COLS * BK;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   // (COLS = 64: the MMA reads 128 token rows from a stage whatever its box holds; what lies behind the box must be shared
   // memory too, and an output row depends on its own row only)
-  uint8_t* out_tile = smem + static_cast<size_t>(kStages) * kStageBytes + (COLS == 64 ? kABytes : 0);
+  uint8_t* ring = smem + (FUSED ? p.kblocks * 1024 : 0);
+  uint8_t* out_tile = ring + static_cast<size_t>(kStages) * kStageBytes + (COLS == 64 ? kABytes : 0);
   SmemTail* s = reinterpret_cast<SmemTail*>(out_tile + C::kStaging);
+  float* x_scale = reinterpret_cast<float*>(s + 1);  // FUSED: [rows][K-blocks]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   // ---- set-up: barriers, TMEM, tile list ------------------------------------------------
@@ -487,6 +531,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
     }
     for (int i = 0; i < 4; ++i) mbar_init(&s->amax_full[i], 2);
     mbar_init(&s->teardown, 1);
+    mbar_init(&s->x_ready, kPromoWarps);
     s->abort_flag = 0;
     fence_mbar_init();
   }
@@ -606,10 +651,10 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
             if (p.stop_after_stages >= 0 && armed_total >= p.stop_after_stages) { ok = false; break; }
             ++armed_total;
             if (!wait_or_abort(&s->empty[stage], phase ^ 1, s, p)) { ok = false; break; }
-            uint8_t* a_dst = smem + static_cast<size_t>(stage) * kStageBytes;
+            uint8_t* a_dst = ring + static_cast<size_t>(stage) * kStageBytes;
             uint8_t* b_dst = a_dst + a_bytes;
             mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
-            tma_load_2d(a_dst, &tm_a, &s->full[stage], kb * BK, c.m0);
+            if (!FUSED) tma_load_2d(a_dst, &tm_a, &s->full[stage], kb * BK, c.m0);
             if (p.weights_once) {
               tma_load_2d_hint(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo, stream_once);
               if (HALVES == 2) tma_load_2d_hint(b_dst + kBHalfBytes, &tm_b, &s->full[stage], kb * BK, row_hi, stream_once);
@@ -633,15 +678,16 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
         constexpr uint32_t idesc = umma_idesc_e4m3_f32(BM, COLS);
         int stage = 0, ks = 0;
         uint32_t phase = 0, acc_phase = 0;
-        bool ok = true;
+        bool ok = !FUSED || wait_or_abort(&s->x_ready, 0, s, p);
         for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
           for (int kb = 0; kb < KB; ++kb) {
             if (!wait_or_abort(&s->tmem_empty[ks], acc_phase ^ 1, s, p)) { ok = false; break; }
             if (!wait_or_abort(&s->full[stage], phase, s, p)) { ok = false; break; }
             tc_fence_after_sync();
-            const uint32_t a_addr = smem_u32(smem + static_cast<size_t>(stage) * kStageBytes);
+            const uint32_t stage_addr = smem_u32(ring + static_cast<size_t>(stage) * kStageBytes);
+            const uint32_t a_addr = FUSED ? smem_u32(smem) + kb * 1024 : stage_addr;
             const uint64_t a_desc = umma_desc_k_sw128(a_addr);
-            const uint64_t b_desc = umma_desc_k_sw128(a_addr + a_bytes);
+            const uint64_t b_desc = umma_desc_k_sw128(stage_addr + a_bytes);
             const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(ks * COLS);
 #pragma unroll
             for (int k4 = 0; k4 < BK / 32; ++k4)  // +32 bytes of K = +2 in the 16-byte address field
@@ -684,19 +730,19 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
         x1 = p.a_scales + static_cast<int64_t>(min(c.m0 + r0 + 32, p.rows_total - 1)) * KB;
         wl = p.b_scales + (static_cast<int64_t>(c.e) * NB + nb_lo) * KB;
         wh = p.b_scales + (static_cast<int64_t>(c.e) * NB + nb_hi) * KB;
-        n0 = __ldg(x0);
-        n1 = __ldg(x1);
+        n0 = FUSED ? x_scale[min(r0, p.rows_total - 1) * KB] : __ldg(x0);
+        n1 = FUSED ? n0 : __ldg(x1);  // (FUSED: rows from 8 on are never used)
         nl = __ldg(wl);
         nh = __ldg(wh);
       };
-      if (first_tile < total_tiles) open_tile(first_tile);
-      bool ok = true;
+      bool ok = !FUSED || warp_wait_or_abort(&s->x_ready, 0, s, p);
+      if (ok && first_tile < total_tiles) open_tile(first_tile);
       for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
         for (int kb = 0; kb < KB; ++kb) {
           const float2 v0 = make_float2(__fmul_rn(n0, nl), __fmul_rn(n0, nh)), v1 = make_float2(__fmul_rn(n1, nl), __fmul_rn(n1, nh));
           if (kb + 1 < KB) {
-            n0 = __ldg(x0 + kb + 1);
-            n1 = __ldg(x1 + kb + 1);
+            n0 = FUSED ? x_scale[min(r0, p.rows_total - 1) * KB + kb + 1] : __ldg(x0 + kb + 1);
+            n1 = FUSED ? n0 : __ldg(x1 + kb + 1);
             nl = __ldg(wl + kb + 1);
             nh = __ldg(wh + kb + 1);
           } else if (T + num_ctas < total_tiles) {
@@ -714,6 +760,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
   } else {
     // =============================== promotion warps ==================================
     setmaxnreg_inc<kPromoRegs>();
+    if constexpr (FUSED) quantize_rows(p, smem, x_scale, s);
     promotion_role<MODE, SAVE, COLS>(tm_o, p, smem, s, first_tile, num_ctas, total_tiles);
   }
 
@@ -753,7 +800,7 @@ CUresult make_tmap(EncodeTiledFn encode, CUtensorMap* m, const void* base, uint6
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
-template <int MODE, bool SAVE, int COLS>
+template <int MODE, bool SAVE, int COLS, bool FUSED = false>
 cudaError_t launch_mode(const Launch& L, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to,
                         const GemmParams& p, int grid) {
   // sticky per function and device; atomic: contexts on several host threads may launch at once (both
@@ -761,18 +808,26 @@ cudaError_t launch_mode(const Launch& L, const CUtensorMap& ta, const CUtensorMa
   static std::atomic<bool> attr_set_dev[64];
   std::atomic<bool>& attr_set = attr_set_dev[L.device & 63];
   if (!attr_set.load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_blockscaled_kernel<MODE, SAVE, COLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(gemm_blockscaled_kernel<MODE, SAVE, COLS, FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(COLS == 64 ? kSmemLimit : kSmemBytes<MODE, SAVE, COLS>));
     if (e != cudaSuccess) return e;
     attr_set.store(true, std::memory_order_release);
   }
   size_t smem = kSmemBytes<MODE, SAVE, COLS>;
-  if (COLS == 64) smem += kABytes + static_cast<size_t>(p.stages) * (p.a_rows + COLS) * BK;
+  if (COLS == 64)
+    smem += kABytes + static_cast<size_t>(p.stages) * (p.a_rows + COLS) * BK + (FUSED ? static_cast<size_t>(p.kblocks) * (1024 + kFusedRows * 4) : 0);
   ++*L.launches;
-  return launch_pdl(gemm_blockscaled_kernel<MODE, SAVE, COLS>, static_cast<unsigned>(grid), kThreads, smem, L.stream, ta, tb, to, p);
+  return launch_pdl(gemm_blockscaled_kernel<MODE, SAVE, COLS, FUSED>, static_cast<unsigned>(grid), kThreads, smem, L.stream, ta, tb, to, p);
 }
 
 }  // namespace
+
+bool linear_fused_applies(const Launch& L, int64_t M, int64_t N, int64_t K) {
+  // One launch instead of two: every CTA quantizes all rows itself, two passes over its 8 warps at most (64 groups), and has
+  // one tile (one token, by graph replay: N = 5120, K = 2048 7.8 -> 6.9 us, N = 2048, K = 768 5.5 -> 4.6; 256 groups
+  // would cost 12.3 against 11.1).
+  return L.gemm_path == 0 && M <= kFusedRows && M * (K / BK) <= 64 && N / 64 <= L.sm_count;
+}
 
 cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a, CUresult* cu_err) {
   *cu_err = CUDA_SUCCESS;
@@ -799,13 +854,17 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
     if (const double c = cost(64, 0.45); c < best) { best = c; cols = 64; }
   }
   GemmParams p{};
-  if (cols == 64) {
+  if (a.x != nullptr) {
+    cols = 64;
+    const size_t room = kSmemLimit - kSmemBytes<kModeLinear, false, 64> - kABytes - static_cast<size_t>(a.K / BK) * (1024 + kFusedRows * 4);
+    p.stages = static_cast<int>(std::min<size_t>({kMaxStages, room / (64 * BK), static_cast<size_t>(a.K / BK)}));
+  } else if (cols == 64) {
     p.a_rows = static_cast<int>(std::min<int64_t>(BM, (a.rows_total + 7) / 8 * 8));
     const size_t room = kSmemLimit - kSmemBytes<kModeLinear, false, 64> - kABytes;
     p.stages = static_cast<int>(std::min<size_t>({kMaxStages, room / (static_cast<size_t>(p.a_rows + 64) * BK), static_cast<size_t>(a.K / BK)}));
   }
   CUtensorMap ta, tb, to{};
-  CUresult r = make_tmap(encode, &ta, a.a_codes, static_cast<uint64_t>(a.rows_total), static_cast<uint64_t>(a.K),
+  CUresult r = a.x != nullptr ? CUDA_SUCCESS : make_tmap(encode, &ta, a.a_codes, static_cast<uint64_t>(a.rows_total), static_cast<uint64_t>(a.K),
                          cols == 64 ? static_cast<uint32_t>(p.a_rows) : BM);
   if (r == CUDA_SUCCESS)
     r = make_tmap(encode, &tb, a.b_codes, static_cast<uint64_t>(a.E * a.N), static_cast<uint64_t>(a.K), cols == 64 ? 64 : BNH);
@@ -815,6 +874,7 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
     *cu_err = r;
     return cudaErrorUnknown;
   }
+  p.x = a.x;
   p.a_scales = a.a_scales;
   p.b_scales = a.b_scales;
   p.offsets = a.offsets;
@@ -850,7 +910,8 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
   const int grid = static_cast<int>(std::min<int64_t>(L.sm_count, m_tiles_max * p.n_tiles));
   switch (a.mode) {
     case kModeLinear:
-      return cols == 64    ? launch_mode<kModeLinear, false, 64>(L, ta, tb, to, p, grid)
+      return a.x != nullptr ? launch_mode<kModeLinear, false, 64, true>(L, tb, tb, to, p, grid)
+             : cols == 64  ? launch_mode<kModeLinear, false, 64>(L, ta, tb, to, p, grid)
              : cols == 128 ? launch_mode<kModeLinear, false, 128>(L, ta, tb, to, p, grid)
                            : launch_mode<kModeLinear, false, 256>(L, ta, tb, to, p, grid);
     case kModeGateUp:

@@ -132,3 +132,17 @@ def test_linear_empty_and_errors(ctx):
     rc = lib.qarl_linear_fwd(ctx.h, None, 4, 128, wc.data_ptr(), ws.data_ptr(), 128, out.data_ptr(),
                              None, wsb.data_ptr(), 4096, None)
     assert rc == -1
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 128, 128), (1, 640, 8192), (1, 256, 8320), (2, 384, 4096), (7, 128, 1152), (8, 5120, 1024),
+                                   (8, 256, 1152), (9, 128, 128), (3, 9472, 256), (3, 9600, 256),
+                                   (65, 128, 256), (127, 384, 512), (300, 640, 384), (1000, 1280, 256)])
+def test_small_dense_tiles_equal_the_prequantized_call(ctx, m, n, k):
+    """Around the limits of the form that quantizes its rows inside the GEMM (8 rows, 64 groups, one 64-column tile per
+    SM) and of the 64- and 128-column tiles: rows equal the pre-quantized call's byte for byte, and the oracle's
+    to the tolerance of the other tests."""
+    case = inputs.linear_case(77 + m + n + k, m, n, k)
+    check_linear(ctx, case)
+    xt = bits_to_torch(case.x)
+    w = ctx.quantize_weight(bits_to_torch(case.w))
+    assert torch.equal(ctx.linear_fwd(xt, *w), ctx.linear_fwd_q(*ctx.quantize_act(xt), *w))
