@@ -449,7 +449,7 @@ class Context:
                       workspace: torch.Tensor | None = None):
         """One routed-expert FFN layer on W4A16 weights; w13 and w2 are (packed, scales, zeros)."""
         if not debug:
-            return _native.moe_fwd_4bit(self, x, topk_ids, topk_weights, w13, w2, out, workspace)
+            return _native.moe_fwd_4bit(self, 3, x, topk_ids, topk_weights, w13, w2, out, workspace)
         assert x.dtype == torch.bfloat16 and x.is_contiguous()
         assert topk_ids.dtype == torch.int32 and topk_weights.dtype == torch.float32
         M, H = x.shape
@@ -507,7 +507,7 @@ class Context:
                        workspace: torch.Tensor | None = None):
         """One routed-expert FFN layer on e2m1 weights; w13 and w2 are (packed, scales)."""
         if not debug:
-            return _native.moe_fwd_4bit(self, x, topk_ids, topk_weights, w13, w2, out, workspace)
+            return _native.moe_fwd_4bit(self, 2, x, topk_ids, topk_weights, w13, w2, out, workspace)
         assert x.dtype == torch.bfloat16 and x.is_contiguous()
         assert topk_ids.dtype == torch.int32 and topk_weights.dtype == torch.float32
         M, H = x.shape

@@ -212,11 +212,10 @@ PyObject* linear_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
 struct LayerArgs {
   int64_t M, H, I, E, k;
   void *x, *ids, *wts;
-  LayerArgs(PyObject* xo, PyObject* ido, PyObject* wto, PyObject* w13o) {
+  LayerArgs(PyObject* xo, PyObject* ido, PyObject* wto, const at::Tensor& w13) {
     const at::Tensor& xt = dense(xo, at::kBFloat16, "x: a contiguous bf16 CUDA tensor");
     const at::Tensor& it = cuda_tensor(ido, at::kInt, "topk_ids: an int32 CUDA tensor");
     const at::Tensor& wt = cuda_tensor(wto, at::kFloat, "topk_weights: a float32 CUDA tensor");
-    const at::Tensor& w13 = tensor(w13o);
     expect(xt.dim() == 2 && it.dim() == 2 && w13.dim() == 3, "x [M, H], topk_ids [M, k], w13 [E, 2I, .]");
     M = xt.size(0);
     H = xt.size(1);
@@ -233,7 +232,7 @@ struct LayerArgs {
 PyObject* moe_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return guarded(n, 12, [&]() -> PyObject* {
     Call c(a[0]);
-    const LayerArgs l(a[1], a[2], a[3], a[4]);
+    const LayerArgs l(a[1], a[2], a[3], tensor(a[4]));
     const at::Tensor& x = tensor(a[1]);
     at::Tensor y = output(a[8], {l.M, l.H}, at::kBFloat16, x);
     at::Tensor ws = c.workspace(a[9], a[9] != Py_None ? 0 : qarl_moe_workspace_bytes(l.M, l.H, l.I, l.E, l.k), x);
@@ -252,43 +251,46 @@ PyObject* moe_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   });
 }
 
-// (self, x, ids, wts, w13, w2, out, workspace) -> out; w13 and w2 are (packed, scales, zeros) for integer
-// codes, (packed, scales) for e2m1
+// (self, parts, x, ids, wts, w13, w2, out, workspace) -> out; w13 and w2 are (packed, scales, zeros) with parts = 3
+// (integer codes), (packed, scales) with parts = 2 (e2m1).  The method that calls says which: what else the caller's
+// tuples hold is not looked at, as in the methods' debug forms.
 PyObject* moe_fwd_4bit(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  return guarded(n, 8, [&]() -> PyObject* {
+  return guarded(n, 9, [&]() -> PyObject* {
     Call c(a[0]);
-    expect(PySequence_Check(a[4]) && PySequence_Check(a[5]), "w13 and w2: (packed, scales[, zeros])");
-    void* w[2][3] = {};
-    Py_ssize_t parts = 0;
-    PyObject* packed13 = nullptr;
-    for (int i = 0; i < 2; ++i) {
-      parts = PySequence_Size(a[4 + i]);
-      expect(parts == 2 || parts == 3, "w13 and w2: (packed, scales[, zeros])");
-      for (Py_ssize_t j = 0; j < parts; ++j) {
-        PyObject* o = PySequence_GetItem(a[4 + i], j);  // the sequence keeps the tensor alive
+    const int parts = static_cast<int>(PyLong_AsLong(a[1]));
+    at::Tensor w[2][3];  // (held until the call returns: a sequence may make its items on request)
+    for (int i = 0; i < 2; ++i)
+      for (int j = 0; j < parts; ++j) {
+        PyObject* at = PyLong_FromLong(j);
+        PyObject* o = at ? PyObject_GetItem(a[5 + i], at) : nullptr;
+        Py_XDECREF(at);
         if (!o) throw Fail{};
+        const bool is_tensor = THPVariable_Check(o);
+        if (is_tensor) w[i][j] = THPVariable_Unpack(o);
+        else PyErr_Format(PyExc_TypeError, "w13 and w2 hold torch.Tensors, got %s", Py_TYPE(o)->tp_name);
         Py_DECREF(o);
-        w[i][j] = ptr(o);
-        if (i == 0 && j == 0) packed13 = o;
+        if (!is_tensor) throw Fail{};
       }
-    }
-    const LayerArgs l(a[1], a[2], a[3], packed13);
-    const at::Tensor& x = tensor(a[1]);
-    at::Tensor y = output(a[6], {l.M, l.H}, at::kBFloat16, x);
-    at::Tensor ws = c.workspace(a[7], a[7] != Py_None ? 0 : qarl_moe_w4a16_workspace_bytes(l.M, l.H, l.I, l.E, l.k), x);
+    const LayerArgs l(a[2], a[3], a[4], w[0][0]);
+    const at::Tensor& x = tensor(a[2]);
+    at::Tensor y = output(a[7], {l.M, l.H}, at::kBFloat16, x);
+    at::Tensor ws = c.workspace(a[8], a[8] != Py_None ? 0 : qarl_moe_w4a16_workspace_bytes(l.M, l.H, l.I, l.E, l.k), x);
     const size_t ws_bytes = static_cast<size_t>(ws.numel());
     void *yp = y.data_ptr(), *wp = ws.data_ptr();
     const int32_t* ids = static_cast<int32_t*>(l.ids);
     const float* wts = static_cast<float*>(l.wts);
-    uint8_t *p13 = static_cast<uint8_t*>(w[0][0]), *p2 = static_cast<uint8_t*>(w[1][0]);
-    uint8_t *z13 = static_cast<uint8_t*>(w[0][2]), *z2 = static_cast<uint8_t*>(w[1][2]);
+    void* d[2][3];
+    for (int i = 0; i < 2; ++i)
+      for (int j = 0; j < 3; ++j) d[i][j] = j < parts ? w[i][j].data_ptr() : nullptr;
+    uint8_t *p13 = static_cast<uint8_t*>(d[0][0]), *p2 = static_cast<uint8_t*>(d[1][0]);
+    uint8_t *z13 = static_cast<uint8_t*>(d[0][2]), *z2 = static_cast<uint8_t*>(d[1][2]);
     c.run([&] {
-      return parts == 3 ? qarl_moe_fwd_w4a16(c.ctx, l.x, ids, wts, l.M, l.H, l.I, l.E, l.k, p13, w[0][1], z13, p2, w[1][1],
+      return parts == 3 ? qarl_moe_fwd_w4a16(c.ctx, l.x, ids, wts, l.M, l.H, l.I, l.E, l.k, p13, d[0][1], z13, p2, d[1][1],
                                              z2, yp, wp, ws_bytes, nullptr, c.stream)
-                        : qarl_moe_fwd_fp4a16(c.ctx, l.x, ids, wts, l.M, l.H, l.I, l.E, l.k, p13, w[0][1], p2, w[1][1], yp,
+                        : qarl_moe_fwd_fp4a16(c.ctx, l.x, ids, wts, l.M, l.H, l.I, l.E, l.k, p13, d[0][1], p2, d[1][1], yp,
                                               wp, ws_bytes, nullptr, c.stream);
     });
-    return wrap_or(a[6], y);
+    return wrap_or(a[7], y);
   });
 }
 

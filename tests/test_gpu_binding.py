@@ -1,0 +1,70 @@
+"""The marshalling of the hot calls (csrc/native_binding.cpp): what it refuses, and with which exception, is what the
+library's own checks and torch's allocations give; what a call is asked for decides what runs."""
+from collections import UserDict
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2604_07853_b200 import binding, build, inputs
+from util import bits_to_torch, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    build.build()
+    c = binding.Context(0)
+    yield c
+    assert c.poll() == 0
+    c.close()
+
+
+@pytest.fixture(scope="module")
+def layer():
+    return inputs.moe_case(6, 5, h=256, i=128, e=4, k=2)
+
+
+def _io(c):
+    return bits_to_torch(c.x), to_dev(c.ids), to_dev(c.weights)
+
+
+class Parts:
+    """A sequence that makes its items on request and keeps none of them."""
+
+    def __init__(self, items):
+        self.items = items
+
+    def __len__(self):
+        return len(self.items)
+
+    def __getitem__(self, i):
+        return self.items[i].clone()
+
+
+def test_four_bit_format_is_the_one_of_the_method(ctx, layer):
+    """The method called says which format runs, whatever the weights' tuples hold besides the parts it takes: without
+    zero points the integer layer raises and launches nothing, and the e2m1 layer looks at the first two parts only, with
+    and without the debug dumps."""
+    io = _io(layer)
+    masters = [bits_to_torch(w) for w in (layer.w13, layer.w2)]
+    w4, fp4 = ([q(w) for w in masters] for q in (ctx.quantize_weight_w4, ctx.quantize_weight_fp4))
+    launches = ctx.launch_count()
+    for pair in ((fp4[0], fp4[1]), (w4[0], fp4[1]), (fp4[0], w4[1])):
+        with pytest.raises(IndexError):
+            ctx.moe_fwd_w4a16(*io, *pair)
+    assert ctx.launch_count() == launches
+    for pair in ((fp4[0], fp4[1]), ((*fp4[0], None), (*fp4[1], None)), (fp4[0], w4[1]), (w4[0], fp4[1]), (w4[0], w4[1])):
+        got = ctx.moe_fwd_fp4a16(*io, *pair).clone()
+        assert torch.equal(got, ctx.moe_fwd_fp4a16(*io, *pair, debug=True)[0])
+    assert torch.equal(ctx.moe_fwd_w4a16(*io, *w4).clone(), ctx.moe_fwd_w4a16(*io, *w4, debug=True)[0])
+
+
+def test_parts_are_kept_while_the_call_runs(ctx, layer):
+    """The parts of a weight may come from any sequence, also one that hands out new tensors."""
+    io = _io(layer)
+    w = [ctx.quantize_weight_fp4(bits_to_torch(w)) for w in (layer.w13, layer.w2)]
+    want = ctx.moe_fwd_fp4a16(*io, *w).clone()
+    assert torch.equal(ctx.moe_fwd_fp4a16(*io, *(list(p) for p in w)), want)
+    assert torch.equal(ctx.moe_fwd_fp4a16(*io, *(Parts(p) for p in w)), want)
