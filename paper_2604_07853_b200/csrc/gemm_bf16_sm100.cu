@@ -526,6 +526,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
               tma_store_3d(m, my_box, col, row0, GROUP == kGroupedContraction ? t.e : 0);
               bulk_commit_group();
             }
+            __syncwarp();  // (an aligned tcgen05 instruction may follow)
           } else {
             __syncwarp();
             const int chunk = lane & 7, c = col + chunk * (16 / es);

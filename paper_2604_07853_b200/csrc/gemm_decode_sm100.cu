@@ -170,6 +170,7 @@ __device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parit
 
 // Barrier among `n` threads that also tells every one of them whether `pred` held for all.
 __device__ __forceinline__ bool named_bar_all(uint32_t id, uint32_t n, bool pred) {
+  __syncwarp();  // (bar.red is an aligned instruction)
   uint32_t r;
   asm volatile(
       "{\n\t"

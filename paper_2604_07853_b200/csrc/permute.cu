@@ -211,7 +211,6 @@ __global__ void __launch_bounds__(kClusterThreads) permute_cluster_kernel(const 
       }
       total[tid] = all;
     }
-    __syncwarp();
     ptx::cluster_arrive();  // (waited for before the exit: the others may still be reading `mine`)
   }
   __syncthreads();
