@@ -11,6 +11,7 @@
 
 #include <ATen/cuda/EmptyTensor.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "../../include/qarl.h"
@@ -132,8 +133,8 @@ PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F&& f) {
     return f();
   } catch (const Fail&) {
     return nullptr;
-  } catch (const std::exception& e) {
-    if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what());
+  } catch (...) {  // torch's errors keep their types (torch.OutOfMemoryError, IndexError, ...)
+    if (!PyErr_Occurred()) torch::translate_exception_to_python(std::current_exception());
     return nullptr;
   }
 }

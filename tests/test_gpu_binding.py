@@ -68,3 +68,13 @@ def test_parts_are_kept_while_the_call_runs(ctx, layer):
     want = ctx.moe_fwd_fp4a16(*io, *w).clone()
     assert torch.equal(ctx.moe_fwd_fp4a16(*io, *(list(p) for p in w)), want)
     assert torch.equal(ctx.moe_fwd_fp4a16(*io, *(Parts(p) for p in w)), want)
+
+
+
+def test_out_of_memory_is_torchs_error(ctx):
+    """Two tebibytes of output: the allocation's own error type, which programs catch to retry with less."""
+    x = torch.zeros((1 << 20, 128), dtype=torch.bfloat16, device="cuda")
+    wc = torch.zeros((1 << 20, 128), dtype=torch.uint8, device="cuda")
+    ws = torch.zeros((1 << 13, 1), dtype=torch.float32, device="cuda")
+    with pytest.raises(torch.OutOfMemoryError):
+        ctx.linear_fwd(x, wc, ws)
