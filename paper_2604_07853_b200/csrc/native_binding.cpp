@@ -66,9 +66,9 @@ struct Call {
   explicit Call(PyObject* ctx_object) : self(ctx_object) {
     PyObject* h = PyObject_GetAttr(self, s_hv);
     if (!h) throw Fail{};
-    ctx = static_cast<qarl_ctx*>(PyLong_AsVoidPtr(h));
+    ctx = static_cast<qarl_ctx*>(PyLong_AsVoidPtr(h));  // null once closed: the library refuses it
     Py_DECREF(h);
-    if (!ctx) fail("the context is closed");
+    if (!ctx && PyErr_Occurred()) throw Fail{};
     stream = c10::cuda::getCurrentCUDAStream().stream();
   }
   // the caller's workspace, or the context's cached scratch, grown if it is too small

@@ -78,3 +78,15 @@ def test_out_of_memory_is_torchs_error(ctx):
     ws = torch.zeros((1 << 13, 1), dtype=torch.float32, device="cuda")
     with pytest.raises(torch.OutOfMemoryError):
         ctx.linear_fwd(x, wc, ws)
+
+
+
+def test_closed_context_is_refused_by_the_library(layer):
+    c = binding.Context(0)
+    w = c.quantize_weight(bits_to_torch(layer.w13[0]))
+    x = bits_to_torch(layer.x)
+    c.close()
+    for call in (lambda: c.linear_fwd(x, *w), lambda: c.quantize_act(x), lambda: c.linear_fwd_q(*w, *w)):
+        with pytest.raises(binding.QarlError) as e:
+            call()
+        assert e.value.status == -1
