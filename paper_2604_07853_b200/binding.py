@@ -286,7 +286,7 @@ class Context:
     # ------------------------------------------------------------------ calls
     def quantize_weight(self, w: torch.Tensor, codes=None, scales=None):
         """w bf16 [E, N, K] or [N, K] -> (codes u8 same shape, scales f32 [.., N/128, K/128])."""
-        return _native.quantize_weight(self, w, codes, scales, None, None)
+        return _native.quantize_weight(self, w, codes, scales)
 
     def quantize_act(self, x: torch.Tensor, codes=None, scales=None):
         """x bf16 [M, K] (rows may be strided) -> (codes u8 [M, K], scales f32 [M, K/128])."""
@@ -533,7 +533,7 @@ class Context:
 
     def quantize_weight_publish(self, w, codes, scales, pub_codes, pub_scales):
         """quantize_weight writing a second, published copy of codes and scales in the same launch."""
-        return _native.quantize_weight(self, w, codes, scales, pub_codes, pub_scales)
+        return _native.quantize_weight_publish(self, w, codes, scales, pub_codes, pub_scales)
 
     # ------------------------------------------------------------------ backward
     def linear_bwd(self, dy, x, w, want_dx_f32: bool = False, dx: bool = True, dw: bool = True):

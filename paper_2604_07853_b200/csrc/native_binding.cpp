@@ -150,9 +150,18 @@ struct WeightShape {
   }
 };
 
-// (self, w, codes, scales, pub_codes, pub_scales) -> (codes, scales)
+void quantize_weight_call(Call& c, const at::Tensor& w, const WeightShape& s, void* codes, void* scales, void* pub_codes,
+                          void* pub_scales) {
+  void* wp = w.data_ptr();
+  c.run([&] {
+    return qarl_quantize_weight_publish(c.ctx, wp, s.E, s.N, s.K, static_cast<uint8_t*>(codes), static_cast<float*>(scales),
+                                        static_cast<uint8_t*>(pub_codes), static_cast<float*>(pub_scales), c.stream);
+  });
+}
+
+// (self, w, codes, scales) -> (codes, scales)
 PyObject* quantize_weight(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  return guarded(n, 6, [&]() -> PyObject* {
+  return guarded(n, 4, [&]() -> PyObject* {
     Call c(a[0]);
     const at::Tensor& w = dense(a[1], at::kBFloat16, "w: a contiguous bf16 CUDA tensor");
     const WeightShape s(w);
@@ -160,12 +169,18 @@ PyObject* quantize_weight(PyObject*, PyObject* const* a, Py_ssize_t n) {
     at::Tensor scales = a[3] != Py_None ? tensor(a[3])
                         : w.dim() == 3  ? empty({s.E, s.N / 128, s.K / 128}, at::kFloat, w)
                                         : empty({s.N / 128, s.K / 128}, at::kFloat, w);
-    void *wp = w.data_ptr(), *cp = codes.data_ptr(), *sp = scales.data_ptr(), *pc = ptr(a[4]), *ps = ptr(a[5]);
-    c.run([&] {
-      return qarl_quantize_weight_publish(c.ctx, wp, s.E, s.N, s.K, static_cast<uint8_t*>(cp), static_cast<float*>(sp),
-                                          static_cast<uint8_t*>(pc), static_cast<float*>(ps), c.stream);
-    });
+    quantize_weight_call(c, w, s, codes.data_ptr(), scales.data_ptr(), nullptr, nullptr);
     return tuple_of(wrap_or(a[2], codes), wrap_or(a[3], scales));
+  });
+}
+
+// (self, w, codes, scales, pub_codes, pub_scales) -> (codes, scales); the buffers are the caller's
+PyObject* quantize_weight_publish(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return guarded(n, 6, [&]() -> PyObject* {
+    Call c(a[0]);
+    const at::Tensor& w = dense(a[1], at::kBFloat16, "w: a contiguous bf16 CUDA tensor");
+    quantize_weight_call(c, w, WeightShape(w), ptr(a[2]), ptr(a[3]), ptr(a[4]), ptr(a[5]));
+    return tuple_of(Py_NewRef(a[2]), Py_NewRef(a[3]));
   });
 }
 
@@ -404,9 +419,9 @@ PyObject* tbpo_loss(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 #define FAST(name, doc) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(name)), METH_FASTCALL, doc}
 PyMethodDef methods[] = {
-    FAST(quantize_weight, "qarl_quantize_weight_publish"), FAST(quantize_act, "qarl_quantize_act"),
-    FAST(linear_fwd, "qarl_linear_fwd"),                   FAST(moe_fwd, "qarl_moe_fwd"),
-    FAST(moe_fwd_4bit, "qarl_moe_fwd_w4a16 / qarl_moe_fwd_fp4a16"),
+    FAST(quantize_weight, "qarl_quantize_weight"),         FAST(quantize_weight_publish, "qarl_quantize_weight_publish"),
+    FAST(quantize_act, "qarl_quantize_act"),               FAST(linear_fwd, "qarl_linear_fwd"),
+    FAST(moe_fwd, "qarl_moe_fwd"),                         FAST(moe_fwd_4bit, "qarl_moe_fwd_w4a16 / qarl_moe_fwd_fp4a16"),
     FAST(router_fwd, "qarl_router_fwd"),                   FAST(linear_bwd, "qarl_linear_bwd"),
     FAST(tbpo_loss, "qarl_tbpo_loss"),                     {nullptr, nullptr, 0, nullptr}};
 #undef FAST

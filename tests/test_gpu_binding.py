@@ -90,3 +90,20 @@ def test_closed_context_is_refused_by_the_library(layer):
         with pytest.raises(binding.QarlError) as e:
             call()
         assert e.value.status == -1
+
+
+
+def test_publish_takes_buffers_it_is_given(ctx, layer):
+    """quantize_weight makes the outputs it is not given, quantize_weight_publish makes none."""
+    w = bits_to_torch(layer.w13)
+    codes, scales = ctx.quantize_weight(w)
+    pub = [torch.zeros_like(t) for t in (codes, scales)]
+    for own in ((None, scales), (codes, None), (None, None)):
+        with pytest.raises(binding.QarlError) as e:
+            ctx.quantize_weight_publish(w, *own, *pub)
+        assert e.value.status == -1
+    with pytest.raises(binding.QarlError):
+        ctx.quantize_weight_publish(w, codes, scales, pub[0], None)
+    got = ctx.quantize_weight_publish(w, codes, scales, *pub)
+    assert got[0] is codes and got[1] is scales
+    assert torch.equal(pub[0], codes) and torch.equal(pub[1], scales)
