@@ -329,9 +329,8 @@ class Context:
         save: dict(gate_up=bf16 [P, 2I], h=bf16 [P, I]) of caller-owned tensors that receive the
         activations the backward needs (expert-sorted order), without the other dumps."""
         if not debug:
-            gate_up, h = (save["gate_up"], save["h"]) if save is not None else (None, None)
             return _native.moe_fwd(self, x, topk_ids, topk_weights, w13_codes, w13_scales, w2_codes, w2_scales, out,
-                                   workspace, gate_up, h)
+                                   workspace, save)
         assert x.dtype == torch.bfloat16 and x.is_contiguous()
         assert topk_ids.dtype == torch.int32 and topk_weights.dtype == torch.float32
         M, H = x.shape

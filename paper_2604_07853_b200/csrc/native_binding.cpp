@@ -18,7 +18,7 @@
 
 namespace {
 
-PyObject *s_hv, *s_ws, *s_check, *s_r, *s_w, *s_J, *s_flags, *s_grad, *s_loss;
+PyObject *s_hv, *s_ws, *s_check, *s_r, *s_w, *s_J, *s_flags, *s_grad, *s_loss, *s_gate_up, *s_h, *s_index[3];
 
 struct Fail {};  // a Python exception is set
 
@@ -50,6 +50,18 @@ const at::Tensor& dense(PyObject* o, at::ScalarType type, const char* what) {
 void* ptr(PyObject* o) { return o == Py_None ? nullptr : tensor(o).data_ptr(); }
 template <typename T>
 T* ptr_as(PyObject* o) { return static_cast<T*>(ptr(o)); }
+
+// The tensor a mapping (or a sequence, with an int key) holds under `key`: a reference of its own.
+at::Tensor item(PyObject* o, PyObject* key) {
+  PyObject* v = PyObject_GetItem(o, key);
+  if (!v) throw Fail{};
+  at::Tensor t;
+  if (THPVariable_Check(v)) t = THPVariable_Unpack(v);
+  else PyErr_Format(PyExc_TypeError, "expected a torch.Tensor, got %s", Py_TYPE(v)->tp_name);
+  Py_DECREF(v);
+  if (!t.defined()) throw Fail{};
+  return t;
+}
 
 at::Tensor empty(at::IntArrayRef shape, at::ScalarType type, const at::Tensor& like) {
   return at::detail::empty_cuda(shape, type, like.device(), std::nullopt);
@@ -232,7 +244,7 @@ struct LayerArgs {
     const at::Tensor& xt = dense(xo, at::kBFloat16, "x: a contiguous bf16 CUDA tensor");
     const at::Tensor& it = cuda_tensor(ido, at::kInt, "topk_ids: an int32 CUDA tensor");
     const at::Tensor& wt = cuda_tensor(wto, at::kFloat, "topk_weights: a float32 CUDA tensor");
-    expect(xt.dim() == 2 && it.dim() == 2 && w13.dim() == 3, "x [M, H], topk_ids [M, k], w13 [E, 2I, .]");
+    expect(xt.dim() == 2 && it.dim() >= 2 && w13.dim() == 3, "x [M, H], topk_ids [M, k], w13 [E, 2I, .]");
     M = xt.size(0);
     H = xt.size(1);
     k = it.size(1);
@@ -244,9 +256,10 @@ struct LayerArgs {
   }
 };
 
-// (self, x, ids, wts, w13_codes, w13_scales, w2_codes, w2_scales, out, workspace, save_gate_up, save_h) -> out
+// (self, x, ids, wts, w13_codes, w13_scales, w2_codes, w2_scales, out, workspace, save) -> out; save: None or a mapping
+// with the tensors gate_up and h
 PyObject* moe_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  return guarded(n, 12, [&]() -> PyObject* {
+  return guarded(n, 11, [&]() -> PyObject* {
     Call c(a[0]);
     const LayerArgs l(a[1], a[2], a[3], tensor(a[4]));
     const at::Tensor& x = tensor(a[1]);
@@ -255,9 +268,12 @@ PyObject* moe_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const size_t ws_bytes = static_cast<size_t>(ws.numel());
     void *c13 = ptr(a[4]), *s13 = ptr(a[5]), *c2 = ptr(a[6]), *s2 = ptr(a[7]), *yp = y.data_ptr(), *wp = ws.data_ptr();
     qarl_moe_debug dbg{};
-    dbg.gate_up_bf16 = ptr(a[10]);
-    dbg.h_bf16 = ptr(a[11]);
-    const bool save = dbg.gate_up_bf16 || dbg.h_bf16;
+    const bool save = a[10] != Py_None;
+    at::Tensor gate_up, h;
+    if (save) {
+      dbg.gate_up_bf16 = (gate_up = item(a[10], s_gate_up)).data_ptr();
+      dbg.h_bf16 = (h = item(a[10], s_h)).data_ptr();
+    }
     c.run([&] {
       return qarl_moe_fwd(c.ctx, l.x, static_cast<int32_t*>(l.ids), static_cast<float*>(l.wts), l.M, l.H, l.I, l.E, l.k,
                           static_cast<uint8_t*>(c13), static_cast<float*>(s13), static_cast<uint8_t*>(c2),
@@ -276,17 +292,7 @@ PyObject* moe_fwd_4bit(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int parts = static_cast<int>(PyLong_AsLong(a[1]));
     at::Tensor w[2][3];  // (held until the call returns: a sequence may make its items on request)
     for (int i = 0; i < 2; ++i)
-      for (int j = 0; j < parts; ++j) {
-        PyObject* at = PyLong_FromLong(j);
-        PyObject* o = at ? PyObject_GetItem(a[5 + i], at) : nullptr;
-        Py_XDECREF(at);
-        if (!o) throw Fail{};
-        const bool is_tensor = THPVariable_Check(o);
-        if (is_tensor) w[i][j] = THPVariable_Unpack(o);
-        else PyErr_Format(PyExc_TypeError, "w13 and w2 hold torch.Tensors, got %s", Py_TYPE(o)->tp_name);
-        Py_DECREF(o);
-        if (!is_tensor) throw Fail{};
-      }
+      for (int j = 0; j < parts; ++j) w[i][j] = item(a[5 + i], s_index[j]);
     const LayerArgs l(a[2], a[3], a[4], w[0][0]);
     const at::Tensor& x = tensor(a[2]);
     at::Tensor y = output(a[7], {l.M, l.H}, at::kBFloat16, x);
@@ -316,7 +322,7 @@ PyObject* router_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     Call c(a[0]);
     const at::Tensor& x = dense(a[1], at::kBFloat16, "x: a contiguous bf16 CUDA tensor");
     const at::Tensor& w = dense(a[2], at::kBFloat16, "w_router: a contiguous bf16 CUDA tensor");
-    expect(x.dim() == 2 && w.dim() == 2, "x [M, H], w_router [E, H]");
+    expect(x.dim() == 2 && w.dim() >= 1, "x [M, H], w_router [E, H]");
     const int64_t k = PyLong_AsLongLong(a[3]);
     if (k == -1 && PyErr_Occurred()) throw Fail{};
     const int64_t M = x.size(0), H = x.size(1), E = w.size(0);
@@ -371,47 +377,51 @@ PyObject* tbpo_loss(PyObject*, PyObject* const* a, Py_ssize_t n) {
       if (prm[i] == -1.0 && PyErr_Occurred()) throw Fail{};
     }
     const qarl_tbpo_params params{prm[0], prm[1], prm[2], prm[3]};
-    PyObject* out;
-    if (a[11] != Py_None) {
-      expect(PyDict_Check(a[11]), "out: a dict of an earlier call");
-      out = Py_NewRef(a[11]);
-    } else {
-      out = PyDict_New();
-      if (!out) throw Fail{};
-      auto put = [&](PyObject* key, PyObject* v) {
-        PyDict_SetItem(out, key, v);
+    struct Output {
+      PyObject* key;
+      at::ScalarType type;
+      int64_t n;
+    };
+    const Output outputs[6] = {{s_r, at::kDouble, B},  {s_w, at::kDouble, B},   {s_J, at::kDouble, B},
+                               {s_flags, at::kInt, B}, {s_grad, at::kFloat, T}, {s_loss, at::kDouble, 1}};
+    at::Tensor t[6];
+    void* p[6] = {};
+    const bool given = a[11] != Py_None;
+    const bool want_grad = !given && PyObject_IsTrue(a[10]) == 1;
+    for (int i = 0; i < 6; ++i) {
+      if (!given) {
+        if (outputs[i].key != s_grad || want_grad) t[i] = empty({outputs[i].n}, outputs[i].type, cur);
+      } else {  // any mapping; an entry may be None (no gradient)
+        PyObject* v = PyObject_GetItem(a[11], outputs[i].key);
+        if (!v) throw Fail{};
+        const bool none = v == Py_None;
+        if (THPVariable_Check(v)) t[i] = THPVariable_Unpack(v);
         Py_DECREF(v);
-      };
-      put(s_r, wrap(empty({B}, at::kDouble, cur)));
-      put(s_w, wrap(empty({B}, at::kDouble, cur)));
-      put(s_J, wrap(empty({B}, at::kDouble, cur)));
-      put(s_flags, wrap(empty({B}, at::kInt, cur)));
-      put(s_grad, PyObject_IsTrue(a[10]) == 1 ? wrap(empty({T}, at::kFloat, cur)) : Py_NewRef(Py_None));
-      put(s_loss, wrap(empty({1}, at::kDouble, cur)));
+        if (!none && !t[i].defined()) fail("out: a mapping of tensors, as an earlier call returned it");
+      }
+      if (t[i].defined()) p[i] = t[i].data_ptr();
     }
-    try {
-      auto of = [&](PyObject* key) {
-        PyObject* v = PyDict_GetItemWithError(out, key);
-        if (!v) {
-          if (!PyErr_Occurred()) PyErr_SetObject(PyExc_KeyError, key);
-          throw Fail{};
-        }
-        return ptr(v);
-      };
-      void *r = of(s_r), *w = of(s_w), *J = of(s_J), *flags = of(s_flags), *grad = of(s_grad), *loss = of(s_loss);
-      at::Tensor ws = c.workspace(a[12], a[12] != Py_None ? 0 : qarl_tbpo_workspace_bytes(B, T), cur);
-      const size_t ws_bytes = static_cast<size_t>(ws.numel());
-      void *p0 = cur.data_ptr(), *p1 = old_l.data_ptr(), *p2 = old_s.data_ptr(), *po = off.data_ptr(), *pa = adv.data_ptr(),
-           *wp = ws.data_ptr();
-      c.run([&] {
-        return qarl_tbpo_loss(c.ctx, static_cast<float*>(p0), static_cast<float*>(p1), static_cast<float*>(p2),
-                              static_cast<int64_t*>(po), static_cast<float*>(pa), B, T, &params, static_cast<double*>(r),
-                              static_cast<double*>(w), static_cast<double*>(J), static_cast<int32_t*>(flags),
-                              static_cast<float*>(grad), static_cast<double*>(loss), wp, ws_bytes, c.stream);
-      });
-    } catch (...) {
-      Py_DECREF(out);
-      throw;
+    at::Tensor ws = c.workspace(a[12], a[12] != Py_None ? 0 : qarl_tbpo_workspace_bytes(B, T), cur);
+    const size_t ws_bytes = static_cast<size_t>(ws.numel());
+    void *p0 = cur.data_ptr(), *p1 = old_l.data_ptr(), *p2 = old_s.data_ptr(), *po = off.data_ptr(), *pa = adv.data_ptr(),
+         *wp = ws.data_ptr();
+    c.run([&] {
+      return qarl_tbpo_loss(c.ctx, static_cast<float*>(p0), static_cast<float*>(p1), static_cast<float*>(p2),
+                            static_cast<int64_t*>(po), static_cast<float*>(pa), B, T, &params, static_cast<double*>(p[0]),
+                            static_cast<double*>(p[1]), static_cast<double*>(p[2]), static_cast<int32_t*>(p[3]),
+                            static_cast<float*>(p[4]), static_cast<double*>(p[5]), wp, ws_bytes, c.stream);
+    });
+    if (given) return Py_NewRef(a[11]);
+    PyObject* out = PyDict_New();
+    if (!out) throw Fail{};
+    for (int i = 0; i < 6; ++i) {
+      PyObject* v = t[i].defined() ? THPVariable_Wrap(t[i]) : Py_NewRef(Py_None);
+      const int rc = v ? PyDict_SetItem(out, outputs[i].key, v) : -1;
+      Py_XDECREF(v);
+      if (rc != 0) {
+        Py_DECREF(out);
+        throw Fail{};
+      }
     }
     return out;
   });
@@ -436,8 +446,11 @@ PyMODINIT_FUNC PyInit__native() {
     PyObject** at;
     const char* text;
   } names[] = {{&s_hv, "_hv"}, {&s_ws, "_ws"}, {&s_check, "_check"}, {&s_r, "r"},      {&s_w, "w"},
-               {&s_J, "J"},    {&s_flags, "flags"}, {&s_grad, "grad"},  {&s_loss, "loss"}};
+               {&s_J, "J"},    {&s_flags, "flags"}, {&s_grad, "grad"},  {&s_loss, "loss"},   {&s_gate_up, "gate_up"},
+               {&s_h, "h"}};
   for (auto& s : names)
     if (!(*s.at = PyUnicode_InternFromString(s.text))) return nullptr;
+  for (long i = 0; i < 3; ++i)
+    if (!(s_index[i] = PyLong_FromLong(i))) return nullptr;
   return PyModule_Create(&module);
 }

@@ -107,3 +107,28 @@ def test_publish_takes_buffers_it_is_given(ctx, layer):
     got = ctx.quantize_weight_publish(w, codes, scales, *pub)
     assert got[0] is codes and got[1] is scales
     assert torch.equal(pub[0], codes) and torch.equal(pub[1], scales)
+
+
+
+def test_shapes_and_containers_the_calls_take(ctx, layer):
+    """Ids with trailing dimensions of one, a router weight with a dimension in between, any mapping as the loss's `out`;
+    a save dict has to hold both tensors."""
+    x, ids, wts = _io(layer)
+    q = [t for w in (layer.w13, layer.w2) for t in ctx.quantize_weight(bits_to_torch(w))]
+    want = ctx.moe_fwd(x, ids, wts, *q).clone()
+    assert torch.equal(ctx.moe_fwd(x, ids.unsqueeze(2), wts.unsqueeze(2), *q), want)
+    gate_up = torch.empty((layer.M * layer.k, 2 * layer.I), dtype=torch.bfloat16, device="cuda")
+    with pytest.raises((AttributeError, TypeError)):
+        ctx.moe_fwd(x, ids, wts, *q, save={"gate_up": gate_up, "h": None})
+    with pytest.raises(KeyError):
+        ctx.moe_fwd(x, ids, wts, *q, save={"gate_up": gate_up})
+    wr = torch.randn((8, 256), device="cuda").to(torch.bfloat16)
+    for a, b in zip(ctx.router_fwd(x, wr, 2), ctx.router_fwd(x, wr.unsqueeze(1), 2)):
+        assert torch.equal(a, b)
+    lp = torch.linspace(-1.0, -0.5, 40, device="cuda")
+    offsets = torch.tensor([0, 10, 40], device="cuda")
+    adv = torch.tensor([1.0, -1.0], device="cuda")
+    first = ctx.tbpo_loss(lp + 1e-3, lp, lp, offsets, adv)
+    again = UserDict({k: torch.zeros_like(v) for k, v in first.items()})
+    assert ctx.tbpo_loss(lp + 1e-3, lp, lp, offsets, adv, out=again) is again
+    assert all(torch.equal(again[k], first[k]) for k in first)
