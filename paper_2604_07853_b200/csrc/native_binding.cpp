@@ -47,6 +47,11 @@ const at::Tensor& dense(PyObject* o, at::ScalarType type, const char* what) {
   expect(t.is_contiguous(), what);
   return t;
 }
+bool truth(PyObject* o) {
+  const int v = PyObject_IsTrue(o);
+  if (v < 0) throw Fail{};
+  return v == 1;
+}
 void* ptr(PyObject* o) { return o == Py_None ? nullptr : tensor(o).data_ptr(); }
 template <typename T>
 T* ptr_as(PyObject* o) { return static_cast<T*>(ptr(o)); }
@@ -220,7 +225,7 @@ PyObject* linear_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const at::Tensor& x = dense(a[1], at::kBFloat16, "x: a contiguous bf16 CUDA tensor");
     expect(x.dim() == 2, "x: [M, K]");
     const int64_t M = x.size(0), K = x.size(1), N = tensor(a[2]).size(0);
-    const bool want_f32 = PyObject_IsTrue(a[5]) == 1;
+    const bool want_f32 = truth(a[5]);
     at::Tensor y = output(a[4], {M, N}, at::kBFloat16, x);
     at::Tensor y32;
     if (want_f32) y32 = empty({M, N}, at::kFloat, x);
@@ -346,7 +351,7 @@ PyObject* linear_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     expect(dy.dim() == 2 && x.dim() == 2 && w.dim() == 2, "dy [M, N], x [M, K], w [N, K]");
     const int64_t M = dy.size(0), N = dy.size(1), K = x.size(1);
     expect(x.size(0) == M && w.size(0) == N && w.size(1) == K, "dy [M, N], x [M, K], w [N, K]");
-    const bool f32 = PyObject_IsTrue(a[4]) == 1, want_dx = PyObject_IsTrue(a[5]) == 1, want_dw = PyObject_IsTrue(a[6]) == 1;
+    const bool f32 = truth(a[4]), want_dx = truth(a[5]), want_dw = truth(a[6]);
     at::Tensor dx, dx32, dw;
     if (want_dx) dx = empty({M, K}, at::kBFloat16, dy);
     if (want_dx && f32) dx32 = empty({M, K}, at::kFloat, dy);
@@ -387,7 +392,7 @@ PyObject* tbpo_loss(PyObject*, PyObject* const* a, Py_ssize_t n) {
     at::Tensor t[6];
     void* p[6] = {};
     const bool given = a[11] != Py_None;
-    const bool want_grad = !given && PyObject_IsTrue(a[10]) == 1;
+    const bool want_grad = !given && truth(a[10]);
     for (int i = 0; i < 6; ++i) {
       if (!given) {
         if (outputs[i].key != s_grad || want_grad) t[i] = empty({outputs[i].n}, outputs[i].type, cur);

@@ -132,3 +132,11 @@ def test_shapes_and_containers_the_calls_take(ctx, layer):
     again = UserDict({k: torch.zeros_like(v) for k, v in first.items()})
     assert ctx.tbpo_loss(lp + 1e-3, lp, lp, offsets, adv, out=again) is again
     assert all(torch.equal(again[k], first[k]) for k in first)
+
+
+
+def test_flags_without_a_truth_value_raise(ctx, layer):
+    x = bits_to_torch(layer.x)
+    w = ctx.quantize_weight(bits_to_torch(layer.w13[0]))
+    with pytest.raises(ValueError):
+        ctx.linear_fwd(x, *w, want_f32=np.ones(2))
