@@ -18,9 +18,9 @@
 //   grouped contraction  C_e = sum over the expert's rows p of A[p, :]^T B[p, :]  (dW of an
 //                        expert projection: both operands MN-major, the contraction runs over a
 //                        ragged row range).  The last 64-row step of an expert also holds rows of
-//                        the next expert: a warp overwrites those rows of the staged A tile with zeros
+//                        the next expert: a warp overwrites those rows of both staged tiles with zeros
 //                        (generic stores + proxy fence) before the step is issued, so
-//                        they contribute nothing whatever B holds there.
+//                        they contribute nothing whatever they hold.
 //
 // Tile 128 x 256 x 64 (or 256 x 256, 128 x 192: see the host).  TMA stages both operands with the 128-byte swizzle (a K-major tile is
 // one box of R rows x 128 bytes; an MN-major tile is one box of 64 c-rows x 128 bytes per 64
@@ -463,8 +463,8 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   } else if (GROUP == kGroupedContraction && warp == C::kFixWarp) {
     // =============================== ragged steps =====================================
     // The last 64-row step of an expert also holds rows of the next one.  This warp zeroes what the last 16-row
-    // slice holds of them in the staged A tile as soon as the step has landed, ahead of the MMA thread (which
-    // did this itself once: ~2000 clocks of a tile's ~12000).
+    // slice holds of them in both staged tiles (in one alone 0 x inf and 0 x NaN would still be NaN) as soon as the
+    // step has landed, ahead of the MMA thread (which did this itself once: ~2000 clocks of a tile's ~12000).
     int stage = 0;
     uint32_t phase = 0;
     // every step is followed (and counted in `empty`): a parity wait tells neighbouring fills apart, no more
@@ -473,12 +473,12 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       const uint32_t step = *reinterpret_cast<volatile uint32_t*>(&list->step[stage]);
       const int valid = static_cast<int>(step >> 3);
       if (valid < BK) {
-        uint8_t* a_tile = smem + static_cast<size_t>(stage) * kStageBytes;
-        const int nrows = -valid & 15;
-        for (int idx = lane; idx < (TM / 64) * nrows * 8; idx += 32) {
-          const int blk = idx / (nrows * 8), rem = idx % (nrows * 8);
-          *reinterpret_cast<uint4*>(a_tile + blk * kBlockBytes + (valid + rem / 8) * 128 + (rem % 8) * 16) = make_uint4(0, 0, 0, 0);
-        }
+        uint8_t* tiles = smem + static_cast<size_t>(stage) * kStageBytes;  // A's blocks of 64 columns, then B's
+        const int chunks = (-valid & 15) * 8;
+#pragma unroll
+        for (int blk = 0; blk < (TM + BN) / 64; ++blk)
+          for (int i = lane; i < chunks; i += 32)  // (rows are 128 bytes: chunk i of the overhang is at valid * 128 + 16 i)
+            *reinterpret_cast<uint4*>(tiles + blk * kBlockBytes + valid * 128 + i * 16) = make_uint4(0, 0, 0, 0);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&s->fixed[stage]);

@@ -235,3 +235,29 @@ def test_moe_layer_backward_token_rows_do_not_depend_on_the_batch(ctx):
     full = run(list(range(128)))
     for rows in ([0], [127], list(range(40, 72))):
         assert torch.equal(run(rows), full[rows])
+
+
+def test_grouped_dw_is_not_touched_by_the_next_experts_rows(ctx):
+    """A 64-row step that an expert's rows do not fill also holds the next expert's: infinities and NaN there must
+    not reach this expert's dW (0 * inf is NaN), in either operand."""
+    sizes = [3, 17, 70, 130, 1, 64, 33]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32)
+    rng = np.random.default_rng(17)
+    P, N, K, E = int(off[-1]), 128, 320, len(sizes)
+    dy, x = (rng.integers(-4, 5, size=(P, n)).astype(np.float32) for n in (N, K))
+    w = torch.zeros((E, N, K), dtype=torch.bfloat16, device="cuda")
+
+    def dw(a, b):
+        t = [torch.from_numpy(v).to(torch.bfloat16).cuda() for v in (a, b)]
+        return ctx.grouped_linear_bwd(*t, w, torch.from_numpy(off).cuda(), dx=False)[2].cpu().numpy()
+
+    want = np.stack([dy[a:b].T @ x[a:b] for a, b in zip(off[:-1], off[1:])])
+    assert np.array_equal(dw(dy, x), want)
+    for e in range(1, E):
+        for which in (0, 1):
+            for bad in (np.inf, np.nan):
+                ops = [dy.copy(), x.copy()]
+                ops[which][off[e]] = bad              # the first row past expert e - 1
+                got = dw(*ops)
+                keep = [i for i in range(E) if i != e]
+                assert np.array_equal(got[keep], want[keep]), (e, which, bad)
