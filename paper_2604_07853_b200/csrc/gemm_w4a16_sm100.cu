@@ -61,7 +61,7 @@ constexpr int kMaxAccBufs = 2;
 constexpr int kDqWarps = 16;       // two groups of eight
 template <int NT>
 struct Cfg {
-  // epilogue warps 0 ..: TMEM quadrant = warp % 4, with eight the token half = warp / 4
+  // epilogue warps 0 ..: TMEM quadrant = warp % 4, warp / 4 = which token columns of it, 16 at a time
   static constexpr int kEpiWarps = 8;
   static constexpr int kCodeWarp = kEpiWarps + kDqWarps;             // producer of the codes
   static constexpr int kTokenWarp = kCodeWarp + 1;                   // producer of the token rows
@@ -111,6 +111,7 @@ struct __align__(8) SmemTail {
   uint64_t teardown[2];
   uint32_t tmem_addr;
   int abort_flag;
+  float weight[2][kWide];      // down: the tile's pair weights, by tile parity
   int32_t off[kMaxExperts + 1];
   int32_t prefix[kMaxExperts + 1];
 };
@@ -485,18 +486,24 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
   } else {
     // =============================== epilogue warps ===================================
     const int wr = (warp & 3) * 32 + lane;  // weight row within a block = TMEM lane
-    constexpr int kShare = NT / (kEpiWarps / 4);  // tokens of a warp
-    const int tc0 = (warp >> 2) * kShare;
+    constexpr int kTurn = 16 * (kEpiWarps / 4);  // the warps of a quadrant take 16 token columns in turn
+    const int tc0 = (warp >> 2) * 16;
     constexpr uint32_t kEpiThreads = kEpiWarps * 32;
     const uint32_t lane_addr = static_cast<uint32_t>((warp & 3) * 32) << 16;
     int acc = 0, cur_e = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
     uint16_t* T16 = reinterpret_cast<uint16_t*>(out_tile);
-    for (int T = first_tile; T < total_tiles; T += num_ctas) {
+    uint32_t par = 0;
+    for (int T = first_tile; T < total_tiles; T += num_ctas, par ^= 1) {
       const TileCoord c = decode_tile(s->off, s->prefix, NT, T, cur_e);
       const int rows = min(NT, c.m_end - c.m0);  // live token rows of this tile (>= 1)
       const int j = c.n_tile;
+      // The pair weights come in while the tile is still being multiplied: loaded where they are used, with the
+      // accumulators waiting, they cost more than the MMAs of a short contraction (I = 256, 65536 pairs of 512 experts:
+      // down 167 us against 145).  (The barrier below is between this and their use, and two tiles share no slot.)
+      if (MODE == kModeDown && threadIdx.x < NT)
+        s->weight[par][threadIdx.x] = __ldg(p.pair_weights + min(c.m0 + static_cast<int>(threadIdx.x), p.rows_total - 1));
       ok = warp_wait_or_abort(&s->tmem_full[acc], acc_phase, s, p);
       ok = named_bar_all(1, kEpiThreads, ok);  // one decision for the four warps; the previous tile's row readers are done
       if (!ok) break;
@@ -504,18 +511,20 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
       const uint32_t t0 = tmem_base + lane_addr + static_cast<uint32_t>(acc) * (2 * NT);
       const int col_lo = 2 * j * BW + wr, col_hi = col_lo + BW;  // down / linear: this thread's two output columns
       const bool hi_ok = col_hi < p.N;
-      // 16 token columns at a time (the register budget of the CTA)
+      auto hand_back = [&]() {  // this warp's share of the accumulator is in registers
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&s->tmem_empty[acc]);
+      };
+      if (tc0 >= rows) hand_back();
+      // 16 token columns at a time (the register budget of the CTA), the live ones only
 #pragma unroll 1
-      for (int tc = tc0; tc < tc0 + kShare; tc += 16) {
+      for (int tc = tc0; tc < rows; tc += kTurn) {
         uint32_t vl[16], vh[16];
         tmem_ld_x16(t0 + tc, vl);
         tmem_ld_x16(t0 + NT + tc, vh);
         tmem_ld_wait();
-        if (tc + 16 == tc0 + kShare) {  // this warp's share of the accumulator is in registers: hand it back
-          tc_fence_before_sync();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&s->tmem_empty[acc]);
-        }
+        if (tc + kTurn >= rows) hand_back();
 #pragma unroll
         for (int u = 0; u < 16; ++u) {
           const int t = tc + u;
@@ -537,7 +546,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
               if (hi_ok) d[col_hi] = hi;
             }
             if (MODE == kModeDown) {  // contribution = bf16( fl(w * y) )
-              const float w = __ldg(p.pair_weights + min(c.m0 + t, p.rows_total - 1));
+              const float w = s->weight[par][t];
               lo = __fmul_rn(w, lo);
               hi = __fmul_rn(w, hi);
             }
