@@ -28,8 +28,8 @@ int qarl_harness_rmsnorm(qarl_ctx* ctx, const void* x_bf16, int64_t M, int64_t H
  * qarl_poll_device_status reports (and clears) the error.  Nothing traps, faults or hangs. */
 int qarl_harness_wait_selftest(qarl_ctx* ctx, uint64_t limit_ns, void* stream);
 
-/* The two calls below exist so that a test can watch the pipeline of the FP8 GEMMs and of the one-launch
- * router give up on a wait (the library never needs them).  Both only store a value in the context (host side, not
+/* The two calls below exist so that a test can watch the pipeline of the GEMMs and of the one-launch
+ * routers give up on a wait (the library never needs them).  Both only store a value in the context (host side, not
  * synchronized with calls running on other threads); it applies to the GEMM kernels launched
  * through `ctx` afterwards.
  *
@@ -56,6 +56,17 @@ int qarl_harness_stop_producer_after(qarl_ctx* ctx, int64_t stages);
  * through each and compare.  A value other than 0 also makes qarl_router_fwd take its two-launch form.
  * Host side only, stored in the context. */
 int qarl_harness_set_gemm_path(qarl_ctx* ctx, int path);
+
+/* The same for two choices by size inside one path, so that a small input reaches the form a large one takes.
+ *
+ * qarl_harness_set_dense_columns: the wide-tile kernel's dense calls (projections of pre-quantized rows or not) take tiles
+ * of 64, 128 or 256 columns (0 restores the choice by size, and with it the form that quantizes its rows itself).
+ *
+ * qarl_harness_set_router_form: qarl_router_fwd takes two launches (1), one launch of persistent CTAs (2; up to 128
+ * experts and top-16) or one launch of clusters (3; up to 128 experts, as many tokens as there are clusters at once);
+ * where a form does not apply, two launches.  0 restores the choice by size. */
+int qarl_harness_set_dense_columns(qarl_ctx* ctx, int columns);
+int qarl_harness_set_router_form(qarl_ctx* ctx, int form);
 
 /* Roofline denominators measured with the library's own instructions (used by the benchmark; the
  * paper has no counterpart).  Both only launch a kernel on `stream`; the caller times it with

@@ -42,7 +42,7 @@ EXPORTS = [
 STATIC_LINEAR_MAX_ELEMS = 4 * 1024 * 1024
 HARNESS_EXPORTS = ["qarl_harness_rmsnorm", "qarl_harness_wait_selftest", "qarl_harness_set_wait_limit_ns",
                    "qarl_harness_stop_producer_after", "qarl_harness_fp8_mma_peak", "qarl_harness_read_stream",
-                   "qarl_harness_set_gemm_path"]
+                   "qarl_harness_set_gemm_path", "qarl_harness_set_dense_columns", "qarl_harness_set_router_form"]
 STAGES = ["quantize_weight", "quantize_act", "linear_gemm", "permute", "gate_up_gemm", "down_gemm",
           "combine", "bwd_dx", "bwd_dw", "tbpo", "router", "bwd_elementwise", "moe_decode_layer"]
 
@@ -167,6 +167,10 @@ def load() -> C.CDLL:
     L.qarl_harness_stop_producer_after.argtypes = [p, i64]
     L.qarl_harness_set_gemm_path.restype = C.c_int
     L.qarl_harness_set_gemm_path.argtypes = [p, C.c_int]
+    L.qarl_harness_set_dense_columns.restype = C.c_int
+    L.qarl_harness_set_dense_columns.argtypes = [p, C.c_int]
+    L.qarl_harness_set_router_form.restype = C.c_int
+    L.qarl_harness_set_router_form.argtypes = [p, C.c_int]
     L.qarl_harness_fp8_mma_peak.restype = C.c_int
     L.qarl_harness_fp8_mma_peak.argtypes = [p, i64, C.POINTER(C.c_double), p]
     L.qarl_harness_read_stream.restype = C.c_int
@@ -257,12 +261,20 @@ class Context:
         self._check(self.lib.qarl_harness_set_wait_limit_ns(self.h, limit_ns))
 
     def harness_stop_producer_after(self, stages: int):
-        """FP8 GEMM TMA producers stop arming stages after `stages` (negative: normal operation)."""
+        """GEMM and one-launch router TMA producers stop arming stages after `stages` (negative: normal operation)."""
         self._check(self.lib.qarl_harness_stop_producer_after(self.h, stages))
 
     def harness_set_gemm_path(self, path: int):
         """0: automatic choice of the grouped FP8 GEMM kernel, 1: wide tiles, 2: decode (swapped operands)."""
         self._check(self.lib.qarl_harness_set_gemm_path(self.h, path))
+
+    def harness_set_dense_columns(self, columns: int):
+        """Columns per tile of the wide-tile kernel's dense calls: 64, 128 or 256; 0: the choice by size."""
+        self._check(self.lib.qarl_harness_set_dense_columns(self.h, columns))
+
+    def harness_set_router_form(self, form: int):
+        """1: two launches, 2: one launch of persistent CTAs, 3: one launch of clusters; 0: the choice by size."""
+        self._check(self.lib.qarl_harness_set_router_form(self.h, form))
 
     def harness_fp8_mma_peak(self, kblocks_per_sm: int) -> float:
         """Launch the dense FP8 MMA peak kernel; returns the floating-point operations it performs."""

@@ -414,6 +414,18 @@ int qarl_harness_set_gemm_path(qarl_ctx* ctx, int path) {
   return QARL_OK;
 }
 
+int qarl_harness_set_dense_columns(qarl_ctx* ctx, int columns) {
+  if (!ctx || (columns != 0 && columns != 64 && columns != 128 && columns != 256)) return QARL_ERR_INVALID_ARG;
+  ctx->dense_columns = columns;
+  return QARL_OK;
+}
+
+int qarl_harness_set_router_form(qarl_ctx* ctx, int form) {
+  if (!ctx || form < 0 || form > 3) return QARL_ERR_INVALID_ARG;
+  ctx->router_form = form;
+  return QARL_OK;
+}
+
 int qarl_harness_stop_producer_after(qarl_ctx* ctx, int64_t stages) {
   if (!ctx) return QARL_ERR_INVALID_ARG;
   ctx->stop_after_stages = stages < 0 ? -1 : static_cast<int>(stages > 0x7FFFFFFF ? 0x7FFFFFFF : stages);

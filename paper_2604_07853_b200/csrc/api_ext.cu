@@ -570,8 +570,9 @@ int qarl_router_fwd(qarl_ctx* ctx, const void* x, int64_t M, int64_t H, const vo
   if (!x || !wr || !logits || !ids || !wts) return QARL_ERR_INVALID_ARG;
   if (!aligned16(x) || !aligned16(wr) || !aligned16(logits)) return QARL_ERR_MISALIGNED;
   Launch L = make_launch(ctx, stream);
-  const bool cluster = L.gemm_path == 0 && router_cluster_applies(L, M, E);
-  if (cluster || (L.gemm_path == 0 && router_fused_applies(E, k))) {  // one launch: selection in the GEMM's epilogue
+  const int form = L.gemm_path != 0 ? 1 : L.router_form;
+  const bool cluster = (form == 0 || form == 3) && router_cluster_applies(L, M, E);
+  if (cluster || ((form == 0 || form == 2) && router_fused_applies(E, k))) {  // one launch: selection in the GEMM's epilogue
     CUresult cu = CUDA_SUCCESS;
     mark(ctx, L.stream, -1);
     cudaError_t e = (cluster ? launch_router_cluster : launch_router_fused)(

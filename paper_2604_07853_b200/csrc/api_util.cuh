@@ -34,6 +34,8 @@ inline Launch make_launch(qarl_ctx* ctx, void* stream) {
   L.wait_limit_ns = ctx->wait_limit_ns;
   L.stop_after_stages = ctx->stop_after_stages;
   L.gemm_path = ctx->gemm_path;
+  L.dense_columns = ctx->dense_columns;
+  L.router_form = ctx->router_form;
   return L;
 }
 

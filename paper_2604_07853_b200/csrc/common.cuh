@@ -62,8 +62,10 @@ struct Launch {
   int* d_status;
   int64_t* launches;  // host counter
   unsigned long long wait_limit_ns = 0;  // bound of every device-side barrier wait (0: the default, 2 s)
-  int stop_after_stages = -1;            // test harness only: FP8 GEMM producers stop after this many stages
+  int stop_after_stages = -1;            // test harness only: GEMM producers stop after this many stages
   int gemm_path = 0;                     // test harness only: 0 = automatic, 1 = wide-tile kernel, 2 = decode kernel (one launch per projection)
+  int dense_columns = 0;                 // test harness only: columns per tile of a dense FP8 call (0 = automatic)
+  int router_form = 0;                   // test harness only: 0 = automatic, 1 = two launches, 2 = one launch, 3 = one launch of clusters
 };
 
 // Launch with the programmatic-stream-serialization attribute (see pdl_wait above).
@@ -295,6 +297,8 @@ struct qarl_ctx {
   unsigned long long wait_limit_ns = 0;  // 0: default; set only by the test harness
   int stop_after_stages = -1;            // -1: off; set only by the test harness
   int gemm_path = 0;                     // 0: automatic; set only by the test harness
+  int dense_columns = 0;                 // the same
+  int router_form = 0;                   // the same
   qarl::EncodeTiledFn encode;
   char err[256];
   // stage timing: marks[i] closes stage mark_stage[i] (-1: an opening mark)

@@ -89,6 +89,7 @@ struct Bf16Params {
   float* c_f32;       // [Mo, No] or nullptr
   int* status;
   unsigned long long wait_limit_ns;
+  int stop_after_stages;  // test harness only (< 0: off): the TMA producer stops arming stages after this many
 };
 
 struct __align__(8) SmemTail {
@@ -311,11 +312,14 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       int stage = 0;
       uint32_t phase = 0;
       uint32_t armed = 0, armed_parity = 0;
+      int armed_total = 0;
       bool ok = true;
       // steps [from, to) of tile t into the ring
       auto feed = [&](const Tile& t, int from, int to, int acc) {
         const int i0 = t.i0, j0 = t.j0;
         for (int ks = from; ks < to; ++ks) {
+          if (p.stop_after_stages >= 0 && armed_total >= p.stop_after_stages) { ok = false; return; }
+          ++armed_total;
           if (!wait_or_abort(&s->empty[stage], phase ^ 1, s, p)) { ok = false; return; }
           uint8_t* a_dst = smem + static_cast<size_t>(stage) * kStageBytes;
           uint8_t* b_dst = a_dst + kABytes;
@@ -747,7 +751,8 @@ cudaError_t launch_gemm_bf16(const Launch& L, EncodeTiledFn encode, const GemmBf
   p.c_bf16 = a.c_bf16;
   p.c_f32 = a.c_f32;
   p.status = L.d_status;
-  p.wait_limit_ns = 2000000000ull;
+  p.wait_limit_ns = L.wait_limit_ns ? L.wait_limit_ns : 2000000000ull;
+  p.stop_after_stages = L.stop_after_stages;
   const int64_t n_tiles = (a.No + BN - 1) / BN;
   const int64_t m_tiles = (a.Mo + TM - 1) / TM;
   if (grouped_rows)  // each expert adds at most one partial row tile

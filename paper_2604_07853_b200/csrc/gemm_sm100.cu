@@ -826,7 +826,7 @@ bool linear_fused_applies(const Launch& L, int64_t M, int64_t N, int64_t K) {
   // One launch instead of two: every CTA quantizes all rows itself, two passes over its 8 warps at most (64 groups), and has
   // one tile (one token, by graph replay: N = 5120, K = 2048 7.8 -> 6.9 us, N = 2048, K = 768 5.5 -> 4.6; 256 groups
   // would cost 12.3 against 11.1).
-  return L.gemm_path == 0 && M <= kFusedRows && M * (K / BK) <= 64 && N / 64 <= L.sm_count;
+  return L.gemm_path == 0 && L.dense_columns == 0 && M <= kFusedRows && M * (K / BK) <= 64 && N / 64 <= L.sm_count;
 }
 
 cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a, CUresult* cu_err) {
@@ -837,8 +837,9 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
   // drawing of tiles (N = 2048, K = 4096, one token, by graph replay: 14.4 us there, 10.2 here; N = 16384, K = 2048:
   // 10.9 there, 13.6 here).
   const bool one_round = a.offsets == nullptr && a.N / 64 <= L.sm_count;
+  const bool forced = L.dense_columns != 0 && a.mode == kModeLinear && a.offsets == nullptr;
   if (L.gemm_path == 2 ? ((a.offsets != nullptr || a.E == 1) && a.K / BK <= 64)
-                       : (L.gemm_path == 0 && !one_round && gemm_decode_applies(a)))
+                       : (L.gemm_path == 0 && !forced && !one_round && gemm_decode_applies(a)))
     return launch_gemm_decode(L, encode, a, cu_err);
   // Columns per tile of a dense call: the width whose full rounds over the SMs cost least.  Per round 128 columns take
   // ~0.6 of what 256 take, 64 ~0.45 (M = 777, N = 2048, K = 4096: 56 tiles of 256 on 148 SMs 23.6 us, 112 of 128
@@ -852,6 +853,7 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
     double best = cost(BN, 1.0);
     if (const double c = cost(128, 0.6); c < best) { best = c; cols = 128; }
     if (const double c = cost(64, 0.45); c < best) { best = c; cols = 64; }
+    if (forced) cols = L.dense_columns;
   }
   GemmParams p{};
   if (a.x != nullptr) {

@@ -97,6 +97,7 @@ struct W4Params {
   const float* pair_weights;
   int* status;
   unsigned long long wait_limit_ns;
+  int stop_after_stages;     // test harness only (< 0: off): the producers stop arming stages after this many
 };
 
 struct __align__(8) SmemTail {
@@ -253,13 +254,13 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
   if (warp == kTokenWarp) {
     // =============================== producer of the token rows =======================
     if (elect_one()) {
-      int xs = 0, cur_e = 0;
+      int xs = 0, cur_e = 0, left = p.stop_after_stages;
       uint32_t x_phase = 0, armed = 0, armed_parity = 0;
       bool ok = true;
       for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
         const TileCoord c = decode_tile(s->off, s->prefix, NT, T, cur_e);
         for (int g = 0; g < KG; ++g) {
-          if (!wait_or_abort(&s->x_empty[xs], x_phase ^ 1, s, p)) { ok = false; break; }
+          if (left-- == 0 || !wait_or_abort(&s->x_empty[xs], x_phase ^ 1, s, p)) { ok = false; break; }
           mbar_arrive_expect_tx(&s->x_full[xs], C::kXBytes);
           uint8_t* dst = x_base + static_cast<size_t>(xs) * C::kXBytes;
           tma_load_2d(dst, &tm_x, &s->x_full[xs], 2 * g * BK, c.m0);
@@ -278,7 +279,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
     // =============================== producer of the codes ============================
     // Per quantization group bulk copies of the two blocks' codes (8 KB each), scales and zero points.
     if (elect_one()) {
-      int qs = 0, cur_e = 0;
+      int qs = 0, cur_e = 0, left = p.stop_after_stages;
       uint32_t q_phase = 0, armed = 0, armed_parity = 0;
       bool ok = true;
       for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
@@ -289,7 +290,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
         tile_blocks<MODE>(p, c.n_tile, nb_lo, nb_hi);
         int64_t sz = static_cast<int64_t>(c.e) * KG * p.N;
         for (int g = 0; g < KG; ++g, sz += p.N) {
-          if (!wait_or_abort(&s->q_empty[qs], q_phase ^ 1, s, p)) { ok = false; break; }
+          if (left-- == 0 || !wait_or_abort(&s->q_empty[qs], q_phase ^ 1, s, p)) { ok = false; break; }
           uint8_t* dst = q_base + static_cast<size_t>(qs) * kGroupBytes;
           uint64_t* bar = &s->q_full[qs];
           mbar_arrive_expect_tx(bar, FMT == kFmtInt4 ? kGroupBytes : kCodeBytes + 4 * BW);
@@ -316,7 +317,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
     // The same for scales and zero points that are not 16-byte aligned (the interface promises 2 and 1): plain loads,
     // lane l rows l, l + 32, ..., written to the stage by this warp; their latency is paid per group (gate_up of 96
     // tokens 94 us instead of 70).
-    int qs = 0, cur_e = 0;
+    int qs = 0, cur_e = 0, left = p.stop_after_stages;
     uint32_t q_phase = 0, armed = 0, armed_parity = 0;
     bool ok = true;
     for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
@@ -335,7 +336,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
           sc[r] = __ldg(p.b_scales + at);
           if constexpr (FMT == kFmtInt4) z[r] = __ldg(p.b_zeros + at);
         }
-        if (!warp_wait_or_abort(&s->q_empty[qs], q_phase ^ 1, s, p)) { ok = false; break; }
+        if (left-- == 0 || !warp_wait_or_abort(&s->q_empty[qs], q_phase ^ 1, s, p)) { ok = false; break; }
         uint8_t* dst = q_base + static_cast<size_t>(qs) * kGroupBytes;
         if (lane == 0) {
           mbar_arrive_expect_tx(&s->q_full[qs], kCodeBytes);
@@ -661,6 +662,7 @@ cudaError_t launch_gemm_w4a16(const Launch& L, EncodeTiledFn encode, const GemmW
   p.pair_weights = a.pair_weights;
   p.status = L.d_status;
   p.wait_limit_ns = L.wait_limit_ns ? L.wait_limit_ns : 2000000000ull;
+  p.stop_after_stages = L.stop_after_stages;
   switch (a.mode) {
     case kModeLinear: return launch_mode<kModeLinear>(L, tx, p, a.fmt, nt);
     case kModeGateUp: return launch_mode<kModeGateUp>(L, tx, p, a.fmt, nt);

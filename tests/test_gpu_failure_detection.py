@@ -74,14 +74,94 @@ def test_gemm_pipeline_wait_expires_and_context_survives(stop_after):
     ctx.close()
 
 
+def _gives_up(ctx, stop_after, call):
+    """`call` with producers that stop: the status says so within the second, nothing else happens; then it is normal again."""
+    ref = [t.clone() for t in call()]
+    assert ctx.poll() == 0
+    ctx.harness_set_wait_limit_ns(1_000_000)
+    ctx.harness_stop_producer_after(stop_after)
+    t0 = time.perf_counter()
+    call()
+    assert ctx.poll() == -7
+    assert time.perf_counter() - t0 < 1.0
+    ctx.harness_stop_producer_after(-1)
+    ctx.harness_set_wait_limit_ns(0)
+    assert ctx.poll() == 0
+    for _ in range(2):
+        out = call()
+        assert all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(out, ref)) and ctx.poll() == 0
+
+
+@pytest.fixture
+def ctx():
+    build.build()
+    c = binding.Context(0)
+    yield c
+    c.close()
+
+
 @pytest.mark.parametrize("stop_after", [0, 1, 5])
-def test_router_pipeline_wait_expires_and_context_survives(stop_after):
-    """The same for the one-launch router: its TMA producer stops arming stages, the MMA role's bounded
+@pytest.mark.parametrize("m,columns", [(300, 64), (300, 128), (300, 256), (8, 0)])
+def test_every_dense_form_gives_up(ctx, m, columns, stop_after):
+    """The dense FP8 call with tiles of 64, 128 and 256 columns, and (8 rows, choice by size) the form that quantizes its
+    rows itself."""
+    case = inputs.linear_case(5, m, 384, 1024)              # 8 K-blocks
+    w = ctx.quantize_weight(bits_to_torch(case.w))
+    x = bits_to_torch(case.x)
+    ctx.harness_set_dense_columns(columns)
+    _gives_up(ctx, stop_after, lambda: [ctx.linear_fwd(x, *w)])
+
+
+def _unaligned(t):
+    """The same values one element further on in memory."""
+    buf = torch.empty(t.numel() + 1, dtype=t.dtype, device="cuda")
+    buf[1:] = t.reshape(-1)
+    return buf[1:].view(t.shape)
+
+
+@pytest.mark.parametrize("stop_after", [0, 1, 3])
+@pytest.mark.parametrize("m", [8, 40, 200])                 # tiles of 32, 64 and 128 token rows
+@pytest.mark.parametrize("aligned", [True, False])
+def test_four_bit_gemm_gives_up(ctx, m, aligned, stop_after):
+    """The 4-bit GEMM, with the bulk copies of scales and zero points and with its own loads of unaligned ones."""
+    case = inputs.linear_case(6, m, 384, 1024)              # 8 quantization groups
+    packed, scales, zeros = ctx.quantize_weight_w4(bits_to_torch(case.w))
+    if not aligned:
+        scales, zeros = _unaligned(scales), _unaligned(zeros)
+    x = bits_to_torch(case.x)
+    _gives_up(ctx, stop_after, lambda: [ctx.linear_fwd_w4a16(x, packed, scales, zeros)])
+
+
+@pytest.mark.parametrize("stop_after", [0, 1, 5])
+def test_dense_backward_gives_up(ctx, stop_after):
+    case = inputs.linear_case(7, 520, 384, 512)
+    dy = torch.randn((520, 384), device="cuda").to(torch.bfloat16)
+    x, w = bits_to_torch(case.x), bits_to_torch(case.w)
+    _gives_up(ctx, stop_after, lambda: [t for t in ctx.linear_bwd(dy, x, w) if t is not None])
+
+
+@pytest.mark.parametrize("stop_after", [0, 1, 3])          # (the longest contraction is 5 steps)
+@pytest.mark.parametrize("dx,dw", [(True, False), (False, True)])
+def test_grouped_backward_gives_up(ctx, dx, dw, stop_after):
+    """Grouped rows (dX) and the grouped contraction (dW: two accumulators, and a warp that follows every step)."""
+    sizes = [300, 0, 17, 70, 1, 130]
+    offsets = torch.tensor(np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32), device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(1)
+    dy, x, w = (torch.randn(s, device="cuda", generator=g).to(torch.bfloat16)
+                for s in ((sum(sizes), 512), (sum(sizes), 256), (len(sizes), 512, 256)))
+    _gives_up(ctx, stop_after, lambda: [t for t in ctx.grouped_linear_bwd(dy, x, w, offsets, dx=dx, dw=dw) if t is not None])
+
+
+@pytest.mark.parametrize("form", [2, 3])
+@pytest.mark.parametrize("stop_after", [0, 1, 5])
+def test_router_pipeline_wait_expires_and_context_survives(stop_after, form):
+    """The same for the one-launch routers (2: persistent CTAs, 3: clusters): the TMA producer stops arming stages, the MMA role's bounded
     wait (1 ms here) runs out, the CTA aborts (epilogue warps leave through the abort flag, logits
     stores in flight are waited for, TMEM is freed), the status word says QARL_ERR_DEVICE_TIMEOUT and
     the next call gives the reference bytes."""
     build.build()
     ctx = binding.Context(0)
+    ctx.harness_set_router_form(form)
     rng = np.random.default_rng(8)
     x = bits_to_torch(inputs.act_bf16(rng, 300, 512))       # 3 tiles of 8 contraction steps each
     wr = bits_to_torch(inputs.weight_bf16(rng, 64, 512))

@@ -139,10 +139,42 @@ def test_linear_empty_and_errors(ctx):
                                    (65, 128, 256), (127, 384, 512), (300, 640, 384), (1000, 1280, 256)])
 def test_small_dense_tiles_equal_the_prequantized_call(ctx, m, n, k):
     """Around the limits of the form that quantizes its rows inside the GEMM (8 rows, 64 groups, one 64-column tile per
-    SM) and of the 64- and 128-column tiles: rows equal the pre-quantized call's byte for byte, and the oracle's
-    to the tolerance of the other tests."""
+    SM): rows equal the pre-quantized call's byte for byte where that form applies, and the oracle's to the tolerance
+    of the other tests there and at the sizes beyond."""
     case = inputs.linear_case(77 + m + n + k, m, n, k)
     check_linear(ctx, case)
     xt = bits_to_torch(case.x)
     w = ctx.quantize_weight(bits_to_torch(case.w))
     assert torch.equal(ctx.linear_fwd(xt, *w), ctx.linear_fwd_q(*ctx.quantize_act(xt), *w))
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 128, 128), (7, 640, 1152), (8, 256, 8192), (9, 384, 4096), (65, 128, 256), (127, 384, 512),
+                                   (129, 640, 2048), (257, 256, 128), (300, 1280, 768), (1000, 1280, 256), (2, 9600, 256)])
+def test_every_tile_width_gives_the_same_bytes(ctx, m, n, k):
+    """One input through tiles of 64, 128 and 256 columns (forced by the harness switch), the decode kernel and the choice by
+    size, on bf16 rows and on quantized ones: the same fp32 sums and the same bf16 rows.  Rows taken out of the batch, in
+    batches that go to other forms, too."""
+    case = inputs.linear_case(500 + m + n + k, m, n, k)
+    x = bits_to_torch(case.x)
+    w = ctx.quantize_weight(bits_to_torch(case.w))
+    xq = ctx.quantize_act(x)
+    y, y32 = (t.clone() for t in ctx.linear_fwd(x, *w, want_f32=True))
+    o32, _ = oracle.linear_q(*(t.cpu().numpy() for t in (*xq, *w)))
+    nx, nw = _dequant_norms(*(t.cpu().numpy() for t in (*xq, *w)))
+    assert (np.abs(y32.cpu().numpy().astype(np.float64) - o32) <= 1e-3 * nx[:, None] * nw[None, :]).all()
+    try:
+        for columns, path in ((64, 0), (128, 0), (256, 0), (0, 2), (0, 0)):
+            ctx.harness_set_dense_columns(columns)
+            ctx.harness_set_gemm_path(path)
+            for got in (ctx.linear_fwd(x, *w, want_f32=True), ctx.linear_fwd_q(*xq, *w, want_f32=True)):
+                assert torch.equal(got[0].view(torch.int16), y.view(torch.int16)), (columns, path)
+                assert torch.equal(got[1].view(torch.int32), y32.view(torch.int32)), (columns, path)
+            assert torch.equal(ctx.linear_fwd_q(*xq, *w).view(torch.int16), y.view(torch.int16))
+    finally:
+        ctx.harness_set_dense_columns(0)
+        ctx.harness_set_gemm_path(0)
+    for rows in (1, 8, 9, 65):
+        if rows < m:
+            at = torch.arange(m - rows, m, device="cuda")
+            assert torch.equal(ctx.linear_fwd(x[at].contiguous(), *w), y[at])
+    assert ctx.poll() == 0

@@ -21,6 +21,25 @@ def ctx():
     c.close()
 
 
+def through_every_form(ctx, x, w, k):
+    """One input through the automatic choice, the persistent one-launch router, the cluster router and the two launches,
+    forced by the harness switch: the same bytes from each.  Returns the automatic choice's outputs."""
+    m, e = x.shape[0], w.shape[0]
+    clusters = e <= 128 and m <= 4096  # (more tokens than that may not fit the clusters of one round)
+    out = []
+    for form, launches in ((0, None), (2, 1 if e <= 128 and k <= 16 else 2), (3, 1 if clusters else None), (1, 2)):
+        ctx.harness_set_router_form(form)
+        before = ctx.launch_count()
+        out.append([t.clone() for t in ctx.router_fwd(x, w, k)])
+        ctx.harness_set_router_form(0)
+        assert launches is None or ctx.launch_count() - before == launches, form
+    assert ctx.poll() == 0
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            assert torch.equal(a.view(torch.int32), b.view(torch.int32))
+    return out[0]
+
+
 def check_router(ctx, seed, m, h, e, k):
     """Logits within the GEMM tolerance of the exact ones; the selection and the weights teacher-forced:
     the oracle's top-k on the GPU's own logits must give the same ids bit for bit (an arg-max decided
@@ -56,13 +75,13 @@ def test_router_ties_and_equal_logits(ctx):
     wr[5] = wr[2]
     wr[9] = wr[2]
     wr[15] = wr[0]
-    logits, ids, wts = ctx.router_fwd(bits_to_torch(x), bits_to_torch(wr), 6)
+    logits, ids, wts = through_every_form(ctx, bits_to_torch(x), bits_to_torch(wr), 6)
     g = logits.cpu().numpy()
     assert np.array_equal(g[:, 5], g[:, 2]) and np.array_equal(g[:, 9], g[:, 2])
     o_ids, o_w = oracle.router_topk(g, 6)
     assert np.array_equal(ids.cpu().numpy(), o_ids)
     zero = torch.zeros((4, 256), dtype=torch.bfloat16, device="cuda")      # all logits equal (0)
-    _, ids0, w0 = ctx.router_fwd(zero, bits_to_torch(wr), 4)
+    _, ids0, w0 = through_every_form(ctx, zero, bits_to_torch(wr), 4)
     assert ids0.cpu().numpy().tolist() == [[0, 1, 2, 3]] * 4 and torch.all(w0 == 0.25)
 
 
@@ -77,21 +96,15 @@ def test_routing_does_not_depend_on_the_batch(ctx):
 @pytest.mark.parametrize("m,h,e,k", [(1, 64, 8, 1), (300, 2048, 128, 8), (1000, 520, 40, 8), (129, 512, 128, 32),
                                      (4133, 1024, 96, 6), (3, 8, 8, 8), (129, 72, 24, 24), (40000, 128, 128, 8)])
 def test_one_launch_router_equals_the_two_launch_router(ctx, m, h, e, k):
-    """Up to 128 experts the selection runs in the epilogue of the logits GEMM (one launch); the harness
-    switch forces the separate selection kernel.  Logits, ids and weights must be the same bytes: the
-    same MMA sequence per row, the same selection rule, the softmax summed in the same order."""
+    """Up to 128 experts the selection runs in the epilogue of the logits GEMM (one launch, persistent CTAs or clusters of
+    CTAs by size); the harness switch forces each and the separate selection kernel.  Logits, ids and weights must
+    be the same bytes: the same MMA sequence per row, the same selection rule, the softmax summed in the same order."""
     rng = np.random.default_rng(900 + m)
     x = bits_to_torch(inputs.act_bf16(rng, m, h))
     wr_bits = inputs.weight_bf16(rng, e, h)
     wr_bits[e - 1] = wr_bits[0]                              # a tie between the first and the last expert
     wr = bits_to_torch(wr_bits)
-    fused = ctx.router_fwd(x, wr, k)
-    ctx.harness_set_gemm_path(1)
-    split = ctx.router_fwd(x, wr, k)
-    ctx.harness_set_gemm_path(0)
-    assert ctx.poll() == 0
-    for a, b in zip(fused, split):
-        assert torch.equal(a.view(torch.int32), b.view(torch.int32))
+    fused = through_every_form(ctx, x, wr, k)
     ids = fused[1].cpu().numpy()
     assert ((ids >= 0) & (ids < e)).all() and all(len(set(r)) == k for r in ids[:: max(1, m // 50)].tolist())
 
@@ -99,9 +112,9 @@ def test_one_launch_router_equals_the_two_launch_router(ctx, m, h, e, k):
 @pytest.mark.parametrize("e,k,hot", [(128, 16, range(0, 16)), (128, 16, range(16, 32)), (128, 8, range(120, 128)),
                                      (40, 16, range(0, 16)), (128, 16, [0, 17, 33, 34, 35, 50, 66, 67, 82, 98, 99, 100, 113, 114, 126, 127])])
 def test_selection_concentrated_in_few_groups(ctx, e, k, hot):
-    """The one-launch router keeps one candidate per group of 16 experts and re-scans only the winner's group:
+    """The persistent one-launch router keeps one candidate per group of 16 experts and re-scans only the winner's group:
     batches whose k largest logits all sit in one group (also the first, which then runs almost empty) or are
-    spread one per group must select what the oracle's plain scan selects on the same logits, in both forms."""
+    spread one per group must select what the oracle's plain scan selects on the same logits, in every form."""
     rng = np.random.default_rng(5 + e + k)
     h = 256
     u = rng.standard_normal(h).astype(np.float32)
@@ -112,13 +125,7 @@ def test_selection_concentrated_in_few_groups(ctx, e, k, hot):
     w[hot[1]] = w[hot[0]]                                                            # and one exact tie
     xt = torch.from_numpy(x).to(torch.bfloat16).cuda()
     wt = torch.from_numpy(w).to(torch.bfloat16).cuda()
-    fused = ctx.router_fwd(xt, wt, k)
-    ctx.harness_set_gemm_path(1)
-    split = ctx.router_fwd(xt, wt, k)
-    ctx.harness_set_gemm_path(0)
-    assert ctx.poll() == 0
-    for a, b in zip(fused, split):
-        assert torch.equal(a.view(torch.int32), b.view(torch.int32))
+    fused = through_every_form(ctx, xt, wt, k)
     o_ids, _ = oracle.router_topk(fused[0].cpu().numpy(), k)
     ids = fused[1].cpu().numpy()
     assert np.array_equal(ids, o_ids)
@@ -127,7 +134,7 @@ def test_selection_concentrated_in_few_groups(ctx, e, k, hot):
 
 def test_router_with_non_finite_activations(ctx):
     """Infinite and NaN activations give infinite and NaN logits; whatever the selection does with them, the
-    ids stay inside [0, E) and distinct, and both forms of the router do the same."""
+    ids stay inside [0, E) and distinct, and every form of the router does the same."""
     rng = np.random.default_rng(77)
     x = bits_to_torch(inputs.act_bf16(rng, 64, 256)).clone()
     x[3, 5] = float("inf")
@@ -136,16 +143,9 @@ def test_router_with_non_finite_activations(ctx):
     x[11, 1] = float("inf")
     x[11, 2] = float("-inf")
     wr = bits_to_torch(inputs.weight_bf16(rng, 32, 256))
-    fused = ctx.router_fwd(x, wr, 4)
-    ctx.harness_set_gemm_path(1)
-    split = ctx.router_fwd(x, wr, 4)
-    ctx.harness_set_gemm_path(0)
-    assert ctx.poll() == 0
+    fused = through_every_form(ctx, x, wr, 4)
     ids = fused[1].cpu().numpy()
     assert ((ids >= 0) & (ids < 32)).all() and all(len(set(r)) == 4 for r in ids.tolist())
-    assert torch.equal(fused[1], split[1])
-    assert torch.equal(fused[0].view(torch.int32), split[0].view(torch.int32))
-    assert torch.equal(fused[2].view(torch.int32), split[2].view(torch.int32))
     o_ids, _ = oracle.router_topk(fused[0].cpu().numpy(), 4)
     assert np.array_equal(ids, o_ids)
 

@@ -415,3 +415,32 @@ def test_quantizer_next_to_every_boundary(ctx, fmt):
     quantize = ctx.quantize_weight_w4 if fmt == "w4" else ctx.quantize_weight_fp4
     packed = (oracle.quantize_weight_w4 if fmt == "w4" else oracle.quantize_weight_fp4)(w)[0]
     assert np.array_equal(unpack_lib(quantize(bits_to_torch(w))[0].cpu().numpy()), unpack_linear(packed))
+
+
+def _shifted(t):
+    """The same values one element further on in memory."""
+    buf = torch.empty(t.numel() + 1, dtype=t.dtype, device="cuda")
+    buf[1:] = t.reshape(-1)
+    return buf[1:].view(t.shape)
+
+
+@pytest.mark.parametrize("fmt", ["w4", "fp4"])
+def test_scales_and_zero_points_need_no_alignment(ctx, fmt):
+    """Scales on any 2-byte and zero points on any byte boundary: read by plain loads instead of bulk copies, the same bytes
+    out, in every tile size (8, 40 and 200 rows; groups of a few and of many rows)."""
+    quantize = ctx.quantize_weight_w4 if fmt == "w4" else ctx.quantize_weight_fp4
+    linear = ctx.linear_fwd_w4a16 if fmt == "w4" else ctx.linear_fwd_fp4a16
+    layer = ctx.moe_fwd_w4a16 if fmt == "w4" else ctx.moe_fwd_fp4a16
+    for m in (8, 40, 200):
+        c = inputs.linear_case(40 + m, m, 384, 1152)
+        x, w = bits_to_torch(c.x), quantize(bits_to_torch(c.w))
+        moved = (w[0], *(_shifted(t) for t in w[1:]))
+        assert all(t.data_ptr() % 16 for t in moved[1:])
+        assert torch.equal(linear(x, *moved), linear(x, *w))
+    for m in (12, 100, 400):
+        c = inputs.moe_case(50 + m, m, h=256, i=384, e=8, k=2)
+        x, ids, wts = bits_to_torch(c.x), torch.from_numpy(c.ids).cuda(), torch.from_numpy(c.weights).cuda()
+        w = [quantize(bits_to_torch(t)) for t in (c.w13, c.w2)]
+        moved = [(t[0], *(_shifted(u) for u in t[1:])) for t in w]
+        assert torch.equal(layer(x, ids, wts, *moved).clone(), layer(x, ids, wts, *w))
+    assert ctx.poll() == 0
