@@ -343,7 +343,7 @@ int qarl_moe_fwd(qarl_ctx* ctx, const void* x, const int32_t* ids, const float* 
   d.offsets = pb.offsets;
   d.out_bf16 = contrib;
   d.out_f32 = dbg ? dbg->down_f32 : nullptr;
-  d.sorted_pair = nullptr;  // contributions stay in sorted order (dense row blocks); the k-sum finds them by position
+  // (contributions stay in sorted order, dense row blocks; the k-sum finds them by position)
   d.pair_weights = sorted_w;
 
   int rc;

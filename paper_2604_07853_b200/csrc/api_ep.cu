@@ -144,7 +144,6 @@ int qarl_moe_experts_fwd(qarl_ctx* ctx, const uint8_t* codes, const float* scale
   d.E = E_local;
   d.offsets = offsets;
   d.out_bf16 = static_cast<uint16_t*>(contrib);
-  d.sorted_pair = nullptr;  // contributions stay in the order the rows came in
   d.pair_weights = row_weights;
   rc = run_gemm(ctx, L, d);
   if (rc != QARL_OK) return rc;

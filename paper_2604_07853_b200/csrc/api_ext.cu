@@ -191,7 +191,7 @@ int moe_w4(qarl_ctx* ctx, int fmt, const void* x, const int32_t* ids, const floa
   d.offsets = pb.offsets;
   d.out_bf16 = contrib;
   d.out_f32 = dbg ? dbg->down_f32 : nullptr;
-  d.sorted_pair = nullptr;  // contributions stay in sorted order (dense row blocks); the k-sum finds them by position
+  // (contributions stay in sorted order, dense row blocks; the k-sum finds them by position)
   d.pair_weights = sorted_w;
   rc = run_gemm_w4(ctx, L, d);
   if (rc != QARL_OK) return rc;

@@ -163,12 +163,11 @@ struct GemmArgs {
   // one group of rows_total rows (dense).
   const int32_t* offsets;
   // outputs
-  uint16_t* out_bf16;        // linear: y [M, N]; gate_up (debug): gate_up [P, 2I]; down: contrib [P, H] by pair id
+  uint16_t* out_bf16;        // linear: y [M, N]; gate_up (debug): gate_up [P, 2I]; down: contributions [P, H] in sorted order
   float* out_f32;            // optional fp32 accumulator dump (linear: [M,N]; down: [P,H] sorted order)
   uint8_t* h_codes;          // gate_up: [P, I]
   float* h_scales;           // gate_up: [P, I/128]
   uint16_t* h_bf16;          // gate_up (debug): [P, I]
-  const int32_t* sorted_pair;   // down: [P]
   const float* pair_weights;    // down: [M*k] by sorted position
   const uint16_t* x;            // linear where linear_fused_applies: the bf16 rows themselves (a_codes, a_scales unused)
 };
@@ -215,10 +214,9 @@ struct GemmW4Args {
   int64_t N;
   int64_t E;
   const int32_t* offsets;   // row groups per expert, or nullptr (dense)
-  uint16_t* out_bf16;       // linear: y [M, N]; gate_up (debug): gate_up [P, 2I]; down: contrib [P, H] by pair id
+  uint16_t* out_bf16;       // linear: y [M, N]; gate_up (debug): gate_up [P, 2I]; down: contributions [P, H] in sorted order
   float* out_f32;           // optional fp32 accumulator dump (linear: [M, N]; down: [P, H] sorted order)
   uint16_t* h_bf16;         // gate_up: h [P, I]
-  const int32_t* sorted_pair;
   const float* pair_weights;
 };
 cudaError_t launch_gemm_w4a16(const Launch& L, EncodeTiledFn encode, const GemmW4Args& a, CUresult* cu_err);

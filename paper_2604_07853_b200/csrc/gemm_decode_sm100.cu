@@ -94,7 +94,6 @@ struct DecodeParams {
   uint8_t* h_codes;
   float* h_scales;
   uint16_t* h_bf16;
-  const int32_t* sorted_pair;
   const float* pair_weights;
   // the layer in one launch
   const int32_t* ids;          // [M, k]
@@ -785,12 +784,10 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         }
       } else {
         for (int t = ew; t < rows; t += kEpiWarps) {  // a warp per output row: 512 bytes, 16 per lane
-          const int row = c.m0 + t;
-          int64_t out_row = row;
-          if (c.mode == kModeDown && p.sorted_pair) out_row = min(max(__ldg(p.sorted_pair + row), 0), p.rows_total - 1);
+          const int64_t row = c.m0 + t;
           const uint4 v = *reinterpret_cast<const uint4*>(out_tile + t * kOutRowBytes + lane * 16);
           const int col = 2 * j * BW + 8 * lane;
-          if (col < N) *reinterpret_cast<uint4*>(p.out_rows + out_row * N + col) = v;
+          if (col < N) *reinterpret_cast<uint4*>(p.out_rows + row * N + col) = v;
         }
       }
       __syncwarp();
@@ -964,7 +961,6 @@ cudaError_t launch_gemm_decode(const Launch& L, EncodeTiledFn encode, const Gemm
   p.h_codes = a.h_codes;
   p.h_scales = a.h_scales;
   p.h_bf16 = a.h_bf16;
-  p.sorted_pair = a.sorted_pair;
   p.pair_weights = a.pair_weights;
   p.status = L.d_status;
   p.wait_limit_ns = L.wait_limit_ns ? L.wait_limit_ns : 2000000000ull;
@@ -1012,7 +1008,6 @@ cudaError_t launch_moe_decode_layer(const Launch& L, EncodeTiledFn encode, const
   p.h_codes = g.h_codes;
   p.h_scales = g.h_scales;
   p.h_bf16 = g.h_bf16;
-  p.sorted_pair = d.sorted_pair;
   p.pair_weights = d.pair_weights;
   p.ids = ids;
   p.pos_of_pair = pos_of_pair;
