@@ -9,6 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libqarl.so")
 NATIVE = os.path.join(HERE, "_native.so")
+NATIVE_KEY = os.path.join(HERE, "_native.key")  # what _native.so was built against
 SOURCES = ["api.cu", "quantize.cu", "permute.cu", "combine.cu", "gemm_sm100.cu", "gemm_decode_sm100.cu", "harness.cu", "linear_static.cu",
            "gemm_w4a16_sm100.cu", "api_ext.cu", "api_ep.cu", "gemm_bf16_sm100.cu", "tbpo.cu", "router.cu", "router_fused_sm100.cu", "router_cluster_sm100.cu", "moe_bwd.cu"]
 HEADERS = ["common.cuh", "quant_device.cuh", "w4_dequant.cuh", "ptx_sm100.cuh", "sched.cuh", "router_select.cuh", "api_util.cuh", os.path.join("..", "..", "include", "qarl.h"),
@@ -28,6 +29,25 @@ def _stale(target: str, sources) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def native_key() -> str:
+    """The interpreter and the torch whose headers and libraries _native.so depends on: built against others it may fail to
+    import, or import and misread their objects."""
+    import importlib.metadata
+    import importlib.util
+    import sysconfig
+
+    where = os.path.dirname(importlib.util.find_spec("torch").origin)
+    return "\n".join((sysconfig.get_config_var("SOABI"), sysconfig.get_paths()["include"], importlib.metadata.version("torch"), where))
+
+
+def _native_is_for_this_python() -> bool:
+    try:
+        with open(NATIVE_KEY) as f:
+            return f.read() == native_key()
+    except OSError:
+        return False
+
+
 def _build_native() -> None:
     import sysconfig
 
@@ -41,6 +61,8 @@ def _build_native() -> None:
         "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10",
         "-Wl,-rpath,$ORIGIN"])
     os.replace(tmp, NATIVE)
+    with open(NATIVE_KEY, "w") as f:
+        f.write(native_key())
 
 
 def _build_library(verbose: bool) -> None:
@@ -58,7 +80,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
     """Compile what is missing or older than its sources; returns the library's path."""
     if force or _stale(LIB, SOURCES + HEADERS):
         _build_library(verbose)
-    if force or _stale(NATIVE, ["native_binding.cpp", os.path.join("..", "..", "include", "qarl.h")]):
+    if (force or not _native_is_for_this_python() or
+            _stale(NATIVE, ["native_binding.cpp", os.path.join("..", "..", "include", "qarl.h")])):
         _build_native()
     return LIB
 
