@@ -840,7 +840,7 @@ def main():
                         f"{tbytes / 1e6:.0f} MB per step, larger than L2",
             "ms_per_step": t_ms, "tokens_per_s": world * Tt / (t_ms * 1e-3),
             "algorithmic_bytes": tbytes, "gbs": tbytes / (t_ms * 1e-3) / 1e9,
-            "frac_hbm_measured": tbytes / (t_ms * 1e-3) / 1e9 / pk["hbm_gbs"], "launches_per_step": 4,
+            "frac_hbm_measured": tbytes / (t_ms * 1e-3) / 1e9 / pk["hbm_gbs"], "launches_per_step": 2,
         }
         del tcase, tout, tws
 

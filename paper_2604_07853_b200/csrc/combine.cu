@@ -1,8 +1,7 @@
 // Top-k weighted combine: out[t] = bf16( sum_j float(c[t,j]) ), the token's k bf16
 // contributions added in ASCENDING EXPERT ID starting from 0.0f -- a fixed order (App. C), so
 // the result does not depend on the caller's slot order or on how the batch was tiled.
-// contrib is [M*k, H] bf16 indexed by flat pair id, or, with `pos_of_pair`, by the pair's position in
-// the expert-sorted order (rows that came back from other GPUs' experts); HBM-bound, 128-bit accesses.
+// contrib is [M*k, H] bf16 in expert-sorted order, a pair's row at pos_of_pair; HBM-bound, 128-bit accesses.
 #include "common.cuh"
 
 namespace qarl {
@@ -27,8 +26,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const uint16_t* __restrict
       if (other < mine || (other == mine && j < tid)) ++rank;
       if (other == mine && j != tid) set_status(status, QARL_ERR_BAD_EXPERT_ID);  // expert repeated in a token
     }
-    const int64_t pair = t * k + tid;
-    order[rank] = pos_of_pair ? min(max(static_cast<int64_t>(pos_of_pair[pair]), int64_t(0)), M * k - 1) : pair;
+    order[rank] = min(max(static_cast<int64_t>(pos_of_pair[t * k + tid]), int64_t(0)), M * k - 1);
   }
   __syncthreads();
   for (int64_t c = static_cast<int64_t>(tid) * 8; c < H; c += 256 * 8) {

@@ -136,9 +136,9 @@ cudaError_t launch_moe_prep_small(const Launch& L, const int32_t* ids, int64_t M
                                   uint8_t* codes, float* scales, float* sorted_w, int32_t* zero = nullptr,
                                   int zero_count = 0);
 
-// pos_of_pair == nullptr: contrib is indexed by flat pair id; else by pos_of_pair[pair] (sorted order)
+// contrib in sorted order: a pair's row is pos_of_pair[pair]
 cudaError_t launch_combine(const Launch& L, const uint16_t* contrib, const int32_t* ids, int64_t M, int64_t k,
-                           int64_t H, int64_t E, uint16_t* out, const int32_t* pos_of_pair = nullptr);
+                           int64_t H, int64_t E, uint16_t* out, const int32_t* pos_of_pair);
 
 cudaError_t launch_wait_selftest(const Launch& L, unsigned long long limit_ns);
 cudaError_t launch_fp8_mma_peak(const Launch& L, int kblocks);

@@ -6,7 +6,7 @@
 // its N side:
 //   D[n, t] = sum_k w^[n, k] x[t, k]      (kind::f16, M = 128, N = NT, K = 16, A from TMEM)
 // The bf16 products are exact, and the whole K reduction accumulates in TMEM in ascending k whatever NT is, so a
-// token's output row has the same bits for every tile size and batch (App. C; the tests compare the two sizes).
+// token's output row has the same bits for every tile size and batch (App. C; the tests compare the sizes).
 //
 // Why tensor memory: expanded weights that travel through shared memory cost a 128-byte-per-clock port 2 bytes of
 // stores and 2 of operand reads per weight.  Measured per 64 KB (256 rows x 128 k) on one SM: 616 clocks of stores with
@@ -14,15 +14,15 @@
 // memory (bound by reading A) against 16 with A in TMEM (its multiply rate).  What is left is the expansion's own
 // arithmetic (measured 740 clocks per 64 KB for integer codes, 920 for e2m1 with its general scale: bf16x2 instructions
 // issue at half rate) and, at decode, the weight stream.  Layer of 96 / 1024 / 4096 tokens (128 experts, top-8): integer 177 /
-// 223 / 562 -> 117 / 200 / 484 us, e2m1 209 / 238 / 585 -> 130 / 210 / 501.
+// 223 / 562 -> 113 / 170 / 467 us, e2m1 209 / 238 / 585 -> 121 / 188 / 472.
 //
 // A tile = (expert e, pair of weight blocks j, chunk of <= NT rows of the expert's group):
 //   gate_up: blocks j (gate rows) and j + I/128 (the matching up rows); down/linear: blocks 2j, 2j+1.
-// CTA: epilogue warps (4, or 8 with NT = 128; thread = weight row: TMEM -> SwiGLU / weighting -> bf16, transposed
+// CTA: 8 epilogue warps (thread = weight row: TMEM -> SwiGLU / weighting -> bf16, transposed
 // through shared memory so that global stores are whole token rows), 16 dequantization warps in two groups that take A
 // stages in turn (thread = one of the pair's 256 weight rows), a producer warp for the codes (bulk copies into a
 // shared-memory ring, scales and zero points with them), one for the token rows (TMA), two MMA issuers (one per block).
-// TMEM: the accumulators of 2 NT columns (two with NT = 32; with NT = 128 one: four A stages instead of two keep
+// TMEM: the accumulators of 2 NT columns (two with NT = 32 and 64; with NT = 128 one: four A stages instead of two keep
 // the tensor pipe fed, and the exposed epilogue costs less), the rest A stages.
 // What the hand-offs cost decides the stage sizes: a step of one issuing thread (two waits, its MMAs, the
 // commits) takes 300-450 clocks whatever the MMAs, so codes and token rows move in 128-element quantization groups, and
@@ -506,7 +506,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
       if (MODE == kModeDown && threadIdx.x < NT)
         s->weight[par][threadIdx.x] = __ldg(p.pair_weights + min(c.m0 + static_cast<int>(threadIdx.x), p.rows_total - 1));
       ok = warp_wait_or_abort(&s->tmem_full[acc], acc_phase, s, p);
-      ok = named_bar_all(1, kEpiThreads, ok);  // one decision for the four warps; the previous tile's row readers are done
+      ok = named_bar_all(1, kEpiThreads, ok);  // one decision for the eight warps; the previous tile's row readers are done
       if (!ok) break;
       tc_fence_after_sync();
       const uint32_t t0 = tmem_base + lane_addr + static_cast<uint32_t>(acc) * (2 * NT);

@@ -2,15 +2,15 @@
 // the experts of a 128-token tile split over the CTAs of a cluster.
 //
 // That kernel gives a token tile to one CTA: at M <= 2048 at most 16 of the 148 SMs work, and the call
-// takes what one SM needs to walk the 128 x H x 128 tile and one thread needs to select a row -- 25 us
-// at M = 1 and at M = 2048 alike.  Here CTA c of a cluster computes the logits of experts
+// takes what one SM needs to walk the 128 x H x 128 tile and one thread needs to select a row -- 13.3 us
+// at M = 1, 14.0 at M = 2048 (H = 2048, 128 experts, by graph replay; 8.2 and 12.7 here).  Here CTA c of a cluster computes the logits of experts
 // [c NC, (c + 1) NC) with an MMA of N = NC columns (the same products in the same order per logit: the
 // bits do not depend on N), every CTA sends the rows it does not own through distributed shared memory,
 // and after one cluster barrier each CTA selects for its share of the rows, a warp per row.
 //
-// NC = 16 while the clusters of 8 fit the SMs at once (M <= 2048), then 32, then 64: fewer columns per
+// NC = 16 while the clusters (of 8 with 128 experts) fit the SMs at once, then 32: fewer columns per
 // CTA mean a shorter walk, but each CTA re-reads the token tile (from L2), so a second round of clusters
-// costs more than it saves.
+// costs more than it saves.  More tokens than that go to the persistent kernel.
 //
 // Structure of a CTA (512 threads, one tile): warps 0-3 epilogue (thread = token row), warps 4 and 6
 // TMA producers (per 64-element step a box of x, and a box of NC rows of W_r: for one token the walk is

@@ -1,8 +1,7 @@
-"""The W4A16 / FP4A16 grouped GEMM has a wide-tile kernel (token rows on the MMA's M side) and a
-swapped-operand kernel for decode-sized groups (expanded weight rows on the M side, at most 32
-token rows on the N side).  Both must give the same bytes for every row (App. C: the fixed
-K-reduction order holds across kernels): one input goes through both, forced by the harness
-switch, and every stage the layer exposes is compared bit for bit; the automatic choice too."""
+"""The W4A16 / FP4A16 grouped GEMM takes 32, 64 or 128 token rows per tile by the size of the groups (the expanded weight
+rows are the MMA's M side in each).  All must give the same bytes for every row (App. C: the fixed K-reduction order
+holds across tile sizes): one input goes through the widest and the narrowest tiles, forced by the harness switch, and
+the choice by size, and every stage the layer exposes is compared bit for bit."""
 import pytest
 import torch
 
@@ -34,7 +33,7 @@ def _layer(ctx, dc, path, debug=True):
 @pytest.mark.parametrize("m,h,i,e,k,zipf", [(256, 2048, 768, 128, 8, None), (64, 512, 256, 8, 2, None), (1, 512, 256, 8, 2, None),
                                              (8, 2048, 768, 128, 8, None), (33, 256, 384, 2, 1, None),
                                              (300, 512, 256, 8, 2, 1.1), (100, 512, 128, 16, 4, 1.5)])
-def test_decode_kernel_equals_wide_kernel_stage_by_stage(ctx, fmt, m, h, i, e, k, zipf):
+def test_tile_sizes_agree_stage_by_stage(ctx, fmt, m, h, i, e, k, zipf):
     c = inputs.moe_case(31, m, h=h, i=i, e=e, k=k, zipf_s=zipf)
     dc = DeviceCase(ctx, c, fmt)
     out_w, d_w = _layer(ctx, dc, 1)
