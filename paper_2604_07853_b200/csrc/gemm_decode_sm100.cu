@@ -655,14 +655,17 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
 #pragma unroll
         for (int t = 0; t < NTH; ++t) acc_lo[t] = acc_hi[t] = 0.0f;
 
+        const int live = rows - tb;  // token columns of this warp that hold a row: the others are not promoted
         for (int kb = 0; kb < KB; ++kb) {
           if (!warp_wait_or_abort(&s->tmem_full[ks], acc_phase, s, p)) { ok = false; break; }
           tc_fence_after_sync();
           const uint32_t t0 = tmem_base + lane_addr + static_cast<uint32_t>(ks) * (2 * NT) + static_cast<uint32_t>(tb);
           uint32_t vl[NTH], vh[NTH];
-          tmem_ld_x16(t0, vl);
-          tmem_ld_x16(t0 + NT, vh);
-          tmem_ld_wait();
+          if (live > 0) {
+            tmem_ld_x16(t0, vl);
+            tmem_ld_x16(t0 + NT, vh);
+            tmem_ld_wait();
+          }
           tc_fence_before_sync();
           __syncwarp();
           if (lane == 0) mbar_arrive(&s->tmem_empty[ks]);  // both reads have landed: hand the accumulator back
@@ -670,6 +673,7 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
           const float2 sw = *reinterpret_cast<const float2*>(sl.sw[kb]);
 #pragma unroll
           for (int t4 = 0; t4 < NTH; t4 += 4) {
+            if (t4 >= live) break;
             const float4 sx = *reinterpret_cast<const float4*>(&sl.sx[kb][tb + t4]);  // same address in every lane: broadcast
             const float sxs[4] = {sx.x, sx.y, sx.z, sx.w};
 #pragma unroll
@@ -697,6 +701,7 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
           uint16_t* T16 = reinterpret_cast<uint16_t*>(out_tile);
 #pragma unroll
           for (int t = 0; t < NTH; ++t) {
+            if (t >= live) break;
             float lo = acc_lo[t], hi = acc_hi[t];
             if (c.mode == kModeDown) {  // contribution = bf16( fl(w * y) )
               const float w = sl.w[tb + t];
