@@ -20,7 +20,7 @@
 //               256-column TMEM accumulators (overwrite on the first), then tcgen05.commit to
 //               free the smem stage and to publish the accumulator;
 //   warps 10-11 scales: fl(s_x s_w) of every row and half for the K-block in each accumulator;
-//   warps 0-7   promotion (224 registers each via setmaxnreg): warp w reads TMEM lanes
+//   warps 0-7   promotion (216 registers each via setmaxnreg): warp w reads TMEM lanes
 //               32*(w%4).. (its hardware quadrant) and the 64-column slice (w/4) of each half,
 //               releases the accumulator, and adds scale * partial into fp32 registers; the
 //               MMA of block kb+1 overlaps the promotion of kb.  At the end of a tile it finishes
@@ -71,9 +71,9 @@ constexpr int kTmaWarp = 8;
 constexpr int kMmaWarp = 9;
 constexpr int kScaleWarp = 10;    // and 11
 constexpr int kThreads = 12 * 32;
-// register re-allocation: 256 x 224 + 128 x 56 = 64512 = 384 x 168 (the launch allocation)
-constexpr int kPromoRegs = 224;
-constexpr int kAuxRegs = 56;
+// register re-allocation: 256 x 216 + 128 x 72 = 64512 = 384 x 168 (the launch allocation)
+constexpr int kPromoRegs = 216;
+constexpr int kAuxRegs = 72;
 constexpr uint32_t kABytes = BM * BK;
 constexpr uint32_t kBHalfBytes = BNH * BK;
 constexpr uint32_t kTmemCols = 512;
@@ -124,7 +124,7 @@ struct Cfg {
   static constexpr int kAccBufs = COLS == 256 ? 2 : 4;
 };
 
-struct __align__(8) SmemTail {
+struct __align__(16) SmemTail {
   uint64_t full[kMaxStages];
   uint64_t empty[kMaxStages];
   uint64_t tmem_full[kMaxAccBufs];
@@ -134,6 +134,10 @@ struct __align__(8) SmemTail {
   uint64_t x_ready;            // FUSED: the rows are quantized
   float2 scale[kMaxAccBufs][BM];  // products of the K-block in each accumulator: row scale x (lo, hi) weight scale
   uint32_t amax[2][2][BM];     // gate_up: [tile parity][column slice][row] |h| maxima (bf16 bits)
+  // Grouped forms: what the promotion warps need to know about a tile, published by the scale warps with its first K-block
+  // (they may be kMaxAccBufs tiles of one K-block ahead, hence twice as many slots).
+  int4 tile[2 * kMaxAccBufs];  // first row, end of the group's rows, column tile
+  float pair_w[4][BM];         // down (two accumulators): combine weight of every row
   uint32_t tmem_addr;
   int abort_flag;
   int32_t off[kMaxExperts + 1];
@@ -297,7 +301,18 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
   };
 
   for (int T = first_tile; T < total_tiles; T += num_ctas, ++tile_iter) {
-    const TileCoord c = decode_tile<C::kTileRows>(s, T, cur_e);
+    // Grouped: looking the tile up and loading the combine weights here would keep the accumulators waiting at every tile's
+    // start and end (1501 tokens, 128 experts: gate_up 88 -> 84 us, down 57 -> 51); a dense call's single group is
+    // looked up faster than the scale warps publish it (M = 777, N = 2048, K = 4096: 17.0 against 17.5).
+    TileCoord c;
+    if constexpr (MODE == kModeLinear) {
+      c = decode_tile<C::kTileRows>(s, T, cur_e);
+      if (!full_wait()) return;
+    } else {
+      if (!full_wait()) return;
+      const int4 at = s->tile[tile_iter & (2 * kMaxAccBufs - 1)];
+      c = TileCoord{0, at.z, at.x, at.y};
+    }
     // a warp whose 32 rows all lie past the group's end (ragged tails, decode-sized groups)
     // keeps the barrier protocol going but reads and accumulates nothing
     const bool warp_live = c.m0 + q * 32 < c.m_end;
@@ -308,9 +323,10 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
     float2* const acc_hi = acc + (HALVES == 2 ? 32 : 0);
 
     if (!warp_live) {
-      for (int kb = 0; kb < KB; ++kb) {
-        if (!full_wait()) return;
+      for (int kb = 0;;) {
         release();
+        if (++kb == KB) break;
+        if (!full_wait()) return;
       }
     } else {
       // The 16-column chunks of the accumulators are one stream across the K-blocks of the tile: while a
@@ -338,7 +354,6 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
         }
         tmem_ld_x16(chunk_at(t0, kChunks - 1), vb);
       };
-      if (!full_wait()) return;
       tc_fence_after_sync();
       tmem_ld_x16(tmem + static_cast<uint32_t>(ks * COLS), va);
       read_scale();
@@ -380,7 +395,7 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
       }
     }
     if (MODE == kModeDown) {  // contribution = bf16( fl(w * y) )
-      const float w = valid ? __ldg(p.pair_weights + row) : 0.0f;
+      const float w = s->pair_w[tile_iter & 3][r];
       const float2 w2 = make_float2(w, w);
 #pragma unroll
       for (int j = 0; j < kSliceCols / 2; ++j) {
@@ -548,9 +563,9 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
       mbar_init(&s->empty[i], 1);
     }
     for (int i = 0; i < kAccBufs * C::kParts; ++i) {
-      mbar_init(&s->tmem_full[i], 3);  // the MMA commit and the two scale warps
+      mbar_init(&s->tmem_full[i], FUSED ? 2 : 3);  // the MMA commit and the two scale warps
       // (PAIR: the even CTA's MMAs write the accumulators of both)
-      mbar_init(&s->tmem_empty[i], kPromoWarps / C::kParts * (PAIR && rank == 0 ? 2 : 1));
+      mbar_init(&s->tmem_empty[i], FUSED ? 2 : kPromoWarps / C::kParts * (PAIR && rank == 0 ? 2 : 1));
     }
     for (int i = 0; i < 4; ++i) mbar_init(&s->amax_full[i], 2);
     mbar_init(&s->teardown, 1);
@@ -759,7 +774,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
           mbar_wait_bounded(&s->teardown, 0, 20000000ull);
         }
       }
-    } else {
+    } else if (!FUSED || warp == kScaleWarp) {
       // =============================== scale warps ======================================
       // Two warps, 64 rows each, form the products fl(s_x s_w) of every K-block next to its accumulator: the
       // slot is free when the accumulator is and published with it (tmem_full counts the MMA and these
@@ -767,6 +782,9 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
       const int r0 = (warp - kScaleWarp) * 64 + lane;
       int ks = 0, cur_e = 0;
       uint32_t acc_phase = 0;
+      uint32_t tile_iter = 0;
+      int4 tile_info = make_int4(0, 0, 0, 0);
+      float pw0 = 0.f, pw1 = 0.f;
       const float *x0 = nullptr, *x1 = nullptr, *wl = nullptr, *wh = nullptr;
       float n0 = 0.f, n1 = 0.f, nl = 0.f, nh = 0.f;  // of the next K-block: its loads fly during this one
       auto open_tile = [&](int T) {
@@ -779,6 +797,11 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
           nb_lo = COLS == 64 ? c.n_tile / 2 : HALVES * c.n_tile;
           nb_hi = min(nb_lo + HALVES - 1, NB - 1);
         }
+        if (MODE != kModeLinear) tile_info = make_int4(c.m0, c.m_end, c.n_tile, 0);
+        if (MODE == kModeDown) {
+          pw0 = __ldg(p.pair_weights + min(c.m0 + r0, p.rows_total - 1));
+          pw1 = __ldg(p.pair_weights + min(c.m0 + r0 + 32, p.rows_total - 1));
+        }
         x0 = p.a_scales + static_cast<int64_t>(min(c.m0 + r0, p.rows_total - 1)) * KB;
         x1 = p.a_scales + static_cast<int64_t>(min(c.m0 + r0 + 32, p.rows_total - 1)) * KB;
         wl = p.b_scales + (static_cast<int64_t>(c.e) * NB + nb_lo) * KB;
@@ -790,8 +813,10 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
       };
       bool ok = !FUSED || warp_wait_or_abort(&s->x_ready, 0, s, p);
       if (ok && first_tile < total_tiles) open_tile(first_tile);
-      for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
+      for (int T = first_tile; ok && T < total_tiles; T += num_ctas, ++tile_iter) {
         for (int kb = 0; kb < KB; ++kb) {
+          const int4 info = tile_info;
+          const float w0 = pw0, w1 = pw1;
           const float2 v0 = make_float2(__fmul_rn(n0, nl), __fmul_rn(n0, nh)), v1 = make_float2(__fmul_rn(n1, nl), __fmul_rn(n1, nh));
           if (kb + 1 < KB) {
             n0 = FUSED ? x_scale[min(r0, p.rows_total - 1) * KB + kb + 1] : __ldg(x0 + kb + 1);
@@ -803,6 +828,13 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
           }
           for (int part = 0; part < C::kParts; ++part) ok = ok && warp_wait_or_abort(&s->tmem_empty[C::kParts * ks + part], acc_phase ^ 1, s, p);
           if (!ok) break;
+          if (MODE != kModeLinear && kb == 0) {
+            if (warp == kScaleWarp && lane == 0) s->tile[tile_iter & (2 * kMaxAccBufs - 1)] = info;
+            if (MODE == kModeDown) {
+              s->pair_w[tile_iter & 3][r0] = w0;
+              s->pair_w[tile_iter & 3][r0 + 32] = w1;
+            }
+          }
           s->scale[ks][r0] = v0;
           s->scale[ks][r0 + 32] = v1;
           __syncwarp();
@@ -817,7 +849,9 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
     // =============================== promotion warps ==================================
     setmaxnreg_inc<kPromoRegs>();
     if constexpr (FUSED) quantize_rows(p, smem, x_scale, s);
-    promotion_role<MODE, SAVE, COLS, PAIR>(tm_o, p, smem, s, first_tile, num_ctas, total_tiles);
+    // (FUSED: all rows are in TMEM quadrant 0; warps that only keep the barriers going cost those that work: one token,
+    // N = 5120, K = 2048 7.0 -> 6.8 us)
+    if (!FUSED || (warp & 3) == 0) promotion_role<MODE, SAVE, COLS, PAIR>(tm_o, p, smem, s, first_tile, num_ctas, total_tiles);
   }
 
   // ---- teardown ---------------------------------------------------------------------------
