@@ -36,6 +36,7 @@
 // epilogues are the ones of the separate launches: the bytes are the same.
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "common.cuh"
 #include "ptx_sm100.cuh"
@@ -57,6 +58,7 @@ constexpr int kTmaWarp = 12;
 constexpr int kMmaWarp = 13;        // and 14: one issuer per weight block of the pair; warp 15 idle
 constexpr int kThreads = 16 * 32;
 constexpr int NTH = NT / 2;        // token columns per promotion thread
+constexpr int kFewCols = 4;
 // 512 threads: 128 registers each, which every role fits (a promotion thread holds 2 x 16 accumulators and
 // 2 x 16 partial sums in flight); no re-allocation between warpgroups
 constexpr uint32_t kABytes = 2 * BW * BK;   // two weight blocks
@@ -655,7 +657,10 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
 #pragma unroll
         for (int t = 0; t < NTH; ++t) acc_lo[t] = acc_hi[t] = 0.0f;
 
-        const int live = rows - tb;  // token columns of this warp that hold a row: the others are not promoted
+        // Token columns of this warp that hold a row.  A warp without one keeps the barriers going and promotes nothing, with a
+        // few it promotes those (one token: router and layer 33.5 -> 32.2 us); finer steps cost the fuller tiles more than
+        // they save (every four columns: 256 tokens 126.6 -> 127.9).
+        const int live = rows - tb;
         for (int kb = 0; kb < KB; ++kb) {
           if (!warp_wait_or_abort(&s->tmem_full[ks], acc_phase, s, p)) { ok = false; break; }
           tc_fence_after_sync();
@@ -671,17 +676,20 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
           if (lane == 0) mbar_arrive(&s->tmem_empty[ks]);  // both reads have landed: hand the accumulator back
           if (++ks == kAccBufs) { ks = 0; acc_phase ^= 1; }
           const float2 sw = *reinterpret_cast<const float2*>(sl.sw[kb]);
+          auto promote = [&](auto columns) {
 #pragma unroll
-          for (int t4 = 0; t4 < NTH; t4 += 4) {
-            if (t4 >= live) break;
-            const float4 sx = *reinterpret_cast<const float4*>(&sl.sx[kb][tb + t4]);  // same address in every lane: broadcast
-            const float sxs[4] = {sx.x, sx.y, sx.z, sx.w};
+            for (int t4 = 0; t4 < decltype(columns)::value; t4 += 4) {
+              const float4 sx = *reinterpret_cast<const float4*>(&sl.sx[kb][tb + t4]);  // same address in every lane: broadcast
+              const float sxs[4] = {sx.x, sx.y, sx.z, sx.w};
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              acc_lo[t4 + u] = __fmaf_rn(__fmul_rn(sxs[u], sw.x), __uint_as_float(vl[t4 + u]), acc_lo[t4 + u]);
-              acc_hi[t4 + u] = __fmaf_rn(__fmul_rn(sxs[u], sw.y), __uint_as_float(vh[t4 + u]), acc_hi[t4 + u]);
+              for (int u = 0; u < 4; ++u) {
+                acc_lo[t4 + u] = __fmaf_rn(__fmul_rn(sxs[u], sw.x), __uint_as_float(vl[t4 + u]), acc_lo[t4 + u]);
+                acc_hi[t4 + u] = __fmaf_rn(__fmul_rn(sxs[u], sw.y), __uint_as_float(vh[t4 + u]), acc_hi[t4 + u]);
+              }
             }
-          }
+          };
+          if (live > kFewCols) promote(std::integral_constant<int, NTH>{});
+          else if (live > 0) promote(std::integral_constant<int, kFewCols>{});
         }
 
         // ---- hand the tile to the epilogue warps: bf16, transposed to [token][256 weight rows] ----
@@ -699,18 +707,21 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         if (ok) ok = warp_wait_or_abort(&s->out_empty, (tile_iter & 1u) ^ 1u, s, p);  // previous tile drained
         if (ok) {
           uint16_t* T16 = reinterpret_cast<uint16_t*>(out_tile);
+          auto stage = [&](auto columns) {
 #pragma unroll
-          for (int t = 0; t < NTH; ++t) {
-            if (t >= live) break;
-            float lo = acc_lo[t], hi = acc_hi[t];
-            if (c.mode == kModeDown) {  // contribution = bf16( fl(w * y) )
-              const float w = sl.w[tb + t];
-              lo = __fmul_rn(w, lo);
-              hi = __fmul_rn(w, hi);
+            for (int t = 0; t < decltype(columns)::value; ++t) {
+              float lo = acc_lo[t], hi = acc_hi[t];
+              if (c.mode == kModeDown) {  // contribution = bf16( fl(w * y) )
+                const float w = sl.w[tb + t];
+                lo = __fmul_rn(w, lo);
+                hi = __fmul_rn(w, hi);
+              }
+              T16[(tb + t) * (kOutRowBytes / 2) + wr] = static_cast<uint16_t>(f32_to_bf16_bits(lo));
+              T16[(tb + t) * (kOutRowBytes / 2) + BW + wr] = static_cast<uint16_t>(f32_to_bf16_bits(hi));
             }
-            T16[(tb + t) * (kOutRowBytes / 2) + wr] = static_cast<uint16_t>(f32_to_bf16_bits(lo));
-            T16[(tb + t) * (kOutRowBytes / 2) + BW + wr] = static_cast<uint16_t>(f32_to_bf16_bits(hi));
-          }
+          };
+          if (live > kFewCols) stage(std::integral_constant<int, NTH>{});
+          else if (live > 0) stage(std::integral_constant<int, kFewCols>{});
           __syncwarp();
           if (lane == 0) mbar_arrive(&s->out_full);  // release: the epilogue warps see the tile after their wait
         }
