@@ -17,8 +17,8 @@
 //                                   the chunk; the last CTA to finish adds all J in index order: loss = -mean J
 // The response of a token is found by a 32-way search of the offsets.  Every sum has a fixed order: results do not
 // depend on the grid or on timing.  1024 responses, 4.2 M tokens (67 MB) on the device: 31.7 us as four launches (response
-// map, CTA per 8192 tokens with a block sum per response, statistics, gradient), 20.2 us so (22.3 with its inputs read evict-first and
-// the finish kernel's chunks fixed at 8192), more than half of it the partial kernel.
+// map, CTA per 8192 tokens with a block sum per response, statistics, gradient), 22.5 us so, of which 13.6 are the partial
+// kernel (3.7 TB/s: ~4 us of its time is launch and first-load latency).
 #include <math.h>
 
 #include <algorithm>
@@ -36,7 +36,6 @@ constexpr int kPieces = 2368;  // most pieces of a call: 16 warps on each of 148
 // chunk of a response repeats its statistics (64 responses, 393,216 tokens: 10.1 with 8192, 10.6 with 1024; 1024 responses, 4.2 M tokens:
 // 22.2 with 8192, 25.9 with 4096; 2048 responses, 12.6 M: 51.9 with 8192, 49.6 with 16384).
 constexpr int kMinChunk = 1024, kMaxChunk = 16384, kFinishCtas = 592;
-constexpr int64_t kCachedTokens = 6 << 20;  // 16 bytes each: 100 of the L2's 126 MB
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 
@@ -92,21 +91,17 @@ struct Step {
   float c[16], o[16], q[16];
 };
 // Loads of the step at token `base`; element e of a lane is token base + 4 lane + 128 (e / 4) + e % 4.
-// VEC: the three arrays are 16-byte aligned.  STREAM: they and the gradient do not fit the L2 and are read evict-first; what
-// fits is left there (1024 responses, 4.2 M tokens: 22.2 -> 20.2 us; 2048 responses, 12.6 M: 51.9 evict-first, 57.7 without).
-template <bool STREAM, typename T>
-__device__ __forceinline__ T load_once(const T* p) {
-  return STREAM ? __ldcs(p) : __ldg(p);
-}
-template <bool VEC, bool STREAM>
+// VEC: the three arrays are 16-byte aligned.  They are read evict-first whatever their size: left in the L2, inputs that fit it cost
+// a call on other inputs more (4.2 M tokens 24.0 -> 25.5 us) than they save one on the same (22.2 -> 20.2).
+template <bool VEC>
 __device__ __forceinline__ void load_step(const TbpoParams& p, Step& s, int64_t base, int64_t hi, int lane) {
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int64_t t = base + 4 * (32 * j + lane);
     if (VEC && t + 4 <= hi) {
-      const float4 a = load_once<STREAM>(reinterpret_cast<const float4*>(p.lp_cur + t));
-      const float4 b = load_once<STREAM>(reinterpret_cast<const float4*>(p.lp_old + t));
-      const float4 d = load_once<STREAM>(reinterpret_cast<const float4*>(p.lp_smp + t));
+      const float4 a = __ldcs(reinterpret_cast<const float4*>(p.lp_cur + t));
+      const float4 b = __ldcs(reinterpret_cast<const float4*>(p.lp_old + t));
+      const float4 d = __ldcs(reinterpret_cast<const float4*>(p.lp_smp + t));
       s.c[4 * j] = a.x, s.c[4 * j + 1] = a.y, s.c[4 * j + 2] = a.z, s.c[4 * j + 3] = a.w;
       s.o[4 * j] = b.x, s.o[4 * j + 1] = b.y, s.o[4 * j + 2] = b.z, s.o[4 * j + 3] = b.w;
       s.q[4 * j] = d.x, s.q[4 * j + 1] = d.y, s.q[4 * j + 2] = d.z, s.q[4 * j + 3] = d.w;
@@ -114,15 +109,15 @@ __device__ __forceinline__ void load_step(const TbpoParams& p, Step& s, int64_t 
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const bool in = t + u < hi;
-        s.c[4 * j + u] = in ? load_once<STREAM>(p.lp_cur + t + u) : 0.0f;
-        s.o[4 * j + u] = in ? load_once<STREAM>(p.lp_old + t + u) : 0.0f;
-        s.q[4 * j + u] = in ? load_once<STREAM>(p.lp_smp + t + u) : 0.0f;
+        s.c[4 * j + u] = in ? __ldcs(p.lp_cur + t + u) : 0.0f;
+        s.o[4 * j + u] = in ? __ldcs(p.lp_old + t + u) : 0.0f;
+        s.q[4 * j + u] = in ? __ldcs(p.lp_smp + t + u) : 0.0f;
       }
     }
   }
 }
 
-template <bool VEC, bool STREAM>
+template <bool VEC>
 __global__ void __launch_bounds__(kThreads, 2) tbpo_partial_kernel(const TbpoParams p) {
   pdl_wait();
   pdl_trigger();  // after the wait: the finish kernel may read the call's inputs before its own wait
@@ -132,7 +127,7 @@ __global__ void __launch_bounds__(kThreads, 2) tbpo_partial_kernel(const TbpoPar
   const int64_t lo = k * p.piece, hi = min(lo + p.piece, p.T);
   if (lo >= p.T) return;
   Step s[2];
-  load_step<VEC, STREAM>(p, s[0], lo, hi, lane);
+  load_step<VEC>(p, s[0], lo, hi, lane);
   int64_t i = response_of(p, lo, lane);
   int64_t t0 = clamp_off(p, i), t1 = clamp_off(p, i + 1);
   double2 acc = make_double2(0.0, 0.0);
@@ -172,10 +167,10 @@ __global__ void __launch_bounds__(kThreads, 2) tbpo_partial_kernel(const TbpoPar
   };
   bool more = true;
   for (int64_t base = lo; more && base < hi; base += 2 * kStep) {
-    if (base + kStep < hi) load_step<VEC, STREAM>(p, s[1], base + kStep, hi, lane);
+    if (base + kStep < hi) load_step<VEC>(p, s[1], base + kStep, hi, lane);
     more = consume(s[0], base);
     if (more && base + kStep < hi) {
-      if (base + 2 * kStep < hi) load_step<VEC, STREAM>(p, s[0], base + 2 * kStep, hi, lane);
+      if (base + 2 * kStep < hi) load_step<VEC>(p, s[0], base + 2 * kStep, hi, lane);
       more = consume(s[1], base + kStep);
     }
   }
@@ -356,10 +351,7 @@ cudaError_t launch_tbpo(const Launch& L, const TbpoArgs& a) {
   const unsigned partial_blocks = static_cast<unsigned>(std::max<int64_t>(1, (pieces_of(a.T) + kWarps - 1) / kWarps));
   const unsigned finish_blocks = static_cast<unsigned>(std::max<int64_t>(1, (a.T + p.chunk - 1) / p.chunk));
   *L.launches += 2;
-  const bool stream = a.T > kCachedTokens;
-  const cudaError_t e = launch_pdl(vec ? (stream ? tbpo_partial_kernel<true, true> : tbpo_partial_kernel<true, false>)
-                                       : (stream ? tbpo_partial_kernel<false, true> : tbpo_partial_kernel<false, false>),
-                                   partial_blocks, kThreads, 0, L.stream, p);
+  const cudaError_t e = launch_pdl(vec ? tbpo_partial_kernel<true> : tbpo_partial_kernel<false>, partial_blocks, kThreads, 0, L.stream, p);
   if (e != cudaSuccess) return e;
   return launch_pdl(tbpo_finish_kernel, finish_blocks, kThreads, 0, L.stream, p);
 }

@@ -55,8 +55,8 @@ def test_many_short_responses_and_one_long(ctx):
 
 @pytest.mark.parametrize("n,mean,longest", [(200, 30, 200), (3, 3000, 6000), (4, 30000, 40000), (900, 700, 3000), (2000, 3700, 12000)])
 def test_every_chunk_length_of_the_finish_kernel(ctx, n, mean, longest):
-    """Token counts and average lengths that give chunks of 1024 (many short responses) to 16384 tokens (few long ones, and a call
-    whose arrays do not fit the L2)."""
+    """Token counts and average lengths that give chunks of 1024 (many short responses) to 16384 tokens (few long ones, or very many
+    tokens)."""
     check(ctx, inputs.tbpo_case(40 + n, inputs.tbpo_lengths(40 + n, n, mean_len=mean, max_len=longest)))
 
 
