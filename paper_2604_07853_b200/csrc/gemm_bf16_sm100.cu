@@ -365,25 +365,25 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
               tma_load_2d_pair(b_dst, &tm_b, bar, ks * BK, t.b_row0 + j);
             }
           } else {
-          mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
-          if (A_MN && p.a3d) {
-            tma_load_3d(a_dst, &tm_a, &s->full[stage], 0, t.a_c0 + ks * BK, i0 / 64);
-          } else if (A_MN) {
+            mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
+            if (A_MN && p.a3d) {
+              tma_load_3d(a_dst, &tm_a, &s->full[stage], 0, t.a_c0 + ks * BK, i0 / 64);
+            } else if (A_MN) {
 #pragma unroll
-            for (int b = 0; b < TM / 64; ++b)
-              tma_load_2d(a_dst + b * kBlockBytes, &tm_a, &s->full[stage], i0 + 64 * b, t.a_c0 + ks * BK);
-          } else {  // one box of TM rows x 128 bytes
-            tma_load_2d(a_dst, &tm_a, &s->full[stage], t.a_c0 + ks * BK, i0);
-          }
-          if (B_MN && p.b3d) {
-            tma_load_3d(b_dst, &tm_b, &s->full[stage], 0, t.b_c0 + ks * BK, j0 / 64);
-          } else if (B_MN) {
+              for (int b = 0; b < TM / 64; ++b)
+                tma_load_2d(a_dst + b * kBlockBytes, &tm_a, &s->full[stage], i0 + 64 * b, t.a_c0 + ks * BK);
+            } else {  // one box of TM rows x 128 bytes
+              tma_load_2d(a_dst, &tm_a, &s->full[stage], t.a_c0 + ks * BK, i0);
+            }
+            if (B_MN && p.b3d) {
+              tma_load_3d(b_dst, &tm_b, &s->full[stage], 0, t.b_c0 + ks * BK, j0 / 64);
+            } else if (B_MN) {
 #pragma unroll
-            for (int b = 0; b < BN / 64; ++b)
-              tma_load_2d(b_dst + b * kBlockBytes, &tm_b, &s->full[stage], j0 + 64 * b, t.b_c0 + ks * BK);
-          } else {
-            tma_load_2d(b_dst, &tm_b, &s->full[stage], ks * BK, t.b_row0 + j0);
-          }
+              for (int b = 0; b < BN / 64; ++b)
+                tma_load_2d(b_dst + b * kBlockBytes, &tm_b, &s->full[stage], j0 + 64 * b, t.b_c0 + ks * BK);
+            } else {
+              tma_load_2d(b_dst, &tm_b, &s->full[stage], ks * BK, t.b_row0 + j0);
+            }
           }
           armed |= 1u << stage;
           armed_parity = (armed_parity & ~(1u << stage)) | (phase << stage);

@@ -704,15 +704,15 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
               tma_load_2d_pair(a_dst, &tm_a, bar, kb * BK, c.m0);
               tma_load_2d_pair(b_dst, &tm_b, bar, kb * BK, rank == 0 ? row_lo : row_hi);
             } else {
-            mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
-            if (!FUSED) tma_load_2d(a_dst, &tm_a, &s->full[stage], kb * BK, c.m0);
-            if (p.weights_once) {
-              tma_load_2d_hint(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo, stream_once);
-              if (HALVES == 2) tma_load_2d_hint(b_dst + kBHalfBytes, &tm_b, &s->full[stage], kb * BK, row_hi, stream_once);
-            } else {
-              tma_load_2d(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo);
-              if (HALVES == 2) tma_load_2d(b_dst + kBHalfBytes, &tm_b, &s->full[stage], kb * BK, row_hi);
-            }
+              mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
+              if (!FUSED) tma_load_2d(a_dst, &tm_a, &s->full[stage], kb * BK, c.m0);
+              if (p.weights_once) {
+                tma_load_2d_hint(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo, stream_once);
+                if (HALVES == 2) tma_load_2d_hint(b_dst + kBHalfBytes, &tm_b, &s->full[stage], kb * BK, row_hi, stream_once);
+              } else {
+                tma_load_2d(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo);
+                if (HALVES == 2) tma_load_2d(b_dst + kBHalfBytes, &tm_b, &s->full[stage], kb * BK, row_hi);
+              }
             }
             armed |= 1u << stage;
             armed_parity = (armed_parity & ~(1u << stage)) | (phase << stage);
