@@ -22,7 +22,7 @@
 //                        (generic stores + proxy fence) before the step is issued, so
 //                        they contribute nothing whatever they hold.
 //
-// Tile 128 x 256 x 64 (or 256 x 256, by one CTA or by a pair of them, 128 x 192: see the host).  TMA stages both operands with the 128-byte swizzle (a K-major tile is
+// Tile 128 x 256 x 64 (or 256 x 256, 128 x 192: see the host).  TMA stages both operands with the 128-byte swizzle (a K-major tile is
 // one box of R rows x 128 bytes; an MN-major tile is one box of 64 c-rows x 128 bytes per 64
 // output indices); one thread issues 4 x tcgen05.mma kind::f16 (128 x 256 x 16) per stage with
 // the matching operand-major bits; two 256-column TMEM accumulators let the epilogue of a tile
@@ -32,8 +32,6 @@
 // 1536 x 2048, 1.6 GB out) 1010 us of which the stores need 250.  Static persistent schedule, row tiles fastest
 // (grouped contraction: long and short tiles in turn, see the producer).  One fixed
 // order of accumulation: a result does not depend on the grid or on the other rows.
-// PAIR: two CTAs (a cluster; tcgen05 cta_group::2) on a tile of 256 x 256: each loads its 128 rows of A and half of B's columns,
-// the even one issues the MMAs for both, each writes its rows out; 32 KB per step and SM instead of 48, six stages.
 // Every wait is bounded (status word + CTA-wide abort flag), as in the other GEMMs.
 #include <algorithm>
 #include <atomic>
@@ -48,7 +46,7 @@ namespace {
 using namespace ptx;
 
 constexpr int BM = 128, BK = 64;
-constexpr int kMaxStages = 6, kMaxAccBufs = 2;
+constexpr int kMaxStages = 4, kMaxAccBufs = 2;
 constexpr uint32_t kAHalfBytes = BM * BK * 2;   // 16 KB: 128 output rows x 64 contraction elements
 // an epilogue warp's rows on their way out: boxes of 32 rows x 128 bytes (128-byte swizzle)
 constexpr uint32_t kOutBoxBytes = 32 * 128;
@@ -58,14 +56,13 @@ constexpr uint32_t kOutBoxBytes = 32 * 128;
 // it leaves one set of accumulators, i.e. an epilogue that is not overlapped, which only pays when
 // the contraction is long enough (MT = 1 for the ragged contraction of the grouped dW).
 enum { kDense = 0, kGroupedRows = 1, kGroupedContraction = 2 };
-template <int GROUP, int MT, int BN, bool PAIR>
+template <int GROUP, int MT, int BN>
 struct Cfg {
-  static constexpr int kRows = (PAIR ? 2 : MT) * BM;    // rows of a tile
-  static constexpr int kCtaCols = PAIR ? BN / 2 : BN;   // columns of B that a CTA loads
+  static constexpr int kRows = MT * BM;
   static constexpr uint32_t kABytes = MT * kAHalfBytes;
-  static constexpr uint32_t kBBytes = kCtaCols * BK * 2;
+  static constexpr uint32_t kBBytes = BN * BK * 2;
   static constexpr uint32_t kStageBytes = kABytes + kBBytes;
-  static constexpr int kStages = PAIR ? 6 : MT == 2 ? 3 : 4;
+  static constexpr int kStages = MT == 2 ? 3 : 4;
   static constexpr int kAccBufs = MT == 1 ? 2 : 1;
   // Warps 0 .. kEpiWarps - 1: TMEM quadrant = warp % 4; with eight, two share a quadrant and take the 128-byte
   // column chunks in turn (each has one box; grouped rows need the shared memory for the tile list).
@@ -117,16 +114,15 @@ struct SmemLists {  // grouped rows: the tile list
   int32_t off[kMaxExperts + 1];
   int32_t prefix[kMaxExperts + 1];
 };
-template <int GROUP, int MT, int BN, bool PAIR = false>
+template <int GROUP, int MT, int BN>
 constexpr size_t smem_bytes() {
-  using C = Cfg<GROUP, MT, BN, PAIR>;
+  using C = Cfg<GROUP, MT, BN>;
   return 1024 + static_cast<size_t>(C::kStages) * C::kStageBytes + C::kOutBytes + sizeof(SmemTail) +
          (GROUP == kGroupedRows ? sizeof(SmemLists) : GROUP == kGroupedContraction ? sizeof(SmemOrder) : 0);
 }
 static_assert(smem_bytes<kDense, 1, 256>() <= 227 * 1024 && smem_bytes<kDense, 1, 192>() <= 227 * 1024 &&
                   smem_bytes<kDense, 2, 256>() <= 227 * 1024 && smem_bytes<kGroupedRows, 1, 256>() <= 227 * 1024 &&
-                  smem_bytes<kGroupedContraction, 1, 256>() <= 227 * 1024 && smem_bytes<kDense, 1, 256, true>() <= 227 * 1024 &&
-                  smem_bytes<kGroupedRows, 1, 256, true>() <= 227 * 1024,
+                  smem_bytes<kGroupedContraction, 1, 256>() <= 227 * 1024,
               "shared memory budget");
 
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, SmemTail* s, const Bf16Params& p) {
@@ -178,14 +174,14 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&b);
 }
 
-template <bool A_MN, bool B_MN, int GROUP, int MT, int BN, bool PAIR>
-__global__ void __launch_bounds__(Cfg<GROUP, MT, BN, PAIR>::kThreads, 1)
+template <bool A_MN, bool B_MN, int GROUP, int MT, int BN>
+__global__ void __launch_bounds__(Cfg<GROUP, MT, BN>::kThreads, 1)
 gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                  const __grid_constant__ CUtensorMap tm_f32, const __grid_constant__ CUtensorMap tm_bf16,
                  const Bf16Params p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  using C = Cfg<GROUP, MT, BN, PAIR>;
+  using C = Cfg<GROUP, MT, BN>;
   constexpr int kStages = C::kStages, kAccBufs = C::kAccBufs, TM = C::kRows;
   constexpr uint32_t kABytes = C::kABytes, kStageBytes = C::kStageBytes;
   constexpr int kEpiWarps = C::kEpiWarps, kTmaWarp = C::kTmaWarp, kMmaWarp = C::kMmaWarp;
@@ -194,7 +190,6 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   SmemLists* lists = reinterpret_cast<SmemLists*>(s + 1);
   SmemOrder* list = reinterpret_cast<SmemOrder*>(s + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rank = PAIR ? static_cast<int>(cluster_ctarank()) : 0;
 
   pdl_trigger();
   if (threadIdx.x == 0) {
@@ -205,7 +200,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     }
     for (int i = 0; i < kAccBufs; ++i) {
       mbar_init(&s->tmem_full[i], 1);
-      mbar_init(&s->tmem_empty[i], PAIR ? 2 * kEpiWarps : kEpiWarps);  // (PAIR: in the even CTA, which issues the MMAs)
+      mbar_init(&s->tmem_empty[i], kEpiWarps);
     }
     mbar_init(&s->teardown, 1);
     s->abort_flag = 0;
@@ -216,13 +211,8 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     prefetch_tensormap(&tm_b);
   }
   if (warp == kMmaWarp) {
-    if constexpr (PAIR) {
-      tmem_alloc_pair(&s->tmem_addr, kTmemCols);
-      tmem_relinquish_pair();
-    } else {
-      tmem_alloc(&s->tmem_addr, kTmemCols);
-      tmem_relinquish();
-    }
+    tmem_alloc(&s->tmem_addr, kTmemCols);
+    tmem_relinquish();
   }
   pdl_wait();
   const int n_tiles = (p.No + BN - 1) / BN;
@@ -249,14 +239,12 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     }
   }
   tc_fence_before_sync();
-  if constexpr (PAIR) cluster_sync();  // (the other CTA's barriers are initialised too)
-  else __syncthreads();
+  __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = s->tmem_addr;
   const int total_tiles = GROUP == kGroupedRows ? lists->prefix[p.E]
                         : GROUP == kGroupedContraction ? p.E * m_tiles * n_tiles : m_tiles * n_tiles;
-  const int grid = PAIR ? gridDim.x / 2 : gridDim.x;  // (pairs)
-  const int cta = PAIR ? blockIdx.x / 2 : blockIdx.x;
+  const int grid = gridDim.x;
 
   // Everything a role needs to know about tile T.  i0 / j0: first output row / column; a_c0 / b_c0:
   // first contraction coordinate of A / B; KS: 64-element contraction steps; last_valid: contraction
@@ -294,7 +282,6 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       t.b_row0 = c.e * p.No;        // K-major B: the expert's [No, Kc] block starts at row e No
       t.row_end = c.m_end;
     }
-    if (PAIR) t.i0 += rank * BM;  // this CTA's rows
     return t;
   };
   // Grouped contraction: this CTA's list holds every grid-th tile of the experts by falling row count, the direction
@@ -341,49 +328,24 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
             *reinterpret_cast<volatile uint32_t*>(&list->step[stage]) =
                 acc | (ks == 0 ? 2u : 0u) | (last ? 4u : 0u) | static_cast<uint32_t>(last ? t.last_valid : BK) << 3;
           }
-          if constexpr (PAIR) {
-            // the bytes of both CTAs count on the even CTA's barrier
-            const uint32_t bar = map_to_cta(smem_u32(&s->full[stage]), 0);
-            if (rank == 0) mbar_arrive_expect_tx(&s->full[stage], 2 * kStageBytes);
-            const int j = j0 + rank * C::kCtaCols;
-            if (A_MN && p.a3d) {
-              tma_load_3d_pair(a_dst, &tm_a, bar, 0, t.a_c0 + ks * BK, i0 / 64);
-            } else if (A_MN) {
+          mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
+          if (A_MN && p.a3d) {
+            tma_load_3d(a_dst, &tm_a, &s->full[stage], 0, t.a_c0 + ks * BK, i0 / 64);
+          } else if (A_MN) {
 #pragma unroll
-              for (int b = 0; b < BM / 64; ++b)
-                tma_load_2d_pair(a_dst + b * kBlockBytes, &tm_a, bar, i0 + 64 * b, t.a_c0 + ks * BK);
-            } else {
-              tma_load_2d_pair(a_dst, &tm_a, bar, t.a_c0 + ks * BK, i0);
-            }
-            if (B_MN && p.b3d) {
-              tma_load_3d_pair(b_dst, &tm_b, bar, 0, t.b_c0 + ks * BK, j / 64);
-            } else if (B_MN) {
+            for (int b = 0; b < TM / 64; ++b)
+              tma_load_2d(a_dst + b * kBlockBytes, &tm_a, &s->full[stage], i0 + 64 * b, t.a_c0 + ks * BK);
+          } else {  // one box of TM rows x 128 bytes
+            tma_load_2d(a_dst, &tm_a, &s->full[stage], t.a_c0 + ks * BK, i0);
+          }
+          if (B_MN && p.b3d) {
+            tma_load_3d(b_dst, &tm_b, &s->full[stage], 0, t.b_c0 + ks * BK, j0 / 64);
+          } else if (B_MN) {
 #pragma unroll
-              for (int b = 0; b < C::kCtaCols / 64; ++b)
-                tma_load_2d_pair(b_dst + b * kBlockBytes, &tm_b, bar, j + 64 * b, t.b_c0 + ks * BK);
-            } else {
-              tma_load_2d_pair(b_dst, &tm_b, bar, ks * BK, t.b_row0 + j);
-            }
+            for (int b = 0; b < BN / 64; ++b)
+              tma_load_2d(b_dst + b * kBlockBytes, &tm_b, &s->full[stage], j0 + 64 * b, t.b_c0 + ks * BK);
           } else {
-            mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
-            if (A_MN && p.a3d) {
-              tma_load_3d(a_dst, &tm_a, &s->full[stage], 0, t.a_c0 + ks * BK, i0 / 64);
-            } else if (A_MN) {
-#pragma unroll
-              for (int b = 0; b < TM / 64; ++b)
-                tma_load_2d(a_dst + b * kBlockBytes, &tm_a, &s->full[stage], i0 + 64 * b, t.a_c0 + ks * BK);
-            } else {  // one box of TM rows x 128 bytes
-              tma_load_2d(a_dst, &tm_a, &s->full[stage], t.a_c0 + ks * BK, i0);
-            }
-            if (B_MN && p.b3d) {
-              tma_load_3d(b_dst, &tm_b, &s->full[stage], 0, t.b_c0 + ks * BK, j0 / 64);
-            } else if (B_MN) {
-#pragma unroll
-              for (int b = 0; b < BN / 64; ++b)
-                tma_load_2d(b_dst + b * kBlockBytes, &tm_b, &s->full[stage], j0 + 64 * b, t.b_c0 + ks * BK);
-            } else {
-              tma_load_2d(b_dst, &tm_b, &s->full[stage], ks * BK, t.b_row0 + j0);
-            }
+            tma_load_2d(b_dst, &tm_b, &s->full[stage], ks * BK, t.b_row0 + j0);
           }
           armed |= 1u << stage;
           armed_parity = (armed_parity & ~(1u << stage)) | (phase << stage);
@@ -417,36 +379,24 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
         }
       } else {
         int cur_e = 0;
-        for (int T = cta; ok && T < total_tiles; T += grid) {
+        for (int T = blockIdx.x; ok && T < total_tiles; T += grid) {
           const Tile t = tile_of(T, cur_e);
           feed(t, 0, t.KS, 0);
         }
       }
       if (!ok) {
         for (int i = 0; i < kStages; ++i)
-          if (rank == 0 && (armed & (1u << i))) mbar_wait_bounded(&s->full[i], (armed_parity >> i) & 1u, 20000000ull);
-        if (PAIR) {  // copies counted on a barrier that is not waited for here: they land in microseconds
-          const uint64_t t0 = globaltimer_ns();
-          while (globaltimer_ns() - t0 < 1000000ull) __nanosleep(1000);
-        }
+          if (armed & (1u << i)) mbar_wait_bounded(&s->full[i], (armed_parity >> i) & 1u, 20000000ull);
       }
     }
   } else if (warp == kMmaWarp) {
-    if (rank == 0 && elect_one()) {
-      constexpr uint32_t idesc = umma_idesc_bf16_f32_major(PAIR ? 2 * BM : BM, BN, A_MN, B_MN);
+    if (elect_one()) {
+      constexpr uint32_t idesc = umma_idesc_bf16_f32_major(BM, BN, A_MN, B_MN);
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
       // the first `slices` 16-element slices of the staged step; 16 contraction elements further on: 32 bytes
       // inside a K-major row, 16 rows of 128 bytes in an MN-major block (start-address field counts 16-byte units)
-      auto mma = [&](uint32_t d, uint64_t ad, uint64_t bd, uint32_t id, uint32_t accumulate) {
-        if constexpr (PAIR) umma_bf16_pair(d, ad, bd, id, accumulate);
-        else umma_bf16(d, ad, bd, id, accumulate);
-      };
-      auto commit = [&](uint64_t* bar) {
-        if constexpr (PAIR) umma_commit_pair(bar);
-        else umma_commit(bar);
-      };
       auto issue = [&](uint32_t d_tmem, bool first, int slices) {
         tc_fence_after_sync();
         const uint32_t a_addr = smem_u32(smem + static_cast<size_t>(stage) * kStageBytes);
@@ -460,13 +410,13 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
           for (int mt = 0; mt < MT; ++mt)  // the 128-row halves of A share the B tile
 #pragma unroll
             for (int k4 = 0; k4 < BK / 16; ++k4)
-              mma(d_tmem + mt * BN, a_desc + mt * (kAHalfBytes >> 4) + a_step * k4, b_desc + b_step * k4, idesc,
+              umma_bf16(d_tmem + mt * BN, a_desc + mt * (kAHalfBytes >> 4) + a_step * k4, b_desc + b_step * k4, idesc,
                         (!first || k4 > 0) ? 1u : 0u);
         } else {  // (MT is 1 in the form that has these)
           for (int k4 = 0; k4 < slices; ++k4)
-            mma(d_tmem, a_desc + a_step * k4, b_desc + b_step * k4, idesc, (!first || k4 > 0) ? 1u : 0u);
+            umma_bf16(d_tmem, a_desc + a_step * k4, b_desc + b_step * k4, idesc, (!first || k4 > 0) ? 1u : 0u);
         }
-        commit(&s->empty[stage]);
+        umma_commit(&s->empty[stage]);
       };
       auto next_stage = [&]() {
         if (++stage == kStages) { stage = 0; phase ^= 1; }
@@ -485,7 +435,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
           }
           issue(tmem_base + acc * BN, (step & 2u) != 0, (valid + 15) / 16);
           if (step & 4u) {
-            commit(&s->tmem_full[acc]);
+            umma_commit(&s->tmem_full[acc]);
             acc_phase ^= 1u << acc;
             ++done;
           }
@@ -494,14 +444,14 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       } else {
         int acc = 0, cur_e = 0;
         uint32_t acc_phase = 0;
-        for (int T = cta; ok && T < total_tiles; T += grid) {
+        for (int T = blockIdx.x; ok && T < total_tiles; T += grid) {
           const Tile t = tile_of(T, cur_e);
           if (t.KS == 0) continue;  // an empty contraction: the epilogue writes zeros, no accumulator is used
           if (!wait_or_abort(&s->tmem_empty[acc], acc_phase ^ 1, s, p)) { ok = false; break; }
           for (int ks = 0; ks < t.KS; ++ks) {
             if (!wait_or_abort(&s->full[stage], phase, s, p)) { ok = false; break; }
             issue(tmem_base + static_cast<uint32_t>(acc * MT) * BN, ks == 0, BK / 16);
-            if (ks == t.KS - 1) commit(&s->tmem_full[acc]);
+            if (ks == t.KS - 1) umma_commit(&s->tmem_full[acc]);
             next_stage();
           }
           if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1; }
@@ -510,7 +460,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       // Nothing of this CTA's tensor work may be in flight when its TMEM and shared memory go
       // away: after an abort some MMAs may still be executing, so wait (bounded) for them.
       if (!ok) {
-        commit(&s->teardown);
+        umma_commit(&s->teardown);
         mbar_wait_bounded(&s->teardown, 0, 20000000ull);
       }
     }
@@ -632,11 +582,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
       if (have_acc) {
         tc_fence_before_sync();
         __syncwarp();
-        if (lane == 0) {
-          // (what is handed over is tensor memory, read completely)
-          if constexpr (PAIR) mbar_arrive_cluster_relaxed(map_to_cta(smem_u32(&s->tmem_empty[acc]), 0));
-          else mbar_arrive(&s->tmem_empty[acc]);
-        }
+        if (lane == 0) mbar_arrive(&s->tmem_empty[acc]);
       }
     };
     if constexpr (GROUP == kGroupedContraction) {
@@ -659,7 +605,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     } else {
       int acc = 0, cur_e = 0;
       uint32_t acc_phase = 0;
-      for (int T = cta; T < total_tiles; T += grid) {
+      for (int T = blockIdx.x; T < total_tiles; T += grid) {
         const Tile t = tile_of(T, cur_e);
         if (t.KS == 0) {
           write_out(t, false, 0);
@@ -675,12 +621,10 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   }
 
   tc_fence_before_sync();
-  if constexpr (PAIR) cluster_sync();  // (nothing reads or signals the other CTA any more)
-  else __syncthreads();
+  __syncthreads();
   if (warp == kMmaWarp) {
     tc_fence_after_sync();
-    if constexpr (PAIR) tmem_dealloc_pair(tmem_base, kTmemCols);
-    else tmem_dealloc(tmem_base, kTmemCols);
+    tmem_dealloc(tmem_base, kTmemCols);
   }
 }
 
@@ -725,38 +669,34 @@ struct Maps {
   CUtensorMap a, b, f32, bf16;
 };
 
-template <bool A_MN, bool B_MN, int GROUP, int MT, int BN, bool PAIR>
+template <bool A_MN, bool B_MN, int GROUP, int MT, int BN>
 cudaError_t launch_variant(const Launch& L, const Maps& tm, const Bf16Params& p, int64_t tiles) {
   // sticky per function and device; atomic: contexts on several host threads may launch at once (both
   // would set the same value)
   static std::atomic<bool> attr_set_dev[64];
   std::atomic<bool>& attr_set = attr_set_dev[L.device & 63];
   if (!attr_set.load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_bf16_kernel<A_MN, B_MN, GROUP, MT, BN, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem_bytes<GROUP, MT, BN, PAIR>()));
+    cudaError_t e = cudaFuncSetAttribute(gemm_bf16_kernel<A_MN, B_MN, GROUP, MT, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(smem_bytes<GROUP, MT, BN>()));
     if (e != cudaSuccess) return e;
     attr_set.store(true, std::memory_order_release);
   }
   // full rounds only: with W = ceil(tiles / SMs) rounds, ceil(tiles / W) CTAs finish in W rounds
   // (for grouped rows `tiles` is an upper bound: the surplus CTAs find no tile and retire)
-  const int64_t workers = PAIR ? L.sm_count / 2 : L.sm_count;
-  const int64_t rounds = std::max<int64_t>(1, (tiles + workers - 1) / workers);
+  const int64_t rounds = std::max<int64_t>(1, (tiles + L.sm_count - 1) / L.sm_count);
   const int grid = static_cast<int>(std::max<int64_t>(1, (tiles + rounds - 1) / rounds));
   ++*L.launches;
-  if constexpr (PAIR)
-    return launch_pdl_cluster(gemm_bf16_kernel<A_MN, B_MN, GROUP, MT, BN, PAIR>, static_cast<unsigned>(2 * grid), 2, Cfg<GROUP, MT, BN, PAIR>::kThreads,
-                              smem_bytes<GROUP, MT, BN, PAIR>(), L.stream, tm.a, tm.b, tm.f32, tm.bf16, p);
-  return launch_pdl(gemm_bf16_kernel<A_MN, B_MN, GROUP, MT, BN, PAIR>, static_cast<unsigned>(grid), Cfg<GROUP, MT, BN, PAIR>::kThreads, smem_bytes<GROUP, MT, BN, PAIR>(), L.stream,
+  return launch_pdl(gemm_bf16_kernel<A_MN, B_MN, GROUP, MT, BN>, static_cast<unsigned>(grid), Cfg<GROUP, MT, BN>::kThreads, smem_bytes<GROUP, MT, BN>(), L.stream,
                     tm.a, tm.b, tm.f32, tm.bf16, p);
 }
 
-template <int GROUP, int MT, int BN, bool PAIR = false>
+template <int GROUP, int MT, int BN>
 cudaError_t launch_majors(const Launch& L, const Maps& tm, const Bf16Params& p, int64_t tiles, bool a_mn, bool b_mn) {
-  if constexpr (GROUP == kGroupedContraction) return launch_variant<true, true, GROUP, MT, BN, PAIR>(L, tm, p, tiles);
+  if constexpr (GROUP == kGroupedContraction) return launch_variant<true, true, GROUP, MT, BN>(L, tm, p, tiles);
   if constexpr (GROUP != kGroupedRows)  // (grouped rows: A is K-major)
     if (a_mn)
-      return b_mn ? launch_variant<true, true, GROUP, MT, BN, PAIR>(L, tm, p, tiles) : launch_variant<true, false, GROUP, MT, BN, PAIR>(L, tm, p, tiles);
-  return b_mn ? launch_variant<false, true, GROUP, MT, BN, PAIR>(L, tm, p, tiles) : launch_variant<false, false, GROUP, MT, BN, PAIR>(L, tm, p, tiles);
+      return b_mn ? launch_variant<true, true, GROUP, MT, BN>(L, tm, p, tiles) : launch_variant<true, false, GROUP, MT, BN>(L, tm, p, tiles);
+  return b_mn ? launch_variant<false, true, GROUP, MT, BN>(L, tm, p, tiles) : launch_variant<false, false, GROUP, MT, BN>(L, tm, p, tiles);
 }
 
 }  // namespace
@@ -770,7 +710,6 @@ cudaError_t launch_gemm_bf16(const Launch& L, EncodeTiledFn encode, const GemmBf
   // tiles cost in proportion.  The grouped forms keep 128 x 256 (ragged groups waste more of a 256-row tile
   // and its single accumulator set exposes the epilogue of short contractions).
   int MT = 1, BN = 256;
-  bool pair = false;
   if (a.group == 0) {
     auto cost = [&](int rows, int cols, double unit) {
       const int64_t tiles = ((a.Mo + rows - 1) / rows) * ((a.No + cols - 1) / cols);
@@ -779,24 +718,8 @@ cudaError_t launch_gemm_bf16(const Launch& L, EncodeTiledFn encode, const GemmBf
     double best = cost(BM, 256, 1.0);
     if (const double c = cost(2 * BM, 256, 2.0 * 0.87); c < best) { best = c; MT = 2; }
     if (const double c = cost(BM, 192, 0.77); c < best) { best = c; MT = 1; BN = 192; }
-    // Two CTAs on a tile of 256 x 256 (PAIR): as many operand bytes as the 256 x 256 tile of one CTA, rounds half as long.
-    // Both directions, one and then the other form in turn: 8192 rows, N = 2048, K = 4096 234 -> 210 us, 6983 rows, 2560 x 3328
-    // 189 -> 181; in a single round it loses (1172 rows, N = 2048, K = 4096: 52 -> 54).
-    const int64_t pair_tiles = ((a.Mo + 2 * BM - 1) / (2 * BM)) * ((a.No + 255) / 256), pairs = L.sm_count / 2;
-    const int64_t pair_rounds = (pair_tiles + pairs - 1) / pairs;
-    pair = pair_rounds > 1 && static_cast<double>(pair_rounds) * 0.96 < best;
-  } else {
-    // Ragged groups waste more of a 256-row tile: from 512 rows per expert on it pays (dX, H x I of the projection: 8192
-    // tokens, 128 experts top-8, 417 -> 380 us, with Zipf popularity 468 -> 468; 4096 tokens, 32 experts top-4 of 4096 x 1536: 433 ->
-    // 403 and 246 -> 218; at 256 and 375 rows 0.80 to 1.10).  The grouped contraction keeps one CTA per tile: its tiles
-    // end when their rows do, and a pair's two epilogues wait for each other (8192 tokens 641 -> 719 us).
-    pair = grouped_rows && a.Mo >= 512 * a.E;
   }
-  if (L.gemm_path != 0) pair = L.gemm_path == 3 && !grouped_k;
-  if (pair) { MT = 1; BN = 256; }
-  const int TM = MT * BM;                   // rows of A and columns of B that a CTA loads
-  const int cta_cols = pair ? BN / 2 : BN;
-  const int tile_rows = pair ? 2 * BM : TM;
+  const int TM = MT * BM;
   // rows of the tensors as TMA sees them
   const int64_t a_rows = a.a_mn_major ? (grouped_k ? a.rows_total : a.Kc) : a.Mo;
   const int64_t b_rows = a.b_mn_major ? (grouped_k ? a.rows_total : (grouped_rows ? a.E * a.Kc : a.Kc))
@@ -806,8 +729,8 @@ cudaError_t launch_gemm_bf16(const Launch& L, EncodeTiledFn encode, const GemmBf
   CUresult r = a3d ? make_tmap_mn3d(encode, &tm.a, a.a, a_rows, a.Mo, TM / 64)
              : a.a_mn_major ? make_tmap(encode, &tm.a, a.a, a_rows, a.Mo, 64, BK) : make_tmap(encode, &tm.a, a.a, a_rows, a.Kc, BK, TM);
   if (r == CUDA_SUCCESS)
-    r = b3d ? make_tmap_mn3d(encode, &tm.b, a.b, b_rows, a.No, cta_cols / 64)
-      : a.b_mn_major ? make_tmap(encode, &tm.b, a.b, b_rows, a.No, 64, BK) : make_tmap(encode, &tm.b, a.b, b_rows, a.Kc, BK, cta_cols);
+    r = b3d ? make_tmap_mn3d(encode, &tm.b, a.b, b_rows, a.No, BN / 64)
+      : a.b_mn_major ? make_tmap(encode, &tm.b, a.b, b_rows, a.No, 64, BK) : make_tmap(encode, &tm.b, a.b, b_rows, a.Kc, BK, BN);
   const uint64_t out_count = grouped_k ? static_cast<uint64_t>(a.E) : 1;
   if (r == CUDA_SUCCESS && a.c_f32) r = make_out_tmap(encode, &tm.f32, a.c_f32, out_count, a.Mo, a.No, 4);
   if (r == CUDA_SUCCESS && a.c_bf16) r = make_out_tmap(encode, &tm.bf16, a.c_bf16, out_count, a.Mo, a.No, 2);
@@ -831,10 +754,7 @@ cudaError_t launch_gemm_bf16(const Launch& L, EncodeTiledFn encode, const GemmBf
   p.wait_limit_ns = L.wait_limit_ns ? L.wait_limit_ns : 2000000000ull;
   p.stop_after_stages = L.stop_after_stages;
   const int64_t n_tiles = (a.No + BN - 1) / BN;
-  const int64_t m_tiles = (a.Mo + tile_rows - 1) / tile_rows;
-  if (pair && grouped_rows)
-    return launch_majors<kGroupedRows, 1, 256, true>(L, tm, p, (a.Mo / tile_rows + a.E) * n_tiles, false, a.b_mn_major);
-  if (pair) return launch_majors<kDense, 1, 256, true>(L, tm, p, m_tiles * n_tiles, a.a_mn_major, a.b_mn_major);
+  const int64_t m_tiles = (a.Mo + TM - 1) / TM;
   if (grouped_rows)  // each expert adds at most one partial row tile
     return launch_majors<kGroupedRows, 1, 256>(L, tm, p, (a.Mo / TM + a.E) * n_tiles, false, a.b_mn_major);
   if (grouped_k) return launch_majors<kGroupedContraction, 1, 256>(L, tm, p, a.E * m_tiles * n_tiles, true, true);

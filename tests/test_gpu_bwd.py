@@ -96,6 +96,22 @@ def test_qkv_projection_shape_sampled(ctx):
     assert (np.abs(g - o_dw) <= tol).all()
 
 
+@pytest.mark.parametrize("m,n,k", [(8192, 2048, 4096), (7001, 2176, 4224)])
+def test_several_tiles_per_cta_sampled(ctx, m, n, k):
+    """Both directions take several tiles per CTA; ragged rows and a last column tile that is half full."""
+    dy, x, w = _case(10 + m, m, n, k)
+    _, dx32, dw32 = ctx.linear_bwd(bits_to_torch(dy), bits_to_torch(x), bits_to_torch(w), want_dx_f32=True)
+    assert ctx.poll() == 0
+    rows = np.array([0, 255, 256, m - 1] + list(np.random.default_rng(2).integers(0, m, 8)))
+    o_dx32, _, _ = oracle.linear_bwd(dy[rows], x[rows], w)
+    tol = 1e-3 * _norms(dy[rows], 1)[:, None] * _norms(w, 0)[None, :]
+    assert (np.abs(dx32[torch.from_numpy(rows).cuda()].cpu().numpy().astype(np.float64) - o_dx32) <= tol).all()
+    feats = np.array([0, 255, 256, n - 1])
+    _, _, o_dw = oracle.linear_bwd(np.ascontiguousarray(dy[:, feats]), x, w[feats])
+    tol = 1e-3 * _norms(dy[:, feats], 0)[:, None] * _norms(x, 0)[None, :]
+    assert (np.abs(dw32[torch.from_numpy(feats).cuda()].cpu().numpy().astype(np.float64) - o_dw) <= tol).all()
+
+
 def test_quantize_weight_publish_writes_two_equal_copies(ctx):
     """Sec. 3.1 item 3: the published tensors are the ones the training forward uses, bit for bit."""
     rng = np.random.default_rng(9)
@@ -167,6 +183,11 @@ def test_grouped_expert_projection_shapes(ctx):
     sizes = [900, 40, 333, 0, 128, 1, 77, 569]
     check_grouped(ctx, 5, sizes, 2048, 768)
     check_grouped(ctx, 6, sizes, 1536, 2048)
+
+
+def test_grouped_many_rows_per_expert(ctx):
+    """Over 512 rows per expert on average, unevenly."""
+    check_grouped(ctx, 8, [1500, 0, 700, 129, 640], 384, 512)
 
 
 # ------------------------------------------------------------------------------ MoE layer backward

@@ -1,0 +1,21 @@
+"""The allocation of tensor memory waits without a limit.  What keeps it from waiting for ever is the order of a few
+instructions, read here from the sources: a GPU that such a wait holds up is lost to its other users, so no run shows it."""
+import os
+import re
+
+import pytest
+
+from paper_2604_07853_b200 import build
+
+ONE_CTA = ["gemm_bf16_sm100.cu"]
+
+
+def source(name):
+    with open(os.path.join(build.CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+@pytest.mark.parametrize("name", ONE_CTA)
+def test_no_kernel_allocates_for_a_pair_of_ctas(name):
+    """`cta_group::2` allocates for two CTAs at once and waits for both: with one of them not begun, or gone, nothing ends it."""
+    assert not re.search(r"cta_group::2|tmem_alloc_pair|umma_\w+_pair", source(name))
