@@ -409,7 +409,7 @@ int qarl_harness_set_wait_limit_ns(qarl_ctx* ctx, uint64_t limit_ns) {
 }
 
 int qarl_harness_set_gemm_path(qarl_ctx* ctx, int path) {
-  if (!ctx || path < 0 || path > 3) return QARL_ERR_INVALID_ARG;
+  if (!ctx || path < 0 || path > 2) return QARL_ERR_INVALID_ARG;
   ctx->gemm_path = path;
   return QARL_OK;
 }

@@ -63,7 +63,7 @@ struct Launch {
   int64_t* launches;  // host counter
   unsigned long long wait_limit_ns = 0;  // bound of every device-side barrier wait (0: the default, 2 s)
   int stop_after_stages = -1;            // test harness only: GEMM producers stop after this many stages
-  int gemm_path = 0;                     // test harness only: 0 = automatic, 1 = wide-tile kernel, 2 = decode kernel (one launch per projection), 3 = wide-tile kernel on pairs of CTAs
+  int gemm_path = 0;                     // test harness only: 0 = automatic, 1 = wide-tile kernel, 2 = decode kernel (one launch per projection)
   int dense_columns = 0;                 // test harness only: columns per tile of a dense FP8 call (0 = automatic)
   int router_form = 0;                   // test harness only: 0 = automatic, 1 = two launches, 2 = one launch, 3 = one launch of clusters
 };

@@ -36,15 +36,6 @@
 // of this one is accumulated), two FMAs per instruction, the loop body without spills (32-column chunks
 // spill and lose), and no epilogue warps (their registers and polling cost more than they hid).
 //
-// Dense calls of many rows: a PAIR of CTAs (a cluster; tcgen05 cta_group::2) shares a tile of 256 rows x 256 columns.  Each
-// CTA loads its 128 rows of A and 128 of the 256 weight rows, the even one issues the MMAs for both and each promotes its own
-// rows, so an SM takes in 32 KB per K-block instead of 48.  That traffic is the other bound of the single-CTA form: MMAs and
-// loads without promotion take ~800 clocks per K-block, MMAs alone 630.  The accumulator is published and handed
-// back in two column parts (64 columns of either half, the slices of warps 0-3 and of warps 4-7; MMAs of N = 128), so that
-// the two warps of an SM sub-partition promote in turn instead of waiting and multiplying at the same time: with whole
-// accumulators the pair's longer hand-over ate what the loads saved (983 clocks per K-block with tile ends, 848 in parts,
-// single CTA 935).
-//
 // Every wait on an mbarrier is bounded; on expiry the thread records
 // QARL_ERR_DEVICE_TIMEOUT, raises a CTA-wide abort flag that all other waits poll, and the
 // CTA drains and frees its TMEM, so a broken pipeline returns an error instead of hanging.
@@ -109,17 +100,14 @@ struct GemmParams {
 
 // SAVE (gate_up only): the call also wants the bf16 gate_up and / or h rows (a training forward, tests)
 // COLS: columns of a tile, 256 (two halves); 128 and 64 are for dense calls that do not fill the SMs with 256
-// PAIR: two CTAs share a tile of 256 rows (see the header)
-template <int MODE, bool SAVE, int COLS, bool PAIR>
+template <int MODE, bool SAVE, int COLS>
 struct Cfg {
   static constexpr bool kStaged = MODE != kModeGateUp || SAVE;  // rows leave through the staging boxes
   static constexpr int kHalves = COLS == 256 ? 2 : 1;
   static constexpr int kSlice = COLS / kHalves / 2;             // columns of each half owned by one promotion warp
   // ring: fixed 48 or 32 KB stages; with 64 columns as many as fit (a decode call's token box is a few rows, see the host)
-  static constexpr int kStages = COLS == 64 ? 0 : COLS == 128 ? 5 : PAIR ? 4 : kStaged ? 3 : 4;
-  static constexpr uint32_t kStageBytes = kABytes + (PAIR ? kBHalfBytes : COLS * BK);
-  static constexpr int kTileRows = PAIR ? 2 * BM : BM;
-  static constexpr int kParts = PAIR ? 2 : 1;  // accumulators are published and handed back in this many column parts
+  static constexpr int kStages = COLS == 64 ? 0 : COLS == 128 ? 5 : kStaged ? 3 : 4;
+  static constexpr uint32_t kStageBytes = kABytes + COLS * BK;
   static constexpr uint32_t kStaging = kStaged && COLS > 64 ? kPromoWarps * kHalves * kOutBoxBytes : 0;
   static constexpr int kAccBufs = COLS == 256 ? 2 : 4;
 };
@@ -144,13 +132,12 @@ struct __align__(16) SmemTail {
   int32_t prefix[kMaxExperts + 1];
 };
 
-template <int MODE, bool SAVE, int COLS, bool PAIR = false>
-constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(Cfg<MODE, SAVE, COLS, PAIR>::kStages) * Cfg<MODE, SAVE, COLS, PAIR>::kStageBytes +
-                              Cfg<MODE, SAVE, COLS, PAIR>::kStaging + sizeof(SmemTail);
+template <int MODE, bool SAVE, int COLS>
+constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(Cfg<MODE, SAVE, COLS>::kStages) * Cfg<MODE, SAVE, COLS>::kStageBytes +
+                              Cfg<MODE, SAVE, COLS>::kStaging + sizeof(SmemTail);
 constexpr size_t kSmemLimit = 227 * 1024;
 static_assert(kSmemBytes<kModeGateUp, false, 256> <= kSmemLimit && kSmemBytes<kModeGateUp, true, 256> <= kSmemLimit &&
-                  kSmemBytes<kModeLinear, false, 128> <= kSmemLimit &&
-                  kSmemBytes<kModeLinear, false, 256, true> <= kSmemLimit,
+                  kSmemBytes<kModeLinear, false, 128> <= kSmemLimit,
               "shared memory budget");
 
 struct TileCoord {
@@ -159,17 +146,15 @@ struct TileCoord {
 
 // Tile T -> (expert, column tile, first row, end of the expert's rows).  Within an expert the
 // row tiles vary fastest, so CTAs running at the same time share one weight tile through L2.
-template <int TILE_ROWS>
 __device__ __forceinline__ TileCoord decode_tile(const SmemTail* s, int T, int& cur_e) {
   while (T >= s->prefix[cur_e + 1]) ++cur_e;
   const int local = T - s->prefix[cur_e];
   const int rows = s->off[cur_e + 1] - s->off[cur_e];
-  const int m_tiles = (rows + TILE_ROWS - 1) / TILE_ROWS;
+  const int m_tiles = (rows + BM - 1) / BM;
   TileCoord c;
   c.e = cur_e;
   c.n_tile = local / m_tiles;
-  c.m0 = s->off[cur_e] + (local % m_tiles) * TILE_ROWS;
-  if (TILE_ROWS > BM) c.m0 += static_cast<int>(cluster_ctarank()) * BM;  // this CTA's rows
+  c.m0 = s->off[cur_e] + (local % m_tiles) * BM;
   c.m_end = s->off[cur_e + 1];
   return c;
 }
@@ -236,10 +221,10 @@ __device__ __forceinline__ void st_global_2x16(void* dst, const uint32_t (&v)[8]
 
 // The promotion warps (see the header).  What they need is read again here instead of being carried over from
 // the kernel's set-up: with 160 registers of sums and partial sums every long-lived value counts.
-template <int MODE, bool SAVE, int COLS, bool PAIR>
+template <int MODE, bool SAVE, int COLS>
 __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const GemmParams& p, uint8_t* smem, SmemTail* s,
                                                const int first_tile, const int num_ctas, const int total_tiles) {
-  using C = Cfg<MODE, SAVE, COLS, PAIR>;
+  using C = Cfg<MODE, SAVE, COLS>;
   constexpr int kAccBufs = C::kAccBufs, HALVES = C::kHalves, kSliceCols = C::kSlice;
   constexpr int kPerHalf = kSliceCols / 16, kChunks = kPerHalf * HALVES;  // 16-column chunks of this warp's slices
   uint32_t tid;
@@ -249,10 +234,8 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
   const int hs = warp >> 2;        // which 64-column slice of each half tile
   const int r = q * 32 + lane;     // row within the tile
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&s->tmem_addr) + (static_cast<uint32_t>(q * 32) << 16) +
-                        static_cast<uint32_t>(hs * (PAIR ? COLS / 2 : kSliceCols));
-  // (PAIR: this warp's slices of the two halves are one part of the accumulator, with barriers of its own)
-  constexpr uint32_t kBarStep = 8 * C::kParts;
-  const uint32_t full_bar = smem_u32(&s->tmem_full[PAIR ? hs : 0]), empty_bar = smem_u32(&s->tmem_empty[PAIR ? hs : 0]);
+                        static_cast<uint32_t>(hs * kSliceCols);
+  const uint32_t full_bar = smem_u32(&s->tmem_full[0]), empty_bar = smem_u32(&s->tmem_empty[0]);
   const uint32_t scale_at = smem_u32(&s->scale[0][r]);
   const int KB = p.kblocks;
   int ks = 0;
@@ -260,15 +243,11 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
   int cur_e = 0;
   uint32_t tile_iter = 0;
 
-  auto full_wait = [&]() -> bool { return __all_sync(0xFFFFFFFFu, wait_or_abort_at(full_bar + kBarStep * ks, acc_phase, s, p)) != 0; };
+  auto full_wait = [&]() -> bool { return __all_sync(0xFFFFFFFFu, wait_or_abort_at(full_bar + 8 * ks, acc_phase, s, p)) != 0; };
   auto release = [&]() {  // this warp's reads of accumulator ks are done: hand it back to the MMA warp
     tc_fence_before_sync();
     __syncwarp();
-    if (lane == 0) {
-      mbar_arrive_at(empty_bar + kBarStep * ks);
-      // (the MMA warp of the pair is in the even CTA; the data handed over is tensor memory, read completely)
-      if (PAIR && cluster_ctarank() != 0) mbar_arrive_cluster_relaxed(map_to_cta(empty_bar + kBarStep * ks, 0));
-    }
+    if (lane == 0) mbar_arrive_at(empty_bar + 8 * ks);
     if (++ks == kAccBufs) { ks = 0; acc_phase ^= 1; }
   };
 
@@ -306,7 +285,7 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
     // looked up faster than the scale warps publish it (M = 777, N = 2048, K = 4096: 17.0 against 17.5).
     TileCoord c;
     if constexpr (MODE == kModeLinear) {
-      c = decode_tile<C::kTileRows>(s, T, cur_e);
+      c = decode_tile(s, T, cur_e);
       if (!full_wait()) return;
     } else {
       if (!full_wait()) return;
@@ -338,7 +317,7 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
         asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(scale.x), "=f"(scale.y)
                      : "r"(scale_at + static_cast<uint32_t>(ks) * static_cast<uint32_t>(sizeof(s->scale[0]))) : "memory");
       };
-      auto chunk_at = [&](uint32_t t0, int c) { return PAIR ? t0 + 16 * c : t0 + (c / kPerHalf) * BNH + 16 * (c % kPerHalf); };
+      auto chunk_at = [&](uint32_t t0, int c) { return t0 + (c / kPerHalf) * BNH + 16 * (c % kPerHalf); };
       auto add = [&](int c, const uint32_t (&v)[16]) { promote16(acc + 8 * c, v, c < kPerHalf ? scale.x : scale.y); };
       auto all_but_last = [&]() {  // every chunk of accumulator ks but the last two sums; on return the last is in flight
         const uint32_t t0 = tmem + static_cast<uint32_t>(ks * COLS);
@@ -362,7 +341,7 @@ __device__ __forceinline__ void promotion_role(const CUtensorMap& tm_o, const Ge
         all_but_last();
         // the next accumulator's barrier: the answer is needed one chunk later
         const int kn = ks + 1 == kAccBufs ? 0 : ks + 1;
-        const bool next_ready = mbar_try_wait_at(full_bar + kBarStep * kn, kn == 0 ? acc_phase ^ 1u : acc_phase);
+        const bool next_ready = mbar_try_wait_at(full_bar + 8 * kn, kn == 0 ? acc_phase ^ 1u : acc_phase);
         add(kChunks - 2, va);
         tmem_ld_wait();
         const float last_scale = HALVES == 2 ? scale.y : scale.x;
@@ -535,15 +514,15 @@ __device__ __forceinline__ void quantize_rows(const GemmParams& p, uint8_t* smem
   if ((threadIdx.x & 31) == 0) mbar_arrive(&s->x_ready);
 }
 
-template <int MODE, bool SAVE, int COLS, bool FUSED, bool PAIR>
+template <int MODE, bool SAVE, int COLS, bool FUSED>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                         const __grid_constant__ CUtensorMap tm_o, const GemmParams p) {
-  using C = Cfg<MODE, SAVE, COLS, PAIR>;
+  using C = Cfg<MODE, SAVE, COLS>;
   constexpr int kAccBufs = C::kAccBufs, HALVES = C::kHalves;
   const int kStages = COLS == 64 ? p.stages : C::kStages;
   const uint32_t a_bytes = FUSED ? 0u : COLS == 64 ? static_cast<uint32_t>(p.a_rows) * BK : kABytes;
-  const uint32_t kStageBytes = PAIR ? C::kStageBytes : a_bytes + COLS * BK;
+  const uint32_t kStageBytes = a_bytes + COLS * BK;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   // (COLS = 64: the MMA reads 128 token rows from a stage whatever its box holds; what lies behind the box must be shared
@@ -553,7 +532,6 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
   SmemTail* s = reinterpret_cast<SmemTail*>(out_tile + C::kStaging);
   float* x_scale = reinterpret_cast<float*>(s + 1);  // FUSED: [rows][K-blocks]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rank = PAIR ? static_cast<int>(cluster_ctarank()) : 0;
 
   // ---- set-up: barriers, TMEM, tile list ------------------------------------------------
   pdl_trigger();
@@ -562,10 +540,9 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
       mbar_init(&s->full[i], 1);
       mbar_init(&s->empty[i], 1);
     }
-    for (int i = 0; i < kAccBufs * C::kParts; ++i) {
+    for (int i = 0; i < kAccBufs; ++i) {
       mbar_init(&s->tmem_full[i], FUSED ? 2 : 3);  // the MMA commit and the two scale warps
-      // (PAIR: the even CTA's MMAs write the accumulators of both)
-      mbar_init(&s->tmem_empty[i], FUSED ? 2 : kPromoWarps / C::kParts * (PAIR && rank == 0 ? 2 : 1));
+      mbar_init(&s->tmem_empty[i], FUSED ? 2 : kPromoWarps);
     }
     for (int i = 0; i < 4; ++i) mbar_init(&s->amax_full[i], 2);
     mbar_init(&s->teardown, 1);
@@ -579,15 +556,10 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
     if (C::kStaging > 0) prefetch_tensormap(&tm_o);
   }
   if (warp == kMmaWarp) {
-    if constexpr (PAIR) {
-      tmem_alloc_pair(&s->tmem_addr, kTmemCols);
-      tmem_relinquish_pair();
-    } else {
-      tmem_alloc(&s->tmem_addr, kTmemCols);
-      tmem_relinquish();
-    }
+    tmem_alloc(&s->tmem_addr, kTmemCols);
+    tmem_relinquish();
   }
-  if (warp == kTmaWarp && lane == 0 && !PAIR && p.early_prefetch > 0) {
+  if (warp == kTmaWarp && lane == 0 && p.early_prefetch > 0) {
     // Decode-sized calls are bound by streaming the weights from HBM, and the kernels before
     // this one in the stream (permute, activation quantization) leave the memory system idle.
     // The weights do not depend on them, so pull this CTA's first weight tiles into L2 now.
@@ -633,7 +605,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
         // with every boundary inside [0, rows_total] the other groups stay inside the tensors
         const int rows = s->off[e + 1] - s->off[e];
         if (rows < 0) set_status(p.status, QARL_ERR_INVALID_ARG);
-        v = ((max(rows, 0) + C::kTileRows - 1) / C::kTileRows) * p.n_tiles;
+        v = ((max(rows, 0) + BM - 1) / BM) * p.n_tiles;
       }
       int inc = v;
 #pragma unroll
@@ -647,8 +619,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
     if (lane == 0) s->prefix[p.E] = carry;
   }
   tc_fence_before_sync();
-  if constexpr (PAIR) cluster_sync();  // (the other CTA's barriers are initialised too)
-  else __syncthreads();
+  __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = s->tmem_addr;
   const int total_tiles = s->prefix[p.E];
@@ -656,13 +627,12 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
   // finish in W rounds; using exactly that many keeps every round full (768 decode tiles: 128 CTAs
   // x 6 instead of 148 CTAs of which 120 idle through the sixth round) and leaves the streaming
   // bandwidth to the CTAs that still have work.  The CTAs beyond that count retire at once.
-  int num_ctas = PAIR ? gridDim.x / 2 : gridDim.x;  // (pairs)
-  const int cta = PAIR ? blockIdx.x / 2 : blockIdx.x;
+  int num_ctas = gridDim.x;
   if (total_tiles > 0) {
     const int rounds = (total_tiles + num_ctas - 1) / num_ctas;
     num_ctas = (total_tiles + rounds - 1) / rounds;
   }
-  const int first_tile = cta < num_ctas ? cta : total_tiles;
+  const int first_tile = static_cast<int>(blockIdx.x) < num_ctas ? static_cast<int>(blockIdx.x) : total_tiles;
   const int KB = p.kblocks;
   const int NB = p.N / BNH;  // weight scale block-rows per expert
 
@@ -689,7 +659,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
           }
         };
         for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
-          const TileCoord c = decode_tile<C::kTileRows>(s, T, cur_e);
+          const TileCoord c = decode_tile(s, T, cur_e);
           int row_lo, row_hi;
           b_rows(c, row_lo, row_hi);
           for (int kb = 0; kb < KB; ++kb) {
@@ -698,69 +668,47 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
             if (!wait_or_abort(&s->empty[stage], phase ^ 1, s, p)) { ok = false; break; }
             uint8_t* a_dst = ring + static_cast<size_t>(stage) * kStageBytes;
             uint8_t* b_dst = a_dst + a_bytes;
-            if constexpr (PAIR) {  // both CTAs' bytes count on the even CTA's barrier; of the tile's columns each loads a half
-              const uint32_t bar = map_to_cta(smem_u32(&s->full[stage]), 0);
-              if (rank == 0) mbar_arrive_expect_tx(&s->full[stage], 2 * kStageBytes);
-              tma_load_2d_pair(a_dst, &tm_a, bar, kb * BK, c.m0);
-              tma_load_2d_pair(b_dst, &tm_b, bar, kb * BK, rank == 0 ? row_lo : row_hi);
+            mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
+            if (!FUSED) tma_load_2d(a_dst, &tm_a, &s->full[stage], kb * BK, c.m0);
+            if (p.weights_once) {
+              tma_load_2d_hint(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo, stream_once);
+              if (HALVES == 2) tma_load_2d_hint(b_dst + kBHalfBytes, &tm_b, &s->full[stage], kb * BK, row_hi, stream_once);
             } else {
-              mbar_arrive_expect_tx(&s->full[stage], kStageBytes);
-              if (!FUSED) tma_load_2d(a_dst, &tm_a, &s->full[stage], kb * BK, c.m0);
-              if (p.weights_once) {
-                tma_load_2d_hint(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo, stream_once);
-                if (HALVES == 2) tma_load_2d_hint(b_dst + kBHalfBytes, &tm_b, &s->full[stage], kb * BK, row_hi, stream_once);
-              } else {
-                tma_load_2d(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo);
-                if (HALVES == 2) tma_load_2d(b_dst + kBHalfBytes, &tm_b, &s->full[stage], kb * BK, row_hi);
-              }
+              tma_load_2d(b_dst, &tm_b, &s->full[stage], kb * BK, row_lo);
+              if (HALVES == 2) tma_load_2d(b_dst + kBHalfBytes, &tm_b, &s->full[stage], kb * BK, row_hi);
             }
             armed |= 1u << stage;
             armed_parity = (armed_parity & ~(1u << stage)) | (phase << stage);
             if (++stage == kStages) { stage = 0; phase ^= 1; }
           }
         }
-        if (!ok && rank != 0) {  // this CTA's copies count on the other's barrier, which is not waited for from here: they land in microseconds
-          const uint64_t t0 = globaltimer_ns();
-          while (globaltimer_ns() - t0 < 1000000ull) __nanosleep(1000);
-        } else if (!ok) {  // let copies in flight land before the CTA's shared memory is released
+        if (!ok) {  // let copies in flight land before the CTA's shared memory is released
           for (int i = 0; i < kStages; ++i)
             if (armed & (1u << i)) mbar_wait_bounded(&s->full[i], (armed_parity >> i) & 1u, 20000000ull);
         }
       }
     } else if (warp == kMmaWarp) {
       // =============================== MMA issuer =======================================
-      if (rank == 0 && elect_one()) {
-        constexpr uint32_t idesc = umma_idesc_e4m3_f32(C::kTileRows, COLS / C::kParts);
+      if (elect_one()) {
+        constexpr uint32_t idesc = umma_idesc_e4m3_f32(BM, COLS);
         int stage = 0, ks = 0;
         uint32_t phase = 0, acc_phase = 0;
         bool ok = !FUSED || wait_or_abort(&s->x_ready, 0, s, p);
         for (int T = first_tile; ok && T < total_tiles; T += num_ctas) {
           for (int kb = 0; kb < KB; ++kb) {
+            if (!wait_or_abort(&s->tmem_empty[ks], acc_phase ^ 1, s, p)) { ok = false; break; }
+            if (!wait_or_abort(&s->full[stage], phase, s, p)) { ok = false; break; }
+            tc_fence_after_sync();
             const uint32_t stage_addr = smem_u32(ring + static_cast<size_t>(stage) * kStageBytes);
             const uint32_t a_addr = FUSED ? smem_u32(smem) + kb * 1024 : stage_addr;
             const uint64_t a_desc = umma_desc_k_sw128(a_addr);
             const uint64_t b_desc = umma_desc_k_sw128(stage_addr + a_bytes);
+            const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(ks * COLS);
 #pragma unroll
-            for (int part = 0; part < C::kParts; ++part) {
-              if (!wait_or_abort(&s->tmem_empty[C::kParts * ks + part], acc_phase ^ 1, s, p)) { ok = false; break; }
-              if (part == 0 && !wait_or_abort(&s->full[stage], phase, s, p)) { ok = false; break; }
-              tc_fence_after_sync();
-              const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(ks * COLS + part * (COLS / C::kParts));
-#pragma unroll
-              for (int k4 = 0; k4 < BK / 32; ++k4) {  // +32 bytes of K = +2 in the 16-byte address field
-                // (part 1: rows 64.. of each CTA's 128 weight rows)
-                if constexpr (PAIR) umma_f8_pair(d_tmem, a_desc + 2 * k4, b_desc + part * (64 * BK / 16) + 2 * k4, idesc, k4 > 0 ? 1u : 0u);
-                else umma_f8(d_tmem, a_desc + 2 * k4, b_desc + 2 * k4, idesc, k4 > 0 ? 1u : 0u);
-              }
-              if constexpr (PAIR) {
-                if (part == C::kParts - 1) umma_commit_pair(&s->empty[stage]);
-                umma_commit_pair(&s->tmem_full[C::kParts * ks + part]);
-              } else {
-                umma_commit(&s->empty[stage]);
-                umma_commit(&s->tmem_full[ks]);
-              }
-            }
-            if (!ok) break;
+            for (int k4 = 0; k4 < BK / 32; ++k4)  // +32 bytes of K = +2 in the 16-byte address field
+              umma_f8(d_tmem, a_desc + 2 * k4, b_desc + 2 * k4, idesc, k4 > 0 ? 1u : 0u);
+            umma_commit(&s->empty[stage]);
+            umma_commit(&s->tmem_full[ks]);
             if (++stage == kStages) { stage = 0; phase ^= 1; }
             if (++ks == kAccBufs) { ks = 0; acc_phase ^= 1; }
           }
@@ -769,8 +717,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
         // go away: after a normal run every MMA has been consumed already; after an abort
         // some may still be executing, so wait (bounded) for all of them.
         if (!ok) {
-          if constexpr (PAIR) umma_commit_pair(&s->teardown);
-          else umma_commit(&s->teardown);
+          umma_commit(&s->teardown);
           mbar_wait_bounded(&s->teardown, 0, 20000000ull);
         }
       }
@@ -788,7 +735,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
       const float *x0 = nullptr, *x1 = nullptr, *wl = nullptr, *wh = nullptr;
       float n0 = 0.f, n1 = 0.f, nl = 0.f, nh = 0.f;  // of the next K-block: its loads fly during this one
       auto open_tile = [&](int T) {
-        const TileCoord c = decode_tile<C::kTileRows>(s, T, cur_e);
+        const TileCoord c = decode_tile(s, T, cur_e);
         int nb_lo, nb_hi;
         if (MODE == kModeGateUp) {
           nb_lo = c.n_tile;
@@ -826,8 +773,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
           } else if (T + num_ctas < total_tiles) {
             open_tile(T + num_ctas);
           }
-          for (int part = 0; part < C::kParts; ++part) ok = ok && warp_wait_or_abort(&s->tmem_empty[C::kParts * ks + part], acc_phase ^ 1, s, p);
-          if (!ok) break;
+          if (!warp_wait_or_abort(&s->tmem_empty[ks], acc_phase ^ 1, s, p)) { ok = false; break; }
           if (MODE != kModeLinear && kb == 0) {
             if (warp == kScaleWarp && lane == 0) s->tile[tile_iter & (2 * kMaxAccBufs - 1)] = info;
             if (MODE == kModeDown) {
@@ -838,9 +784,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
           s->scale[ks][r0] = v0;
           s->scale[ks][r0 + 32] = v1;
           __syncwarp();
-          if (lane == 0) {
-            for (int part = 0; part < C::kParts; ++part) mbar_arrive(&s->tmem_full[C::kParts * ks + part]);
-          }
+          if (lane == 0) mbar_arrive(&s->tmem_full[ks]);
           if (++ks == kAccBufs) { ks = 0; acc_phase ^= 1; }
         }
       }
@@ -851,17 +795,15 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
     if constexpr (FUSED) quantize_rows(p, smem, x_scale, s);
     // (FUSED: all rows are in TMEM quadrant 0; warps that only keep the barriers going cost those that work: one token,
     // N = 5120, K = 2048 7.0 -> 6.8 us)
-    if (!FUSED || (warp & 3) == 0) promotion_role<MODE, SAVE, COLS, PAIR>(tm_o, p, smem, s, first_tile, num_ctas, total_tiles);
+    if (!FUSED || (warp & 3) == 0) promotion_role<MODE, SAVE, COLS>(tm_o, p, smem, s, first_tile, num_ctas, total_tiles);
   }
 
   // ---- teardown ---------------------------------------------------------------------------
   tc_fence_before_sync();
-  if constexpr (PAIR) cluster_sync();  // (nothing reads or signals the other CTA any more)
-  else __syncthreads();
+  __syncthreads();
   if (warp == kMmaWarp) {
     tc_fence_after_sync();
-    if constexpr (PAIR) tmem_dealloc_pair(tmem_base, kTmemCols);
-    else tmem_dealloc(tmem_base, kTmemCols);
+    tmem_dealloc(tmem_base, kTmemCols);
   }
 }
 
@@ -892,7 +834,7 @@ CUresult make_tmap(EncodeTiledFn encode, CUtensorMap* m, const void* base, uint6
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
-template <int MODE, bool SAVE, int COLS, bool FUSED = false, bool PAIR = false>
+template <int MODE, bool SAVE, int COLS, bool FUSED = false>
 cudaError_t launch_mode(const Launch& L, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to,
                         const GemmParams& p, int grid) {
   // sticky per function and device; atomic: contexts on several host threads may launch at once (both
@@ -900,18 +842,16 @@ cudaError_t launch_mode(const Launch& L, const CUtensorMap& ta, const CUtensorMa
   static std::atomic<bool> attr_set_dev[64];
   std::atomic<bool>& attr_set = attr_set_dev[L.device & 63];
   if (!attr_set.load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_blockscaled_kernel<MODE, SAVE, COLS, FUSED, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(COLS == 64 ? kSmemLimit : kSmemBytes<MODE, SAVE, COLS, PAIR>));
+    cudaError_t e = cudaFuncSetAttribute(gemm_blockscaled_kernel<MODE, SAVE, COLS, FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(COLS == 64 ? kSmemLimit : kSmemBytes<MODE, SAVE, COLS>));
     if (e != cudaSuccess) return e;
     attr_set.store(true, std::memory_order_release);
   }
-  size_t smem = kSmemBytes<MODE, SAVE, COLS, PAIR>;
+  size_t smem = kSmemBytes<MODE, SAVE, COLS>;
   if (COLS == 64)
     smem += kABytes + static_cast<size_t>(p.stages) * (p.a_rows + COLS) * BK + (FUSED ? static_cast<size_t>(p.kblocks) * (1024 + kFusedRows * 4) : 0);
   ++*L.launches;
-  if constexpr (PAIR)
-    return launch_pdl_cluster(gemm_blockscaled_kernel<MODE, SAVE, COLS, FUSED, PAIR>, static_cast<unsigned>(grid), 2, kThreads, smem, L.stream, ta, tb, to, p);
-  return launch_pdl(gemm_blockscaled_kernel<MODE, SAVE, COLS, FUSED, PAIR>, static_cast<unsigned>(grid), kThreads, smem, L.stream, ta, tb, to, p);
+  return launch_pdl(gemm_blockscaled_kernel<MODE, SAVE, COLS, FUSED>, static_cast<unsigned>(grid), kThreads, smem, L.stream, ta, tb, to, p);
 }
 
 }  // namespace
@@ -938,11 +878,7 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
   // Columns per tile of a dense call: the width whose full rounds over the SMs cost least.  Per round 128 columns take
   // ~0.6 of what 256 take, 64 ~0.45 (M = 777, N = 2048, K = 4096: 56 tiles of 256 on 148 SMs 23.6 us, 112 of 128
   // columns 16.5; M = 65: 12.9 us with 128 columns, 11.6 with 64).
-  // Two CTAs on 256 rows x 256 columns: see the header; a round of pairs takes 0.93 of one of single CTAs (8192 rows, N = 5120,
-  // K = 2048: 103 -> 95 us; 2048 rows 30.8 -> 29.1).  Row groups keep one CTA per tile: they waste more of a 256-row
-  // tile than the pair gains (32768 tokens, Zipf popularity: gate_up 1030 -> 1013, down 609 -> 643 us; 8192: both slower).
   int cols = BN;
-  bool pair = false;
   if (a.mode == kModeLinear && a.offsets == nullptr) {
     auto cost = [&](int c, double unit) {
       const int64_t tiles = ((a.rows_total + BM - 1) / BM) * ((a.N + c - 1) / c);
@@ -951,11 +887,7 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
     double best = cost(BN, 1.0);
     if (const double c = cost(128, 0.6); c < best) { best = c; cols = 128; }
     if (const double c = cost(64, 0.45); c < best) { best = c; cols = 64; }
-    const int64_t pair_tiles = ((a.rows_total + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN), pairs = L.sm_count / 2;
-    pair = static_cast<double>((pair_tiles + pairs - 1) / pairs) * 0.93 < best;
-    if (L.gemm_path != 0) pair = L.gemm_path == 3;
-    if (forced) { cols = L.dense_columns; pair = false; }
-    if (pair) cols = BN;
+    if (forced) cols = L.dense_columns;
   }
   GemmParams p{};
   if (a.x != nullptr) {
@@ -1010,10 +942,6 @@ cudaError_t launch_gemm(const Launch& L, EncodeTiledFn encode, const GemmArgs& a
   }
   // upper bound on the tile count (group sizes live on the device): each expert adds at most
   // one partial row tile
-  if (pair) {
-    const int64_t tiles = (a.rows_total + 2 * BM - 1) / (2 * BM) * p.n_tiles;
-    return launch_mode<kModeLinear, false, 256, false, true>(L, ta, tb, to, p, 2 * static_cast<int>(std::min<int64_t>(L.sm_count / 2, tiles)));
-  }
   const int64_t m_tiles_max = a.rows_total / BM + a.E;
   const int grid = static_cast<int>(std::min<int64_t>(L.sm_count, m_tiles_max * p.n_tiles));
   switch (a.mode) {

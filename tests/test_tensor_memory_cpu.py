@@ -7,7 +7,7 @@ import pytest
 
 from paper_2604_07853_b200 import build
 
-ONE_CTA = ["gemm_bf16_sm100.cu"]
+FILES = sorted(f for f in os.listdir(build.CSRC) if f.endswith((".cu", ".cuh")))
 
 
 def source(name):
@@ -15,7 +15,7 @@ def source(name):
         return re.sub(r"//[^\n]*", "", f.read())
 
 
-@pytest.mark.parametrize("name", ONE_CTA)
+@pytest.mark.parametrize("name", FILES)
 def test_no_kernel_allocates_for_a_pair_of_ctas(name):
     """`cta_group::2` allocates for two CTAs at once and waits for both: with one of them not begun, or gone, nothing ends it."""
     assert not re.search(r"cta_group::2|tmem_alloc_pair|umma_\w+_pair", source(name))
