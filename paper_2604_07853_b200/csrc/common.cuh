@@ -48,6 +48,10 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // (its successor may start launching) and pdl_wait() before its first access to global memory
 // (the predecessor, and transitively everything before it, has completed and is visible).
 // Only barrier set-up, TMEM allocation and other memory-free preamble runs ahead of the wait.
+// A kernel that takes tensor memory triggers after it has it.  The allocation waits without a limit, in no promised
+// order: of three small kernels whose CTAs share an SM (71 KB of shared memory each in the 64-column dense form), the third could
+// otherwise be given the columns that the first frees and hold them for the end of the second, which waits for them.
+// So a CTA that holds tensor memory only ever waits for kernels that hold all of theirs.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -191,7 +191,6 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   SmemOrder* list = reinterpret_cast<SmemOrder*>(s + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) {
       mbar_init(&s->full[i], 1);
@@ -212,6 +211,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   }
   if (warp == kMmaWarp) {
     tmem_alloc(&s->tmem_addr, kTmemCols);
+    pdl_trigger();  // not before the allocation: see pdl_trigger
     tmem_relinquish();
   }
   pdl_wait();

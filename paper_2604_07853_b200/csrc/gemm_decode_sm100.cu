@@ -344,7 +344,6 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr bool kLayer = MODE == kModeLayer;
 
-  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) {
       mbar_init(&s->full[i], 1);
@@ -375,6 +374,7 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   }
   if (warp == kMmaWarp) {
     tmem_alloc(&s->tmem_addr, kTmemCols);
+    pdl_trigger();  // not before the allocation: see pdl_trigger
     tmem_relinquish();
   }
   if (warp == kTmaWarp && lane == 0 && p.early_prefetch > 0) {

@@ -534,7 +534,6 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   // ---- set-up: barriers, TMEM, tile list ------------------------------------------------
-  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) {
       mbar_init(&s->full[i], 1);
@@ -557,6 +556,7 @@ gemm_blockscaled_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_c
   }
   if (warp == kMmaWarp) {
     tmem_alloc(&s->tmem_addr, kTmemCols);
+    pdl_trigger();  // not before the allocation: see pdl_trigger
     tmem_relinquish();
   }
   if (warp == kTmaWarp && lane == 0 && p.early_prefetch > 0) {

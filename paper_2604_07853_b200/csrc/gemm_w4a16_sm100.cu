@@ -189,7 +189,6 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   // ---- set-up: barriers, TMEM, tile list ------------------------------------------------
-  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int i = 0; i < kXStages; ++i) {
       mbar_init(&s->x_full[i], 1);
@@ -215,6 +214,7 @@ gemm_w4a16_kernel(const __grid_constant__ CUtensorMap tm_x, const W4Params p) {
   if (warp == kTokenWarp && lane == 0) prefetch_tensormap(&tm_x);
   if (warp == kMmaWarp) {
     tmem_alloc(&s->tmem_addr, kTmemCols);
+    pdl_trigger();  // not before the allocation: see pdl_trigger
     tmem_relinquish();
   }
   const int KS = p.ksteps;

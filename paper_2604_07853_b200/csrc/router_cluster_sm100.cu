@@ -103,7 +103,6 @@ router_cluster_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
   const int tile = blockIdx.x / cluster;
   const int KS = (p.H + RK - 1) / RK;  // a ragged last step reads zeros (TMA out-of-range fill)
 
-  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int i = 0; i < p.stages; ++i) {
       mbar_init(&s->full[i], 2);  // the two producers
@@ -121,6 +120,7 @@ router_cluster_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
   }
   if (warp == kMmaWarp) {
     tmem_alloc(&s->tmem_addr, kTmemCols);
+    pdl_trigger();  // not before the allocation: see pdl_trigger
     tmem_relinquish();
   }
   tc_fence_before_sync();

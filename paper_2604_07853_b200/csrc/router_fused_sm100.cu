@@ -105,7 +105,6 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
   SmemTail* s = reinterpret_cast<SmemTail*>(logit_tile + kLogitBytes + kScratchBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) {
       mbar_init(&s->full[i], 1);
@@ -126,6 +125,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
   }
   if (warp == kMmaWarp) {
     tmem_alloc(&s->tmem_addr, kTmemCols);
+    pdl_trigger();  // not before the allocation: see pdl_trigger
     tmem_relinquish();
   }
   pdl_wait();

@@ -178,3 +178,26 @@ def test_every_tile_width_gives_the_same_bytes(ctx, m, n, k):
             at = torch.arange(m - rows, m, device="cuda")
             assert torch.equal(ctx.linear_fwd(x[at].contiguous(), *w), y[at])
     assert ctx.poll() == 0
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 2048, 512), (8, 9472, 384), (9, 2048, 512)])
+def test_small_calls_in_a_row_on_two_streams(ctx, m, n, k):
+    """Several calls of this size fit on an SM at once, and each takes all of its tensor memory: a call that has not got it yet must
+    not be overtaken by the ones behind it.  A router's call, which takes a few columns, comes in between."""
+    x, router = (torch.randn((r, k), device="cuda").to(torch.bfloat16) for r in (m, 64))
+    w = ctx.quantize_weight((0.02 * torch.randn((n, k), device="cuda")).to(torch.bfloat16))
+    want, logits = ctx.linear_fwd(x, *w).clone(), ctx.router_fwd(x, router, 4)[0].clone()
+    each = [(binding.Context(0), torch.cuda.Stream()) for _ in range(2)]  # (a context keeps one scratch buffer)
+    torch.cuda.synchronize()
+    got = []
+    for i in range(200):
+        for c, stream in each:
+            with torch.cuda.stream(stream):
+                got.append((c.linear_fwd(x, *w), want))
+                if i % 3 == 0:
+                    got.append((c.router_fwd(x, router, 4)[0], logits))
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in got)
+    for c, _ in each:
+        assert c.poll() == 0
+        c.close()

@@ -19,3 +19,11 @@ def source(name):
 def test_no_kernel_allocates_for_a_pair_of_ctas(name):
     """`cta_group::2` allocates for two CTAs at once and waits for both: with one of them not begun, or gone, nothing ends it."""
     assert not re.search(r"cta_group::2|tmem_alloc_pair|umma_\w+_pair", source(name))
+
+
+@pytest.mark.parametrize("name", [f for f in FILES if "tmem_alloc(" in source(f) and "pdl_" in source(f) and f != "ptx_sm100.cuh"])
+def test_dependents_may_start_once_the_tensor_memory_is_held(name):
+    """A kernel that lets its successor start first may find that the successor holds the columns and waits for its end."""
+    text = source(name)
+    held = re.findall(r"tmem_alloc\([^;]*;\s*pdl_trigger\(\);", text)
+    assert len(held) == len(re.findall(r"tmem_alloc\(", text)) == len(re.findall(r"pdl_trigger\(\)", text)) > 0
