@@ -30,8 +30,9 @@ namespace {
 
 constexpr int kStep = 512;     // tokens a warp of the partial kernel takes at a time: 16 per lane
 constexpr int kPieces = 2368;  // most pieces of a call: 16 warps on each of 148 SMs (a fixed number: the cut depends on T alone)
-// Tokens per CTA of the finish kernel: a power of two, half an average response or more, and so that at most kFinishCtas make
-// the call.  A CTA takes the responses of its chunk one after the other, so a call of few tokens in short responses wants short
+// Tokens per CTA of the finish kernel: the smallest power of two from kMinChunk that is half an average response or more and leaves the
+// call kFinishCtas CTAs or fewer, at most kMaxChunk: calls over 592 x 16384 tokens have more CTAs, responses of over 32768 tokens on
+// average more chunks each.  A CTA takes the responses of its chunk one after the other, so a call of few tokens in short responses wants short
 // chunks (64 responses, 32,768 tokens: 22.4 us with 8192, 13.0 with 1024; 300 responses, 233,100 tokens: 21.4 and 12.9), while every
 // chunk of a response repeats its statistics (64 responses, 393,216 tokens: 10.1 with 8192, 10.6 with 1024; 1024 responses, 4.2 M tokens:
 // 22.2 with 8192, 25.9 with 4096; 2048 responses, 12.6 M: 51.9 with 8192, 49.6 with 16384).

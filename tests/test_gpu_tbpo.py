@@ -53,11 +53,22 @@ def test_many_short_responses_and_one_long(ctx):
     check(ctx, inputs.tbpo_case(2, lens))
 
 
-@pytest.mark.parametrize("n,mean,longest", [(200, 30, 200), (3, 3000, 6000), (4, 30000, 40000), (900, 700, 3000), (2000, 3700, 12000)])
-def test_every_chunk_length_of_the_finish_kernel(ctx, n, mean, longest):
+def chunk_of(b, t):
+    """Tokens per CTA of the second launch, as the host picks them."""
+    chunk = 1024
+    while chunk < 16384 and (-(-t // chunk) > 592 or 2 * chunk * b < t):
+        chunk *= 2
+    return chunk
+
+
+@pytest.mark.parametrize("chunk,n,mean,longest", [(1024, 200, 30, 200), (2048, 3, 3000, 6000), (16384, 4, 30000, 40000), (2048, 900, 700, 3000),
+                                                  (16384, 2000, 3700, 12000), (4096, 64, 6144, 12000), (8192, 3, 15000, 30000)])
+def test_every_chunk_length_of_the_finish_kernel(ctx, chunk, n, mean, longest):
     """Token counts and average lengths that give chunks of 1024 (many short responses) to 16384 tokens (few long ones, or very many
     tokens)."""
-    check(ctx, inputs.tbpo_case(40 + n, inputs.tbpo_lengths(40 + n, n, mean_len=mean, max_len=longest)))
+    lens = inputs.tbpo_lengths(40 + n, n, mean_len=mean, max_len=longest)
+    assert chunk_of(n, int(lens.sum())) == chunk
+    check(ctx, inputs.tbpo_case(40 + n, lens))
 
 
 def test_single_response_and_single_token(ctx):
