@@ -125,3 +125,42 @@ def test_bad_offsets_are_clamped_not_followed(ctx):
         assert ctx.poll() == -1                             # QARL_ERR_INVALID_ARG from the device
         g_out.check("experts output")
         g_ws.check("experts workspace")
+
+
+def _guarded_backward(ctx, rows_of_dx, n, k, experts, call):
+    """`call` writes dX in bf16 and fp32 and dW through the pointers given to it; returns them."""
+    dev = torch.device("cuda", 0)
+    shapes = ((rows_of_dx, k), (rows_of_dx, k), (experts, n, k))
+    types = (torch.bfloat16, torch.float32, torch.float32)
+    bufs = [Guarded(int(np.prod(s)) * t.itemsize, dev) for s, t in zip(shapes, types)]
+    ctx._check(call(*(b.view.data_ptr() for b in bufs)))
+    assert ctx.poll() == 0
+    for b, what in zip(bufs, ("dX", "dX in fp32", "dW")):
+        b.check(what)
+    return [b.view[:b.exact].view(t).view(s) for b, s, t in zip(bufs, shapes, types)]
+
+
+def _rand(seed, *shape):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.empty(shape, dtype=torch.bfloat16, device="cuda").normal_(0.0, 1.0, generator=g)
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 128, 128), (129, 384, 512), (257, 640, 256), (300, 136, 72)])
+def test_linear_backward_leaves_surroundings_untouched(ctx, M, N, K):
+    dy, x, w = _rand(1, M, N), _rand(2, M, K), _rand(3, N, K)
+    got = _guarded_backward(ctx, M, N, K, 1, lambda *out: ctx.lib.qarl_linear_bwd(
+        ctx.h, dy.data_ptr(), x.data_ptr(), w.data_ptr(), M, N, K, *out, binding._stream()))
+    ref = ctx.linear_bwd(dy, x, w, want_dx_f32=True)
+    assert all(torch.equal(a, b.view(a.shape)) for a, b in zip(got, ref))
+
+
+@pytest.mark.parametrize("sizes", [[0, 1, 127, 129, 0, 64, 3, 300, 0], [0, 0, 5]])
+@pytest.mark.parametrize("N,K", [(256, 128), (384, 520)])
+def test_grouped_backward_leaves_surroundings_untouched(ctx, sizes, N, K):
+    off = torch.tensor(np.concatenate([[0], np.cumsum(sizes)]), dtype=torch.int32, device="cuda")
+    P, E = sum(sizes), len(sizes)
+    dy, x, w = _rand(4, P, N), _rand(5, P, K), _rand(6, E, N, K)
+    got = _guarded_backward(ctx, P, N, K, E, lambda *out: ctx.lib.qarl_grouped_linear_bwd(
+        ctx.h, dy.data_ptr(), x.data_ptr(), w.data_ptr(), off.data_ptr(), P, N, K, E, *out, binding._stream()))
+    ref = ctx.grouped_linear_bwd(dy, x, w, off, want_dx_f32=True)
+    assert all(torch.equal(a, b) for a, b in zip(got, ref))
