@@ -10,6 +10,7 @@
 // so that no transposed copy of dY, X or W is ever made:
 //   dX[m, k] = sum_n dY[m, n] W[n, k]:  A = dY (K-major),  B = W  (MN-major, [c = n][j = k])
 //   dW[n, k] = sum_m dY[m, n] X[m, k]:  A = dY (MN-major, [c = m][i = n]),  B = X (MN-major)
+// (The two-launch router's logits, sum_h x[m, h] w[e, h], take A and B K-major.)
 //
 // Two grouped forms serve the expert GEMMs of the MoE layer, both on the forward's expert-sorted
 // row layout (expert e owns rows offsets[e] .. offsets[e+1]-1), with no padding and no copies:
@@ -32,7 +33,7 @@
 // 1536 x 2048, 1.6 GB out) 1010 us of which the stores need 250.  Static persistent schedule, row tiles fastest
 // (grouped contraction: long and short tiles in turn, see the producer).  One fixed
 // order of accumulation: a result does not depend on the grid or on the other rows.
-// Every wait is bounded (status word + CTA-wide abort flag), as in the other GEMMs.
+// Every wait on an mbarrier is bounded (status word + CTA-wide abort flag), as in the other GEMMs.
 #include <algorithm>
 #include <atomic>
 
@@ -52,9 +53,8 @@ constexpr uint32_t kAHalfBytes = BM * BK * 2;   // 16 KB: 128 output rows x 64 c
 constexpr uint32_t kOutBoxBytes = 32 * 128;
 // A tile holds MT x 128 output rows.  The kernel is bound by the bytes it can keep in flight from
 // L2/HBM (shared-memory capacity over load latency: throughput grew linearly with the ring depth),
-// so MT = 2 -- both 128-row halves share one B tile, a third fewer bytes per flop -- is the default;
-// it leaves one set of accumulators, i.e. an epilogue that is not overlapped, which only pays when
-// the contraction is long enough (MT = 1 for the ragged contraction of the grouped dW).
+// so dense calls may take MT = 2 (the host picks by rounds): both 128-row halves share one B tile, a
+// third fewer bytes per flop, but one set of accumulators is left, i.e. an epilogue that is not overlapped.
 enum { kDense = 0, kGroupedRows = 1, kGroupedContraction = 2 };
 template <int GROUP, int MT, int BN>
 struct Cfg {

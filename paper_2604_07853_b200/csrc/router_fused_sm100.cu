@@ -20,7 +20,7 @@
 //            of the selection (the best of eight per-group candidates, then a re-scan of the winner's
 //            16-expert group) and the softmax in double (exp of logit - max, summed in selection
 //            order), while the next tile's main loop runs.
-// Every wait is bounded (status word + CTA-wide abort flag), as in the GEMMs.
+// Every wait on an mbarrier is bounded (status word + CTA-wide abort flag), as in the GEMMs.
 #include <algorithm>
 #include <atomic>
 #include <math.h>
