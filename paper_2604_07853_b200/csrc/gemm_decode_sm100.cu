@@ -658,8 +658,9 @@ gemm_decode_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         for (int t = 0; t < NTH; ++t) acc_lo[t] = acc_hi[t] = 0.0f;
 
         // Token columns of this warp that hold a row.  A warp without one keeps the barriers going and promotes nothing, with a
-        // few it promotes those (one token: router and layer 33.5 -> 32.2 us); finer steps cost the fuller tiles more than
-        // they save (every four columns: 256 tokens 126.6 -> 127.9).
+        // few it promotes those (one token, router and layer: 33.5 -> 32.4 us on weights that the L2 holds, 53.8 -> 53.0 on
+        // weights read for the first time); finer steps cost the fuller tiles more than they save (every four columns: 256
+        // tokens 126.6 -> 127.9).
         const int live = rows - tb;
         for (int kb = 0; kb < KB; ++kb) {
           if (!warp_wait_or_abort(&s->tmem_full[ks], acc_phase, s, p)) { ok = false; break; }

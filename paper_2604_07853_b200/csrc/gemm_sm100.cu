@@ -27,11 +27,11 @@
 //               its 128 values itself: gate_up = SwiGLU, 1x128 amax / scale / e4m3 codes from registers;
 //               linear, down = bf16 rows through a swizzled staging box and a TMA store.
 //
-// What bounds it: the promotion next to the MMA.  Per K-block it reads 128 KB of TMEM and does 32768 FMAs
-// (256 clocks of the FP32 pipes; reads and FMAs alone measure 360) against 512 clocks of MMAs, so what it must
-// not do is wait or spill.  With scale loads, waits and separate epilogue warps inline a K-block took ~1210
-// clocks; as below ~960 (dense M = 8192, N = 5120, K = 2048: 103 -> 84 us on the same part, at the clock
-// the power cap allows).  What did it: scales from two warps of their own through shared memory, one stream
+// What bounds it: the promotion next to the MMA, and close to it the 48 KB per K-block that come into the SM (MMAs and loads
+// alone ~800 clocks).  Per K-block the promotion reads 128 KB of TMEM and does 32768 FMAs (256 clocks of the FP32 pipes; alone it
+// measures 573) against 512 clocks of MMAs, so what it must not do is wait or spill.  With scale loads, waits and separate
+// epilogue warps inline a K-block took ~1210 clocks; as below 870 to 890, 935 with the tile ends of K = 2048 (dense M = 8192,
+// N = 5120, K = 2048: 92 us in short runs).  What did it: scales from two warps of their own through shared memory, one stream
 // of TMEM reads across K-blocks (the first chunk of the next accumulator is on its way before the last chunk
 // of this one is accumulated), two FMAs per instruction, the loop body without spills (32-column chunks
 // spill and lose), and no epilogue warps (their registers and polling cost more than they hid).
